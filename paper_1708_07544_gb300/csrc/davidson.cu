@@ -1,9 +1,9 @@
 // FP64 Davidson for the lowest eigenpair on a fixed determinant space:
 // the minimum of the energy functional Eq. (variational) with the
 // normalisation multiplier (Sec. II.A: after each enlargement of V the new
-// ground state is found with Davidson's method).  Vector operations, the subspace eigenproblem
-// (cyclic Jacobi on one warp) and the phase convention all run on the GPU;
-// the host only reads the Ritz value and the residual norm per iteration.
+// ground state is found with Davidson's method).  Vector operations, the
+// subspace eigenproblem (one block) and the phase convention all run on the
+// GPU; the host only reads the Ritz value and the residual norm per iteration.
 #include <cmath>
 
 #include "hci_internal.cuh"
@@ -17,15 +17,14 @@ constexpr int DBLOCK = 256;
 
 struct DavDev {
   double G[LDG * LDG];
-  double Qp[LDG * LDG];   // eigenvectors of the previous subspace matrix (kq x kq)
+  float X[LDG * LDG];        // FP32 eigenvectors of the last subspace matrix (kx x kx), start of the next
+  double Y[DAV_KEEP][LDG];   // the lowest eigenvectors of the subspace matrix, orthonormal (k_lowest<DAV_KEEP>)
   double y[LDG];
   double dots[LDG];
-  double ev[LDG];         // eigenvalues of the subspace matrix (columns of Qp)
   double theta;
   double nrm2;
   double ols[4];          // |r|^2, x . M^-1 r, x . M^-1 x (Olsen correction)
-  int amax_idx;
-  int kq;                 // size of Qp (0: none)
+  int kx, ky;             // sizes of X and of y (0: none)
   unsigned int ticket;    // blocks of the running k_dots that have finished
   int stall;              // a correction fell inside the subspace (k_scale_unit)
 };
@@ -93,77 +92,91 @@ __global__ void __launch_bounds__(DBLOCK) k_dots(const double* __restrict__ V, i
   if (threadIdx.x == 0) gd->ticket = 0u;
 }
 
-// Lowest eigenpair of the k x k subspace matrix by parallel-order Jacobi on
-// one block of JW warps: in each round the indices are paired by a
-// round-robin schedule and all disjoint pairs rotate at once (their
-// rotations commute), so a sweep is k-1 rounds of parallel row and column
-// updates, the pairs split over the warps.  An off-diagonal
-// element too small to change either diagonal partner in floating point
-// (even scaled by 100) is zeroed; the sweeps stop when a sweep rotates none.
+// ---------------------------------------------------------------------------
+// Lowest eigenpair(s) of the k x k subspace matrix G, one block.
 //
-// When the matrix is the previous one bordered by one row and column, the
-// sweeps start from the previous eigenvectors Q0 = diag(Qp, 1): Q0^T G Q0 is
-// diagonal but for its last row and column, and takes a few sweeps instead
-// of a full diagonalisation.
-constexpr int JW = 4;   // warps of k_jacobi: one per SM sub-partition (FP64 issue is the limit)
+// FP64 is the scarce unit: a warp's FP64 instruction takes 64 cycles of its
+// sub-partition whatever its active lanes, so a full FP64 Jacobi (about 70
+// of them per round, 23 rounds per sweep) is bound by that pipe.  Only the
+// lowest pair is needed, so FP64 is kept for the residual and everything
+// else runs in FP32 on G shifted by G_00 (which takes the large common part
+// of the energies away).
+//
+// NV = 1 (lowest_newton), from the last lowest vector y: y is turned by the
+// 2 x 2 problem of y and the newly added direction, then
+//   rho = y.Gy / y.y,  r = Gy - rho y                       (FP64)
+//   y <- y - B^-1 r,   B = G - rho + s y y^T                (FP32 inverse)
+// until the next residual is predicted below 2e-16 of the spectrum's
+// spread.  B lifts y by the spread s, so it is positive definite exactly
+// when no other eigenvalue lies below rho: its pivots (Gauss-Jordan, one
+// row per lane) decide whether the pair found is the lowest one.  A pivot
+// below 1e-5 s (a neighbour too close for FP32), or no convergence, and
+// every NV > 1 call, takes the second way.
+//
+// Second way: Jacobi in FP32 (round-robin schedule; thread (s, t) owns the
+// 2 x 2 block of pairs s and t, reads it and both pairs' rotations from one
+// copy of A and writes the rotated block to the other, so that a round takes
+// one barrier), started from the last eigenvectors when the matrix is the
+// last one or that bordered by one row and column, then the same refinement
+// of the NV lowest vectors, one warp each, with the FP32 eigenvectors x_m:
+//   y <- y - sum_{m != lowest} x_m (x_m . r) / (e_m - rho).
+// Neighbours closer than 2e-5 of the spread, or no convergence: FP64 Jacobi.
+//
+// (12e,12o) space, k up to 24, about 840 calls: 219 us per call with an
+// FP64 Jacobi started from the last eigenvectors, 45 us by the second way,
+// 12.4 us by the first.
+constexpr int LW_X = 160;             // threads below: 2 x 2 blocks of A; from here on: rows of X
+constexpr int LW_T = 320;
+constexpr float LW_SKIP = 1e-6f;      // rotations below this angle are skipped
+constexpr float LW_GAP = 2e-5f;       // least gap (of the spread) that FP32 resolves
 
-__global__ void __launch_bounds__(JW * 32) k_jacobi(DavDev* d, int k) {
-  __shared__ double A[32][33];
-  __shared__ double Q[32][33];
-  __shared__ double T[32][33];
-  __shared__ double rc[16], rs[16];
-  __shared__ int rp[16], rq[16];
-  __shared__ int s_rot, s_m;
-  const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const bool warm = k > 1 && d->kq == k - 1;
-  for (int j = w; j < 32; j += JW) {
-    A[l][j] = (l < k && j < k) ? d->G[l * LDG + j] : 0.0;
-    double q0 = (l == j) ? 1.0 : 0.0;
-    if (warm && l < k - 1 && j < k - 1) q0 = d->Qp[l * LDG + j];
-    Q[l][j] = q0;
+// pair t of round r, m players (index m - 1 stays, the others rotate)
+__device__ __forceinline__ void rr_pair(int r, int t, int m, int& p, int& q) {
+  int a = r, b = m - 1;
+  if (t > 0) {
+    a = r + t;
+    if (a >= m - 1) a -= m - 1;
+    b = r - t;
+    if (b < 0) b += m - 1;
   }
-  __syncthreads();
-  if (warm) {
-    // T = G Q0 (lane = row, warps split the columns), then A = Q0^T T
-    // (lane = column, warps split the rows)
-    if (l < k)
-      for (int j = w; j < k; j += JW) {
-        double t = 0.0;
-        for (int mm = 0; mm < k; ++mm) t = fma(A[l][mm], Q[mm][j], t);
-        T[l][j] = t;
-      }
-    __syncthreads();
-    if (l < k)
-      for (int i = w; i < k; i += JW) {
-        double t = 0.0;
-        for (int mm = 0; mm < k; ++mm) t = fma(Q[mm][i], T[mm][l], t);
-        A[i][l] = t;
-      }
-    __syncthreads();
-  }
+  p = a < b ? a : b;
+  q = a < b ? b : a;
+}
+
+__device__ __forceinline__ bool rot32(const float (*a)[LDG + 1], int p, int q, float& c, float& s) {
+  const float apq = a[p][q], dd = a[q][q] - a[p][p];
+  c = 1.0f;
+  s = 0.0f;
+  if (fabsf(apq) <= LW_SKIP * fabsf(dd)) return false;
+  const float e2 = 2.0f * apq, h = dd * dd + e2 * e2;
+  const float t = __fdividef(copysignf(e2, dd * e2), fabsf(dd) + h * rsqrtf(h));
+  c = rsqrtf(1.0f + t * t);
+  s = t * c;
+  return true;
+}
+
+// Full FP64 Jacobi of A (overwritten; diagonal = eigenvalues), Q = vectors
+__device__ void jacobi_fp64(int k, double (*A)[LDG + 1], double (*Q)[LDG + 1], double* rc, double* rs, int* rp,
+                            int* rq) {
+  const int l = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int m = (k + 1) & ~1;          // even number of players (index k is a dummy when k is odd)
   const int npairs = m / 2;
   for (int sweep = 0; sweep < 50 && k > 1; ++sweep) {
-    if (threadIdx.x == 0) s_rot = 0;
-    __syncthreads();
+    int rotated = 0;
     for (int r = 0; r < m - 1; ++r) {
-      // thread t < npairs: pair t of round r
+      int active = 0;
       if (threadIdx.x < npairs) {
         const int t = threadIdx.x;
-        int a, b;
-        if (t == 0) { a = r; b = m - 1; }
-        else { a = (r + t) % (m - 1); b = (r - t + (m - 1)) % (m - 1); }
-        int p = a < b ? a : b, q = a < b ? b : a;
+        int p, q;
+        rr_pair(r, t, m, p, q);
         double c = 1.0, sn = 0.0;
-        int active = 0;
         if (q < k) {
           const double apq = A[p][q], app = A[p][p], aqq = A[q][q];
           const double g = 100.0 * fabs(apq);
+          // an element too small to change either diagonal partner (even
+          // scaled by 100) is zeroed
           if (!((fabs(app) + g == fabs(app) && fabs(aqq) + g == fabs(aqq)) || fabs(apq) < 1e-300)) {
-            // tan of the rotation angle, t = sgn(tau) / (|tau| + sqrt(1 +
-            // tau^2)) with tau = (aqq - app) / (2 apq), written without the
-            // division for tau (one square root, one division and one
-            // reciprocal square root on this part's narrow FP64 pipe; the
+            // tan of the rotation angle without the division for tau (the
             // entries are Rayleigh quotients of normalised vectors, far
             // from overflow)
             const double dd = aqq - app, e2 = 2.0 * apq;
@@ -175,12 +188,11 @@ __global__ void __launch_bounds__(JW * 32) k_jacobi(DavDev* d, int k) {
         }
         rp[t] = p; rq[t] = q; rc[t] = c; rs[t] = active ? sn : 0.0;
         if (!active && q < k) { A[p][q] = 0.0; A[q][p] = 0.0; }
-        if (active) s_rot = 1;
       }
-      __syncthreads();
-      // columns: A <- A J, Q <- Q J (lane = row; warp w takes pairs w, w + JW, ...)
+      rotated |= __syncthreads_or(active);
+      // columns: A <- A J, Q <- Q J (lane = row)
       if (l < k) {
-        for (int t = w; t < npairs; t += JW) {
+        for (int t = w; t < npairs; t += nw) {
           const double s2 = rs[t];
           if (s2 == 0.0) continue;
           const int p = rp[t], q = rq[t];
@@ -196,7 +208,7 @@ __global__ void __launch_bounds__(JW * 32) k_jacobi(DavDev* d, int k) {
       __syncthreads();
       // rows: A <- J^T A (lane = column)
       if (l < k) {
-        for (int t = w; t < npairs; t += JW) {
+        for (int t = w; t < npairs; t += nw) {
           const double s2 = rs[t];
           if (s2 == 0.0) continue;
           const int p = rp[t], q = rq[t];
@@ -213,24 +225,357 @@ __global__ void __launch_bounds__(JW * 32) k_jacobi(DavDev* d, int k) {
       }
       __syncthreads();
     }
-    const int rotated = s_rot;
-    __syncthreads();
     if (!rotated) break;
   }
-  if (threadIdx.x == 0) {
-    int mm = 0;
-    for (int j = 1; j < k; ++j)
-      if (A[j][j] < A[mm][mm]) mm = j;
-    s_m = mm;
-    d->theta = A[mm][mm];
+}
+
+// The first way (see above) for k <= K: G64 / G32 the shifted matrix, zero
+// beyond k; on success y0 = the normalised lowest vector, *rho0 its shifted
+// eigenvalue.  All threads of the block call it; warp 0 decides.
+template <int K>
+__device__ bool lowest_newton(int k, const double (*G64)[LDG + 1], const float (*G32)[LDG + 1], const double* yprev,
+                              int ky, double (*P)[LDG + 1], double* y0, double* rho0) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  constexpr unsigned ALL = 0xffffffffu;
+  double y = 0.0;
+  if (w == 0) {
+    if (ky == k - 1) {
+      y = lane < ky ? yprev[lane] : 0.0;
+      // 2 x 2 problem of y and e_{k-1}
+      double g = 0.0;
+      if (lane < ky) g = y * G64[lane][k - 1];
+      float gf = (float)g, hf = 0.0f;
+      for (int j = 0; j < ky; ++j) hf = fmaf(G32[lane][j], __shfl_sync(ALL, (float)y, j), hf);
+      hf *= (float)y;
+      for (int b = 16; b; b >>= 1) {
+        gf += __shfl_xor_sync(ALL, gf, b);
+        hf += __shfl_xor_sync(ALL, hf, b);
+      }
+      const float dd = G32[k - 1][k - 1] - hf, e2 = 2.0f * gf;
+      // lowest vector of [[hf, gf], [gf, hf + dd]]: (1, t) with t below
+      const float q = sqrtf(fmaf(dd, dd, e2 * e2));
+      if (dd >= 0.0f) {
+        const float t = e2 == 0.0f ? 0.0f : -e2 / (dd + q);
+        if (lane == k - 1) y = t;
+      } else {
+        const float t = e2 == 0.0f ? 0.0f : -e2 / (q - dd);
+        y = lane == k - 1 ? 1.0 : y * (double)t;
+      }
+    } else {
+      // no vector of the last matrix: its lowest diagonal element
+      const float dl = lane < k ? G32[lane][lane] : INFINITY;
+      float mn = dl;
+      for (int b = 16; b; b >>= 1) mn = fminf(mn, __shfl_xor_sync(ALL, mn, b));
+      const int at = __ffs(__ballot_sync(ALL, dl == mn)) - 1;
+      y = lane == at ? 1.0 : 0.0;
+    }
+    y0[lane] = y;
+  }
+  float inv[K];
+  float prev = 0.0f, scale = 0.0f;
+  bool fresh = false;
+  int verdict = 0;                      // 1: converged, 2: give up
+  for (int it = 0; it < 10; ++it) {
+    __syncthreads();
+    if (w < 4) {
+      double g = 0.0;
+      for (int j = w; j < k; j += 4) g = fma(G64[lane][j], y0[j], g);
+      P[w][lane] = g;
+    }
+    __syncthreads();
+    if (w == 0) {
+      const double g = (P[0][lane] + P[1][lane]) + (P[2][lane] + P[3][lane]);
+      // y.y in the lower half of the warp, y.g in the upper
+      const double a = y * y, c = y * g;
+      const bool up = lane & 16;
+      double t = (up ? c : a) + __shfl_xor_sync(ALL, up ? a : c, 16);
+      for (int b = 8; b; b >>= 1) t += __shfl_xor_sync(ALL, t, b);
+      const double s0 = __shfl_sync(ALL, t, 0), s1 = __shfl_sync(ALL, t, 16);
+      const double rho = s1 / s0;
+      const float rf = (float)(g - rho * y);
+      if (!fresh) {
+        // B^-1 at this y (row per lane)
+        const float yf = (float)y, dg = (float)(G64[lane][lane] - rho);
+        float sc = lane < k ? fabsf(dg) : 0.0f;
+        for (int b = 16; b; b >>= 1) sc = fmaxf(sc, __shfl_xor_sync(ALL, sc, b));
+        scale = sc;
+        const float sy = sc / (float)s0 * yf;
+#pragma unroll
+        for (int m = 0; m < K; ++m) {
+          const float ym = __shfl_sync(ALL, yf, m);
+          inv[m] = fmaf(sy, ym, m == lane ? dg : G32[lane][m]);
+          if (m >= k) inv[m] = m == lane ? sc : 0.0f;   // padding: a multiple of the identity
+        }
+        bool pos = sc > 0.0f;
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+          const float piv = __shfl_sync(ALL, inv[j], j);
+          pos = pos && piv > 1e-5f * sc;
+          const float ip = 1.0f / piv;
+          const float f = lane == j ? 0.0f : inv[j];
+#pragma unroll
+          for (int m = 0; m < K; ++m)
+            if (m != j) {
+              const float rj = __shfl_sync(ALL, inv[m], j) * ip;
+              inv[m] = lane == j ? rj : fmaf(-f, rj, inv[m]);
+            }
+          inv[j] = lane == j ? ip : -f * ip;
+        }
+        if (!pos) verdict = 2;
+        fresh = true;
+      }
+      float de = 0.0f;
+#pragma unroll
+      for (int m = 0; m < K; ++m) de = fmaf(inv[m], __shfl_sync(ALL, rf, m), de);
+      float rr = rf * rf, d2 = lane < k ? de * de : 0.0f;
+      for (int b = 16; b; b >>= 1) {
+        rr += __shfl_xor_sync(ALL, rr, b);
+        d2 += __shfl_xor_sync(ALL, d2, b);
+      }
+      if (lane < k) y -= (double)de;
+      const float s0f = (float)s0, rn = sqrtf(rr / s0f);
+      d2 /= s0f;
+      if (verdict == 0) {
+        const float ratio = it > 0 ? fminf(rn / prev, 1.0f) : 1.0f;
+        if (rn * ratio <= 2e-16f * scale && d2 < 1e-6f) verdict = 1;
+        else if (it >= 3 && rn > 0.5f * prev) verdict = rn <= 1e-14f * scale ? 1 : 2;
+        else if (!(d2 < 1.0f)) verdict = 2;
+      }
+      if (d2 > 1e-4f) fresh = false;    // y moved by more than 1e-2: invert again
+      prev = rn;
+      if (verdict == 1) {
+        double q = y * y;
+        for (int b = 16; b; b >>= 1) q += __shfl_xor_sync(ALL, q, b);
+        y *= 1.0 / sqrt(q);
+        if (lane == 0) *rho0 = rho;
+      }
+      y0[lane] = y;
+    }
+    const int v = __syncthreads_or(w == 0 ? verdict : 0);
+    if (v) return __syncthreads_or(w == 0 && verdict == 1) != 0;
+  }
+  return false;
+}
+
+// NV = 1: theta, y = the lowest eigenpair.  NV > 1: also Y[0 .. min(NV, k))
+// = the lowest eigenvectors, ascending, orthonormal.
+template <int NV>
+__global__ void __launch_bounds__(LW_T) k_lowest(DavDev* d, int k) {
+  __shared__ double G[LDG][LDG + 1];
+  __shared__ float A[2][LDG][LDG + 1];
+  __shared__ float X[LDG][LDG + 1];
+  __shared__ float ev[LDG];
+  __shared__ int order[LDG];
+  __shared__ double Ys[NV][LDG], th[NV];
+  __shared__ float Rs[NV][LDG], Cs[NV][LDG];
+  __shared__ double A64[LDG][LDG + 1], Q64[LDG][LDG + 1];
+  __shared__ double rc[LDG / 2], rs[LDG / 2];
+  __shared__ int rp[LDG / 2], rq[LDG / 2];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const double sh = d->G[0];
+  const int kx = (d->kx == k || d->kx == k - 1) ? d->kx : 0, ky = d->ky;
+  for (int e = tid; e < LDG * LDG; e += LW_T) {
+    const int i = e / LDG, j = e % LDG;
+    const double g = (i < k && j < k) ? d->G[e] - (i == j ? sh : 0.0) : 0.0;
+    G[i][j] = g;
+    A[0][i][j] = (float)g;
+    A[1][i][j] = 0.0f;
+    X[i][j] = (i < kx && j < kx) ? d->X[e] : (i == j ? 1.0f : 0.0f);
+  }
+  if (tid < LDG) order[tid] = tid;
+  __syncthreads();
+  if (NV == 1) {
+    bool ok;
+    if (k == 1) {
+      if (tid < LDG) Ys[0][tid] = tid == 0 ? 1.0 : 0.0;
+      if (tid == 0) th[0] = 0.0;
+      __syncthreads();
+      ok = G[0][0] == 0.0;               // false for a non-finite matrix
+    } else if (k <= 8) {
+      ok = lowest_newton<8>(k, G, A[0], d->y, ky, Q64, Ys[0], th);
+    } else if (k <= 16) {
+      ok = lowest_newton<16>(k, G, A[0], d->y, ky, Q64, Ys[0], th);
+    } else {
+      ok = lowest_newton<MAXSUB>(k, G, A[0], d->y, ky, Q64, Ys[0], th);
+    }
+    if (ok) {
+      if (w == 0) d->y[lane] = Ys[0][lane];
+      if (tid == 0) {
+        d->theta = th[0] + sh;
+        d->ky = k;
+      }
+      return;
+    }
+  }
+  if (kx > 0) {
+    for (int e = tid; e < k * k; e += LW_T) {
+      const int i = e / k, j = e % k;
+      float t = 0.0f;
+      for (int m = 0; m < k; ++m) t = fmaf(A[0][i][m], X[m][j], t);
+      A[1][i][j] = t;
+    }
+    __syncthreads();
+    for (int e = tid; e < k * k; e += LW_T) {
+      const int i = e / k, j = e % k;
+      float t = 0.0f;
+      for (int m = 0; m < k; ++m) t = fmaf(X[m][i], A[1][m][j], t);
+      A[0][i][j] = t;
+    }
+    __syncthreads();
+  }
+  int cur = 0;
+  if (k > 1) {
+    const int m = (k + 1) & ~1, np = m / 2;
+    int idle = 0, r = 0;
+    for (int round = 0; round < 40 * (m - 1); ++round) {
+      const float(*a)[LDG + 1] = A[cur];
+      float(*b)[LDG + 1] = A[cur ^ 1];
+      bool act = false;
+      if (tid < np * np) {
+        const int si = tid / np, ti = tid - si * np;
+        int p1, q1, p2, q2;
+        rr_pair(r, si, m, p1, q1);
+        rr_pair(r, ti, m, p2, q2);
+        float c1, s1, c2, s2;
+        act = rot32(a, p1, q1, c1, s1);
+        rot32(a, p2, q2, c2, s2);
+        const float xpp = a[p1][p2], xpq = a[p1][q2], xqp = a[q1][p2], xqq = a[q1][q2];
+        const float ypp = c2 * xpp - s2 * xpq, ypq = s2 * xpp + c2 * xpq;
+        const float yqp = c2 * xqp - s2 * xqq, yqq = s2 * xqp + c2 * xqq;
+        b[p1][p2] = c1 * ypp - s1 * yqp;
+        b[p1][q2] = c1 * ypq - s1 * yqq;
+        b[q1][p2] = s1 * ypp + c1 * yqp;
+        b[q1][q2] = s1 * ypq + c1 * yqq;
+      } else if (tid >= LW_X) {
+        for (int it = tid - LW_X; it < np * k; it += LW_T - LW_X) {
+          const int ti = it / k, l = it - ti * k;
+          int p, q;
+          rr_pair(r, ti, m, p, q);
+          float c, s;
+          if (rot32(a, p, q, c, s)) {
+            const float u = X[l][p], v = X[l][q];
+            X[l][p] = c * u - s * v;
+            X[l][q] = s * u + c * v;
+          }
+        }
+      }
+      const int any = __syncthreads_or(act);
+      cur ^= 1;
+      idle = any ? 0 : idle + 1;
+      if (idle >= m - 1) break;
+      if (++r == m - 1) r = 0;
+    }
+  }
+  if (w == 0) {
+    const float e = lane < k ? A[cur][lane][lane] : 0.0f;
+    int rank = 0;
+    for (int j = 0; j < k; ++j) {
+      const float o = __shfl_sync(0xffffffffu, e, j);
+      rank += (o < e || (o == e && j < lane)) ? 1 : 0;
+    }
+    if (lane < k) {
+      ev[lane] = e;
+      order[rank] = lane;
+    }
   }
   __syncthreads();
-  const int mi = s_m;
-  if (w == 0 && l < LDG) d->y[l] = (l < k) ? Q[l][mi] : 0.0;
-  if (l < k)
-    for (int j = w; j < k; j += JW) d->Qp[l * LDG + j] = Q[l][j];
-  if (w == 0 && l < k) d->ev[l] = A[l][l];
-  if (threadIdx.x == 0) d->kq = k;
+  const int kk = k < NV ? k : NV;
+  const float spread = ev[order[k - 1]] - ev[order[0]];
+  bool good = true;
+  for (int t = 0; t < kk && t + 1 < k; ++t) good = good && ev[order[t + 1]] - ev[order[t]] > LW_GAP * spread;
+  if (good && w < kk) {
+    // warp w refines the w-th lowest vector; lane = row
+    const int o = order[w];
+    double y = lane < k ? (double)X[lane][o] : 0.0, rho = 0.0;
+    float prev = 0.0f;
+    good = false;
+    for (int it = 0; it < 12; ++it) {
+      Ys[w][lane] = y;
+      __syncwarp();
+      double g = 0.0;
+      for (int j = 0; j < k; ++j) g = fma(G[lane][j], Ys[w][j], g);
+      double s0 = y * y, s1 = y * g;
+      for (int b = 16; b; b >>= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, b);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, b);
+      }
+      rho = s1 / s0;
+      const float rf = (float)(g - rho * y);
+      float rr = rf * rf;
+      for (int b = 16; b; b >>= 1) rr += __shfl_xor_sync(0xffffffffu, rr, b);
+      const float rn = sqrtf(rr);
+      Rs[w][lane] = rf;
+      __syncwarp();
+      float am = 0.0f;
+      if (lane < k && lane != o) {
+        for (int i = 0; i < k; ++i) am = fmaf(X[i][lane], Rs[w][i], am);
+        am = -am / (ev[lane] - (float)rho);
+      }
+      Cs[w][lane] = am;
+      __syncwarp();
+      float de = 0.0f;
+      for (int j = 0; j < k; ++j) de = fmaf(X[lane][j], Cs[w][j], de);
+      if (lane < k) y += (double)de;
+      const float ratio = it > 0 ? fminf(rn / prev, 1.0f) : 1.0f;
+      if (rn * ratio <= 2e-16f * spread) { good = true; break; }
+      if (it >= 3 && rn > 0.5f * prev) { good = rn <= 1e-14f * spread; break; }
+      prev = rn;
+    }
+    double s0 = y * y;
+    for (int b = 16; b; b >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, b);
+    Ys[w][lane] = y * (1.0 / sqrt(s0));
+    if (lane == 0) th[w] = rho + sh;
+  }
+  if (__syncthreads_and(good)) {
+    if (NV > 1 && w == 0) {
+      // orthogonal to about the refinement's accuracy: one Gram-Schmidt pass
+      for (int t = 1; t < kk; ++t) {
+        double y = Ys[t][lane];
+        for (int u = 0; u < t; ++u) {
+          double dt = Ys[u][lane] * y;
+          for (int b = 16; b; b >>= 1) dt += __shfl_xor_sync(0xffffffffu, dt, b);
+          y = fma(-dt, Ys[u][lane], y);
+        }
+        double s0 = y * y;
+        for (int b = 16; b; b >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, b);
+        Ys[t][lane] = y * (1.0 / sqrt(s0));
+        __syncwarp();
+      }
+    }
+  } else {
+    for (int e = tid; e < LDG * LDG; e += LW_T) {
+      A64[e / LDG][e % LDG] = G[e / LDG][e % LDG];
+      Q64[e / LDG][e % LDG] = e / LDG == e % LDG ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    jacobi_fp64(k, A64, Q64, rc, rs, rp, rq);
+    if (tid == 0) {
+      bool used[LDG];
+      for (int j = 0; j < k; ++j) used[j] = false;
+      for (int t = 0; t < kk; ++t) {
+        int b = -1;
+        for (int j = 0; j < k; ++j)
+          if (!used[j] && (b < 0 || A64[j][j] < A64[b][b])) b = j;
+        used[b] = true;
+        order[t] = b;
+        th[t] = A64[b][b] + sh;
+      }
+    }
+    __syncthreads();
+    if (w < kk) Ys[w][lane] = lane < k ? Q64[lane][order[w]] : 0.0;
+    for (int e = tid; e < LDG * LDG; e += LW_T) X[e / LDG][e % LDG] = (float)Q64[e / LDG][e % LDG];
+  }
+  __syncthreads();
+  for (int e = tid; e < LDG * LDG; e += LW_T) d->X[e] = X[e / LDG][e % LDG];
+  if (w == 0) {
+    d->y[lane] = Ys[0][lane];
+    if (NV > 1)
+      for (int t = 0; t < kk; ++t) d->Y[t % DAV_KEEP][lane] = Ys[t % NV][lane];
+  }
+  if (tid == 0) {
+    d->theta = th[0];
+    d->kx = d->ky = k;
+  }
 }
 
 // x = V y, wy = W y, r = wy - theta x, t = M^-1 r with M = theta - diag
@@ -298,28 +643,12 @@ __global__ void __launch_bounds__(DBLOCK) k_ritz(const double* __restrict__ V, c
 }
 
 // The kk <= DAV_KEEP lowest Ritz vectors of the current subspace (ascending Ritz value)
-// and their H products: Qo[t] = sum_j Qp[j][o_t] V[j], Wo[t] likewise from W.
+// and their H products: Qo[t] = sum_j Y[t][j] V[j], Wo[t] likewise from W.
 __global__ void __launch_bounds__(DBLOCK) k_keep(const double* __restrict__ V, const double* __restrict__ W,
                                                  int64_t ld, int k, const DavDev* __restrict__ d, int kk, int64_t n,
                                                  double* __restrict__ Qo, double* __restrict__ Wo) {
   __shared__ double ys[DAV_KEEP][LDG];
-  __shared__ int order[DAV_KEEP];
-  if (threadIdx.x == 0) {
-    bool used[LDG];
-    for (int j = 0; j < k; ++j) used[j] = false;
-    for (int t = 0; t < kk; ++t) {
-      int b = -1;
-      for (int j = 0; j < k; ++j)
-        if (!used[j] && (b < 0 || d->ev[j] < d->ev[b])) b = j;
-      used[b] = true;
-      order[t] = b;
-    }
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < kk * k; e += blockDim.x) {
-    const int t = e / k, j = e % k;
-    ys[t][j] = d->Qp[j * LDG + order[t]];
-  }
+  for (int e = threadIdx.x; e < kk * k; e += blockDim.x) ys[e / k][e % k] = d->Y[e / k][e % k];
   __syncthreads();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     double qv[DAV_KEEP], wv[DAV_KEEP];
@@ -703,7 +1032,7 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
   // one host synchronisation per iteration: the Ritz value, the residual
   // and whether the previous correction fell inside the subspace
   auto ritz = [&](double& th, double& r, int& stall) -> hci_status {
-    HCI_LAUNCH(k_jacobi, 1, JW * 32, 0, st)(D.d, k);
+    HCI_LAUNCH(k_lowest<1>, 1, LW_T, 0, st)(D.d, k);
     HCI_LAUNCH(k_ritz, D.nblk, DBLOCK, 0, st)(D.V, D.W, D.ld, k, D.d, diag, nV, D.x, D.wy, D.t, D.part);
     HCI_CUDA(ctx, cudaGetLastError());
     double hv[2];
@@ -767,6 +1096,7 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
   if (m == 0 && converged) {
     const int kk = k < DAV_KEEP ? k : DAV_KEEP;
     if (ensure_buf(ctx, K.Q, (size_t)D.ld * kk * 8) == HCI_OK && ensure_buf(ctx, K.W, (size_t)D.ld * kk * 8) == HCI_OK) {
+      HCI_LAUNCH(k_lowest<DAV_KEEP>, 1, LW_T, 0, st)(D.d, k);
       HCI_LAUNCH(k_keep, D.nblk, DBLOCK, 0, st)(D.V, D.W, D.ld, k, D.d, kk, nV, bp<double>(K.Q), bp<double>(K.W));
       K.valid = true;
       K.epoch = G.epoch;
