@@ -15,27 +15,126 @@ constexpr int DAV_KEEP = 4;         // Ritz vectors kept for the next, grown spa
 constexpr int LDG = 32;             // leading dimension of the subspace matrix
 constexpr int DBLOCK = 256;
 
+// what the host reads of an iteration
+struct DavReport {
+  double theta;           // Ritz value
+  double ols[3];          // |r|^2, x . M^-1 r, x . M^-1 x (Olsen correction)
+  int stall;              // a correction fell inside the subspace
+};
+
 struct DavDev {
   double G[LDG * LDG];
   float X[LDG * LDG];        // FP32 eigenvectors of the last subspace matrix (kx x kx), start of the next
   double Y[DAV_KEEP][LDG];   // the lowest eigenvectors of the subspace matrix, orthonormal (k_lowest<DAV_KEEP>)
   double y[LDG];
   double dots[LDG];
-  double theta;
+  DavReport rep;
   double nrm2;
-  double ols[4];          // |r|^2, x . M^-1 r, x . M^-1 x (Olsen correction)
   int kx, ky;             // sizes of X and of y (0: none)
-  unsigned int ticket;    // blocks of the running k_dots that have finished
-  int stall;              // a correction fell inside the subspace (k_scale_unit)
+  unsigned int ticket;    // blocks of the running reduction that have finished
 };
 
-// out[j] = V_j . w (j < k).  Each block writes partial[b][j], its share of
-// the sums; the vectors come in groups of DOTS_GROUP (blockIdx.y = group),
-// which keeps the accumulators few and the kernel at full occupancy for any
-// k.  The last block to finish (a ticket counter) sums the partials in a
-// fixed order (lanes over blocks, then a shuffle tree), so the
-// result does not depend on the order in which blocks finish; with
-// gcol >= 0 it also stores out[j] as G[j][gcol] = G[gcol][j], j <= gcol.
+// ---------------------------------------------------------------------------
+// Grid-wide sums of NA accumulators per thread.
+//
+// The vector passes below are bound by FP64 issue long before memory (a
+// warp's FP64 instruction takes 64 cycles of its sub-partition): a plain
+// shuffle tree costs 5 additions per accumulator and warp, more than the
+// products themselves at a few elements per thread.  warp_sums halves the
+// values held per lane at every step instead (27 additions for 24
+// accumulators, not 120), and the reducing passes run one or two blocks per
+// SM, so that each warp reduces once for several elements.
+// ---------------------------------------------------------------------------
+template <int H, int OFF>
+__device__ __forceinline__ void warp_sums(double* a, int lane) {
+  if constexpr (OFF > 0) {
+    if constexpr (H % 2 == 0) {
+      const bool up = lane & OFF;
+#pragma unroll
+      for (int q = 0; q < H / 2; ++q) {
+        const double keep = up ? a[q + H / 2] : a[q], give = up ? a[q] : a[q + H / 2];
+        a[q] = keep + __shfl_xor_sync(0xffffffffu, give, OFF);
+      }
+      warp_sums<H / 2, OFF / 2>(a, lane);
+    } else {
+#pragma unroll
+      for (int q = 0; q < H; ++q) a[q] += __shfl_xor_sync(0xffffffffu, a[q], OFF);
+      warp_sums<H, OFF / 2>(a, lane);
+    }
+  }
+}
+// lanes that hold sums after warp_sums: first index of a lane's values
+// (`left` values, the same in the lanes that differ only in `spare` bits)
+template <int H, int OFF>
+__device__ __forceinline__ int sums_base(int lane, int& left, int& spare) {
+  left = H;
+  if constexpr (OFF > 0) {
+    if constexpr (H % 2 == 0) {
+      const int b = (lane & OFF) ? H / 2 : 0;
+      return b + sums_base<H / 2, OFF / 2>(lane, left, spare);
+    } else {
+      spare = 2 * OFF - 1;
+    }
+  }
+  return 0;
+}
+
+// Sums of acc[0 .. NA) over the grid, taken by the last block to finish (a
+// ticket counter) from the blocks' partial sums, in a fixed order, so that
+// the result does not depend on the order in which blocks finish.  True in
+// that block, whose threads t < NA then hold sum t in *total.  Blocks of the
+// grid: (x, y), partial sums at [x][j0 .. j0 + NA) for the y-th group.
+template <int NA>
+__device__ __forceinline__ bool grid_sums(double* acc, int j0, int ncol, double* partial, unsigned int* ticket,
+                                          double* total) {
+  __shared__ double red[DBLOCK / 32][LDG];
+  __shared__ bool s_last;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  warp_sums<NA, 16>(acc, lane);
+  int left = 0, spare = 0;
+  const int base = sums_base<NA, 16>(lane, left, spare);
+  if ((lane & spare) == 0)
+    for (int q = 0; q < left; ++q) red[wid][base + q] = acc[q];
+  __syncthreads();
+  if (threadIdx.x < NA && j0 + (int)threadIdx.x < ncol) {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < DBLOCK / 32; ++w) s += red[w][threadIdx.x];
+    partial[(int64_t)blockIdx.x * LDG + j0 + threadIdx.x] = s;
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x * gridDim.y - 1u;
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  // the columns rounded up to a power of two share the block's threads, so
+  // that a thread adds few partial sums (304 blocks: 2 for one column, 38
+  // for 24), four loads in flight
+  int cp = 1;
+  while (cp < ncol) cp <<= 1;
+  const int col = threadIdx.x & (cp - 1);
+  double s = 0.0;
+  if (col < ncol) {
+    const double* pc = partial + col;
+#pragma unroll 4
+    for (int b = threadIdx.x / cp; b < (int)gridDim.x; b += DBLOCK / cp) s += __ldcg(pc + (int64_t)b * LDG);
+  }
+  for (int o = cp; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane < cp) red[wid][lane] = s;
+  __syncthreads();
+  s = 0.0;
+  if ((int)threadIdx.x < ncol)
+#pragma unroll
+    for (int w = 0; w < DBLOCK / 32; ++w) s += red[w][threadIdx.x];
+  *total = s;
+  if (threadIdx.x == 0) *ticket = 0u;
+  return true;
+}
+
+// out[j] = V_j . w (j < k <= 32), vectors in groups of DOTS_GROUP (blockIdx.y
+// = group).  With gcol >= 0 out[j] is also stored as G[j][gcol] = G[gcol][j],
+// j <= gcol.
 constexpr int DOTS_GROUP = 8;
 
 __global__ void __launch_bounds__(DBLOCK) k_dots(const double* __restrict__ V, int64_t ld, int k,
@@ -53,43 +152,97 @@ __global__ void __launch_bounds__(DBLOCK) k_dots(const double* __restrict__ V, i
     for (int j = 0; j < DOTS_GROUP; ++j)
       if (j < kg) acc[j] = fma(Vg[(int64_t)j * ld + i], wv, acc[j]);
   }
-  __shared__ double red[DBLOCK / 32][DOTS_GROUP];
-  __shared__ bool s_last;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double s;
+  if (!grid_sums<DOTS_GROUP>(acc, j0, k, partial, &gd->ticket, &s)) return;
+  const int j = threadIdx.x;
+  if (j < k) {
+    out[j] = s;
+    if (gcol >= 0 && j <= gcol) {
+      gd->G[j * LDG + gcol] = s;
+      gd->G[gcol * LDG + j] = s;
+    }
+  }
+}
+
+// The vector passes of one iteration between the Ritz step and the next
+// product, each one launch over the k subspace vectors (NA >= their number):
+//   OLSEN: t <- t - eps u (the Olsen correction, see k_ritz), dots_j = V_j . t
+//   ORTH:  t <- t - sum_j dots_j V_j, dots_j = V_j . t of the result (the
+//          second Gram-Schmidt pass's products, from the values of V_j that
+//          the first one's subtraction has in registers)
+//   NORM:  V_k <- t - sum_j dots_j V_j, nrm2 = |V_k|^2
+//   GCOL:  after W_k = H V_k: V_k and W_k scaled by 1 / sqrt(nrm2), then
+//          G[j][k] = G[k][j] = V_j . W_k, j <= k.  A correction of norm^2 at
+//          most 1e-26 lies in the subspace: V_k = W_k = 0 and stall = 1.
+// Bound by FP64 issue (2 k + 1 operations per element) at 1e5 elements, by
+// the k vectors' bytes beyond L2.  (12e,12o) space, 1.4e5 elements, k <= 24,
+// per iteration: 4 x 24 us (products, norm), 2 x 5 (subtractions), 7 (Olsen)
+// and 6 (scaling) as separate passes with plain shuffle trees, 53 us so.
+enum { PASS_OLSEN = 0, PASS_ORTH = 1, PASS_NORM = 2, PASS_GCOL = 3 };
+
+template <int OP, int NA>
+__global__ void __launch_bounds__(DBLOCK, 2) k_pass(double* __restrict__ V, double* __restrict__ W, int64_t ld, int k,
+                                                    int64_t n, double* __restrict__ t, const double* __restrict__ u,
+                                                    DavDev* __restrict__ d, double* __restrict__ partial) {
+  __shared__ double cs[LDG];
+  if (threadIdx.x < LDG) cs[threadIdx.x] = d->dots[threadIdx.x];
+  __syncthreads();
+  double eps = 0.0, f = 0.0;
+  if (OP == PASS_OLSEN) {
+    const double den = d->rep.ols[2];
+    eps = den != 0.0 ? d->rep.ols[1] / den : 0.0;
+  }
+  if (OP == PASS_GCOL) {
+    const double n2 = d->nrm2;
+    f = n2 > 1e-26 ? 1.0 / sqrt(n2) : 0.0;
+  }
+  constexpr int NS = OP == PASS_NORM ? 1 : NA;
+  double acc[NS];
 #pragma unroll
-  for (int j = 0; j < DOTS_GROUP; ++j) {
-    if (j < kg) {
-      double a = acc[j];
-      for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-      if (lane == 0) red[wid][j] = a;
+  for (int j = 0; j < NS; ++j) acc[j] = 0.0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    double v[NA];
+#pragma unroll
+    for (int j = 0; j < NA; ++j) v[j] = j < k ? V[(int64_t)j * ld + i] : 0.0;
+    double w, vk = 0.0;
+    if (OP == PASS_OLSEN) {
+      w = fma(-eps, u[i], t[i]);
+      t[i] = w;
+    } else if (OP == PASS_GCOL) {
+      vk = f != 0.0 ? V[(int64_t)k * ld + i] * f : 0.0;
+      w = f != 0.0 ? W[(int64_t)k * ld + i] * f : 0.0;
+      V[(int64_t)k * ld + i] = vk;
+      W[(int64_t)k * ld + i] = w;
+    } else {
+      w = t[i];
+#pragma unroll
+      for (int j = 0; j < NA; ++j)
+        if (j < k) w = fma(-cs[j], v[j], w);
+      if (OP == PASS_ORTH) t[i] = w;
+      else V[(int64_t)k * ld + i] = w;
+    }
+    if (OP == PASS_NORM) {
+      acc[0] = fma(w, w, acc[0]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < NS; ++j)
+        if (j < k + (OP == PASS_GCOL)) acc[j] = fma(OP == PASS_GCOL && j >= k ? vk : v[j], w, acc[j]);
     }
   }
-  __syncthreads();
-  if (threadIdx.x < kg) {
-    double s = 0.0;
-    for (int w2 = 0; w2 < DBLOCK / 32; ++w2) s += red[w2][threadIdx.x];
-    partial[(int64_t)blockIdx.x * LDG + j0 + threadIdx.x] = s;
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&gd->ticket, 1u) == gridDim.x * gridDim.y - 1u;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  const int nblocks = (int)gridDim.x;
-  for (int j = wid; j < k; j += DBLOCK / 32) {
-    double s = 0.0;
-    for (int b = lane; b < nblocks; b += 32) s += __ldcg(partial + (int64_t)b * LDG + j);
-    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-      out[j] = s;
-      if (gcol >= 0 && j <= gcol) {
-        gd->G[j * LDG + gcol] = s;
-        gd->G[gcol * LDG + j] = s;
-      }
+  double s;
+  if (!grid_sums<NS>(acc, 0, OP == PASS_NORM ? 1 : OP == PASS_GCOL ? k + 1 : k, partial, &d->ticket, &s)) return;
+  const int j = threadIdx.x;
+  if (OP == PASS_NORM) {
+    if (j == 0) d->nrm2 = s;
+  } else if (OP == PASS_GCOL) {
+    if (j <= k) {
+      d->G[j * LDG + k] = s;
+      d->G[k * LDG + j] = s;
     }
+    if (j == 0 && f == 0.0) d->rep.stall = 1;
+  } else if (j < k) {
+    d->dots[j] = s;
   }
-  if (threadIdx.x == 0) gd->ticket = 0u;
 }
 
 // ---------------------------------------------------------------------------
@@ -401,7 +554,7 @@ __global__ void __launch_bounds__(LW_T) k_lowest(DavDev* d, int k) {
     if (ok) {
       if (w == 0) d->y[lane] = Ys[0][lane];
       if (tid == 0) {
-        d->theta = th[0] + sh;
+        d->rep.theta = th[0] + sh;
         d->ky = k;
       }
       return;
@@ -573,73 +726,65 @@ __global__ void __launch_bounds__(LW_T) k_lowest(DavDev* d, int k) {
       for (int t = 0; t < kk; ++t) d->Y[t % DAV_KEEP][lane] = Ys[t % NV][lane];
   }
   if (tid == 0) {
-    d->theta = th[0];
+    d->rep.theta = th[0];
     d->kx = d->ky = k;
   }
 }
 
-// x = V y, wy = W y, r = wy - theta x, t = M^-1 r with M = theta - diag
-// (guarded away from zero); partial[b][0..2] = block sums of r^2, x t and
-// x M^-1 x for the Olsen correction.
+// x = V y, wy = W y, r = wy - theta x, t = M^-1 r and u = M^-1 x with M =
+// theta - diag (guarded away from zero), and the sums r^2, x t and x u of
+// the Olsen correction t - eps u, eps = (x M^-1 r) / (x M^-1 x), which is
+// orthogonal to x to first order.  2 k + 16 FP64 operations per element (one
+// division, not two) bound it at 1e5 elements, 16 k bytes beyond L2: 22.1 ->
+// 15.4 us on the (12e,12o) space.
 __global__ void __launch_bounds__(DBLOCK) k_ritz(const double* __restrict__ V, const double* __restrict__ W, int64_t ld,
                                                  int k, DavDev* __restrict__ d, const double* __restrict__ diag,
                                                  int64_t n, double* __restrict__ x, double* __restrict__ wy,
-                                                 double* __restrict__ t, double* __restrict__ partial) {
+                                                 double* __restrict__ t, double* __restrict__ u,
+                                                 double* __restrict__ partial) {
   __shared__ double ys[LDG];
-  __shared__ double red[3][DBLOCK / 32];
-  __shared__ bool s_last;
   if (threadIdx.x < LDG) ys[threadIdx.x] = d->y[threadIdx.x];
   __syncthreads();
-  const double theta = d->theta;
-  double acc = 0.0, axt = 0.0, axx = 0.0;
+  const double theta = d->rep.theta;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     double xv = 0.0, wv = 0.0;
-    for (int j = 0; j < k; ++j) {
-      xv = fma(ys[j], V[(int64_t)j * ld + i], xv);
-      wv = fma(ys[j], W[(int64_t)j * ld + i], wv);
+    const double* v = V + i;
+    const double* w = W + i;
+    int j = 0;
+    for (; j + 4 <= k; j += 4) {
+      const double v0 = v[0], v1 = v[ld], v2 = v[2 * ld], v3 = v[3 * ld];
+      const double w0 = w[0], w1 = w[ld], w2 = w[2 * ld], w3 = w[3 * ld];
+      xv = fma(ys[j], v0, xv);
+      wv = fma(ys[j], w0, wv);
+      xv = fma(ys[j + 1], v1, xv);
+      wv = fma(ys[j + 1], w1, wv);
+      xv = fma(ys[j + 2], v2, xv);
+      wv = fma(ys[j + 2], w2, wv);
+      xv = fma(ys[j + 3], v3, xv);
+      wv = fma(ys[j + 3], w3, wv);
+      v += 4 * ld;
+      w += 4 * ld;
     }
-    double r = wv - theta * xv;
+    for (; j < k; ++j, v += ld, w += ld) {
+      xv = fma(ys[j], v[0], xv);
+      wv = fma(ys[j], w[0], wv);
+    }
+    const double r = wv - theta * xv;
     double den = theta - diag[i];
     if (fabs(den) < 1e-8) den = den >= 0.0 ? 1e-8 : -1e-8;
-    const double tv = r / den;
+    const double inv = 1.0 / den, tv = r * inv, uv = xv * inv;
     x[i] = xv;
     wy[i] = wv;
     t[i] = tv;
-    acc = fma(r, r, acc);
-    axt = fma(xv, tv, axt);
-    axx = fma(xv, xv / den, axx);
+    u[i] = uv;
+    acc[0] = fma(r, r, acc[0]);
+    acc[1] = fma(xv, tv, acc[1]);
+    acc[2] = fma(xv, uv, acc[2]);
   }
-  for (int o = 16; o; o >>= 1) {
-    acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    axt += __shfl_xor_sync(0xffffffffu, axt, o);
-    axx += __shfl_xor_sync(0xffffffffu, axx, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    red[0][threadIdx.x >> 5] = acc;
-    red[1][threadIdx.x >> 5] = axt;
-    red[2][threadIdx.x >> 5] = axx;
-  }
-  __syncthreads();
-  if (threadIdx.x < 3) {
-    double s = 0.0;
-    for (int w = 0; w < DBLOCK / 32; ++w) s += red[threadIdx.x][w];
-    partial[(int64_t)blockIdx.x * LDG + threadIdx.x] = s;
-  }
-  // the last block to finish sums the partials into ols[0..2] (as k_dots)
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&d->ticket, 1u) == gridDim.x - 1u;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (wid < 3) {
-    double s = 0.0;
-    for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(partial + (int64_t)b * LDG + wid);
-    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) d->ols[wid] = s;
-  }
-  if (threadIdx.x == 0) d->ticket = 0u;
+  double s;
+  if (!grid_sums<4>(acc, 0, 3, partial, &d->ticket, &s)) return;
+  if (threadIdx.x < 3) d->rep.ols[threadIdx.x] = s;
 }
 
 // The kk <= DAV_KEEP lowest Ritz vectors of the current subspace (ascending Ritz value)
@@ -715,18 +860,13 @@ __global__ void k_parity_project(double* __restrict__ v, const int32_t* __restri
   }
 }
 
-// Olsen correction: t = M^-1 (r - eps x) with eps = (x M^-1 r) / (x M^-1 x),
-// which makes the correction orthogonal to x to first order.
-__global__ void __launch_bounds__(DBLOCK) k_olsen(const DavDev* __restrict__ d, const double* __restrict__ diag,
-                                                  int64_t n, const double* __restrict__ x, double* __restrict__ t) {
-  const double den_x = d->ols[2];
-  const double eps = den_x != 0.0 ? d->ols[1] / den_x : 0.0;
-  const double theta = d->theta;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    double den = theta - diag[i];
-    if (fabs(den) < 1e-8) den = den >= 0.0 ? 1e-8 : -1e-8;
-    t[i] -= eps * x[i] / den;
-  }
+// t <- t - eps u (the Olsen correction, see k_ritz)
+__global__ void __launch_bounds__(DBLOCK) k_olsen(const DavDev* __restrict__ d, int64_t n,
+                                                  const double* __restrict__ u, double* __restrict__ t) {
+  const double den_x = d->rep.ols[2];
+  const double eps = den_x != 0.0 ? d->rep.ols[1] / den_x : 0.0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    t[i] = fma(-eps, u[i], t[i]);
 }
 
 // v[i] += a * (a hash of i mapped to [-1, 1)): a start component in every
@@ -778,41 +918,61 @@ __global__ void k_scale_unit(const double* __restrict__ x, int64_t n, DavDev* __
   const double f = ok ? 1.0 / sqrt(nrm2) : 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     y[i] = ok ? x[i] * f : 0.0;
-  if (!ok && blockIdx.x == 0 && threadIdx.x == 0) d->stall = 1;
+  if (!ok && blockIdx.x == 0 && threadIdx.x == 0) d->rep.stall = 1;
 }
 
-// argmax |x| (first index on ties): block partials then a final reduce
-__global__ void k_amax_part(const double* __restrict__ x, int64_t n, double* __restrict__ pv, int64_t* __restrict__ pi) {
+// best (value, index) over the grid: the largest value, the lowest index on
+// ties; true in the last block to finish, whose thread 0 gets it
+__device__ __forceinline__ bool grid_best(double& bv, int64_t& bi, double* pv, int64_t* pi, unsigned int* ticket) {
+  __shared__ double sv[DBLOCK / 32];
+  __shared__ int64_t si[DBLOCK / 32];
+  __shared__ bool s_last;
+  auto block_best = [&]() {
+    for (int o = 16; o; o >>= 1) {
+      const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+      const int64_t oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
+    }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) { sv[threadIdx.x >> 5] = bv; si[threadIdx.x >> 5] = bi; }
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int w = 1; w < DBLOCK / 32; ++w)
+        if (sv[w] > bv || (sv[w] == bv && si[w] < bi)) { bv = sv[w]; bi = si[w]; }
+  };
+  block_best();
+  if (threadIdx.x == 0) {
+    pv[blockIdx.x] = bv;
+    pi[blockIdx.x] = bi;
+    __threadfence();
+    s_last = atomicAdd(ticket, 1u) == gridDim.x - 1u;
+  }
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  bv = -INFINITY;
+  bi = INT64_MAX;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += DBLOCK) {
+    const double v = __ldcg(pv + b);
+    const int64_t q = __ldcg(pi + b);
+    if (v > bv || (v == bv && q < bi)) { bv = v; bi = q; }
+  }
+  block_best();
+  if (threadIdx.x == 0) *ticket = 0u;
+  return true;
+}
+
+// sign of the entry of largest magnitude (first index on ties)
+__global__ void __launch_bounds__(DBLOCK) k_phase_sign(const double* __restrict__ x, int64_t n, double* __restrict__ pv,
+                                                       int64_t* __restrict__ pi, DavDev* __restrict__ d,
+                                                       double* __restrict__ sgn) {
   double bv = -1.0;
   int64_t bi = 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    double a = fabs(x[i]);
-    if (a > bv || (a == bv && i < bi)) { bv = a; bi = i; }
+    const double a = fabs(x[i]);
+    if (a > bv) { bv = a; bi = i; }
   }
-  for (int o = 16; o; o >>= 1) {
-    double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-    int64_t oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-  }
-  __shared__ double sv[32];
-  __shared__ int64_t si[32];
-  if ((threadIdx.x & 31) == 0) { sv[threadIdx.x >> 5] = bv; si[threadIdx.x >> 5] = bi; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-      if (sv[w] > bv || (sv[w] == bv && si[w] < bi)) { bv = sv[w]; bi = si[w]; }
-    pv[blockIdx.x] = bv;
-    pi[blockIdx.x] = bi;
-  }
-}
-
-__global__ void k_phase_sign(const double* __restrict__ x, const double* __restrict__ pv,
-                             const int64_t* __restrict__ pi, int nb, double* __restrict__ sgn) {
-  double bv = -1.0;
-  int64_t bi = 0;
-  for (int b = 0; b < nb; ++b)
-    if (pv[b] > bv || (pv[b] == bv && pi[b] < bi)) { bv = pv[b]; bi = pi[b]; }
-  *sgn = x[bi] < 0.0 ? -1.0 : 1.0;
+  if (grid_best(bv, bi, pv, pi, &d->ticket) && threadIdx.x == 0) *sgn = x[bi] < 0.0 ? -1.0 : 1.0;
 }
 
 __global__ void k_apply_sign(double* __restrict__ x, int64_t n, const double* __restrict__ sgn) {
@@ -822,37 +982,47 @@ __global__ void k_apply_sign(double* __restrict__ x, int64_t n, const double* __
     x[i] = -x[i];
 }
 
-__global__ void k_unit_min_diag(double* __restrict__ x, const double* __restrict__ diag, int64_t n) {
-  // single block: index of the smallest diagonal element (first on ties)
-  double bv = 1e300;
+// x[i] = 1 at the smallest diagonal element (first on ties); x zeroed before
+__global__ void __launch_bounds__(DBLOCK) k_unit_min_diag(double* __restrict__ x, const double* __restrict__ diag,
+                                                          int64_t n, double* __restrict__ pv, int64_t* __restrict__ pi,
+                                                          DavDev* __restrict__ d) {
+  double bv = -INFINITY;
   int64_t bi = 0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-    double a = diag[i];
-    if (a < bv || (a == bv && i < bi)) { bv = a; bi = i; }
-  }
-  __shared__ double sv[1024];
-  __shared__ int64_t si[1024];
-  sv[threadIdx.x] = bv;
-  si[threadIdx.x] = bi;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int t = 1; t < (int)blockDim.x; ++t)
-      if (sv[t] < bv || (sv[t] == bv && si[t] < bi)) { bv = sv[t]; bi = si[t]; }
-    x[bi] = 1.0;
-  }
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    if (-diag[i] > bv) { bv = -diag[i]; bi = i; }
+  if (grid_best(bv, bi, pv, pi, &d->ticket) && threadIdx.x == 0) x[bi] = 1.0;
 }
 
 struct Dav {
   hci_ctx* ctx;
   int64_t n, ld;
-  double *V, *W, *x, *wy, *t, *part;
+  double *V, *W, *x, *wy, *t, *u, *part;
   DavDev* d;
-  int nblk;
+  int nblk;     // blocks of the elementwise passes
+  // blocks of the reducing passes: each warp pays the reduction once, so few
+  // blocks (one per SM: 18.6 / 24.8 / 13.4 us for OLSEN / ORTH / NORM at
+  // 1.2e5 elements and k = 22, two 20.6 / 28.1 / 14.3, three 30.7 / 37.8 /
+  // 16.5); k_ritz and GCOL, which also store two to four vectors, take two
+  // (GCOL 24.7, one 28.9; k_ritz 65.9 at 5e5 elements, one 84.2)
+  int rblk, rblk2;
 
   // out[j] = Vb_j . w, j < k; with gcol >= 0 also column gcol of G
   hci_status dots(const double* Vb, int k, const double* w, double* out, int gcol = -1) {
-    const dim3 grid((unsigned)nblk, (unsigned)((k + DOTS_GROUP - 1) / DOTS_GROUP));
+    const dim3 grid((unsigned)rblk, (unsigned)((k + DOTS_GROUP - 1) / DOTS_GROUP));
     HCI_LAUNCH(k_dots, grid, DBLOCK, 0, ctx->st)(Vb, ld, k, w, n, part, out, d, gcol);
+    HCI_CUDA(ctx, cudaGetLastError());
+    return HCI_OK;
+  }
+  template <int OP>
+  hci_status pass(int k) {
+    const int na = k + (OP == PASS_GCOL);
+    const int g = OP == PASS_GCOL ? rblk2 : rblk;
+    if (na <= 8)
+      HCI_LAUNCH((k_pass<OP, 8>), g, DBLOCK, 0, ctx->st)(V, W, ld, k, n, t, u, d, part);
+    else if (na <= 16)
+      HCI_LAUNCH((k_pass<OP, 16>), g, DBLOCK, 0, ctx->st)(V, W, ld, k, n, t, u, d, part);
+    else
+      HCI_LAUNCH((k_pass<OP, MAXSUB>), g, DBLOCK, 0, ctx->st)(V, W, ld, k, n, t, u, d, part);
     HCI_CUDA(ctx, cudaGetLastError());
     return HCI_OK;
   }
@@ -904,7 +1074,9 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
   D.n = nV;
   D.ld = (nV + 31) & ~(int64_t)31;
   D.nblk = grid_for(nV, DBLOCK, ctx->nsm * 8);
-  HCI_TRY(ensure_buf(ctx, ctx->d_vb, (size_t)D.ld * (MAXSUB + 3) * 8));
+  D.rblk = grid_for(nV, DBLOCK, ctx->nsm);
+  D.rblk2 = grid_for(nV, DBLOCK, ctx->nsm * 2);
+  HCI_TRY(ensure_buf(ctx, ctx->d_vb, (size_t)D.ld * (MAXSUB + 4) * 8));
   HCI_TRY(ensure_buf(ctx, ctx->d_wb, (size_t)D.ld * MAXSUB * 8));
   HCI_TRY(ensure_buf(ctx, ctx->d_part, (size_t)(D.nblk + 1) * LDG * 8));
   HCI_TRY(ensure_buf(ctx, ctx->d_small, sizeof(DavDev) + (size_t)(D.nblk + 1) * 16));
@@ -913,6 +1085,7 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
   D.x = D.V + (int64_t)MAXSUB * D.ld;
   D.wy = D.x + D.ld;
   D.t = D.wy + D.ld;
+  D.u = D.t + D.ld;
   D.part = bp<double>(ctx->d_part);
   D.d = bp<DavDev>(ctx->d_small);
   double* amax_v = reinterpret_cast<double*>(bp<char>(ctx->d_small) + sizeof(DavDev));
@@ -972,7 +1145,7 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
   }
   if (!(nrm2 > 0.0) || !std::isfinite(nrm2)) {
     HCI_CUDA(ctx, cudaMemsetAsync(V0, 0, (size_t)nV * 8, st));
-    HCI_LAUNCH(k_unit_min_diag, 1, 1024, 0, st)(V0, diag, nV);
+    HCI_LAUNCH(k_unit_min_diag, D.rblk, DBLOCK, 0, st)(V0, diag, nV, amax_v, amax_i, D.d);
     if (m > 0 || ctx->spin_parity != 0)
       HCI_LAUNCH(k_add_hash, D.nblk, DBLOCK, 0, st)(V0, nV, 1e-2 / std::sqrt((double)nV));
     if (ctx->spin_parity != 0) {
@@ -1014,7 +1187,7 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
       if (nrm2 > 1e-20) break;
       if (attempt == 1) return hci_fail(ctx, HCI_ERR_INVALID, "hci_davidson_roots: no start vector outside the roots");
       HCI_CUDA(ctx, cudaMemsetAsync(D.V, 0, (size_t)nV * 8, st));
-      HCI_LAUNCH(k_unit_min_diag, 1, 1024, 0, st)(D.V, diag, nV);
+      HCI_LAUNCH(k_unit_min_diag, D.rblk, DBLOCK, 0, st)(D.V, diag, nV, amax_v, amax_i, D.d);
       HCI_LAUNCH(k_add_hash, D.nblk, DBLOCK, 0, st)(D.V, nV, 1e-2 / std::sqrt((double)nV));
       parity_project(ctx, D.V, nV, D.nblk);
     }
@@ -1033,15 +1206,14 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
   // and whether the previous correction fell inside the subspace
   auto ritz = [&](double& th, double& r, int& stall) -> hci_status {
     HCI_LAUNCH(k_lowest<1>, 1, LW_T, 0, st)(D.d, k);
-    HCI_LAUNCH(k_ritz, D.nblk, DBLOCK, 0, st)(D.V, D.W, D.ld, k, D.d, diag, nV, D.x, D.wy, D.t, D.part);
+    HCI_LAUNCH(k_ritz, D.rblk2, DBLOCK, 0, st)(D.V, D.W, D.ld, k, D.d, diag, nV, D.x, D.wy, D.t, D.u, D.part);
     HCI_CUDA(ctx, cudaGetLastError());
-    double hv[2];
-    HCI_CUDA(ctx, cudaMemcpyAsync(&hv[0], &D.d->theta, 8, cudaMemcpyDeviceToHost, st));
-    HCI_CUDA(ctx, cudaMemcpyAsync(&hv[1], &D.d->ols[0], 8, cudaMemcpyDeviceToHost, st));
-    HCI_CUDA(ctx, cudaMemcpyAsync(&stall, &D.d->stall, 4, cudaMemcpyDeviceToHost, st));
+    DavReport h;
+    HCI_CUDA(ctx, cudaMemcpyAsync(&h, &D.d->rep, sizeof h, cudaMemcpyDeviceToHost, st));
     HCI_CUDA(ctx, cudaStreamSynchronize(st));
-    th = hv[0];
-    r = std::sqrt(hv[1]);
+    th = h.theta;
+    r = std::sqrt(h.ols[0]);
+    stall = h.stall;
     return HCI_OK;
   };
   for (; it < maxit; ++it) {
@@ -1072,9 +1244,18 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
       HCI_TRY(D.dots(D.V, 1, D.W, D.d->dots, 0));
       k = 1;
     }
-    HCI_LAUNCH(k_olsen, D.nblk, DBLOCK, 0, st)(D.d, diag, nV, D.x, D.t);
-    parity_project(ctx, D.t, nV, D.nblk);
     // orthogonalise the correction twice, normalise
+    if (m == 0 && ctx->spin_parity == 0) {
+      HCI_TRY(D.pass<PASS_OLSEN>(k));
+      HCI_TRY(D.pass<PASS_ORTH>(k));
+      HCI_TRY(D.pass<PASS_NORM>(k));
+      HCI_TRY(D.sigma(k));
+      HCI_TRY(D.pass<PASS_GCOL>(k));
+      ++k;
+      continue;
+    }
+    HCI_LAUNCH(k_olsen, D.nblk, DBLOCK, 0, st)(D.d, nV, D.u, D.t);
+    parity_project(ctx, D.t, nV, D.nblk);
     for (int pass = 0; pass < 2; ++pass) {
       HCI_TRY(D.dots(D.V, k, D.t, D.d->dots));
       HCI_LAUNCH(k_orth, D.nblk, DBLOCK, 0, st)(D.V, D.ld, k, D.d, D.t, nV);
@@ -1113,8 +1294,7 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
   HCI_TRY(D.dots(D.x, 1, D.x, &D.d->nrm2));
   HCI_LAUNCH(k_scale_by, D.nblk, DBLOCK, 0, st)(D.x, nullptr, nV, &D.d->nrm2);
   HCI_TRY(to_sorted(ctx, D.x, c_inout, 1));
-  HCI_LAUNCH(k_amax_part, D.nblk, DBLOCK, 0, st)(c_inout, nV, amax_v, amax_i);
-  HCI_LAUNCH(k_phase_sign, 1, 1, 0, st)(c_inout, amax_v, amax_i, D.nblk, &D.d->dots[0]);
+  HCI_LAUNCH(k_phase_sign, D.rblk, DBLOCK, 0, st)(c_inout, nV, amax_v, amax_i, D.d, &D.d->dots[0]);
   HCI_LAUNCH(k_apply_sign, D.nblk, DBLOCK, 0, st)(c_inout, nV, &D.d->dots[0]);
   HCI_CUDA(ctx, cudaGetLastError());
   prof_toc(ctx, HCI_PH_DAVIDSON);
