@@ -116,16 +116,23 @@ __global__ void k_rdm_pairs(int n, const ulonglong2* __restrict__ V, const doubl
 // Occupation correlation sum_a w_a n(a) n(a)^T of the distinct targets (the
 // first pair of each run of equal keys, w_a = d_a^2), over spin orbitals
 // (alpha 0..n-1, beta n..2n-1), split about the aufbau occupations n_R:
-// n(a) = n_R + delta_a, so acc = [W = sum w, u = sum w delta (2n),
-// Q = sum w delta delta^T (2n x 2n)], block-local in shared memory first.
-__global__ void k_dd_acc(int n, const ulonglong2* __restrict__ tgt, const double* __restrict__ d, int64_t m,
-                         uint64_t ra, uint64_t rb, double* __restrict__ acc) {
-  extern __shared__ double s_acc[];
-  const int mm = 2 * n, nacc = 1 + mm + mm * mm;
-  for (int t = threadIdx.x; t < nacc; t += blockDim.x) s_acc[t] = 0.0;
-  __syncthreads();
-  double* su = s_acc + 1;
-  double* sq = s_acc + 1 + mm;
+// n(a) = n_R + delta_a.  A changed spin orbital k has delta_k = s_k, -1 when
+// n_R holds it and +1 when not, so only the weights P_kl = sum of w over the
+// targets that change both k and l are accumulated (k <= l, P_kk among them),
+// with W = sum w: about 36 additions per target.  They go to L2 as FP64
+// reductions without return, spread over DD_COPIES copies [W, P (2n x 2n)]
+// so that the frontier orbitals' entries do not queue up at one address.
+// FP64 additions in shared memory are compare-and-swap loops: block-local
+// copies there took 71.4 ms for the pairs of a (44e,44o) state at eps2 = 2e-5,
+// this 4.7 ms.
+constexpr int DD_COPIES = 64;
+
+__global__ void __launch_bounds__(256) k_dd_acc(int n, const ulonglong2* __restrict__ tgt, const double* __restrict__ d,
+                                                int64_t m, uint64_t ra, uint64_t rb, double* __restrict__ acc) {
+  const int mm = 2 * n;
+  double* A = acc + (int64_t)(blockIdx.x % DD_COPIES) * (1 + mm * mm);
+  double* P = A + 1;
+  double wsum = 0.0;
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
     const ulonglong2 key = tgt[j];
     if (j > 0) {
@@ -135,38 +142,45 @@ __global__ void k_dd_acc(int n, const ulonglong2* __restrict__ tgt, const double
     const double dj = d[j];
     if (dj == 0.0) continue;
     const double w = dj * dj;
-    atomicAdd(&s_acc[0], w);
+    wsum += w;
     const uint64_t da = key.x ^ ra, db = key.y ^ rb;
-    for (int sk = 0; sk < 2; ++sk)
-      for (uint64_t x = sk ? db : da; x; x &= x - 1) {
-        const int ko = __ffsll((long long)x) - 1;
-        const int k = sk * n + ko;
-        const double dk = (((sk ? key.y : key.x) >> ko) & 1ull) ? 1.0 : -1.0;
-        atomicAdd(&su[k], w * dk);
-        for (int sl = 0; sl < 2; ++sl)
-          for (uint64_t y = sl ? db : da; y; y &= y - 1) {
-            const int lo = __ffsll((long long)y) - 1;
-            const double dl = (((sl ? key.y : key.x) >> lo) & 1ull) ? 1.0 : -1.0;
-            atomicAdd(&sq[k * mm + sl * n + lo], w * dk * dl);
-          }
-      }
+    for (uint64_t x = da; x; x &= x - 1) {
+      double* row = P + (__ffsll((long long)x) - 1) * mm;
+      for (uint64_t y = x; y; y &= y - 1) atomicAdd(row + __ffsll((long long)y) - 1, w);
+      for (uint64_t y = db; y; y &= y - 1) atomicAdd(row + n + __ffsll((long long)y) - 1, w);
+    }
+    for (uint64_t x = db; x; x &= x - 1) {
+      double* row = P + (n + __ffsll((long long)x) - 1) * mm + n;
+      for (uint64_t y = x; y; y &= y - 1) atomicAdd(row + __ffsll((long long)y) - 1, w);
+    }
   }
-  __syncthreads();
-  for (int t = threadIdx.x; t < nacc; t += blockDim.x)
-    if (s_acc[t] != 0.0) atomicAdd(&acc[t], s_acc[t]);
+  for (int o = 16; o; o >>= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
+  if ((threadIdx.x & 31) == 0 && wsum != 0.0) atomicAdd(A, wsum);
 }
 
-// M = W n_R n_R^T + n_R u^T + u n_R^T + Q, the layout k_diag_rdm reads
-__global__ void k_dd_matrix(int n, const double* __restrict__ acc, uint64_t ra, uint64_t rb, double* __restrict__ M) {
+// sum[t] = sum of the copies' entries t, in order
+__global__ void k_dd_sum(int cnt, const double* __restrict__ acc, double* __restrict__ sum) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= cnt) return;
+  double s = 0.0;
+#pragma unroll 8
+  for (int c = 0; c < DD_COPIES; ++c) s += acc[(int64_t)c * cnt + t];
+  sum[t] = s;
+}
+
+// M = W n_R n_R^T + n_R u^T + u n_R^T + Q, u_k = s_k P_kk, Q_kl = s_k s_l
+// P_kl, the layout k_diag_rdm reads
+__global__ void k_dd_matrix(int n, const double* __restrict__ sum, uint64_t ra, uint64_t rb, double* __restrict__ M) {
   const int mm = 2 * n;
-  const double W = acc[0];
-  const double* u = acc + 1;
-  const double* Q = acc + 1 + mm;
+  const double W = sum[0];
+  const double* P = sum + 1;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < mm * mm; t += gridDim.x * blockDim.x) {
     const int k = t / mm, l = t % mm;
     const double nk = (k < n ? ((ra >> k) & 1ull) : ((rb >> (k - n)) & 1ull)) ? 1.0 : 0.0;
     const double nl = (l < n ? ((ra >> l) & 1ull) : ((rb >> (l - n)) & 1ull)) ? 1.0 : 0.0;
-    M[t] = W * nk * nl + nk * u[l] + u[k] * nl + Q[t];
+    const double sk = 1.0 - 2.0 * nk, sl = 1.0 - 2.0 * nl;
+    const double p = k < l ? P[k * mm + l] : P[l * mm + k];
+    M[t] = W * nk * nl + nk * (sl * P[l * mm + l]) + (sk * P[k * mm + k]) * nl + sk * sl * p;
   }
 }
 
@@ -497,21 +511,20 @@ hci_status pt2_rdm_begin(hci_ctx* ctx) {
   const size_t n = (size_t)ctx->n, n2 = n * n, n4 = n2 * n2, m = 2 * n;
   HCI_TRY(ensure_buf(ctx, ctx->s_rdmh, (n4 + 2 * n2 + 2 * n2 * n) * 8));
   HCI_CUDA(ctx, cudaMemsetAsync(ctx->s_rdmh.p, 0, (n4 + 2 * n2 + 2 * n2 * n) * 8, ctx->st));
-  HCI_TRY(ensure_buf(ctx, ctx->p2_dd, (1 + m + 2 * m * m) * 8));
-  HCI_CUDA(ctx, cudaMemsetAsync(ctx->p2_dd.p, 0, (1 + m + 2 * m * m) * 8, ctx->st));
+  // the copies, their sum and M
+  HCI_TRY(ensure_buf(ctx, ctx->p2_dd, ((DD_COPIES + 1) * (1 + m * m) + m * m) * 8));
+  HCI_CUDA(ctx, cudaMemsetAsync(ctx->p2_dd.p, 0, DD_COPIES * (1 + m * m) * 8, ctx->st));
   return HCI_OK;
 }
 
 hci_status pt2_rdm_pairs(hci_ctx* ctx, const ulonglong2* V, const double* c, const ulonglong2* tgt, const int32_t* src,
                          const double* d, int64_t m) {
   if (m <= 0) return HCI_OK;
-  const int n = ctx->n, mm = 2 * n;
+  const int n = ctx->n;
   RdmAcc R = pt2_acc(ctx);
   HCI_LAUNCH(k_rdm_pairs, grid_for(m, 256), 256, 0, ctx->st)(n, V, c, tgt, src, d, m, R);
-  const size_t sm = (size_t)(1 + mm + mm * mm) * 8;
-  HCI_CUDA(ctx, cudaFuncSetAttribute(k_dd_acc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  HCI_LAUNCH(k_dd_acc, grid_for(m, 256, ctx->nsm * 2), 256, sm, ctx->st)(n, tgt, d, m, R.ref_a, R.ref_b,
-                                                                     bp<double>(ctx->p2_dd));
+  HCI_LAUNCH(k_dd_acc, grid_for(m, 256, ctx->nsm * 8), 256, 0, ctx->st)(n, tgt, d, m, R.ref_a, R.ref_b,
+                                                                       bp<double>(ctx->p2_dd));
   HCI_CUDA(ctx, cudaGetLastError());
   return HCI_OK;
 }
@@ -524,9 +537,12 @@ hci_status pt2_rdm_finish(hci_ctx* ctx, double* r1dd, double* r2dd, double* r1dc
   HCI_CUDA(ctx, cudaMemsetAsync(r1dc, 0, n2 * 8, st));
   HCI_CUDA(ctx, cudaMemsetAsync(r2dc, 0, n4 * 8, st));
   HCI_LAUNCH(k_rdm_finish, grid_for((int64_t)n4, 256, ctx->nsm * 8), 256, 0, st)(n, R, r1dc, r2dc, 0);
+  const int cnt = 1 + mm * mm;
   double* acc = bp<double>(ctx->p2_dd);
-  double* M = acc + 1 + mm + mm * mm;
-  HCI_LAUNCH(k_dd_matrix, grid_for((int64_t)mm * mm, 256), 256, 0, st)(n, acc, R.ref_a, R.ref_b, M);
+  double* sum = acc + (int64_t)DD_COPIES * cnt;
+  double* M = sum + cnt;
+  HCI_LAUNCH(k_dd_sum, (unsigned)((cnt + 255) / 256), 256, 0, st)(cnt, acc, sum);
+  HCI_LAUNCH(k_dd_matrix, grid_for((int64_t)mm * mm, 256), 256, 0, st)(n, sum, R.ref_a, R.ref_b, M);
   HCI_CUDA(ctx, cudaMemsetAsync(r1dd, 0, n2 * 8, st));
   HCI_CUDA(ctx, cudaMemsetAsync(r2dd, 0, n4 * 8, st));
   HCI_LAUNCH(k_diag_rdm, grid_for((int64_t)n2, 256), 256, 0, st)(n, M, r1dd, r2dd);
