@@ -127,7 +127,7 @@ struct hci_ctx {
   Graph graph;
   // scratch
   DevBuf s_cand, s_cand2, s_flags, s_scan, s_misc, s_counter, s_hist, s_walkstat, s_items, s_rdmw, s_rdmh;
-  DevBuf p2_vals, p2_vals2, p2_ref, p2_src, p2_src2, p2_d, p2_dd;   // perturbative correction
+  DevBuf p2_vals, p2_vals2, p2_ref, p2_src, p2_src2, p2_d, p2_dd, p2_tab;   // perturbative correction
   DevBuf ss_w, ss_draw, ss_draw2, ss_run, ss_src;                 // sampled perturbative correction
   DevBuf g_ua, g_ga, g_ia, g_ub, g_gb, g_ib, g_permb, g_bkeys, g_bkeys2, g_nbr_ptr, g_nbr, g_cnt;
   DevBuf g_bnbr_ptr, g_bnbr, g_costa, g_costb, g_htab, g_hval, g_posb, g_vb, g_ba;
@@ -228,6 +228,11 @@ hci_status sort_keys(hci_ctx* ctx, uint64_t* keys, uint64_t* tmp, int64_t n, int
 // (idx, with itmp as scratch) per key; either may be NULL
 hci_status sort_pairs(hci_ctx* ctx, uint64_t* keys, uint64_t* tmp, double* vals, double* vtmp, int32_t* idx,
                       int32_t* itmp, int64_t n, int bits_a, int bits_b);
+// The pairs grouped by key instead of sorted: ordered by the low `*bits` bits
+// of group_hash(key), so that equal keys lie in one run of equal hash, among
+// the few other keys that share it (first_of_key, below, tells them apart).
+hci_status group_pairs(hci_ctx* ctx, uint64_t* keys, uint64_t* tmp, double* vals, double* vtmp, int32_t* idx,
+                       int32_t* itmp, int64_t n, int* bits);
 // 64-bit content hash of a key array (device result).
 hci_status hash_keys(hci_ctx* ctx, const uint64_t* keys, int64_t n, uint64_t* hash_host);
 // Checks that keys are strictly ascending (device reduction); *ok_host = 1 if sorted.
@@ -246,13 +251,50 @@ hci_status direct_rdm(hci_ctx* ctx, const double* c, const RdmAcc& R);
 // density matrices of the perturbative correction (rdm.cu)
 hci_status pt2_rdm_begin(hci_ctx* ctx);
 hci_status pt2_rdm_pairs(hci_ctx* ctx, const ulonglong2* V, const double* c, const ulonglong2* tgt, const int32_t* src,
-                         const double* d, int64_t m);
+                         const double* d, int64_t m, const int64_t* list, const unsigned long long* nlist);
 hci_status pt2_rdm_finish(hci_ctx* ctx, double* r1dd, double* r2dd, double* r1dc, double* r2dc);
 // vectors between the caller's (sorted) order and the graph's internal order
 hci_status to_internal(hci_ctx* ctx, const double* sorted, double* internal, int nvec);
 hci_status to_sorted(hci_ctx* ctx, const double* internal, double* sorted, int nvec);
 
 // device helpers -------------------------------------------------------------
+__device__ __forceinline__ uint64_t key_mix(ulonglong2 k) {
+  uint64_t x = k.x * 0x9E3779B97F4A7C15ull ^ (k.y + 0x632BE59BD9B4E019ull + (k.x << 6) + (k.x >> 2));
+  x ^= x >> 31; x *= 0xBF58476D1CE4E5B9ull; x ^= x >> 29;
+  return x;
+}
+__device__ __forceinline__ bool key_eq(ulonglong2 a, ulonglong2 b) { return a.x == b.x && a.y == b.y; }
+
+// order of grouped pairs (the low bits of key_mix choose the hash class)
+__device__ __forceinline__ uint64_t group_hash(ulonglong2 k) { return key_mix(k) >> 16; }
+
+// In grouped pairs t: is i the first pair of its key?  The pair before
+// decides but where two keys share a hash.
+__device__ __forceinline__ bool first_of_key(const ulonglong2* __restrict__ t, int64_t i, ulonglong2 key, uint64_t mask) {
+  if (i == 0) return true;
+  ulonglong2 p = t[i - 1];
+  if (key_eq(p, key)) return false;
+  const uint64_t h = group_hash(key) & mask;
+  for (int64_t j = i - 1; (group_hash(p) & mask) == h;) {
+    if (--j < 0) break;
+    p = t[j];
+    if (key_eq(p, key)) return false;
+  }
+  return true;
+}
+// Next pair of the key after e in its run, or m
+__device__ __forceinline__ int64_t next_of_key(const ulonglong2* __restrict__ t, int64_t e, int64_t m, ulonglong2 key,
+                                               uint64_t mask) {
+  if (++e >= m || key_eq(t[e], key)) return e;
+  const uint64_t h = group_hash(key) & mask;
+  for (; e < m; ++e) {
+    const ulonglong2 k = t[e];
+    if (key_eq(k, key)) return e;
+    if ((group_hash(k) & mask) != h) return m;
+  }
+  return m;
+}
+
 __device__ __forceinline__ int popc64(uint64_t x) { return __popcll(x); }
 
 // (-1)^(number of set bits of s strictly between orbitals p and r)

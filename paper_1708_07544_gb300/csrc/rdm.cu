@@ -114,7 +114,7 @@ __global__ void k_rdm_pairs(int n, const ulonglong2* __restrict__ V, const doubl
 }
 
 // Occupation correlation sum_a w_a n(a) n(a)^T of the distinct targets (the
-// first pair of each run of equal keys, w_a = d_a^2), over spin orbitals
+// listed pairs j = list[0 .. *nlist), w_a = d_j^2), over spin orbitals
 // (alpha 0..n-1, beta n..2n-1), split about the aufbau occupations n_R:
 // n(a) = n_R + delta_a.  A changed spin orbital k has delta_k = s_k, -1 when
 // n_R holds it and +1 when not, so only the weights P_kl = sum of w over the
@@ -128,19 +128,19 @@ __global__ void k_rdm_pairs(int n, const ulonglong2* __restrict__ V, const doubl
 constexpr int DD_COPIES = 64;
 
 __global__ void __launch_bounds__(256) k_dd_acc(int n, const ulonglong2* __restrict__ tgt, const double* __restrict__ d,
-                                                int64_t m, uint64_t ra, uint64_t rb, double* __restrict__ acc) {
+                                                const int64_t* __restrict__ list,
+                                                const unsigned long long* __restrict__ nlist, uint64_t ra, uint64_t rb,
+                                                double* __restrict__ acc) {
   const int mm = 2 * n;
   double* A = acc + (int64_t)(blockIdx.x % DD_COPIES) * (1 + mm * mm);
   double* P = A + 1;
   double wsum = 0.0;
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
-    const ulonglong2 key = tgt[j];
-    if (j > 0) {
-      const ulonglong2 prev = tgt[j - 1];
-      if (prev.x == key.x && prev.y == key.y) continue;
-    }
+  const int64_t nt = (int64_t)*nlist;
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nt; q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t j = list[q];
     const double dj = d[j];
     if (dj == 0.0) continue;
+    const ulonglong2 key = tgt[j];
     const double w = dj * dj;
     wsum += w;
     const uint64_t da = key.x ^ ra, db = key.y ^ rb;
@@ -518,12 +518,12 @@ hci_status pt2_rdm_begin(hci_ctx* ctx) {
 }
 
 hci_status pt2_rdm_pairs(hci_ctx* ctx, const ulonglong2* V, const double* c, const ulonglong2* tgt, const int32_t* src,
-                         const double* d, int64_t m) {
+                         const double* d, int64_t m, const int64_t* list, const unsigned long long* nlist) {
   if (m <= 0) return HCI_OK;
   const int n = ctx->n;
   RdmAcc R = pt2_acc(ctx);
   HCI_LAUNCH(k_rdm_pairs, grid_for(m, 256), 256, 0, ctx->st)(n, V, c, tgt, src, d, m, R);
-  HCI_LAUNCH(k_dd_acc, grid_for(m, 256, ctx->nsm * 8), 256, 0, ctx->st)(n, tgt, d, m, R.ref_a, R.ref_b,
+  HCI_LAUNCH(k_dd_acc, grid_for(m, 256, ctx->nsm * 8), 256, 0, ctx->st)(n, tgt, d, list, nlist, R.ref_a, R.ref_b,
                                                                        bp<double>(ctx->p2_dd));
   HCI_CUDA(ctx, cudaGetLastError());
   return HCI_OK;

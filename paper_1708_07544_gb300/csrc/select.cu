@@ -52,12 +52,6 @@ struct WalkArgs {
   const double* eri;
 };
 
-__device__ __forceinline__ uint64_t key_mix(ulonglong2 k) {
-  uint64_t x = k.x * 0x9E3779B97F4A7C15ull ^ (k.y + 0x632BE59BD9B4E019ull + (k.x << 6) + (k.x >> 2));
-  x ^= x >> 31; x *= 0xBF58476D1CE4E5B9ull; x ^= x >> 29;
-  return x;
-}
-
 // perturbative mode: keep the term and the target?
 __device__ __forceinline__ bool pt_keep(const WalkArgs& A, ulonglong2 key, double term) {
   return fabs(term) > A.eps1 && (A.npart <= 1 || (int)(key_mix(key) % (uint64_t)A.npart) == A.part);
@@ -395,7 +389,6 @@ __global__ void __launch_bounds__(SEL_WARPS * 32) k_singles(WalkArgs A) {
 __device__ __forceinline__ bool key_less(ulonglong2 a, ulonglong2 b) {
   return a.x < b.x || (a.x == b.x && a.y < b.y);
 }
-__device__ __forceinline__ bool key_eq(ulonglong2 a, ulonglong2 b) { return a.x == b.x && a.y == b.y; }
 
 // number of elements of sorted arr[0,n) strictly less than key
 __device__ __forceinline__ int64_t lower_bound(const ulonglong2* __restrict__ arr, int64_t n, ulonglong2 key) {
@@ -612,7 +605,7 @@ extern "C" hci_status hci_merge(hci_ctx* ctx, const uint64_t* keys, const double
 // ---------------------------------------------------------------------------
 // Second-order Epstein-Nesbet correction with screening (Sec. II.B,
 // Eq. pt_hci): the walk and the singles emit every target D_a with its term
-// H_ai c_i when |H_ai c_i| > eps2; the (target, term) pairs are sorted by
+// H_ai c_i when |H_ai c_i| > eps2; the (target, term) pairs are grouped by
 // target, targets in V are dropped, and each remaining target contributes
 // (sum of its terms)^2 / (E0 - H_aa).  The targets are processed in hash
 // classes so that at most max_pairs pairs are held at once.
@@ -622,41 +615,45 @@ namespace {
 // Aufbau reference R for diagonal elements by differences, over spin
 // orbitals k (alpha 0..n-1, beta n..2n-1): g_kl = (kk|ll) - [same spin] (kl|lk),
 // F_k = h_kk + sum_{l in R, l != k} g_kl, E_R = e_core + sum_{k in R} h_kk +
-// sum_{k<l in R} g_kl.  out = [E_R, F (2n), g (2n x 2n)].
-__global__ void k_pt2_ref(int n, const double* __restrict__ h, const double* __restrict__ eri, double ecore,
-                          uint64_t ra, uint64_t rb, double* __restrict__ out) {
-  const int m = 2 * n;
-  double* F = out + 1;
-  double* g = out + 1 + m;
-  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-    const int k = t / m, l = t % m, p = k % n, q = l % n;
+// sum_{k<l in R} g_kl.  A spin orbital k where a determinant differs from R
+// is emptied (d_k = -1) when R holds it, else filled (d_k = +1), so the
+// signs go into the table: out = [E_R, d_k F_k (2n), d_k d_l g_kl (2n x 2n)].
+// One block per k; k_pt2_eref adds E_R.
+__global__ void k_pt2_ref(int n, const double* __restrict__ h, const double* __restrict__ eri, uint64_t ra, uint64_t rb,
+                          double* __restrict__ out) {
+  extern __shared__ double s_g[];
+  const int m = 2 * n, k = blockIdx.x, p = k % n;
+  auto occ = [&](int l) { return (l < n ? (ra >> l) : (rb >> (l - n))) & 1ull; };
+  const double dk = occ(k) ? -1.0 : 1.0;
+  for (int l = threadIdx.x; l < m; l += blockDim.x) {
+    const int q = l % n;
     double v = eri[(((int64_t)p * n + p) * n + q) * n + q];
     if ((k < n) == (l < n)) v -= eri[(((int64_t)p * n + q) * n + q) * n + p];
-    g[t] = k == l ? 0.0 : v;
+    if (k == l) v = 0.0;
+    s_g[l] = v;
+    out[1 + m + k * m + l] = dk * (occ(l) ? -v : v);
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < m; k += blockDim.x) {
-    double f = h[(k % n) * n + (k % n)];
-    for (int l = 0; l < m; ++l) {
-      const bool occ = l < n ? ((ra >> l) & 1ull) : ((rb >> (l - n)) & 1ull);
-      if (occ && l != k) f += g[k * m + l];
-    }
-    F[k] = f;
-  }
   if (threadIdx.x == 0) {
-    double e = ecore;
-    for (int k = 0; k < m; ++k) {
-      if (!(k < n ? ((ra >> k) & 1ull) : ((rb >> (k - n)) & 1ull))) continue;
-      e += h[(k % n) * n + (k % n)];
-      for (int l = k + 1; l < m; ++l)
-        if (l < n ? ((ra >> l) & 1ull) : ((rb >> (l - n)) & 1ull)) e += g[k * m + l];
-    }
-    out[0] = e;
+    double f = h[p * n + p];
+    for (int l = 0; l < m; ++l)
+      if (occ(l)) f += s_g[l];
+    out[1 + k] = dk * f;
   }
+}
+// E_R = e_core + sum_{k in R} (h_kk + F_k) / 2
+__global__ void k_pt2_eref(int n, const double* __restrict__ h, double ecore, uint64_t ra, uint64_t rb,
+                           double* __restrict__ out) {
+  const int lane = threadIdx.x;
+  double e = 0.0;
+  for (int k = lane; k < 2 * n; k += 32)
+    if ((k < n ? (ra >> k) : (rb >> (k - n))) & 1ull) e += h[(k % n) * n + (k % n)] - out[1 + k];
+  for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+  if (lane == 0) out[0] = ecore + 0.5 * e;
 }
 
 // H_aa = E_R + sum_k d_k F_k + sum_{k<l} d_k d_l g_kl over the spin orbitals
-// where D_a differs from R (d = +1 occupied in D_a only, -1 in R only)
+// where D_a differs from R
 __device__ __forceinline__ double pt2_diag(const double* s_ref, int n, ulonglong2 key, uint64_t ra, uint64_t rb) {
   const int m = 2 * n;
   const double* F = s_ref + 1;
@@ -665,65 +662,124 @@ __device__ __forceinline__ double pt2_diag(const double* s_ref, int n, ulonglong
   double e = s_ref[0];
   for (uint64_t x = da; x; x &= x - 1) {
     const int k = __ffsll((long long)x) - 1;
-    const double dk = ((key.x >> k) & 1ull) ? 1.0 : -1.0;
-    e += dk * F[k];
-    for (uint64_t y = x & (x - 1); y; y &= y - 1) {
-      const int l = __ffsll((long long)y) - 1;
-      e += dk * (((key.x >> l) & 1ull) ? 1.0 : -1.0) * g[k * m + l];
-    }
-    for (uint64_t y = db; y; y &= y - 1) {
-      const int l = __ffsll((long long)y) - 1;
-      e += dk * (((key.y >> l) & 1ull) ? 1.0 : -1.0) * g[k * m + n + l];
-    }
+    const double* gk = g + k * m;
+    e += F[k];
+    for (uint64_t y = x & (x - 1); y; y &= y - 1) e += gk[__ffsll((long long)y) - 1];
+    for (uint64_t y = db; y; y &= y - 1) e += gk[n + __ffsll((long long)y) - 1];
   }
   for (uint64_t x = db; x; x &= x - 1) {
     const int k = __ffsll((long long)x) - 1;
-    const double dk = ((key.y >> k) & 1ull) ? 1.0 : -1.0;
-    e += dk * F[n + k];
-    for (uint64_t y = x & (x - 1); y; y &= y - 1) {
-      const int l = __ffsll((long long)y) - 1;
-      e += dk * (((key.y >> l) & 1ull) ? 1.0 : -1.0) * g[(n + k) * m + n + l];
-    }
+    const double* gk = g + (n + k) * m + n;
+    e += F[n + k];
+    for (uint64_t y = x & (x - 1); y; y &= y - 1) e += gk[__ffsll((long long)y) - 1];
   }
   return e;
 }
 
-// On the first pair of every run of equal targets (sorted): the run's terms
-// summed, the target dropped when it is in V, else contrib = sum^2 /
-// (e0 - H_aa) and ext = 1; zero on every other pair.
-__global__ void k_pt2_terms(const ulonglong2* __restrict__ t, const double* __restrict__ v, int64_t m,
-                            const ulonglong2* __restrict__ V, int64_t nV, int n, const double* __restrict__ ref,
-                            uint64_t ra, uint64_t rb, double e0, double* __restrict__ contrib,
-                            int64_t* __restrict__ ext, double* __restrict__ dpair, const double* __restrict__ cvec,
-                            const int32_t* __restrict__ src) {
+// Hash table of the determinants of V (their positions; -1 empty), at least
+// twice as many slots, linear probing: one or two look-ups tell whether a
+// target belongs to V, where a binary search takes log2 nV dependent ones.
+__global__ void k_space_insert(const ulonglong2* __restrict__ V, int64_t nV, int32_t* __restrict__ tab, uint64_t mask) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nV; i += (int64_t)gridDim.x * blockDim.x) {
+    uint64_t h = key_mix(V[i]) & mask;
+    for (uint64_t probe = 0; probe <= mask; ++probe, h = (h + 1) & mask)
+      if (atomicCAS(&tab[h], -1, (int32_t)i) == -1) break;
+  }
+}
+__device__ __forceinline__ bool in_space(const ulonglong2* __restrict__ V, const int32_t* __restrict__ tab,
+                                         uint64_t mask, ulonglong2 key) {
+  uint64_t h = key_mix(key) & mask;
+  for (uint64_t probe = 0; probe <= mask; ++probe, h = (h + 1) & mask) {
+    const int32_t j = tab[h];
+    if (j < 0) return false;
+    if (key_eq(V[j], key)) return true;
+  }
+  return false;
+}
+
+// list = the first pairs of the targets outside V (in any order; *count of
+// them); with dpair, 0 on every pair of a target in V
+__global__ void __launch_bounds__(256) k_pt2_targets(const ulonglong2* __restrict__ t, int64_t m, uint64_t gmask,
+                                                     const ulonglong2* __restrict__ V, const int32_t* __restrict__ tab,
+                                                     uint64_t tmask, int64_t* __restrict__ list,
+                                                     unsigned long long* __restrict__ count,
+                                                     double* __restrict__ dpair) {
+  __shared__ int s_n[8];
+  __shared__ unsigned long long s_base;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int64_t i0 = (int64_t)blockIdx.x * 256; i0 < m; i0 += (int64_t)gridDim.x * 256) {
+    const int64_t i = i0 + threadIdx.x;
+    bool ext = false;
+    if (i < m) {
+      const ulonglong2 key = t[i];
+      if (first_of_key(t, i, key, gmask)) {
+        ext = !in_space(V, tab, tmask, key);
+        if (!ext && dpair)
+          for (int64_t e = i; e < m; e = next_of_key(t, e, m, key, gmask)) dpair[e] = 0.0;
+      }
+    }
+    const unsigned b = __ballot_sync(0xffffffffu, ext);
+    if (lane == 0) s_n[w] = __popc(b);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int tot = 0;
+      for (int q = 0; q < 8; ++q) {
+        const int c = s_n[q];
+        s_n[q] = tot;
+        tot += c;
+      }
+      s_base = tot ? atomicAdd(count, (unsigned long long)tot) : 0ull;
+    }
+    __syncthreads();
+    if (ext) list[s_base + s_n[w] + __popc(b & ((1u << lane) - 1u))] = i;
+    __syncthreads();
+  }
+}
+
+// One listed target per thread: its terms summed, sum^2 / (e0 - H_aa) added
+// to the block's part_e (threads in order, then a fixed tree), and with dpair
+// the first-order coefficient d_a on every pair of the target.  Bound by FP64
+// issue (about 55 operations per target, most of them H_aa's), so the targets
+// are listed first: taken in place, where only the first pair of a run works,
+// 2 to 3 lanes of 4 idle through all of them.
+__global__ void __launch_bounds__(256) k_pt2_terms(const ulonglong2* __restrict__ t, const double* __restrict__ v,
+                                                   int64_t m, uint64_t gmask, const int64_t* __restrict__ list,
+                                                   const unsigned long long* __restrict__ count, int n,
+                                                   const double* __restrict__ ref, uint64_t ra, uint64_t rb, double e0,
+                                                   double* __restrict__ part_e, double* __restrict__ dpair,
+                                                   const double* __restrict__ cvec, const int32_t* __restrict__ src) {
   extern __shared__ double s_ref[];
+  __shared__ double red_e[8];
   const int nref = 1 + 2 * n + 4 * n * n;
   for (int u = threadIdx.x; u < nref; u += blockDim.x) s_ref[u] = ref[u];
   __syncthreads();
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    double cv = 0.0;
-    int64_t e = 0;
+  double esum = 0.0;
+  const int64_t nt = (int64_t)*count;
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nt; q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = list[q];
     const ulonglong2 key = t[i];
-    if (i == 0 || !key_eq(key, t[i - 1])) {
-      const int64_t pos = lower_bound(V, nV, key);
-      double da = 0.0;
-      int64_t end = i + 1;
-      if (!(pos < nV && key_eq(V[pos], key))) {
-        double num = 0.0;
-        for (end = i; end < m && key_eq(t[end], key); ++end) num += src ? v[end] * cvec[src[end]] : v[end];
-        da = num / (e0 - pt2_diag(s_ref, n, key, ra, rb));
-        cv = num * da;
-        e = 1;
-      } else if (dpair) {
-        while (end < m && key_eq(t[end], key)) ++end;
-      }
-      // first-order coefficient d_a on every pair of the run (0 for D_a in V)
-      if (dpair)
-        for (int64_t j = i; j < end; ++j) dpair[j] = da;
-    }
-    contrib[i] = cv;
-    ext[i] = e;
+    double num = 0.0;
+    for (int64_t e = i; e < m; e = next_of_key(t, e, m, key, gmask)) num += src ? v[e] * cvec[src[e]] : v[e];
+    const double da = num / (e0 - pt2_diag(s_ref, n, key, ra, rb));
+    esum = fma(num, da, esum);
+    if (dpair)
+      for (int64_t e = i; e < m; e = next_of_key(t, e, m, key, gmask)) dpair[e] = da;
   }
+  for (int o = 16; o; o >>= 1) esum += __shfl_xor_sync(0xffffffffu, esum, o);
+  if ((threadIdx.x & 31) == 0) red_e[threadIdx.x >> 5] = esum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double e = 0.0;
+    for (int w = 0; w < 8; ++w) e += red_e[w];
+    part_e[blockIdx.x] = e;
+  }
+}
+
+__global__ void k_pt2_total(const double* __restrict__ part_e, int np, double* __restrict__ out) {
+  double e = 0.0;
+  for (int b = threadIdx.x; b < np; b += 32) e += part_e[b];
+  for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+  if (threadIdx.x == 0) *out = e;
 }
 
 // dE2/dc_i = 2 sum over the screened pairs of d_a H_ai (the pairs fixed)
@@ -825,10 +881,16 @@ extern "C" hci_status hci_pt2(hci_ctx* ctx, double eps2, const uint64_t* keys, c
   const size_t nref = 1 + 2 * (size_t)n + 4 * (size_t)n * n;
   HCI_TRY(ensure_buf(ctx, ctx->p2_ref, nref * 8 + (PT2_SUM_BLOCKS + 2) * 8));
   double* ref = bp<double>(ctx->p2_ref);
-  double* part = ref + nref;
-  double* dsum = part + PT2_SUM_BLOCKS;
-  HCI_LAUNCH(k_pt2_ref, 1, 256, 0, st)(n, bp<double>(ctx->h), bp<double>(ctx->eri), ctx->ecore, A.ref_a, A.ref_b,
-                                       ref);
+  HCI_LAUNCH(k_pt2_ref, 2 * n, 64, (size_t)2 * n * 8, st)(n, bp<double>(ctx->h), bp<double>(ctx->eri), A.ref_a, A.ref_b,
+                                                         ref);
+  HCI_LAUNCH(k_pt2_eref, 1, 32, 0, st)(n, bp<double>(ctx->h), ctx->ecore, A.ref_a, A.ref_b, ref);
+  HCI_CUDA(ctx, cudaGetLastError());
+  // hash table of V
+  uint64_t tsize = 1024;
+  while (tsize < 2 * (uint64_t)nV) tsize <<= 1;
+  HCI_TRY(ensure_buf(ctx, ctx->p2_tab, (size_t)tsize * 4));
+  HCI_CUDA(ctx, cudaMemsetAsync(ctx->p2_tab.p, 0xFF, (size_t)tsize * 4, st));
+  HCI_LAUNCH(k_space_insert, grid_for(nV, 256), 256, 0, st)(A.keys, nV, bp<int32_t>(ctx->p2_tab), tsize - 1);
   HCI_CUDA(ctx, cudaGetLastError());
   const int64_t per = max_pairs > 0 ? max_pairs : ((int64_t)1 << 28);
   double acc = 0.0;
@@ -868,33 +930,37 @@ extern "C" hci_status hci_pt2(hci_ctx* ctx, double eps2, const uint64_t* keys, c
       src2 = bp<int32_t>(ctx->p2_src2);
       dpair = bp<double>(ctx->p2_d);
     }
-    HCI_TRY(sort_pairs(ctx, bp<uint64_t>(ctx->s_cand), bp<uint64_t>(ctx->s_cand2), bp<double>(ctx->p2_vals),
-                       bp<double>(ctx->p2_vals2), src, src2, m, n, n));
-    HCI_TRY(ensure_buf(ctx, ctx->s_flags, (size_t)(2 * m + 1) * 8));
-    int64_t* ext = bp<int64_t>(ctx->s_flags);
-    int64_t* ext_scan = ext + m;
-    double* contrib = bp<double>(ctx->p2_vals2);
+    int gbits = 0;
+    HCI_TRY(group_pairs(ctx, bp<uint64_t>(ctx->s_cand), bp<uint64_t>(ctx->s_cand2), bp<double>(ctx->p2_vals),
+                        bp<double>(ctx->p2_vals2), src, src2, m, &gbits));
+    const uint64_t gmask = ((uint64_t)1 << gbits) - 1;
+    const int tb = grid_for(m, 256, ctx->nsm * 8);
+    // [E2, targets outside V], the blocks' sums, the list of the targets
+    HCI_TRY(ensure_buf(ctx, ctx->s_flags, (size_t)(2 + tb + m) * 8));
+    double* esum = bp<double>(ctx->s_flags);
+    unsigned long long* count = reinterpret_cast<unsigned long long*>(esum + 1);
+    double* part_e = esum + 2;
+    int64_t* list = reinterpret_cast<int64_t*>(part_e + tb);
+    HCI_CUDA(ctx, cudaMemsetAsync(count, 0, 8, st));
+    HCI_LAUNCH(k_pt2_targets, grid_for(m, 256), 256, 0, st)(bp<ulonglong2>(ctx->s_cand), m, gmask, A.keys,
+                                                          bp<int32_t>(ctx->p2_tab), tsize - 1, list, count, dpair);
     const size_t sm = nref * 8;
     HCI_CUDA(ctx, cudaFuncSetAttribute(k_pt2_terms, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    HCI_LAUNCH(k_pt2_terms, grid_for(m, 256), 256, sm, st)(bp<ulonglong2>(ctx->s_cand), bp<double>(ctx->p2_vals), m,
-                                                          A.keys, nV, n, ref, A.ref_a, A.ref_b, e0, contrib, ext,
-                                                          dpair, c, src);
+    HCI_LAUNCH(k_pt2_terms, tb, 256, sm, st)(bp<ulonglong2>(ctx->s_cand), bp<double>(ctx->p2_vals), m, gmask, list,
+                                             count, n, ref, A.ref_a, A.ref_b, e0, part_e, dpair, c, src);
     if (grad_c)
       HCI_LAUNCH(k_pt2_grad, grid_for(m, 256), 256, 0, st)(src, bp<double>(ctx->p2_vals), dpair, m, grad_c);
-    if (want_rdm) HCI_TRY(pt2_rdm_pairs(ctx, A.keys, c, bp<ulonglong2>(ctx->s_cand), src, dpair, m));
-    HCI_CUDA(ctx, cudaGetLastError());
-    HCI_LAUNCH(k_sum_slices_d, PT2_SUM_BLOCKS, 256, 0, st)(contrib, m, part);
-    HCI_LAUNCH(k_sum_parts_d, 1, 32, 0, st)(part, PT2_SUM_BLOCKS, dsum);
-    int64_t* cnt_dev = reinterpret_cast<int64_t*>(bp<char>(ctx->s_counter) + 40);
-    HCI_TRY(scan_i64(ctx, ext, ext_scan, m, cnt_dev));
+    if (want_rdm)
+      HCI_TRY(pt2_rdm_pairs(ctx, A.keys, c, bp<ulonglong2>(ctx->s_cand), src, dpair, m, list, count));
+    HCI_LAUNCH(k_pt2_total, 1, 32, 0, st)(part_e, tb, esum);
     HCI_CUDA(ctx, cudaGetLastError());
     double hs = 0.0;
-    int64_t hc = 0;
-    HCI_CUDA(ctx, cudaMemcpyAsync(&hs, dsum, 8, cudaMemcpyDeviceToHost, st));
-    HCI_CUDA(ctx, cudaMemcpyAsync(&hc, cnt_dev, 8, cudaMemcpyDeviceToHost, st));
+    unsigned long long hc = 0;
+    HCI_CUDA(ctx, cudaMemcpyAsync(&hs, esum, 8, cudaMemcpyDeviceToHost, st));
+    HCI_CUDA(ctx, cudaMemcpyAsync(&hc, count, 8, cudaMemcpyDeviceToHost, st));
     HCI_CUDA(ctx, cudaStreamSynchronize(st));
     acc += hs;
-    next_total += hc;
+    next_total += (int64_t)hc;
     return HCI_OK;
   };
   HCI_TRY(ensure_buf(ctx, ctx->s_cand, (size_t)4096 * 16));
@@ -1061,11 +1127,12 @@ __global__ void k_ss_gather(int64_t j0, int64_t j1, int64_t ndist, int64_t m, co
   }
 }
 
-// On the first pair of every run of equal targets (sorted; element H_aj and
+// On the first pair of every target (grouped pairs; element H_aj and
 // source j on each pair): targets in V give 0, the others their estimate
 // with the eps2 screen (every emitted pair) and with eps2_det.
 __global__ void k_ss_terms(const ulonglong2* __restrict__ t, const double* __restrict__ v,
-                           const int32_t* __restrict__ src, int64_t m, const ulonglong2* __restrict__ V, int64_t nV,
+                           const int32_t* __restrict__ src, int64_t m, uint64_t gmask,
+                           const ulonglong2* __restrict__ V, const int32_t* __restrict__ tab, uint64_t tmask,
                            const double* __restrict__ sc, const double* __restrict__ sf, double eps2_det,
                            double nd, int n, const double* __restrict__ ref, uint64_t ra, uint64_t rb, double e0,
                            double* __restrict__ out_t, double* __restrict__ out_d) {
@@ -1076,11 +1143,10 @@ __global__ void k_ss_terms(const ulonglong2* __restrict__ t, const double* __res
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
     double et = 0.0, ed = 0.0;
     const ulonglong2 key = t[i];
-    if (i == 0 || !key_eq(key, t[i - 1])) {
-      const int64_t pos = lower_bound(V, nV, key);
-      if (!(pos < nV && key_eq(V[pos], key))) {
+    if (first_of_key(t, i, key, gmask)) {
+      if (!in_space(V, tab, tmask, key)) {
         double S[2] = {0.0, 0.0}, T[2] = {0.0, 0.0}, U[2] = {0.0, 0.0};
-        for (int64_t e = i; e < m && key_eq(t[e], key); ++e) {
+        for (int64_t e = i; e < m; e = next_of_key(t, e, m, key, gmask)) {
           const int32_t j = src[e];
           const double x = v[e] * sc[j], f = sf[j];
           for (int k = 0; k < 2; ++k) {
@@ -1183,7 +1249,10 @@ extern "C" hci_status hci_pt2_stochastic(hci_ctx* ctx, const uint64_t* keys, con
   ulonglong2* sk = bp<ulonglong2>(ctx->ss_src);
   double* sc = reinterpret_cast<double*>(sk + maxsrc);
   double* sf = sc + maxsrc;
-  // the reference of the diagonal elements (written by hci_pt2 above)
+  // the reference of the diagonal elements and the hash table of V (written
+  // by hci_pt2 above)
+  uint64_t tsize = 1024;
+  while (tsize < 2 * (uint64_t)nV) tsize <<= 1;
   WalkArgs A;
   HCI_TRY(pt_walk_args(ctx, A, reinterpret_cast<const uint64_t*>(sk), sc, 0, eps2));
   const size_t nref = 1 + 2 * (size_t)n + 4 * (size_t)n * n;
@@ -1222,12 +1291,14 @@ extern "C" hci_status hci_pt2_stochastic(hci_ctx* ctx, const uint64_t* keys, con
     HCI_TRY(ensure_buf(ctx, ctx->p2_vals2, (size_t)mp * 8));
     HCI_TRY(ensure_buf(ctx, ctx->p2_src2, (size_t)mp * 4));
     HCI_TRY(ensure_buf(ctx, ctx->p2_d, (size_t)mp * 8));
-    HCI_TRY(sort_pairs(ctx, bp<uint64_t>(ctx->s_cand), bp<uint64_t>(ctx->s_cand2), bp<double>(ctx->p2_vals),
-                       bp<double>(ctx->p2_vals2), bp<int32_t>(ctx->p2_src), bp<int32_t>(ctx->p2_src2), mp, n, n));
+    int gbits = 0;
+    HCI_TRY(group_pairs(ctx, bp<uint64_t>(ctx->s_cand), bp<uint64_t>(ctx->s_cand2), bp<double>(ctx->p2_vals),
+                        bp<double>(ctx->p2_vals2), bp<int32_t>(ctx->p2_src), bp<int32_t>(ctx->p2_src2), mp, &gbits));
     double* ct = bp<double>(ctx->p2_vals2);
     double* cd = bp<double>(ctx->p2_d);
     HCI_LAUNCH(k_ss_terms, grid_for(mp, 256), 256, smref, st)(bp<ulonglong2>(ctx->s_cand), bp<double>(ctx->p2_vals),
-                                                              bp<int32_t>(ctx->p2_src), mp, Vk, nV, sc, sf, eps2_det,
+                                                              bp<int32_t>(ctx->p2_src), mp, ((uint64_t)1 << gbits) - 1, Vk,
+                                                              bp<int32_t>(ctx->p2_tab), tsize - 1, sc, sf, eps2_det,
                                                               (double)nd, n, ref, A.ref_a, A.ref_b, e0, ct, cd);
     HCI_LAUNCH(k_sum_slices_d, PT2_SUM_BLOCKS, 256, 0, st)(ct, mp, part);
     HCI_LAUNCH(k_sum_parts_d, 1, 32, 0, st)(part, PT2_SUM_BLOCKS, dsum);
