@@ -104,8 +104,32 @@ __device__ __forceinline__ bool before(double ma, int ia, double mb, int ib) {
   return ma > mb || (ma == mb && ia < ib);
 }
 
+// m (descending, ties by id ascending) and id sorted in place in shared memory
+__device__ __forceinline__ void bitonic_desc(double* m, int* id, int P) {
+  for (int k = 2; k <= P; k <<= 1) {
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      for (int i = threadIdx.x; i < P; i += blockDim.x) {
+        int l = i ^ j;
+        if (l > i) {
+          bool up = (i & k) == 0;   // ascending in "before" order
+          double mi = m[i], ml = m[l];
+          int ii = id[i], il = id[l];
+          bool swap = up ? before(ml, il, mi, ii) : before(mi, ii, ml, il);
+          if (swap) {
+            m[i] = ml; m[l] = mi;
+            id[i] = il; id[l] = ii;
+          }
+        }
+      }
+      __syncthreads();
+    }
+  }
+}
+
 // One CTA per list: gather |v| for every target, bitonic sort (|v| desc,
-// target index asc), write magnitudes and packed targets.
+// target index asc), write magnitudes and packed targets (r | s << 8 | sign
+// of v << 15, so that a walk that needs the element reads it in list order
+// instead of gathering the integral).
 __global__ void k_build_lists(int n, const double* __restrict__ eri, int same, int L, int P,
                               double* __restrict__ mag_out, uint16_t* __restrict__ tgt_out) {
   extern __shared__ double sm_d[];
@@ -128,39 +152,74 @@ __global__ void k_build_lists(int n, const double* __restrict__ eri, int same, i
         v = eri[(((int64_t)p * n + r) * n + q) * n + s];
       }
       m[e] = fabs(v);
-      id[e] = e;
+      id[e] = 2 * e + (signbit(v) ? 1 : 0);
     } else {
       m[e] = -1.0;
       id[e] = INT_MAX;
     }
   }
   __syncthreads();
-  for (int k = 2; k <= P; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        int l = i ^ j;
-        if (l > i) {
-          bool up = (i & k) == 0;   // ascending in "before" order
-          double mi = m[i], ml = m[l];
-          int ii = id[i], il = id[l];
-          bool swap = up ? before(ml, il, mi, ii) : before(mi, ii, ml, il);
-          if (swap) {
-            m[i] = ml; m[l] = mi;
-            id[i] = il; id[l] = ii;
-          }
-        }
-      }
-      __syncthreads();
-    }
-  }
+  bitonic_desc(m, id, P);
   for (int e = threadIdx.x; e < L; e += blockDim.x) {
-    int src = id[e];
+    int src = id[e] >> 1;
     int r, s;
     if (same) tri_decode(src, r, s);
     else { r = src / n; s = src % n; }
     mag_out[(int64_t)list * L + e] = m[e];
-    tgt_out[(int64_t)list * L + e] = (uint16_t)(r | (s << 8));
+    tgt_out[(int64_t)list * L + e] = (uint16_t)(r | (s << 8) | ((id[e] & 1) << 15));
   }
+}
+
+// The single excitations p -> r by descending bound (one block), packed
+// p | r << 8 with the bound rounded up to FP32
+__global__ void k_sort_singles(int n, const double* __restrict__ bound, int P, uint16_t* __restrict__ pr,
+                               float* __restrict__ bf) {
+  extern __shared__ double sm_d[];
+  double* m = sm_d;
+  int* id = reinterpret_cast<int*>(m + P);
+  const int L = n * n;
+  for (int e = threadIdx.x; e < P; e += blockDim.x) {
+    m[e] = e < L ? bound[e] : -1.0;
+    id[e] = e < L ? e : INT_MAX;
+  }
+  __syncthreads();
+  bitonic_desc(m, id, P);
+  for (int e = threadIdx.x; e < L; e += blockDim.x) {
+    pr[e] = (uint16_t)((id[e] / n) | ((id[e] % n) << 8));
+    bf[e] = __double2float_ru(m[e]);
+  }
+}
+
+// |jk_same|, |j_opp| and |f_ref| rounded up to FP32: [n^3][n^3][2 n^2]
+__global__ void k_single_f32(int n, const double* __restrict__ jk_same, const double* __restrict__ j_opp,
+                             const double* __restrict__ f_ref, float* __restrict__ out) {
+  const int64_t n3 = (int64_t)n * n * n, tot = 2 * n3 + 2 * n * n;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tot; t += (int64_t)gridDim.x * blockDim.x) {
+    const double v = t < n3 ? jk_same[t] : t < 2 * n3 ? j_opp[t - n3] : f_ref[t - 2 * n3];
+    out[t] = __double2float_ru(fabs(v));
+  }
+}
+
+// For each sorted single the parts of a bound that needs only the numbers of
+// orbitals in which a determinant differs from the aufbau one, rounded up:
+// |F_R| (alpha, beta) with the margin of the FP64 sums' rounding, and the
+// largest same-spin and other-spin term
+__global__ void k_single_max(int n, const uint16_t* __restrict__ pr, const float* __restrict__ f32,
+                             const float* __restrict__ bf, float4* __restrict__ out) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n * n) return;
+  const int64_t n3 = (int64_t)n * n * n;
+  const int p = pr[e] & 63, r = pr[e] >> 8;
+  const float* js = f32 + ((int64_t)p * n + r) * n;
+  float ms = 0.0f, mo = 0.0f;
+  for (int k = 0; k < n; ++k) {
+    ms = fmaxf(ms, js[k]);
+    mo = fmaxf(mo, js[n3 + k]);
+  }
+  const float add = __fmul_ru(2e-13f, bf[e]), up = 1.000002f;
+  out[e] = make_float4(__fmul_ru(__fadd_ru(f32[2 * n3 + p * n + r], add), up),
+                       __fmul_ru(__fadd_ru(f32[2 * n3 + (int64_t)n * n + p * n + r], add), up), __fmul_ru(ms, up),
+                       __fmul_ru(mo, up));
 }
 
 // f_ref[s][p][r] = h_pr + sum_{k occ in spin s of R} ((pr|kk) - (pk|kr))
@@ -310,7 +369,8 @@ extern "C" hci_status hci_destroy(hci_ctx* ctx) {
   cudaStream_t st = ctx->st;
   DevBuf* bufs[] = {&ctx->h, &ctx->eri, &ctx->jk_same, &ctx->j_opp, &ctx->lists.opp_mag, &ctx->lists.opp_tgt,
                     &ctx->lists.list_max, &ctx->lists.f_ref, &ctx->s_items,
-                    &ctx->lists.same_mag, &ctx->lists.same_tgt, &ctx->lists.single_bound,
+                    &ctx->lists.same_mag, &ctx->lists.same_tgt, &ctx->lists.single_bound, &ctx->lists.single_pr, &ctx->lists.single_bf,
+                    &ctx->lists.single_f32, &ctx->lists.single_max,
                     &ctx->graph.rowptr, &ctx->graph.rowstart, &ctx->graph.diag, &ctx->graph.keys,
                     &ctx->s_cand, &ctx->s_cand2, &ctx->s_flags, &ctx->s_scan, &ctx->s_misc, &ctx->s_counter,
                     &ctx->s_hist, &ctx->g_ua, &ctx->g_ga, &ctx->g_ia, &ctx->g_ub, &ctx->g_gb, &ctx->g_ib,
@@ -380,6 +440,22 @@ extern "C" hci_status hci_build_lists(hci_ctx* ctx) {
   if (L.npair_same > 0)
     HCI_LAUNCH(k_gather_first, (L.npair_same + 255) / 256, 256, 0, ctx->st)(
         bp<double>(L.same_mag), L.npair_same, L.len_same, bp<double>(L.list_max) + n * n);
+  {
+    const int64_t n3 = (int64_t)n * n * n;
+    HCI_TRY(ensure_buf(ctx, L.single_pr, (size_t)n * n * 2));
+    HCI_TRY(ensure_buf(ctx, L.single_bf, (size_t)n * n * 4));
+    HCI_TRY(ensure_buf(ctx, L.single_f32, (size_t)(2 * n3 + 2 * n * n) * 4));
+    const int P = next_pow2(n * n);
+    HCI_CUDA(ctx, cudaFuncSetAttribute(k_sort_singles, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
+    HCI_LAUNCH(k_sort_singles, 1, 1024, (size_t)P * 12, ctx->st)(n, bp<double>(L.single_bound), P,
+                                                                bp<uint16_t>(L.single_pr), bp<float>(L.single_bf));
+    HCI_LAUNCH(k_single_f32, grid_for(2 * n3, 256), 256, 0, ctx->st)(n, bp<double>(ctx->jk_same), bp<double>(ctx->j_opp),
+                                                                    bp<double>(L.f_ref), bp<float>(L.single_f32));
+    HCI_TRY(ensure_buf(ctx, L.single_max, (size_t)n * n * 16));
+    HCI_LAUNCH(k_single_max, (n * n + 127) / 128, 128, 0, ctx->st)(n, bp<uint16_t>(L.single_pr), bp<float>(L.single_f32),
+                                                                  bp<float>(L.single_bf), bp<float4>(L.single_max));
+    HCI_CUDA(ctx, cudaGetLastError());
+  }
   HCI_TRY(ensure_buf(ctx, ctx->s_misc, 64));
   double* dm = bp<double>(ctx->s_misc);
   HCI_CUDA(ctx, cudaMemsetAsync(dm, 0, 64, ctx->st));

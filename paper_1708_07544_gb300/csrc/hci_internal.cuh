@@ -82,9 +82,12 @@ struct Lists {
   int n = 0;
   int len_opp = 0, len_same = 0;     // entries per list
   int npair_same = 0;                // n(n-1)/2
-  DevBuf opp_mag, opp_tgt;           // [n*n][len_opp] double / uint16 (r | s<<8)
+  DevBuf opp_mag, opp_tgt;           // [n*n][len_opp] double / uint16 (r | s<<8 | sign of the element<<15)
   DevBuf same_mag, same_tgt;         // [npair_same][len_same]
   DevBuf single_bound;               // [n*n] upper bound of |H| for single p->r
+  DevBuf single_pr, single_bf;       // [n*n] p | r<<8 by descending bound; the bounds rounded up to FP32
+  DevBuf single_max;                 // float4 [n*n], sorted as single_pr: |F_R| of both spins, largest terms
+  DevBuf single_f32;                 // |jk_same|, |j_opp| [n^3 each] and |f_ref| [2 n^2] rounded up to FP32
   DevBuf list_max;                   // [n*n + npair_same] first (largest) magnitude of each list
   DevBuf f_ref;                      // [2][n][n] single-excitation rows of the aufbau determinant (set at create)
   double max_opp = 0, max_same = 0, max_single = 0;

@@ -32,6 +32,10 @@ struct WalkArgs {
   const double* jk_same;
   const double* j_opp;
   const double* single_bound;
+  const uint16_t* single_pr;       // singles by descending bound, the bounds and the tables of the
+  const float* single_bf;          // tight bound rounded up to FP32
+  const float* single_f32;
+  const float4* single_max;        // per sorted single: |F_R| alpha, beta, largest same- and other-spin term
   double max_single;
   ulonglong2* out;
   int64_t cap;
@@ -65,22 +69,72 @@ __device__ __forceinline__ void tri_decode_dev(int t, int& lo, int& hi) {
   lo = t - h * (h - 1) / 2;
 }
 
-// Warp-aggregated append of one optional key (and term) per lane.
-__device__ __forceinline__ void warp_emit(bool emit, ulonglong2 key, double term, int src, const WalkArgs& A) {
+// Emitted keys (with terms and sources) of a warp, gathered in shared memory
+// and appended 64 or more at a time: an append per 32 tried targets is bound
+// by the one counter's atomic rate (1e7 of them: 5 ms).
+constexpr int EM_CAP = 96, EM_FLUSH = 64;
+struct EmitBuf {
+  ulonglong2 key[EM_CAP];
+  double term[EM_CAP];
+  int32_t src[EM_CAP];
+};
+
+__device__ __forceinline__ void emit_flush(EmitBuf& B, int& cnt, const WalkArgs& A) {
   const int lane = threadIdx.x & 31;
-  unsigned m = __ballot_sync(0xffffffffu, emit);
-  if (!m) return;
+  __syncwarp();
+  if (cnt == 0) return;
   unsigned long long base = 0;
-  if (lane == 0) base = atomicAdd(&A.counter[0], (unsigned long long)__popc(m));
+  if (lane == 0) base = atomicAdd(&A.counter[0], (unsigned long long)cnt);
   base = __shfl_sync(0xffffffffu, base, 0);
-  if (emit) {
-    unsigned long long idx = base + __popc(m & ((1u << lane) - 1u));
+  for (int k = lane; k < cnt; k += 32) {
+    const unsigned long long idx = base + k;
     if ((int64_t)idx < A.cap) {
-      A.out[idx] = key;
-      if (A.vals) A.vals[idx] = term;
-      if (A.srcs) A.srcs[idx] = src;
+      A.out[idx] = B.key[k];
+      if (A.vals) A.vals[idx] = B.term[k];
+      if (A.srcs) A.srcs[idx] = B.src[k];
     }
   }
+  cnt = 0;
+  __syncwarp();
+}
+
+// one optional key (and term) per lane
+__device__ __forceinline__ void warp_emit(bool emit, ulonglong2 key, double term, int src, EmitBuf& B, int& cnt,
+                                          const WalkArgs& A) {
+  const unsigned m = __ballot_sync(0xffffffffu, emit);
+  if (!m) return;
+  if (emit) {
+    const int at = cnt + __popc(m & ((1u << (threadIdx.x & 31)) - 1u));
+    B.key[at] = key;
+    if (A.vals) B.term[at] = term;
+    if (A.srcs) B.src[at] = src;
+  }
+  cnt += __popc(m);
+  if (cnt >= EM_FLUSH) emit_flush(B, cnt, A);
+}
+
+// flip the sign of v for an odd count
+__device__ __forceinline__ double flip_sign(double v, int odd) {
+  return __longlong_as_double(__double_as_longlong(v) ^ ((long long)(odd & 1) << 63));
+}
+// number of set bits of s strictly between orbitals p and r
+__device__ __forceinline__ int bits_between(uint64_t s, int p, int r) {
+  const int lo = p < r ? p : r, hi = p < r ? r : p;
+  return __popcll(s & ((1ull << hi) - 1ull) & ~((2ull << lo) - 1ull));
+}
+
+// The warp's next 32 determinants, one per lane (nV or above: none), or -1
+// at the queue's end.  An atomic per determinant would bound spaces of small
+// coefficients; the 32 lie nV / 32 apart, because determinants of large
+// coefficients are neighbours (32 consecutive ones: 3.9 ms of k_singles where
+// these take 0.3).
+__device__ __forceinline__ int64_t next_dets(const WalkArgs& A) {
+  const int lane = threadIdx.x & 31;
+  const int64_t stride = (A.nV + 31) >> 5;
+  unsigned long long q = 0;
+  if (lane == 0) q = atomicAdd(&A.counter[1], 1ull);
+  q = __shfl_sync(0xffffffffu, q, 0);
+  return (int64_t)q < stride ? (int64_t)q + lane * stride : -1;
 }
 
 // Compact the occupied orbitals of a spin string into smem (ascending).
@@ -97,34 +151,29 @@ __device__ __forceinline__ void occ_list(uint64_t s, int n, int* occ) {
   __syncwarp();
 }
 
-// Largest L with mag[L-1]*absc > eps1 (mag sorted descending).
-__device__ __forceinline__ int prefix_len(const double* __restrict__ mag, int len, double absc, double eps1) {
-  int lo = 0, hi = len;       // invariant: entries [0,lo) pass, [hi,len) fail
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (mag[mid] * absc > eps1) lo = mid + 1;
-    else hi = mid;
-  }
-  return lo;
-}
+// Doubles, planning pass: 32 determinants at a time from a queue (an atomic
+// each would bound a space of small coefficients, most of which the largest
+// element cannot lift over the threshold), one warp per remaining one.  For
+// every occupied pair whose largest element passes in FP32 (maximum and
+// coefficient rounded up, threshold down) the length L of the list prefix
+// with |v||c_i| > eps1 is found by binary search in FP64 (four pairs of a
+// lane side by side: the dependent loads of a single determinant of large
+// coefficient are the kernel's tail), and the prefix is cut into work items of at most WALK_CHUNK entries, so that a determinant
+// with a large coefficient (whose prefixes cover most of the lists) is
+// spread over many warps.
+constexpr int PLAN_ILP = 4;
 
-// Doubles, planning pass: one warp per determinant (dynamic queue).  For
-// every occupied pair the length L of the list prefix with |v||c_i| > eps1
-// is found by binary search, and the prefix is cut into work items of at
-// most WALK_CHUNK entries, so that a determinant with a large coefficient
-// (whose prefixes cover most of the lists) is spread over many warps.
 __global__ void __launch_bounds__(SEL_WARPS * 32) k_walk_plan(WalkArgs A) {
-  // shared: list maxima (n*n + n(n-1)/2 doubles), then the triangular
-  // decode table t -> (lo, hi) of occupied-pair indices (bytes)
-  extern __shared__ double s_dyn[];
+  // shared: list maxima (n*n + n(n-1)/2), then the triangular decode table
+  // t -> (lo, hi) of occupied-pair indices (bytes)
+  extern __shared__ float s_max[];
   __shared__ int s_occ[SEL_WARPS][2][HCI_MAXORB];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int nmax = A.n * A.n + A.n * (A.n - 1) / 2;
-  double* s_max = s_dyn;
-  unsigned char* s_tlo = reinterpret_cast<unsigned char*>(s_dyn + nmax);
+  unsigned char* s_tlo = reinterpret_cast<unsigned char*>(s_max + nmax);
   const int ntri = HCI_MAXORB * (HCI_MAXORB - 1) / 2;
   unsigned char* s_thi = s_tlo + ntri;
-  for (int t = threadIdx.x; t < nmax; t += blockDim.x) s_max[t] = A.list_max[t];
+  for (int t = threadIdx.x; t < nmax; t += blockDim.x) s_max[t] = __double2float_ru(A.list_max[t]);
   for (int t = threadIdx.x; t < ntri; t += blockDim.x) {
     int lo, hi;
     tri_decode_dev(t, lo, hi);
@@ -137,76 +186,109 @@ __global__ void __launch_bounds__(SEL_WARPS * 32) k_walk_plan(WalkArgs A) {
   const int Paa = A.na * (A.na - 1) / 2, Pbb = A.nb * (A.nb - 1) / 2, Pab = A.na * A.nb;
   const int P = Paa + Pbb + Pab;
   const int nn = A.n * A.n;
+  const float epsf = __double2float_rd(A.eps1);
+  unsigned long long walked = 0;
   while (true) {
-    unsigned long long i = 0;
-    if (lane == 0) i = atomicAdd(&A.counter[1], 1ull);
-    i = __shfl_sync(0xffffffffu, i, 0);
-    if ((int64_t)i >= A.nV) break;
-    const double absc = fabs(A.c[i]);
-    if (!A.accept_all && !(A.max_dbl * absc > A.eps1)) continue;
-    const ulonglong2 k = A.keys[i];
-    occ_list(k.x, A.n, occA);
-    occ_list(k.y, A.n, occB);
-    for (int base = 0; base < P; base += 32) {
-      int t = base + lane;
-      int kind = -1, p = 0, q = 0, L = 0;
-      int listid = 0;
-      if (t < P) {
-        int len;
-        double first;
-        const double* mag;
-        if (t < Paa) {
-          p = occA[s_tlo[t]]; q = occA[s_thi[t]]; kind = 0;
-          listid = q * (q - 1) / 2 + p;
-          first = s_max[nn + listid];
-          mag = A.same_mag + (int64_t)listid * A.Ls; len = A.Ls;
-        } else if (t < Paa + Pbb) {
-          p = occB[s_tlo[t - Paa]]; q = occB[s_thi[t - Paa]]; kind = 1;
-          listid = q * (q - 1) / 2 + p;
-          first = s_max[nn + listid];
-          mag = A.same_mag + (int64_t)listid * A.Ls; len = A.Ls;
-        } else {
-          int u = t - Paa - Pbb;
-          p = occA[u / A.nb]; q = occB[u % A.nb]; kind = 2;
-          listid = p * A.n + q;
-          first = s_max[listid];
-          mag = A.opp_mag + (int64_t)listid * A.Lo; len = A.Lo;
+    const int64_t i_l = next_dets(A);
+    if (i_l < 0) break;
+    const double absc_l = i_l < A.nV ? fabs(A.c[i_l]) : 0.0;
+    unsigned go = __ballot_sync(0xffffffffu, i_l < A.nV && (A.accept_all || A.max_dbl * absc_l > A.eps1));
+    while (go) {
+      const int from = __ffs(go) - 1;
+      go &= go - 1;
+      const int64_t i = __shfl_sync(0xffffffffu, i_l, from);
+      const double absc = __shfl_sync(0xffffffffu, absc_l, from);
+      const float cf = __double2float_ru(absc);
+      const ulonglong2 k = A.keys[i];
+      __syncwarp();
+      occ_list(k.x, A.n, occA);
+      occ_list(k.y, A.n, occB);
+      for (int base = 0; base < P; base += 32 * PLAN_ILP) {
+        int code[PLAN_ILP], L[PLAN_ILP], hi[PLAN_ILP];
+        const double* mag[PLAN_ILP];
+#pragma unroll
+        for (int u = 0; u < PLAN_ILP; ++u) {
+          const int t = base + 32 * u + lane;
+          int kind = 0, p = 0, q = 0, listid = 0;
+          L[u] = hi[u] = 0;
+          mag[u] = A.opp_mag;
+          if (t < P) {
+            int len;
+            float first;
+            if (t < Paa + Pbb) {
+              const bool al = t < Paa;
+              const int u2 = al ? t : t - Paa;
+              const int* occ = al ? occA : occB;
+              kind = al ? 0 : 1;
+              p = occ[s_tlo[u2]]; q = occ[s_thi[u2]];
+              listid = q * (q - 1) / 2 + p;
+              first = s_max[nn + listid];
+              mag[u] = A.same_mag + (int64_t)listid * A.Ls; len = A.Ls;
+            } else {
+              const int u2 = t - Paa - Pbb;
+              p = occA[u2 / A.nb]; q = occB[u2 % A.nb]; kind = 2;
+              listid = p * A.n + q;
+              first = s_max[listid];
+              mag[u] = A.opp_mag + (int64_t)listid * A.Lo; len = A.Lo;
+            }
+            if (A.accept_all) L[u] = hi[u] = len;
+            else if (__fmul_ru(first, cf) > epsf) hi[u] = len;
+          }
+          code[u] = kind | (p << 2) | (q << 8) | (listid << 14);
         }
-        if (A.accept_all) L = len;
-        else if (first * absc > A.eps1) L = prefix_len(mag, len, absc, A.eps1);
-      }
-      {
-        unsigned long long tot = (unsigned long long)L;
-        for (int o = 16; o; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-        if (lane == 0 && tot) atomicAdd(&A.walkstat[0], tot);
-      }
-      // work items of at most WALK_CHUNK entries (det, kind|p|q|list, start, end)
-      int nit = L > 0 ? (L + WALK_CHUNK - 1) / WALK_CHUNK : 0;
-      int incl = nit;
-      for (int o = 1; o < 32; o <<= 1) {
-        int t2 = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t2;
-      }
-      const int tot_it = __shfl_sync(0xffffffffu, incl, 31);
-      if (tot_it > 0) {
-        unsigned long long base = 0;
-        if (lane == 31) base = atomicAdd(A.nitems, (unsigned long long)tot_it);
-        base = __shfl_sync(0xffffffffu, base, 31);
-        const int code = kind | (p << 2) | (q << 8) | (listid << 14);
-        for (int j = 0; j < nit; ++j) {
-          const unsigned long long idx = base + (incl - nit) + j;
-          if ((int64_t)idx < A.item_cap)
-            A.items[idx] = make_int4((int)i, code, j * WALK_CHUNK, min(L, (j + 1) * WALK_CHUNK));
+        // the searches side by side: entries [0, L) pass, [hi, len) fail
+        while (true) {
+          bool more = false;
+#pragma unroll
+          for (int u = 0; u < PLAN_ILP; ++u) more = more || L[u] < hi[u];
+          if (!more) break;
+          double v[PLAN_ILP];
+#pragma unroll
+          for (int u = 0; u < PLAN_ILP; ++u) v[u] = L[u] < hi[u] ? mag[u][(L[u] + hi[u]) >> 1] : 0.0;
+#pragma unroll
+          for (int u = 0; u < PLAN_ILP; ++u)
+            if (L[u] < hi[u]) {
+              const int mid = (L[u] + hi[u]) >> 1;
+              if (v[u] * absc > A.eps1) L[u] = mid + 1;
+              else hi[u] = mid;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < PLAN_ILP; ++u) {
+          walked += L[u];
+          // work items of at most WALK_CHUNK entries (det, kind|p|q|list, start, end)
+          const int nit = (L[u] + WALK_CHUNK - 1) / WALK_CHUNK;
+          if (!__any_sync(0xffffffffu, nit > 0)) continue;
+          int incl = nit;
+          for (int o = 1; o < 32; o <<= 1) {
+            int t2 = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t2;
+          }
+          unsigned long long base_it = 0;
+          if (lane == 31) base_it = atomicAdd(A.nitems, (unsigned long long)incl);
+          base_it = __shfl_sync(0xffffffffu, base_it, 31);
+          for (int j = 0; j < nit; ++j) {
+            const unsigned long long idx = base_it + (incl - nit) + j;
+            if ((int64_t)idx < A.item_cap)
+              A.items[idx] = make_int4((int)i, code[u], j * WALK_CHUNK, min(L[u], (j + 1) * WALK_CHUNK));
+          }
         }
       }
     }
   }
+  for (int o = 16; o; o >>= 1) walked += __shfl_xor_sync(0xffffffffu, walked, o);
+  if (lane == 0 && walked) atomicAdd(&A.walkstat[0], walked);
 }
 
 // Walk the planned list ranges: one warp per work item; every target whose
-// orbitals are empty in the source determinant is emitted.
+// orbitals are empty in the source determinant is emitted.  In perturbative
+// mode the element is the list's magnitude with the sign kept beside the
+// target and the determinant's two phases, one FP64 product per target.
 __global__ void __launch_bounds__(SEL_WARPS * 32) k_walk_exec(WalkArgs A, int64_t nitems) {
+  __shared__ EmitBuf s_emit[SEL_WARPS];
   const int lane = threadIdx.x & 31;
+  EmitBuf& B = s_emit[threadIdx.x >> 5];
+  int cnt = 0;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t it = warp; it < nitems; it += nwarps) {
@@ -214,8 +296,8 @@ __global__ void __launch_bounds__(SEL_WARPS * 32) k_walk_exec(WalkArgs A, int64_
     const ulonglong2 k = A.keys[w.x];
     const int sk = w.y & 3, sp = (w.y >> 2) & 63, sq = (w.y >> 8) & 63, sl = w.y >> 14;
     const uint16_t* tg = sk == 2 ? A.opp_tgt + (int64_t)sl * A.Lo : A.same_tgt + (int64_t)sl * A.Ls;
+    const double* mg = sk == 2 ? A.opp_mag + (int64_t)sl * A.Lo : A.same_mag + (int64_t)sl * A.Ls;
     const double ci = A.vals ? A.c[w.x] : 0.0;
-    const int64_t n = A.n;
     for (int k0 = w.z; k0 < w.w; k0 += 32) {
       const int e = k0 + lane;
       bool emit = false;
@@ -223,167 +305,223 @@ __global__ void __launch_bounds__(SEL_WARPS * 32) k_walk_exec(WalkArgs A, int64_
       double term = 0.0, elem = 0.0;
       if (e < w.w) {
         const uint16_t tt = tg[e];
-        const int r = tt & 0xff, s2 = tt >> 8;
-        if (sk == 0) {
-          if (!((k.x >> r) & 1ull) && !((k.x >> s2) & 1ull)) {
-            emit = true;
-            key.x = k.x ^ (1ull << sp) ^ (1ull << sq) ^ (1ull << r) ^ (1ull << s2);
+        const int r = tt & 63, s2 = (tt >> 8) & 63;
+        const uint64_t sa = sk == 1 ? k.y : k.x, sb = sk == 0 ? k.x : k.y;   // strings of p -> r and q -> s
+        emit = !((sa >> r) & 1ull) && !((sb >> s2) & 1ull);
+        if (emit) {
+          const uint64_t ma = (1ull << sp) ^ (1ull << r), mb = (1ull << sq) ^ (1ull << s2);
+          if (sk != 1) key.x ^= sk == 0 ? ma ^ mb : ma;
+          if (sk != 0) key.y ^= sk == 1 ? ma ^ mb : mb;
+          if (A.vals) {
+            // signed <D_a|H|D_i> (same rule as the graph's elements), times c_i
+            const int odd = bits_between(sa, sp, r) + bits_between(sk == 2 ? sb : sa ^ ma, sq, s2) + (tt >> 15);
+            elem = flip_sign(mg[e], odd);
+            term = elem * ci;
+            emit = pt_keep(A, key, term);
           }
-        } else if (sk == 1) {
-          if (!((k.y >> r) & 1ull) && !((k.y >> s2) & 1ull)) {
-            emit = true;
-            key.y = k.y ^ (1ull << sp) ^ (1ull << sq) ^ (1ull << r) ^ (1ull << s2);
-          }
-        } else {
-          if (!((k.x >> r) & 1ull) && !((k.y >> s2) & 1ull)) {
-            emit = true;
-            key.x = k.x ^ (1ull << sp) ^ (1ull << r);
-            key.y = k.y ^ (1ull << sq) ^ (1ull << s2);
-          }
-        }
-        if (emit && A.vals) {
-          // signed <D_a|H|D_i> (same rule as the graph's elements), times c_i
-          double v;
-          if (sk == 2) {
-            v = exc_phase(k.x, sp, r) * exc_phase(k.y, sq, s2) * A.eri[((sp * n + r) * n + sq) * n + s2];
-          } else {
-            const uint64_t s0 = sk == 0 ? k.x : k.y;
-            const double ph = exc_phase(s0, sp, r) * exc_phase(s0 ^ (1ull << sp) ^ (1ull << r), sq, s2);
-            v = ph * (A.eri[((sp * n + r) * n + sq) * n + s2] - A.eri[((sp * n + s2) * n + sq) * n + r]);
-          }
-          term = v * ci;
-          elem = v;
-          emit = pt_keep(A, key, term);
         }
       }
-      warp_emit(emit, key, A.srcs ? elem : term, w.x, A);
+      warp_emit(emit, key, A.srcs ? elem : term, w.x, B, cnt, A);
     }
   }
+  emit_flush(B, cnt, A);
 }
 
-// Bound on |H_ai| of the single p->r (spin S) of a determinant D from the
-// aufbau reference R: H = F_R + sum over the orbitals where D and R differ of
-// +-(pr|kk)-(pk|kr) (same spin) or +-(pr|kk) (other spin), so |H| is at most
-// |F_R| plus the absolute values of those few terms; the margin covers the
-// rounding of both sums (at most 2n+1 terms bounded by the loose bound B).
-__device__ __forceinline__ double single_tight(const WalkArgs& A, int spin, int p, int r, uint64_t s, uint64_t o,
-                                               double B) {
+// Upper bound, in FP32 rounded up, of |H_ai| of the single p->r (spin S) of
+// a determinant D from the aufbau reference R: H = F_R + sum over the
+// orbitals where D and R differ of +-(pr|kk)-(pk|kr) (same spin) or +-(pr|kk)
+// (other spin), so |H| is at most |F_R| plus the absolute values of those few
+// terms; the margins cover the rounding of both FP64 sums (at most 2n+1
+// terms bounded by the loose bound).
+__device__ __forceinline__ float single_tight(const WalkArgs& A, int spin, int p, int r, uint64_t s, uint64_t o) {
   const int n = A.n;
   const uint64_t ds = s ^ (spin == 0 ? A.ref_a : A.ref_b);
   const uint64_t dot = o ^ (spin == 0 ? A.ref_b : A.ref_a);
-  const double* js = A.jk_same + ((int64_t)p * n + r) * n;
-  const double* jo = A.j_opp + ((int64_t)p * n + r) * n;
-  double t = fabs(A.f_ref[((int64_t)spin * n + p) * n + r]);
-  uint64_t x = ds;
-  while (x) {
-    const int k = __ffsll((long long)x) - 1;
-    x &= x - 1;
-    t += fabs(js[k]);
-  }
-  x = dot;
-  while (x) {
-    const int k = __ffsll((long long)x) - 1;
-    x &= x - 1;
-    t += fabs(jo[k]);
-  }
-  return (t + 1e-13 * B) * (1.0 + 1e-12);
+  const int64_t n3 = (int64_t)n * n * n;
+  const float* js = A.single_f32 + ((int64_t)p * n + r) * n;
+  const float* jo = js + n3;
+  float t = A.single_f32[2 * n3 + ((int64_t)spin * n + p) * n + r];
+  for (uint64_t x = ds; x; x &= x - 1) t = __fadd_ru(t, js[__ffsll((long long)x) - 1]);
+  for (uint64_t x = dot; x; x &= x - 1) t = __fadd_ru(t, jo[__ffsll((long long)x) - 1]);
+  t = __fadd_ru(t, __fmul_ru(2e-13f, __double2float_ru(A.single_bound[p * n + r])));
+  return __fmul_ru(t, 1.000002f);
 }
 
-// Singles: one warp per determinant; each lane screens (p->r) with the
-// determinant-independent bound, then evaluates H_ai exactly in the same
-// summation order as the textbook rule (k ascending, same spin then
-// opposite spin per k).
+// Singles.  FP64 operations bound this kernel (64 cycles of a sub-partition
+// each, whatever the active lanes), so they are left to the few singles that
+// need them, 32 at a time:
+//  1. 32 determinants from the queue; each one's prefix of the singles sorted
+//     by their determinant-independent bound (FP32, bound and coefficient
+//     rounded up); the prefix's singles that are occupied -> empty are queued;
+//  2. queued singles against the determinant's own bound (single_tight);
+//  3. the rest in FP64: in selection exactly, in the summation order of the
+//     textbook rule (k ascending, same spin then opposite spin per k), so
+//     that decisions are bit-identical to it; in perturbative mode from the
+//     aufbau value plus the orbitals where the strings differ.
+// The queues (per warp) run on from one determinant to the next.  (44e,44o),
+// 4.1e5 determinants at eps1 = 1.5e-4: 914 us with one determinant per warp
+// and FP64 bounds, 439 us so.
+constexpr int SQ_CAP = 64;
+
 __global__ void __launch_bounds__(SEL_WARPS * 32) k_singles(WalkArgs A) {
-  extern __shared__ double s_bound[];          // n*n single-excitation bounds
-  __shared__ int s_ov[SEL_WARPS][2][2][HCI_MAXORB];   // [warp][spin][occ/vir][]
+  extern __shared__ float s_bf[];              // n*n bounds, then the n*n packed singles
+  __shared__ EmitBuf s_emit[SEL_WARPS];
+  __shared__ uint64_t s_q1[SEL_WARPS][SQ_CAP], s_q2[SEL_WARPS][SQ_CAP];   // determinant << 20 | spin << 16 | r << 8 | p
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int n = A.n;
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) s_bound[t] = A.single_bound[t];
+  const unsigned lt = (1u << lane) - 1u;
+  const int n = A.n, nn = n * n;
+  uint16_t* s_pr = reinterpret_cast<uint16_t*>(s_bf + nn);
+  for (int t = threadIdx.x; t < nn; t += blockDim.x) {
+    s_bf[t] = A.single_bf[t];
+    s_pr[t] = A.single_pr[t];
+  }
   __syncthreads();
-  const int Pa = A.na * (n - A.na), Pb = A.nb * (n - A.nb);
-  const int P = Pa + Pb;
-  while (true) {
-    unsigned long long i = 0;
-    if (lane == 0) i = atomicAdd(&A.counter[1], 1ull);
-    i = __shfl_sync(0xffffffffu, i, 0);
-    if ((int64_t)i >= A.nV) break;
-    const double absc = fabs(A.c[i]);
-    if (!A.accept_all && !(A.max_single * absc > A.eps1)) continue;
-    const ulonglong2 k = A.keys[i];
-    for (int sp = 0; sp < 2; ++sp) {
-      const uint64_t x = sp == 0 ? k.x : k.y;
-      int bo = 0, bv = 0;
-      for (int p0 = 0; p0 < n; p0 += 32) {
-        const int pp = p0 + lane;
-        const bool in = pp < n;
-        const bool o = in && ((x >> pp) & 1ull);
-        const unsigned mo = __ballot_sync(0xffffffffu, o);
-        const unsigned mv = __ballot_sync(0xffffffffu, in && !o);
-        const unsigned lt = (1u << lane) - 1u;
-        if (o) s_ov[w][sp][0][bo + __popc(mo & lt)] = pp;
-        if (in && !o) s_ov[w][sp][1][bv + __popc(mv & lt)] = pp;
-        bo += __popc(mo);
-        bv += __popc(mv);
+  EmitBuf& B = s_emit[w];
+  uint64_t* q1 = s_q1[w];
+  uint64_t* q2 = s_q2[w];
+  int cnt = 0, n1 = 0, n2 = 0;
+  unsigned long long exact = 0;
+  const float epsf = __double2float_rd(A.eps1);
+
+  // the first m <= 32 entries of q2 evaluated
+  auto evaluate = [&](int m) {
+    __syncwarp();
+    bool emit = false;
+    ulonglong2 key = make_ulonglong2(0, 0);
+    double term = 0.0, elem = 0.0;
+    int64_t i = 0;
+    if (lane < m) {
+      const uint64_t q = q2[lane];
+      const int p = (int)(q & 63), r = (int)((q >> 8) & 63), spin = (int)((q >> 16) & 1);
+      i = (int64_t)(q >> 20);
+      key = A.keys[i];
+      const uint64_t s = spin == 0 ? key.x : key.y, o = spin == 0 ? key.y : key.x;
+      const double* js = A.jk_same + ((int64_t)p * n + r) * n;
+      const double* jo = A.j_opp + ((int64_t)p * n + r) * n;
+      double v;
+      if (A.vals) {
+        const uint64_t rs = spin == 0 ? A.ref_a : A.ref_b, ro = spin == 0 ? A.ref_b : A.ref_a;
+        v = A.f_ref[((int64_t)spin * n + p) * n + r];
+        for (uint64_t mm = s & ~rs; mm; mm &= mm - 1) v += js[__ffsll((long long)mm) - 1];
+        for (uint64_t mm = rs & ~s; mm; mm &= mm - 1) v -= js[__ffsll((long long)mm) - 1];
+        for (uint64_t mm = o & ~ro; mm; mm &= mm - 1) v += jo[__ffsll((long long)mm) - 1];
+        for (uint64_t mm = ro & ~o; mm; mm &= mm - 1) v -= jo[__ffsll((long long)mm) - 1];
+        elem = flip_sign(v, bits_between(s, p, r));
+        term = elem * A.c[i];
+        emit = true;
+      } else {
+        v = A.h[p * n + r];
+#pragma unroll 4
+        for (int x = 0; x < n; ++x) {
+          if ((s >> x) & 1ull) v += js[x];
+          if ((o >> x) & 1ull) v += jo[x];
+        }
+        emit = fabs(v) * fabs(A.c[i]) > A.eps1;
+      }
+      const uint64_t flip = (1ull << p) ^ (1ull << r);
+      if (spin == 0) key.x ^= flip;
+      else key.y ^= flip;
+      if (A.vals) emit = pt_keep(A, key, term);
+    }
+    if (!A.vals) exact += m;
+    warp_emit(emit, key, A.srcs ? elem : term, (int)i, B, cnt, A);
+    // the entries behind move to the front
+    __syncwarp();
+    const uint64_t q = lane + m < n2 ? q2[lane + m] : 0;
+    __syncwarp();
+    if (lane + m < n2) q2[lane] = q;
+    n2 -= m;
+    __syncwarp();
+  };
+  // the first m <= 32 entries of q1 against their own bounds
+  auto screen = [&](int m) {
+    __syncwarp();
+    bool pass = false;
+    uint64_t q = 0;
+    if (lane < m) {
+      q = q1[lane];
+      pass = true;
+      if (!A.accept_all) {
+        const int p = (int)(q & 63), r = (int)((q >> 8) & 63), spin = (int)((q >> 16) & 1);
+        const int64_t i = (int64_t)(q >> 20);
+        const ulonglong2 k = A.keys[i];
+        const float t = single_tight(A, spin, p, r, spin == 0 ? k.x : k.y, spin == 0 ? k.y : k.x);
+        pass = __fmul_ru(t, __double2float_ru(fabs(A.c[i]))) > epsf;
       }
     }
+    const unsigned b = __ballot_sync(0xffffffffu, pass);
+    if (pass) q2[n2 + __popc(b & lt)] = q;
+    n2 += __popc(b);
+    if (n2 >= 32) evaluate(32);
     __syncwarp();
-    for (int base = 0; base < P; base += 32) {
-      int t = base + lane;
-      bool emit = false, exact = false;
-      ulonglong2 key = k;
-      double term = 0.0, elem = 0.0;
-      if (t < P) {
-        int spin = t < Pa ? 0 : 1;
-        int u = spin == 0 ? t : t - Pa;
-        uint64_t s = spin == 0 ? k.x : k.y;
-        uint64_t o = spin == 0 ? k.y : k.x;
-        int nocc = spin == 0 ? A.na : A.nb;
-        int nvirt = n - nocc;
-        const int p = s_ov[w][spin][0][u / nvirt], r = s_ov[w][spin][1][u % nvirt];
-        if (A.accept_all && !A.vals) {
-          emit = true;
-        } else if (A.vals) {
-          // perturbative mode: the element from the aufbau value plus the
-          // orbitals where the strings differ (no bit-exact decision needed)
-          if (A.accept_all || s_bound[p * n + r] * absc > A.eps1) {
-            const uint64_t rs = spin == 0 ? A.ref_a : A.ref_b, ro = spin == 0 ? A.ref_b : A.ref_a;
-            const double* js = A.jk_same + ((int64_t)p * n + r) * n;
-            const double* jo = A.j_opp + ((int64_t)p * n + r) * n;
-            double v = A.f_ref[((int64_t)spin * n + p) * n + r];
-            for (uint64_t mm = s & ~rs; mm; mm &= mm - 1) v += js[__ffsll((long long)mm) - 1];
-            for (uint64_t mm = rs & ~s; mm; mm &= mm - 1) v -= js[__ffsll((long long)mm) - 1];
-            for (uint64_t mm = o & ~ro; mm; mm &= mm - 1) v += jo[__ffsll((long long)mm) - 1];
-            for (uint64_t mm = ro & ~o; mm; mm &= mm - 1) v -= jo[__ffsll((long long)mm) - 1];
-            elem = exc_phase(s, p, r) * v;
-            term = elem * A.c[i];
-            emit = true;
-          }
-        } else if (A.accept_all || (s_bound[p * n + r] * absc > A.eps1 &&
-                                    single_tight(A, spin, p, r, s, o, s_bound[p * n + r]) * absc > A.eps1)) {
-          exact = true;
-          double v = A.h[p * n + r];
-          const double* js = A.jk_same + ((int64_t)p * n + r) * n;
-          const double* jo = A.j_opp + ((int64_t)p * n + r) * n;
-          for (int x = 0; x < n; ++x) {
-            if ((s >> x) & 1ull) v += js[x];
-            if ((o >> x) & 1ull) v += jo[x];
-          }
-          emit = fabs(v) * absc > A.eps1;
-          elem = exc_phase(s, p, r) * v;
-          term = elem * A.c[i];
+    const uint64_t rest = lane + m < n1 ? q1[lane + m] : 0;
+    __syncwarp();
+    if (lane + m < n1) q1[lane] = rest;
+    n1 -= m;
+    __syncwarp();
+  };
+
+  while (true) {
+    const int64_t i_l = next_dets(A);
+    if (i_l < 0) break;
+    const bool in = i_l < A.nV;
+    int len = 0;                                 // singles of this lane's determinant to look at
+    if (in) {
+      if (A.accept_all) {
+        len = nn;
+      } else {
+        const float cf = __double2float_ru(fabs(A.c[i_l]));
+        int lo = 0, hi = nn;
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (__fmul_ru(s_bf[mid], cf) > epsf) lo = mid + 1;
+          else hi = mid;
         }
-        if (emit) {
-          uint64_t ns = s ^ (1ull << p) ^ (1ull << r);
-          if (spin == 0) key.x = ns; else key.y = ns;
-          if (A.vals) emit = pt_keep(A, key, term);
+        len = lo;
+      }
+    }
+    unsigned go = __ballot_sync(0xffffffffu, len > 0);
+    while (go) {
+      const int from = __ffs(go) - 1;
+      go &= go - 1;
+      const uint64_t i = (uint64_t)__shfl_sync(0xffffffffu, i_l, from);
+      const int L = __shfl_sync(0xffffffffu, len, from);
+      const ulonglong2 k = A.keys[i];
+      const float cf = __double2float_ru(fabs(A.c[i]));
+      const float da = (float)__popcll(k.x ^ A.ref_a), db = (float)__popcll(k.y ^ A.ref_b);
+      for (int e0 = 0; e0 < L; e0 += 32) {
+        const int e = e0 + lane;
+        const int pr = e < L ? s_pr[e] : 0;
+        const float4 mx = e < L ? A.single_max[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const int p = pr & 63, r = pr >> 8;
+#pragma unroll
+        for (int spin = 0; spin < 2; ++spin) {
+          const uint64_t s = spin == 0 ? k.x : k.y;
+          bool ok = e < L && ((s >> p) & 1ull) && !((s >> r) & 1ull);
+          if (!A.accept_all) {
+            const float t = __fmaf_ru(spin == 0 ? da : db, mx.z, __fmaf_ru(spin == 0 ? db : da, mx.w, spin == 0 ? mx.x : mx.y));
+            ok = ok && __fmul_ru(t, cf) > epsf;
+          }
+          const unsigned b = __ballot_sync(0xffffffffu, ok);
+          if (A.accept_all && !A.vals) {
+            ulonglong2 key = k;
+            const uint64_t flip = (1ull << p) ^ (1ull << r);
+            if (spin == 0) key.x ^= flip;
+            else key.y ^= flip;
+            warp_emit(ok, key, 0.0, (int)i, B, cnt, A);
+          } else if (b) {
+            if (ok) q1[n1 + __popc(b & lt)] = (i << 20) | ((uint64_t)spin << 16) | (uint64_t)pr;
+            n1 += __popc(b);
+            if (n1 >= 32) screen(32);
+          }
         }
       }
-      // exact evaluations counted once per warp (one atomic, not 32)
-      const unsigned mex = __ballot_sync(0xffffffffu, exact);
-      if (lane == 0 && mex) atomicAdd(&A.walkstat[1], (unsigned long long)__popc(mex));
-      warp_emit(emit, key, A.srcs ? elem : term, (int)i, A);
     }
   }
+  if (n1 > 0) screen(n1);
+  if (n2 > 0) evaluate(n2);
+  emit_flush(B, cnt, A);
+  if (lane == 0 && exact) atomicAdd(&A.walkstat[1], exact);
 }
 
 __device__ __forceinline__ bool key_less(ulonglong2 a, ulonglong2 b) {
@@ -461,7 +599,7 @@ static hci_status run_walk(hci_ctx* ctx, WalkArgs& A, int64_t* total) {
   prof_tic(ctx, HCI_PH_WALK);
   HCI_CUDA(ctx, cudaMemsetAsync(A.counter, 0, 16, ctx->st));
   const int grid = ctx->nsm * 8;
-  const size_t smw = (size_t)(A.n * A.n + A.n * (A.n - 1) / 2) * 8 + HCI_MAXORB * (HCI_MAXORB - 1);
+  const size_t smw = (size_t)(A.n * A.n + A.n * (A.n - 1) / 2) * 4 + HCI_MAXORB * (HCI_MAXORB - 1);
   HCI_CUDA(ctx, cudaFuncSetAttribute(k_walk_plan, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
   for (int attempt = 0; attempt < 2; ++attempt) {
     HCI_TRY(ensure_buf(ctx, ctx->s_items, (size_t)(ctx->s_items.bytes > 0 ? ctx->s_items.bytes : (1 << 20) * 16)));
@@ -485,7 +623,7 @@ static hci_status run_walk(hci_ctx* ctx, WalkArgs& A, int64_t* total) {
   prof_tic(ctx, HCI_PH_SINGLES);
   HCI_CUDA(ctx, cudaMemsetAsync(A.counter + 1, 0, 8, ctx->st));
   HCI_CUDA(ctx, cudaFuncSetAttribute(k_singles, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
-  HCI_LAUNCH(k_singles, grid, SEL_WARPS * 32, (size_t)A.n * A.n * 8, ctx->st)(A);
+  HCI_LAUNCH(k_singles, grid, SEL_WARPS * 32, (size_t)A.n * A.n * 6, ctx->st)(A);
   HCI_CUDA(ctx, cudaGetLastError());
   prof_toc(ctx, HCI_PH_SINGLES);
   unsigned long long cnt = 0, ws[2] = {0, 0};
@@ -521,6 +659,8 @@ extern "C" hci_status hci_select(hci_ctx* ctx, double eps1, const uint64_t* keys
   A.max_dbl = L.max_opp > L.max_same ? L.max_opp : L.max_same;
   A.h = bp<double>(ctx->h); A.jk_same = bp<double>(ctx->jk_same); A.j_opp = bp<double>(ctx->j_opp);
   A.single_bound = bp<double>(L.single_bound); A.max_single = L.max_single;
+  A.single_pr = bp<uint16_t>(L.single_pr); A.single_bf = bp<float>(L.single_bf);
+  A.single_f32 = bp<float>(L.single_f32); A.single_max = bp<float4>(L.single_max);
   A.list_max = bp<double>(L.list_max);
   A.f_ref = bp<double>(L.f_ref);
   A.ref_a = ctx->na == 64 ? ~0ull : ((1ull << ctx->na) - 1ull);
@@ -831,6 +971,8 @@ static hci_status pt_walk_args(hci_ctx* ctx, WalkArgs& A, const uint64_t* keys, 
   A.max_dbl = L.max_opp > L.max_same ? L.max_opp : L.max_same;
   A.h = bp<double>(ctx->h); A.jk_same = bp<double>(ctx->jk_same); A.j_opp = bp<double>(ctx->j_opp);
   A.single_bound = bp<double>(L.single_bound); A.max_single = L.max_single;
+  A.single_pr = bp<uint16_t>(L.single_pr); A.single_bf = bp<float>(L.single_bf);
+  A.single_f32 = bp<float>(L.single_f32); A.single_max = bp<float4>(L.single_max);
   A.list_max = bp<double>(L.list_max);
   A.f_ref = bp<double>(L.f_ref);
   A.ref_a = ctx->na == 64 ? ~0ull : ((1ull << ctx->na) - 1ull);

@@ -1,0 +1,63 @@
+"""Selection and screened pairs at the edges of the 32-wide queues of the walk
+and of the singles (32 determinants fetched at a time, 32 queued singles
+evaluated at a time), with coefficients over six orders of magnitude, zeros
+among them, and more than 32 orbitals: the selected set against the oracle's
+enumeration, bit for bit but for its listed ties, and E2 with its pairs."""
+import numpy as np
+import pytest
+import torch
+
+import hci_inputs as hi
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def _problem(norb, na, nb, nV):
+    inst = hi.random_tiny(norb, na, nb, 100 + norb)
+    keys = hi.random_det_keys(norb, na, nb, nV, nV + 3)
+    rng = np.random.default_rng(nV)
+    c = rng.choice([-1.0, 1.0], len(keys)) * 10.0 ** rng.uniform(-6, 0, len(keys))
+    c[:: 7] = 0.0
+    c[len(keys) // 2] = 0.5
+    return inst, keys, c
+
+
+def _dev(a):
+    return torch.tensor(np.ascontiguousarray(a).astype(np.int64) if a.dtype == np.uint64 else a, device="cuda")
+
+
+def _solver(inst):
+    import paper_1708_07544_gb300 as pkg
+
+    return pkg.HCISolver(inst.norb, inst.nalpha, inst.nbeta, _dev(inst.h), _dev(inst.eri), inst.e_core)
+
+
+SPACES = [(12, 6, 5, 1), (12, 6, 5, 31), (12, 6, 5, 32), (12, 6, 5, 33), (12, 6, 5, 65), (12, 6, 5, 1025), (33, 3, 2, 40),
+          (40, 1, 0, 20), (9, 9, 4, 12), (9, 0, 4, 12)]
+
+
+@pytest.mark.parametrize("space", SPACES)
+@pytest.mark.parametrize("eps1", [1e-4, 2e-2, 10.0])
+def test_selection(space, eps1):
+    inst, keys, c = _problem(*space)
+    want, _, ties = oracle.select(inst, keys, c, eps1)
+    with _solver(inst) as s:
+        got = s.select(eps1, _dev(keys), _dev(c)).cpu().numpy().view(np.uint64).reshape(-1, 2)
+    as_set = lambda k: set(map(tuple, np.asarray(k).tolist()))  # noqa: E731
+    assert as_set(got) - as_set(ties) == as_set(want) - as_set(ties)
+    assert len(as_set(got)) == len(got)
+
+
+@pytest.mark.parametrize("space", SPACES)
+@pytest.mark.parametrize("eps2", [1e-3, 0.0, -1.0])
+def test_screened_pairs(space, eps2):
+    inst, keys, c = _problem(*space)
+    if space[0] > 30 and eps2 <= 0.0:
+        pytest.skip("every pair of many orbitals")
+    e0 = float(oracle.diag(inst, keys).min()) - 60.0
+    e2, n = oracle.pt2(inst, keys, c, eps2, e0)
+    with _solver(inst) as s:
+        got = s.pt2(_dev(keys), _dev(c), eps2, e0)
+    assert got[1] == n
+    assert abs(got[0] - e2) <= 1e-11 * max(abs(e2), 1e-12)
