@@ -204,10 +204,10 @@ int64_t hci_fail_alloc_env();
 
 // Quarter transform of the integral rotation, out[J][p] = sum_a in[a][J]
 // M[a][p] for J < n^3 (qtrans_tc.cu): exact digit products on the bf16
-// tensor cores, rounded once to FP64.  qtrans_tc_check() reports (and
-// clears) a launch on stream st that gave up waiting for its products (it
-// reads a device flag on st and synchronises st).
-hci_status qtrans_tc(cudaStream_t st, int n, const double* in, const double* M, double* out);
+// tensor cores, rounded once to FP64.  A launch that gives up waiting for its
+// products sets *timeout (device), or with NULL a flag that qtrans_tc_check()
+// reports and clears (it reads the flag on st and synchronises st).
+hci_status qtrans_tc(cudaStream_t st, int n, const double* in, const double* M, double* out, int* timeout);
 hci_status qtrans_tc_check(cudaStream_t st);
 
 inline int grid_for(int64_t work, int block, int max_blocks = -1) {

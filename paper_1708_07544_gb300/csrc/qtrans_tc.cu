@@ -58,8 +58,8 @@ constexpr int QTC_S = 7;          // balanced base-256 digits per operand entry
 constexpr int QTC_TMEM_COLS = 512;
 constexpr long QTC_WAIT_LIMIT = 1L << 20;   // mbarrier polls before giving up
 
-// set when a CTA gave up waiting for its products (never expected); read
-// and cleared by the host after the rotation's final synchronisation
+// set when a CTA of a launch without a flag of its own gave up waiting for
+// its products (never expected); read and cleared by qtrans_tc_check
 __device__ int g_qtc_timeout;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -270,7 +270,7 @@ __device__ __forceinline__ void issue_products(uint32_t tmem, uint32_t As_a, uin
 template <int NP>
 __global__ void __launch_bounds__(QtcCfg<NP>::THREADS, 1) k_qtrans_tc(int n, const double* __restrict__ in,
                                                              const double* __restrict__ M, double* __restrict__ out,
-                                                             int64_t ntiles) {
+                                                             int64_t ntiles, int* __restrict__ timeout) {
   using C = QtcCfg<NP>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(QtcCfg<NP>::THREADS, 1) k_qtrans_tc(int n, con
     if (warp == 0) {
       ok = mbar_wait_bounded(mbar_a, phase);
       if (!ok) {
-        atomicExch(&g_qtc_timeout, 1);
+        atomicExch(timeout ? timeout : &g_qtc_timeout, 1);
         mbar_wait_bounded(mbar_a, phase);   // let products still in flight finish
       }
     }
@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(QtcCfg<NP>::THREADS, 1) k_qtrans_tc(int n, con
 int g_qtc_nsm[HCI_MAXORB];   // SM count per device ordinal (0: not looked up)
 
 template <int NP>
-hci_status launch(cudaStream_t st, int n, const double* in, const double* M, double* out) {
+hci_status launch(cudaStream_t st, int n, const double* in, const double* M, double* out, int* timeout) {
   using C = QtcCfg<NP>;
   static bool attr_set[HCI_MAXORB] = {};
   int dev = 0;
@@ -470,18 +470,18 @@ hci_status launch(cudaStream_t st, int n, const double* in, const double* M, dou
   const int64_t N3 = (int64_t)n * n * n;
   const int64_t ntiles = (N3 + QTC_M - 1) / QTC_M;
   const int grid = (int)(ntiles < g_qtc_nsm[dev] ? ntiles : g_qtc_nsm[dev]);
-  HCI_LAUNCH(k_qtrans_tc<NP>, grid, C::THREADS, C::SMEM, st)(n, in, M, out, ntiles);
+  HCI_LAUNCH(k_qtrans_tc<NP>, grid, C::THREADS, C::SMEM, st)(n, in, M, out, ntiles, timeout);
   return cudaGetLastError() == cudaSuccess ? HCI_OK : HCI_ERR_CUDA;
 }
 
 }  // namespace
 
-hci_status qtrans_tc(cudaStream_t st, int n, const double* in, const double* M, double* out) {
+hci_status qtrans_tc(cudaStream_t st, int n, const double* in, const double* M, double* out, int* timeout) {
   if (n < 1 || n > HCI_MAXORB) return HCI_ERR_INVALID;
-  if (n <= 16) return launch<16>(st, n, in, M, out);
-  if (n <= 32) return launch<32>(st, n, in, M, out);
-  if (n <= 48) return launch<48>(st, n, in, M, out);
-  return launch<64>(st, n, in, M, out);
+  if (n <= 16) return launch<16>(st, n, in, M, out, timeout);
+  if (n <= 32) return launch<32>(st, n, in, M, out, timeout);
+  if (n <= 48) return launch<48>(st, n, in, M, out, timeout);
+  return launch<64>(st, n, in, M, out, timeout);
 }
 
 hci_status qtrans_tc_check(cudaStream_t st) {

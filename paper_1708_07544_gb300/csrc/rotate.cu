@@ -7,17 +7,20 @@
 //           that each rotate the leading index to the back.
 // Backward: dE/dh = U g1 U^T, dE/d(ab|cd) = sum D_pqrs U_ap U_bq U_cr U_ds
 //           with D = rdm2/2, and dE/dU = h U g1^T + h^T U g1 + 4 sum_bcd
-//           (xb|cd) T[y][b][c][d], T = D with its last three indices
+//           (xb|cd) T[d][c][b][y], T = D with its first three indices
 //           back-transformed (the four index positions of a real state with
-//           8-fold symmetric integrals contribute equally);
+//           8-fold symmetric integrals contribute equally, so the position
+//           left out is the last: T is three quarter transforms of D, and
+//           the fourth gives dE/d(ab|cd));
 //           dE/dkappa = L_exp(kappa^T, dE/dU), the Frechet derivative of
-//           exp at kappa^T, read off exp([[k^T, G], [0, k^T]]).
+//           exp at kappa^T, by the derivative of every step of exp.
 // The quarter transforms (the n^5 part) run on the bf16 tensor cores as
 // exact digit products rounded once to FP64 (qtrans_tc.cu); the n x n
 // matrix work stays on the FP64 pipe.
 #include <cuda.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <mutex>
 
@@ -25,82 +28,323 @@
 
 namespace {
 
-// C = alpha * op(A) op(B) + beta * C, m x m row-major, one thread per entry
-__global__ void k_mm(int m, const double* __restrict__ A, int tA, const double* __restrict__ B, int tB,
-                     double* __restrict__ C, double alpha, double beta) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= m * m) return;
-  int i = t / m, j = t % m;
-  double acc = 0.0;
-  for (int k = 0; k < m; ++k) {
-    double a = tA ? A[k * m + i] : A[i * m + k];
-    double b = tB ? B[j * m + k] : B[k * m + j];
-    acc = fma(a, b, acc);
+// ---------------------------------------------------------------------------
+// n x n matrix chains (n <= 64) in one launch: one thread-block cluster, each
+// CTA owning a block of the entries of every matrix; a product reads its
+// operands from global memory (L2) into shared memory, and the cluster's
+// barrier separates the products that depend on one another.
+//
+// exp(X) is the Taylor polynomial of degree 16 of X = kappa / 2^s, |X|_1 <=
+// 1/2 (remainder below 3e-20), with its blocks of four powers by Horner's rule in
+// X^4 (Paterson and Stockmeyer, SIAM J. Comput. 1973): 6 products where the
+// term-by-term rule takes 17, then s squarings.  On FP64 issue alone a
+// product of 44 x 44 matrices takes 1.4 us over 16 SMs; as separate launches
+// (6.9 us a product, 1.5 us a Horner step, and the host's wait for the norm)
+// exp took 200 us, the chain 45 us.
+// ---------------------------------------------------------------------------
+constexpr int CLM_T = 128;          // threads per CTA: one warp per FP64 pipe
+constexpr int CLM_NU = 4;           // entries per thread at most (8 CTAs: 16 x 32 of 64 x 64)
+constexpr int CLM_BI = 16, CLM_BJ = 32;
+
+__device__ __forceinline__ void cl_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ int cl_rank() {
+  int r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ int cl_size() {
+  int r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+
+// this CTA's block of every matrix
+struct Tile {
+  int i0, j0, ni, nj, cnt;
+};
+__device__ __forceinline__ Tile cl_tile(int n) {
+  const int c = cl_size(), r = cl_rank();
+  const int R = c >= 4 ? 4 : 1, C = c / R;
+  const int bi = (n + R - 1) / R, bj = (n + C - 1) / C;
+  Tile t;
+  t.i0 = (r % R) * bi;
+  t.j0 = (r / R) * bj;
+  t.ni = min(bi, n - t.i0);
+  t.nj = min(bj, n - t.j0);
+  if (t.ni < 0) t.ni = 0;
+  if (t.nj < 0) t.nj = 0;
+  t.cnt = t.ni * t.nj;
+  return t;
+}
+
+struct MM {
+  const double* A;
+  const double* B;
+  int tA, tB;            // transposed
+};
+
+// epi(u, i, j, v) for every entry (i, j) of the CTA's block, v = sum over the
+// terms of (op(A) op(B))_ij, u < CLM_NU the thread's entry number (the same
+// entry in every call).  Operands written in this kernel are read through
+// L2, after cl_sync.
+template <int NT, class F>
+__device__ __forceinline__ void cl_mm(int n, const Tile& t, const MM (&terms)[NT], double* sA, double* sB, F epi) {
+  double acc[CLM_NU];
+#pragma unroll
+  for (int u = 0; u < CLM_NU; ++u) acc[u] = 0.0;
+#pragma unroll
+  for (int q = 0; q < NT; ++q) {
+    const MM& m = terms[q];
+    __syncthreads();
+#pragma unroll 4
+    for (int e = threadIdx.x; e < t.ni * n; e += CLM_T) {
+      const int i = e / n, k = e - i * n;
+      sA[e] = __ldcg(m.tA ? m.A + k * n + t.i0 + i : m.A + (t.i0 + i) * n + k);
+    }
+#pragma unroll 4
+    for (int e = threadIdx.x; e < n * t.nj; e += CLM_T) {
+      const int k = e / t.nj, j = e - k * t.nj;
+      sB[e] = __ldcg(m.tB ? m.B + (t.j0 + j) * n + k : m.B + k * n + t.j0 + j);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < CLM_NU; ++u) {
+      const int o = threadIdx.x + u * CLM_T;
+      if (o >= t.cnt) break;
+      const int i = o / t.nj, j = o - i * t.nj;
+      const double* a = sA + i * n;
+      const double* b = sB + j;
+      double v = acc[u];
+#pragma unroll 4
+      for (int k = 0; k < n; ++k) v = fma(a[k], b[k * t.nj], v);
+      acc[u] = v;
+    }
   }
-  C[t] = beta == 0.0 ? alpha * acc : fma(alpha, acc, beta * C[t]);
-}
-
-// E = I + X * E / k   (Horner step of the Taylor series), X E in tmp
-__global__ void k_horner(int m, const double* __restrict__ XE, double* __restrict__ E, double invk) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= m * m) return;
-  int i = t / m, j = t % m;
-  E[t] = (i == j ? 1.0 : 0.0) + XE[t] * invk;
-}
-
-__global__ void k_eye_plus(int m, const double* __restrict__ X, double s, double* __restrict__ E) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= m * m) return;
-  int i = t / m, j = t % m;
-  E[t] = (i == j ? 1.0 : 0.0) + s * X[t];
-}
-
-__global__ void k_scale_copy(int64_t cnt, const double* __restrict__ in, double s, double* __restrict__ out) {
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x)
-    out[t] = s * in[t];
-}
-
-// max column abs-sum (1-norm) of an m x m matrix, single block
-__global__ void k_norm1(int m, const double* __restrict__ A, double* out) {
-  __shared__ double s[1024];
-  double v = 0.0;
-  for (int j = threadIdx.x; j < m; j += blockDim.x) {
-    double cs = 0.0;
-    for (int i = 0; i < m; ++i) cs += fabs(A[i * m + j]);
-    v = fmax(v, cs);
-  }
-  s[threadIdx.x] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double r = 0.0;
-    for (int t = 0; t < (int)blockDim.x; ++t) r = fmax(r, s[t]);
-    *out = r;
+#pragma unroll
+  for (int u = 0; u < CLM_NU; ++u) {
+    const int o = threadIdx.x + u * CLM_T;
+    if (o >= t.cnt) break;
+    const int i = o / t.nj;
+    epi(u, t.i0 + i, t.j0 + (o - i * t.nj), acc[u]);
   }
 }
 
-// block matrix [[K^T, G], [0, K^T]] of size 2n
-__global__ void k_frechet_block(int n, const double* __restrict__ K, const double* __restrict__ G, double* __restrict__ B) {
-  int m = 2 * n;
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= m * m) return;
-  int i = t / m, j = t % m;
-  double v = 0.0;
-  if (i < n && j < n) v = K[j * n + i];
-  else if (i >= n && j >= n) v = K[(j - n) * n + (i - n)];
-  else if (i < n && j >= n) v = G[i * n + (j - n)];
-  B[t] = v;
+// 1 / k!
+__device__ constexpr double INV_FACT[17] = {
+    1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120, 1.0 / 720, 1.0 / 5040, 1.0 / 40320, 1.0 / 362880, 1.0 / 3628800,
+    1.0 / 39916800, 1.0 / 479001600, 1.0 / 6227020800.0, 1.0 / 87178291200.0, 1.0 / 1307674368000.0,
+    1.0 / 20922789888000.0};
+
+// Work matrices of the chains (n x n each) and their status words.
+enum { W_X = 0, W_X2, W_X3, W_X4, W_S0, W_S1, W_S2, W_E, W_F, W_T, W_T2, W_UT, W_UTH, W_GU, W_FWD_COUNT = W_T + 1,
+       W_D1 = W_GU + 1, W_D2, W_D3, W_D4, W_DS0, W_DS1, W_DS2, W_DE, W_DF, W_COUNT };
+struct RotStatus {
+  int nonfinite;     // |kappa|_1 is not finite
+  int timeout;       // a quarter transform gave up waiting for its products
+  int squarings;
+  int bad_gradient;  // dE/dU is infinite
+};
+
+struct ChainArgs {
+  int n;
+  const double* kappa;
+  const double* h;
+  double* U;
+  double* h_out;        // forward: U^T h U, exactly symmetric
+  const double* g1;     // backward
+  double* dh;           // backward: U g1 U^T, or NULL
+  int want_gu;          // backward: h-part of dE/dU
+  double* ws;
+  RotStatus* status;
+};
+
+template <bool BWD>
+__global__ void __launch_bounds__(CLM_T) k_exp_chain(ChainArgs A) {
+  __shared__ double sA[CLM_BI * HCI_MAXORB], sB[HCI_MAXORB * CLM_BJ];
+  __shared__ double s_nrm[CLM_T];
+  const int n = A.n, nn = n * n, tid = threadIdx.x;
+  double* ws = A.ws;
+  auto W = [&](int k) { return ws + (size_t)k * nn; };
+  // 1-norm, by every CTA for itself: thread = column, rows in halves
+  {
+    const int j = tid & 63, half = tid >> 6;
+    double c = 0.0;
+    if (j < n)
+      for (int i = half; i < n; i += 2) c += fabs(A.kappa[i * n + j]);
+    s_nrm[tid] = c;
+    __syncthreads();
+    if (tid < 64) s_nrm[tid] += s_nrm[tid + 64];
+    __syncthreads();
+    if (tid < 32) {
+      double v = fmax(fmax(0.0, s_nrm[tid]), s_nrm[tid + 32]);
+      for (int o = 16; o; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+      if (tid == 0) s_nrm[0] = v;
+    }
+    __syncthreads();
+  }
+  const double nrm = s_nrm[0];
+  if (!isfinite(nrm)) {
+    if (cl_rank() == 0 && tid == 0) A.status->nonfinite = 1;
+    return;   // the same in every CTA
+  }
+  int s = 0;
+  while (ldexp(nrm, -s) > 0.5) ++s;
+  const double sc = ldexp(1.0, -s);
+  if (cl_rank() == 0 && tid == 0) A.status->squarings = s;
+  const Tile t = cl_tile(n);
+  double x[CLM_NU], x2[CLM_NU], x3[CLM_NU];
+  const MM m2[1] = {{A.kappa, A.kappa, 0, 0}};
+  cl_mm(n, t, m2, sA, sB, [&](int u, int i, int j, double v) {
+    x[u] = A.kappa[i * n + j] * sc;
+    x2[u] = v * sc * sc;
+    if (BWD) W(W_X)[i * n + j] = x[u];
+    W(W_X2)[i * n + j] = x2[u];
+  });
+  cl_sync();
+  const MM m3[1] = {{W(W_X2), A.kappa, 0, 0}};
+  cl_mm(n, t, m3, sA, sB, [&](int u, int i, int j, double v) {
+    x3[u] = v * sc;
+    if (BWD) W(W_X3)[i * n + j] = x3[u];
+  });
+  const MM m4[1] = {{W(W_X2), W(W_X2), 0, 0}};
+  auto blk = [&](int b, int u, int i, int j) {
+    double v = i == j ? INV_FACT[b] : 0.0;
+    v = fma(INV_FACT[b + 1], x[u], v);
+    v = fma(INV_FACT[b + 2], x2[u], v);
+    return fma(INV_FACT[b + 3], x3[u], v);
+  };
+  cl_mm(n, t, m4, sA, sB, [&](int u, int i, int j, double v) {
+    W(W_X4)[i * n + j] = v;
+    W(W_S0)[i * n + j] = fma(INV_FACT[16], v, blk(12, u, i, j));
+  });
+  cl_sync();
+  const MM h1[1] = {{W(W_X4), W(W_S0), 0, 0}}, h2[1] = {{W(W_X4), W(W_S1), 0, 0}}, h3[1] = {{W(W_X4), W(W_S2), 0, 0}};
+  cl_mm(n, t, h1, sA, sB, [&](int u, int i, int j, double v) { W(W_S1)[i * n + j] = v + blk(8, u, i, j); });
+  cl_sync();
+  cl_mm(n, t, h2, sA, sB, [&](int u, int i, int j, double v) { W(W_S2)[i * n + j] = v + blk(4, u, i, j); });
+  cl_sync();
+  auto store_u = [&](int i, int j, double v) {
+    A.U[i * n + j] = v;
+    if (BWD) {
+      W(W_UT)[j * n + i] = v;
+      W(W_UTH)[j * n + i] = 0.5 * v;
+    }
+  };
+  cl_mm(n, t, h3, sA, sB, [&](int u, int i, int j, double v) {
+    v += blk(0, u, i, j);
+    W(W_E)[i * n + j] = v;
+    if (s == 0) store_u(i, j, v);
+  });
+  cl_sync();
+  // squarings (the backward keeps W_E, the exponential of the scaled matrix)
+  int from = W_E, to = W_F;
+  for (int q = 0; q < s; ++q) {
+    const MM sq[1] = {{W(from), W(from), 0, 0}};
+    cl_mm(n, t, sq, sA, sB, [&](int u, int i, int j, double v) {
+      W(to)[i * n + j] = v;
+      if (q == s - 1) store_u(i, j, v);
+    });
+    cl_sync();
+    const int old = from;
+    from = to;
+    to = old == W_E ? W_T : old;
+  }
+  if (!BWD) {
+    const MM a[1] = {{A.h, A.U, 0, 0}};
+    cl_mm(n, t, a, sA, sB, [&](int u, int i, int j, double v) { W(W_S0)[i * n + j] = v; });
+    cl_sync();
+    // the upper triangle's values on both sides
+    const MM b[1] = {{A.U, W(W_S0), 1, 0}};
+    cl_mm(n, t, b, sA, sB, [&](int u, int i, int j, double v) {
+      if (i <= j) {
+        A.h_out[i * n + j] = v;
+        A.h_out[j * n + i] = v;
+      }
+    });
+  } else {
+    const MM a[1] = {{A.g1, A.U, 0, 1}}, b[1] = {{A.h, A.U, 0, 0}}, c[1] = {{A.h, A.U, 1, 0}};
+    if (A.dh) cl_mm(n, t, a, sA, sB, [&](int u, int i, int j, double v) { W(W_D1)[i * n + j] = v; });
+    if (A.want_gu) {
+      cl_mm(n, t, b, sA, sB, [&](int u, int i, int j, double v) { W(W_T)[i * n + j] = v; });
+      cl_mm(n, t, c, sA, sB, [&](int u, int i, int j, double v) { W(W_T2)[i * n + j] = v; });
+    }
+    cl_sync();
+    if (A.want_gu) {
+      const MM d[2] = {{W(W_T), A.g1, 0, 1}, {W(W_T2), A.g1, 0, 0}};
+      cl_mm(n, t, d, sA, sB, [&](int u, int i, int j, double v) { W(W_GU)[i * n + j] = v; });
+    }
+    if (A.dh) {
+      cl_sync();          // dh may be g1's or h's own buffer
+      const MM e[1] = {{A.U, W(W_D1), 0, 0}};
+      cl_mm(n, t, e, sA, sB, [&](int u, int i, int j, double v) { A.dh[i * n + j] = v; });
+    }
+  }
 }
 
-__global__ void k_upper_right(int n, const double* __restrict__ B, double* __restrict__ out) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n * n) return;
-  int i = t / n, j = t % n;
-  out[t] = B[i * 2 * n + n + j];
-}
-
-__global__ void k_eye(int n, double* __restrict__ I) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n * n) I[t] = (t / n == t % n) ? 1.0 : 0.0;
+// dkappa = L_exp(kappa^T, G), G = W_GU: the derivative of every step of the
+// chain above at X^T (whose powers are the stored ones transposed) along
+// dX = G / 2^s; 12 products.
+__global__ void __launch_bounds__(CLM_T) k_exp_adjoint(ChainArgs A, double* __restrict__ dkappa) {
+  __shared__ double sA[CLM_BI * HCI_MAXORB], sB[HCI_MAXORB * CLM_BJ];
+  if (A.status->nonfinite) return;
+  const int n = A.n, nn = n * n, s = A.status->squarings;
+  const double sc = ldexp(1.0, -s);
+  double* ws = A.ws;
+  auto W = [&](int k) { return ws + (size_t)k * nn; };
+  const Tile t = cl_tile(n);
+  double d1[CLM_NU], d2[CLM_NU], d3[CLM_NU];
+  // products with G itself, scaled in the epilogue
+  const MM p2[2] = {{W(W_X), W(W_GU), 1, 0}, {W(W_GU), W(W_X), 0, 1}};
+  cl_mm(n, t, p2, sA, sB, [&](int u, int i, int j, double v) {
+    const double g = __ldcg(W(W_GU) + i * n + j);
+    if (isinf(g)) A.status->bad_gradient = 1;
+    d1[u] = g * sc;
+    d2[u] = v * sc;
+    W(W_D1)[i * n + j] = d1[u];
+    W(W_D2)[i * n + j] = d2[u];
+  });
+  cl_sync();
+  const MM p3[2] = {{W(W_X2), W(W_D1), 1, 0}, {W(W_D2), W(W_X), 0, 1}};
+  cl_mm(n, t, p3, sA, sB, [&](int u, int i, int j, double v) { d3[u] = v; });
+  const MM p4[2] = {{W(W_X2), W(W_D2), 1, 0}, {W(W_D2), W(W_X2), 0, 1}};
+  auto blk = [&](int b, int u) {
+    return fma(INV_FACT[b + 1], d1[u], fma(INV_FACT[b + 2], d2[u], INV_FACT[b + 3] * d3[u]));
+  };
+  cl_mm(n, t, p4, sA, sB, [&](int u, int i, int j, double v) {
+    W(W_D4)[i * n + j] = v;
+    W(W_DS0)[i * n + j] = fma(INV_FACT[16], v, blk(12, u));
+  });
+  cl_sync();
+  const MM q1[2] = {{W(W_X4), W(W_DS0), 1, 0}, {W(W_D4), W(W_S0), 0, 1}};
+  cl_mm(n, t, q1, sA, sB, [&](int u, int i, int j, double v) { W(W_DS1)[i * n + j] = v + blk(8, u); });
+  cl_sync();
+  const MM q2[2] = {{W(W_X4), W(W_DS1), 1, 0}, {W(W_D4), W(W_S1), 0, 1}};
+  cl_mm(n, t, q2, sA, sB, [&](int u, int i, int j, double v) { W(W_DS2)[i * n + j] = v + blk(4, u); });
+  cl_sync();
+  const MM q3[2] = {{W(W_X4), W(W_DS2), 1, 0}, {W(W_D4), W(W_S2), 0, 1}};
+  cl_mm(n, t, q3, sA, sB, [&](int u, int i, int j, double v) {
+    v += blk(0, u);
+    if (s == 0) dkappa[i * n + j] = v;
+    else W(W_DE)[i * n + j] = v;
+  });
+  // E <- E^2, dE <- E^T dE + dE E^T
+  int e0 = W_E, e1 = W_F, f0 = W_DE, f1 = W_DF;
+  for (int q = 0; q < s; ++q) {
+    cl_sync();
+    const MM r[2] = {{W(e0), W(f0), 1, 0}, {W(f0), W(e0), 0, 1}};
+    cl_mm(n, t, r, sA, sB, [&](int u, int i, int j, double v) {
+      if (q == s - 1) dkappa[i * n + j] = v;
+      else W(f1)[i * n + j] = v;
+    });
+    if (q < s - 1) {
+      const MM sq[1] = {{W(e0), W(e0), 0, 0}};
+      cl_mm(n, t, sq, sA, sB, [&](int u, int i, int j, double v) { W(e1)[i * n + j] = v; });
+    }
+    int w = e0; e0 = e1; e1 = w;
+    w = f0; f0 = f1; f1 = w;
+  }
 }
 
 // The solver reads different permutations of one integral (heat-bath lists,
@@ -122,43 +366,89 @@ __global__ void k_sym8(int n, double* __restrict__ eri) {
     if (rep != t) eri[t] = eri[rep];
   }
 }
-__global__ void k_symh(int n, double* __restrict__ h) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n * n) return;
-  const int p = t / n, q = t % n;
-  if (p > q) h[t] = h[q * n + p];
-}
-
-// partial[b][x][y] = sum_{J in chunk b} A[x][J] B[y][J]  (A, B: n x K)
-constexpr int NT_CH = 64;
-__global__ void __launch_bounds__(256) k_gemm_nt_part(int n, int64_t K, const double* __restrict__ A,
-                                                      const double* __restrict__ B, double* __restrict__ partial) {
+// part[b][x][y] = block b's share of sum_J eri[J][x] T[y][J], J = (d, c, b):
+// the leading pair's symmetry of eri, (dc|bx) = (cd|bx), leaves the pairs
+// d <= c with T[y][d][c][b] + T[y][c][d][b] (d < c), half the FP64 products
+// that bound this contraction.  Every block takes an equal share of the
+// n^2 (n + 1) / 2 rows, NT_CH staged at a time; thread t owns entries
+// t, t + 256, ... (44 orbitals: 302 us for all of J, 179 us so).
+constexpr int NT_CH = 48;
+template <int NACC>
+__global__ void __launch_bounds__(256) k_gemm_nt_part(int n, int64_t rows, const double* __restrict__ eri,
+                                                      const double* __restrict__ T, double* __restrict__ part) {
   extern __shared__ double sm[];
-  double* At = sm;                 // n * NT_CH
-  double* Bt = sm + n * NT_CH;     // n * NT_CH
-  const int64_t J0 = (int64_t)blockIdx.x * NT_CH;
-  for (int t = threadIdx.x; t < n * NT_CH; t += blockDim.x) {
-    int x = t / NT_CH, jj = t % NT_CH;
-    int64_t J = J0 + jj;
-    At[t] = J < K ? A[(int64_t)x * K + J] : 0.0;
-    Bt[t] = J < K ? B[(int64_t)x * K + J] : 0.0;
+  double* sE = sm;                 // [NT_CH][n] (x fastest)
+  double* sT = sm + NT_CH * n;     // [NT_CH][n + 1] (y fastest)
+  const int nn = n * n, ld = n + 1;
+  const int64_t n3 = (int64_t)nn * n;
+  const int64_t r0 = rows * blockIdx.x / gridDim.x, r1 = rows * (blockIdx.x + 1) / gridDim.x;
+  double acc[NACC];
+#pragma unroll
+  for (int u = 0; u < NACC; ++u) acc[u] = 0.0;
+  for (int64_t rr = r0; rr < r1; rr += NT_CH) {
+    const int cnt = r1 - rr < NT_CH ? (int)(r1 - rr) : NT_CH;
+    __syncthreads();
+    // row q = (pair t = c (c + 1) / 2 + d with d <= c, b)
+    for (int e = threadIdx.x; e < cnt * n; e += 256) {
+      const int k = e / n, x = e - k * n;
+      const int64_t q = rr + k;
+      const int tp = (int)(q / n), b = (int)(q - (int64_t)tp * n);
+      int c = (int)((sqrtf(8.0f * (float)tp + 1.0f) - 1.0f) * 0.5f);
+      while (c * (c + 1) / 2 > tp) --c;
+      while ((c + 1) * (c + 2) / 2 <= tp) ++c;
+      const int d = tp - c * (c + 1) / 2;
+      sE[k * n + x] = eri[((int64_t)(d * n + c) * n + b) * n + x];
+    }
+    for (int e = threadIdx.x; e < cnt * n; e += 256) {
+      const int y = e / cnt, k = e - y * cnt;
+      const int64_t q = rr + k;
+      const int tp = (int)(q / n), b = (int)(q - (int64_t)tp * n);
+      int c = (int)((sqrtf(8.0f * (float)tp + 1.0f) - 1.0f) * 0.5f);
+      while (c * (c + 1) / 2 > tp) --c;
+      while ((c + 1) * (c + 2) / 2 <= tp) ++c;
+      const int d = tp - c * (c + 1) / 2;
+      double v = T[(int64_t)y * n3 + (int64_t)(d * n + c) * n + b];
+      if (d != c) v += T[(int64_t)y * n3 + (int64_t)(c * n + d) * n + b];
+      sT[k * ld + y] = v;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < NACC; ++u) {
+      const int o = threadIdx.x + 256 * u;
+      if (o < nn) {
+        const int x = o % n, y = o / n;
+        double v = acc[u];
+#pragma unroll 8
+        for (int k = 0; k < cnt; ++k) v = fma(sE[k * n + x], sT[k * ld + y], v);
+        acc[u] = v;
+      }
+    }
   }
-  __syncthreads();
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-    int x = t / n, y = t % n;
-    double acc = 0.0;
-    for (int jj = 0; jj < NT_CH; ++jj) acc = fma(At[x * NT_CH + jj], Bt[y * NT_CH + jj], acc);
-    partial[(int64_t)blockIdx.x * n * n + t] = acc;
+#pragma unroll
+  for (int u = 0; u < NACC; ++u) {
+    const int o = threadIdx.x + 256 * u;
+    if (o < nn) part[(int64_t)blockIdx.x * nn + o] = acc[u];
   }
 }
 
-__global__ void k_sum_parts(int nn, int nparts, const double* __restrict__ partial, double scale,
-                            double* __restrict__ out) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nn) return;
+// out[x][y] += scale * sum of the parts' [y][x], 32 entries per block, the
+// parts in eight slices
+__global__ void __launch_bounds__(256) k_sum_parts(int n, int nparts, const double* __restrict__ part, double scale,
+                                                   double* __restrict__ out) {
+  __shared__ double red[8][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int o = blockIdx.x * 32 + lane, nn = n * n;
   double s = 0.0;
-  for (int b = 0; b < nparts; ++b) s += partial[(int64_t)b * nn + t];
-  out[t] += scale * s;
+  if (o < nn)
+#pragma unroll 4
+    for (int b = w; b < nparts; b += 8) s += part[(int64_t)b * nn + o];
+  red[w][lane] = s;
+  __syncthreads();
+  if (w == 0 && o < nn) {
+    s = 0.0;
+    for (int k = 0; k < 8; ++k) s += red[k][lane];
+    out[(o % n) * n + o / n] += scale * s;
+  }
 }
 
 struct Scratch {
@@ -181,59 +471,97 @@ struct Scratch {
 
 inline unsigned blocks(int64_t work, int b = 256) { return (unsigned)((work + b - 1) / b); }
 
-hci_status mm(cudaStream_t st, int m, const double* A, int tA, const double* B, int tB, double* C, double alpha,
-              double beta) {
-  HCI_LAUNCH(k_mm, blocks((int64_t)m * m), 256, 0, st)(m, A, tA, B, tB, C, alpha, beta);
-  return HCI_OK;
+// CTAs of a chain's cluster: one for 16 orbitals or fewer (a product is then
+// shorter than the cluster's barrier), else 16 where the device can hold
+// such a cluster (an opt-in size), or the portable 8.  Looked up once per
+// device.
+int chain_ctas(int n) {
+  if (n <= 16) return 1;
+  static std::atomic<int> known[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 8;
+  int c = known[dev].load();
+  if (c) return c;
+  c = 8;
+  const void* fns[3] = {(const void*)k_exp_chain<false>, (const void*)k_exp_chain<true>, (const void*)k_exp_adjoint};
+  bool ok = true;
+  for (const void* f : fns) ok = ok && cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+  if (ok) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(16);
+    cfg.blockDim = dim3(CLM_T);
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 16;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int nc = 0;
+    for (const void* f : fns) {
+      ok = ok && cudaOccupancyMaxActiveClusters(&nc, f, &cfg) == cudaSuccess && nc >= 1;
+    }
+    if (ok) c = 16;
+  }
+  cudaGetLastError();
+  known[dev].store(c);
+  return c;
 }
 
-// E = exp(A) for an m x m matrix; w1, w2, w3 scratch of m*m
-hci_status expm_dev(cudaStream_t st, int m, const double* A, double* E, double* w1, double* w2, double* w3,
-                    double* dscal) {
-  HCI_LAUNCH(k_norm1, 1, 256, 0, st)(m, A, dscal);
-  double nrm = 0.0;
-  if (cudaMemcpyAsync(&nrm, dscal, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess) return HCI_ERR_CUDA;
-  if (cudaStreamSynchronize(st) != cudaSuccess) return HCI_ERR_CUDA;
-  if (!std::isfinite(nrm)) return HCI_ERR_INVALID;
-  int s = 0;
-  while (nrm / std::ldexp(1.0, s) > 0.5) ++s;
-  const double sc = std::ldexp(1.0, -s);
-  HCI_LAUNCH(k_scale_copy, blocks((int64_t)m * m), 256, 0, st)((int64_t)m * m, A, sc, w1);   // X
-  // Horner: E = I + X/18; E = I + X E / k for k = 17..1
-  const int deg = 18;
-  HCI_LAUNCH(k_eye_plus, blocks((int64_t)m * m), 256, 0, st)(m, w1, 1.0 / deg, E);
-  for (int k = deg - 1; k >= 1; --k) {
-    mm(st, m, w1, 0, E, 0, w2, 1.0, 0.0);
-    HCI_LAUNCH(k_horner, blocks((int64_t)m * m), 256, 0, st)(m, w2, E, 1.0 / k);
-  }
-  for (int i = 0; i < s; ++i) {
-    mm(st, m, E, 0, E, 0, w3, 1.0, 0.0);
-    cudaMemcpyAsync(E, w3, (size_t)m * m * 8, cudaMemcpyDeviceToDevice, st);
-  }
-  return cudaGetLastError() == cudaSuccess ? HCI_OK : HCI_ERR_CUDA;
+template <class... P, class... Q>
+cudaError_t launch_chain(cudaStream_t st, int n, void (*k)(P...), Q... args) {
+  cudaLaunchConfig_t cfg = {};
+  const int c = chain_ctas(n);
+  cfg.gridDim = dim3((unsigned)c);
+  cfg.blockDim = dim3(CLM_T);
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)c;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  hci_count_launch();
+  return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
 // out[J*n + p] = sum_a in[a*N3 + J] * M[a*n + p], J < N3 = n^3
-#define QTRANS(who, in, M, out)                                                              \
+#define QTRANS(who, in, M, out, flag)                                                        \
   do {                                                                                       \
-    if (qtrans_tc(st, n, in, M, out) != HCI_OK)                                              \
+    if (qtrans_tc(st, n, in, M, out, flag) != HCI_OK)                                            \
       return hci_fail(nullptr, HCI_ERR_CUDA, who ": quarter transform launch failed: %s",     \
                       cudaGetErrorString(cudaGetLastError()));                               \
   } while (0)
 
-// after the final synchronisation: the quarter transforms completed
-#define QTRANS_CHECK(who)                                                                        \
-  do {                                                                                           \
-    if (qtrans_tc_check(st) != HCI_OK)                                                             \
-      return hci_fail(nullptr, HCI_ERR_CUDA, who ": a quarter transform gave up waiting for its " \
-                      "tensor-core products");                                                   \
-  } while (0)
+// the call's status words read and judged (synchronises st)
+hci_status chain_status(const char* who, cudaStream_t st, const RotStatus* dev) {
+  RotStatus h = {};
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, dev, sizeof h, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return hci_fail(nullptr, HCI_ERR_CUDA, "%s: %s", who, cudaGetErrorString(e));
+  if (h.nonfinite) return hci_fail(nullptr, HCI_ERR_INVALID, "%s: matrix exponential failed", who);
+  if (h.bad_gradient) return hci_fail(nullptr, HCI_ERR_INVALID, "%s: Frechet exponential failed", who);
+  if (h.timeout)
+    return hci_fail(nullptr, HCI_ERR_CUDA, "%s: a quarter transform gave up waiting for its tensor-core products", who);
+  return HCI_OK;
+}
 
-// exact permutational symmetry of the rotated integrals (see k_sym8)
-void symmetrize(cudaStream_t st, int n, double* h, double* eri) {
-  const int64_t n4 = (int64_t)n * n * n * n;
-  HCI_LAUNCH(k_symh, blocks((int64_t)n * n), 256, 0, st)(n, h);
-  HCI_LAUNCH(k_sym8, (unsigned)std::min<int64_t>(blocks(n4), 4096), 256, 0, st)(n, eri);
+// ws: W_FWD_COUNT n x n matrices and the status words; t4: n^4
+hci_status rotate_core(const char* who, cudaStream_t st, int n, const double* kappa, const double* h, const double* eri,
+                       double* U, double* h_out, double* eri_out, double* ws, double* t4) {
+  RotStatus* status = reinterpret_cast<RotStatus*>(ws + (size_t)W_FWD_COUNT * n * n);
+  ChainArgs A = {};
+  A.n = n; A.kappa = kappa; A.h = h; A.U = U; A.h_out = h_out; A.ws = ws; A.status = status;
+  cudaError_t e = cudaMemsetAsync(status, 0, sizeof(RotStatus), st);
+  if (e == cudaSuccess) e = launch_chain(st, n, k_exp_chain<false>, A);
+  if (e != cudaSuccess) return hci_fail(nullptr, HCI_ERR_CUDA, "%s: %s", who, cudaGetErrorString(e));
+  QTRANS("hci_rotate", eri, U, t4, &status->timeout);
+  QTRANS("hci_rotate", t4, U, eri_out, &status->timeout);
+  QTRANS("hci_rotate", eri_out, U, t4, &status->timeout);
+  QTRANS("hci_rotate", t4, U, eri_out, &status->timeout);
+  // exact permutational symmetry of the rotated integrals (see k_sym8)
+  HCI_LAUNCH(k_sym8, (unsigned)std::min<int64_t>(blocks((int64_t)n * n * n * n), 4096), 256, 0, st)(n, eri_out);
+  return chain_status(who, st, status);
 }
 
 }  // namespace
@@ -247,25 +575,11 @@ extern "C" hci_status hci_rotate(int norb, const double* kappa, const double* h,
   cudaStream_t st = (cudaStream_t)stream;
   Scratch S{st};
   const size_t n2 = (size_t)n * n, n4 = n2 * n2;
-  double *w1 = S.get(n2), *w2 = S.get(n2), *w3 = S.get(n2), *ds = S.get(8), *t4 = S.get(n4);
-  if (!w1 || !w2 || !w3 || !ds || !t4)
+  double *ws = S.get(W_FWD_COUNT * n2 + 2), *t4 = S.get(n4);
+  if (!ws || !t4)
     return hci_fail(nullptr, HCI_ERR_NOMEM, "hci_rotate: allocation failed%s",
                     S.left == 0 ? " (injected by HCI_FAIL_ALLOC_AFTER)" : "");
-  hci_status s = expm_dev(st, n, kappa, U, w1, w2, w3, ds);
-  if (s != HCI_OK) return hci_fail(nullptr, s, "hci_rotate: matrix exponential failed");
-  mm(st, n, h, 0, U, 0, w1, 1.0, 0.0);          // h U
-  mm(st, n, U, 1, w1, 0, h_out, 1.0, 0.0);      // U^T h U
-  QTRANS("hci_rotate", eri, U, t4);
-  QTRANS("hci_rotate", t4, U, eri_out);
-  QTRANS("hci_rotate", eri_out, U, t4);
-  QTRANS("hci_rotate", t4, U, eri_out);
-  symmetrize(st, n, h_out, eri_out);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return hci_fail(nullptr, HCI_ERR_CUDA, "hci_rotate: %s", cudaGetErrorString(e));
-  e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return hci_fail(nullptr, HCI_ERR_CUDA, "hci_rotate: %s", cudaGetErrorString(e));
-  QTRANS_CHECK("hci_rotate");
-  return HCI_OK;
+  return rotate_core("hci_rotate", st, n, kappa, h, eri, U, h_out, eri_out, ws, t4);
 }
 
 extern "C" hci_status hci_rotate_backward(int norb, const double* kappa, const double* h, const double* eri,
@@ -279,63 +593,42 @@ extern "C" hci_status hci_rotate_backward(int norb, const double* kappa, const d
   cudaStream_t st = (cudaStream_t)stream;
   Scratch S{st};
   const size_t n2 = (size_t)n * n, n4 = n2 * n2;
-  const int m2 = 2 * n;
-  double *U = S.get(n2), *Ut = S.get(n2), *I = S.get(n2), *w1 = S.get(n2), *gU = S.get(n2);
-  double *b1 = S.get((size_t)m2 * m2), *b2 = S.get((size_t)m2 * m2), *b3 = S.get((size_t)m2 * m2),
-         *b4 = S.get((size_t)m2 * m2), *b5 = S.get((size_t)m2 * m2), *ds = S.get(8);
-  double *D = S.get(n4), *t4 = S.get(n4);
-  if (!U || !Ut || !I || !w1 || !gU || !b1 || !b2 || !b3 || !b4 || !b5 || !ds || !D || !t4)
+  const int64_t rows = (int64_t)n2 * (n + 1) / 2;
+  const int nparts = (int)std::min<int64_t>(2 * hci_nsm(), (rows + 15) / 16);
+  double *ws = S.get(W_COUNT * n2 + 2), *U = S.get(n2), *ta = S.get(n4), *tb = S.get(n4);
+  double* part = dkappa ? S.get((size_t)nparts * n2) : nullptr;
+  if (!ws || !U || !ta || !tb || (dkappa && !part))
     return hci_fail(nullptr, HCI_ERR_NOMEM, "hci_rotate_backward: allocation failed%s",
                     S.left == 0 ? " (injected by HCI_FAIL_ALLOC_AFTER)" : "");
-  cudaFuncSetAttribute(k_gemm_nt_part, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 64 * NT_CH * 8);
-  hci_status s = expm_dev(st, n, kappa, U, w1, b1, b2, ds);
-  if (s != HCI_OK) return hci_fail(nullptr, s, "hci_rotate_backward: matrix exponential failed");
-  HCI_LAUNCH(k_eye, blocks((int64_t)n2), 256, 0, st)(n, I);
-  // U^T as a matrix for the back-transforms: M[a][p] = U[p][a]
-  mm(st, n, U, 1, I, 0, Ut, 1.0, 0.0);
-  if (dh) {
-    mm(st, n, rdm1, 0, U, 1, w1, 1.0, 0.0);     // g1 U^T
-    mm(st, n, U, 0, w1, 0, dh, 1.0, 0.0);       // U g1 U^T
-  }
-  HCI_LAUNCH(k_scale_copy, blocks((int64_t)n4), 256, 0, st)((int64_t)n4, rdm2, 0.5, D);
-  if (deri) {
-    QTRANS("hci_rotate_backward", D, Ut, t4);
-    QTRANS("hci_rotate_backward", t4, Ut, deri);
-    QTRANS("hci_rotate_backward", deri, Ut, t4);
-    QTRANS("hci_rotate_backward", t4, Ut, deri);
+  RotStatus* status = reinterpret_cast<RotStatus*>(ws + W_COUNT * n2);
+  ChainArgs A = {};
+  A.n = n; A.kappa = kappa; A.h = h; A.U = U; A.g1 = rdm1; A.dh = dh; A.want_gu = dkappa != nullptr; A.ws = ws;
+  A.status = status;
+  cudaError_t e = cudaMemsetAsync(status, 0, sizeof(RotStatus), st);
+  if (e == cudaSuccess) e = launch_chain(st, n, k_exp_chain<true>, A);
+  if (e != cudaSuccess) return hci_fail(nullptr, HCI_ERR_CUDA, "hci_rotate_backward: %s", cudaGetErrorString(e));
+  // D = rdm2 / 2 back-transformed: the half goes into the first U^T; three
+  // transforms leave T[y][d][c][b] in ta, the fourth is dE/d(dc|ba)
+  const double *Ut = ws + (size_t)W_UT * n2, *Uth = ws + (size_t)W_UTH * n2;
+  if (deri || dkappa) {
+    QTRANS("hci_rotate_backward", rdm2, Uth, ta, &status->timeout);
+    QTRANS("hci_rotate_backward", ta, Ut, tb, &status->timeout);
+    QTRANS("hci_rotate_backward", tb, Ut, ta, &status->timeout);
   }
   if (dkappa) {
-    // h-part: h U g1^T + h^T U g1
-    mm(st, n, h, 0, U, 0, w1, 1.0, 0.0);
-    mm(st, n, w1, 0, rdm1, 1, gU, 1.0, 0.0);
-    mm(st, n, h, 1, U, 0, w1, 1.0, 0.0);
-    mm(st, n, w1, 0, rdm1, 0, gU, 1.0, 1.0);
-    // T[y][b][c][d] = sum_qrs U_bq U_cr U_ds D[y][q][r][s]
-    double* T = t4;
-    QTRANS("hci_rotate_backward", D, I, T);          // (q r s y)
-    QTRANS("hci_rotate_backward", T, Ut, D);         // (r s y b)
-    QTRANS("hci_rotate_backward", D, Ut, T);         // (s y b c)
-    QTRANS("hci_rotate_backward", T, Ut, D);         // (y b c d)
-    const int64_t K = (int64_t)n * n * n;
-    const int nparts = (int)((K + NT_CH - 1) / NT_CH);
-    double* part = S.get((size_t)nparts * n2);
-    if (!part)
-      return hci_fail(nullptr, HCI_ERR_NOMEM, "hci_rotate_backward: allocation failed%s",
-                      S.left == 0 ? " (injected by HCI_FAIL_ALLOC_AFTER)" : "");
-    HCI_LAUNCH(k_gemm_nt_part, nparts, 256, (size_t)2 * n * NT_CH * 8, st)(n, K, eri, D, part);
-    HCI_LAUNCH(k_sum_parts, blocks((int64_t)n2), 256, 0, st)((int)n2, nparts, part, 4.0, gU);
-    // dkappa = L_exp(kappa^T, gU)
-    HCI_LAUNCH(k_frechet_block, blocks((int64_t)m2 * m2), 256, 0, st)(n, kappa, gU, b1);
-    s = expm_dev(st, m2, b1, b2, b3, b4, b5, ds);
-    if (s != HCI_OK) return hci_fail(nullptr, s, "hci_rotate_backward: Frechet exponential failed");
-    HCI_LAUNCH(k_upper_right, blocks((int64_t)n2), 256, 0, st)(n, b2, dkappa);
+    const size_t sm = (size_t)NT_CH * (2 * n + 1) * 8;
+    if (n2 <= 2048) {
+      HCI_LAUNCH(k_gemm_nt_part<8>, nparts, 256, sm, st)(n, rows, eri, ta, part);
+    } else {
+      cudaFuncSetAttribute(k_gemm_nt_part<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, NT_CH * 129 * 8);
+      HCI_LAUNCH(k_gemm_nt_part<16>, nparts, 256, sm, st)(n, rows, eri, ta, part);
+    }
+    HCI_LAUNCH(k_sum_parts, (unsigned)((n2 + 31) / 32), 256, 0, st)(n, nparts, part, 4.0, ws + (size_t)W_GU * n2);
+    e = launch_chain(st, n, k_exp_adjoint, A, dkappa);
+    if (e != cudaSuccess) return hci_fail(nullptr, HCI_ERR_CUDA, "hci_rotate_backward: %s", cudaGetErrorString(e));
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return hci_fail(nullptr, HCI_ERR_CUDA, "hci_rotate_backward: %s", cudaGetErrorString(e));
-  e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return hci_fail(nullptr, HCI_ERR_CUDA, "hci_rotate_backward: %s", cudaGetErrorString(e));
-  QTRANS_CHECK("hci_rotate_backward");
-  return HCI_OK;
+  if (deri) QTRANS("hci_rotate_backward", ta, Ut, deri, &status->timeout);
+  return chain_status("hci_rotate_backward", st, status);
 }
 
 extern "C" hci_status hci_qtrans(int norb, const double* in, const double* M, double* out, int check,
@@ -344,8 +637,9 @@ extern "C" hci_status hci_qtrans(int norb, const double* in, const double* M, do
   if (n < 1 || n > HCI_MAXORB) return hci_fail(nullptr, HCI_ERR_INVALID, "hci_qtrans: norb=%d outside [1,64]", n);
   if (!in || !M || !out) return hci_fail(nullptr, HCI_ERR_INVALID, "hci_qtrans: null pointer");
   cudaStream_t st = (cudaStream_t)stream;
-  QTRANS("hci_qtrans", in, M, out);
-  if (check) QTRANS_CHECK("hci_qtrans");
+  QTRANS("hci_qtrans", in, M, out, nullptr);
+  if (check && qtrans_tc_check(st) != HCI_OK)
+    return hci_fail(nullptr, HCI_ERR_CUDA, "hci_qtrans: a quarter transform gave up waiting for its tensor-core products");
   return HCI_OK;
 }
 
@@ -367,7 +661,7 @@ namespace {
 constexpr int NOALLOC_MAXORB = 32;
 constexpr size_t NOALLOC_T4 = (size_t)NOALLOC_MAXORB * NOALLOC_MAXORB * NOALLOC_MAXORB * NOALLOC_MAXORB;
 constexpr size_t NOALLOC_M = (size_t)NOALLOC_MAXORB * NOALLOC_MAXORB;
-constexpr size_t NOALLOC_DOUBLES = NOALLOC_T4 + 3 * NOALLOC_M + 32;   // 8.02 MiB
+constexpr size_t NOALLOC_DOUBLES = NOALLOC_T4 + W_FWD_COUNT * NOALLOC_M + 32;   // 8.08 MiB
 
 static __device__ __align__(256) double g_noalloc_scratch[NOALLOC_DOUBLES];
 
@@ -455,24 +749,5 @@ extern "C" hci_status hci_rotate_noalloc(int norb, const double* kappa, const do
   // every scratch element read below is written first in the same call, so
   // nothing has to be cleared; calls that overlap on the GPU share the array
   // and race
-  double* t4 = base;
-  double* w1 = base + NOALLOC_T4;
-  double* w2 = w1 + NOALLOC_M;
-  double* w3 = w2 + NOALLOC_M;
-  double* ds = w3 + NOALLOC_M;
-  s = expm_dev(st, n, kappa, U, w1, w2, w3, ds);
-  if (s != HCI_OK) return hci_fail(nullptr, s, "hci_rotate_noalloc: matrix exponential failed");
-  mm(st, n, h, 0, U, 0, w1, 1.0, 0.0);          // h U
-  mm(st, n, U, 1, w1, 0, h_out, 1.0, 0.0);      // U^T h U
-  QTRANS("hci_rotate_noalloc", eri, U, t4);
-  QTRANS("hci_rotate_noalloc", t4, U, eri_out);
-  QTRANS("hci_rotate_noalloc", eri_out, U, t4);
-  QTRANS("hci_rotate_noalloc", t4, U, eri_out);
-  symmetrize(st, n, h_out, eri_out);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return hci_fail(nullptr, HCI_ERR_CUDA, "hci_rotate_noalloc: %s", cudaGetErrorString(e));
-  e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return hci_fail(nullptr, HCI_ERR_CUDA, "hci_rotate_noalloc: %s", cudaGetErrorString(e));
-  QTRANS_CHECK("hci_rotate_noalloc");
-  return HCI_OK;
+  return rotate_core("hci_rotate_noalloc", st, n, kappa, h, eri, U, h_out, eri_out, base + NOALLOC_T4, base);
 }
