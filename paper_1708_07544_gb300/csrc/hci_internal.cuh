@@ -306,3 +306,25 @@ __device__ __forceinline__ double exc_phase(uint64_t s, int p, int r) {
   uint64_t mask = ((hi >= 64) ? ~0ull : ((1ull << hi) - 1ull)) & ~((2ull << lo) - 1ull);
   return (__popcll(s & mask) & 1) ? -1.0 : 1.0;
 }
+
+// flip the sign of v for an odd count
+__device__ __forceinline__ double flip_sign(double v, int odd) {
+  return __longlong_as_double(__double_as_longlong(v) ^ ((long long)(odd & 1) << 63));
+}
+// number of set bits of s strictly between orbitals p and r
+__device__ __forceinline__ int bits_between(uint64_t s, int p, int r) {
+  const int lo = p < r ? p : r, hi = p < r ? r : p;
+  return __popcll(s & ((1ull << hi) - 1ull) & ~((2ull << lo) - 1ull));
+}
+
+// the row of logical entry e < rowptr[nV] (the last row that starts at or
+// before it and is not empty there)
+__device__ __forceinline__ int64_t row_of_entry(const int64_t* __restrict__ rowptr, int64_t nV, int64_t e) {
+  int64_t lo = 0, hi = nV;         // first row with rowptr[row + 1] > e
+  while (lo < hi) {
+    const int64_t mid = (lo + hi) >> 1;
+    if (rowptr[mid + 1] > e) hi = mid;
+    else lo = mid + 1;
+  }
+  return lo;
+}

@@ -16,8 +16,8 @@
 // One orientation of each connected pair is accumulated (the graph stores
 // one, or both) and the other added as its transpose.  The diagonal part is
 // reduced through the weighted
-// occupation correlation M[sp][tq] = sum_i c_i^2 n_sp(i) n_tq(i), folded over
-// the alpha and beta string groups of the graph.
+// occupation correlation M[sp][tq] = sum_i c_i^2 n_sp(i) n_tq(i), summed from
+// the orbitals in which each determinant differs from the aufbau one.
 #include "hci_internal.cuh"
 #include "rdm_acc.cuh"
 
@@ -26,34 +26,128 @@ namespace {
 constexpr int R_WARPS = 8;
 
 
-// One warp per row from a queue.  One-orientation graphs: every stored entry
-// is one orientation of a connected pair; both-orientation graphs: the
-// entries with j > i are.
-__global__ void __launch_bounds__(R_WARPS * 32) k_rdm_offdiag(int n, const ulonglong2* __restrict__ V, int64_t nV,
-                                                              const double* __restrict__ c,
+// A determinant with its coefficient, one 32-byte sector, gathered by one
+// 32-byte load per lane: gathers and additions each take a lane's turn in
+// the L1's address stage (one per clock per SM), which bounds the kernels
+// below, so the key and the coefficient take one turn instead of two.
+struct __align__(32) DetC {
+  uint64_t a, b;
+  double c;
+  uint64_t pad;
+};
+__global__ void k_pack_det(const ulonglong2* __restrict__ V, const double* __restrict__ c, int64_t nV,
+                           DetC* __restrict__ out) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nV; i += (int64_t)gridDim.x * blockDim.x)
+    out[i] = DetC{V[i].x, V[i].y, c[i], 0ull};
+}
+__device__ __forceinline__ void load_det(const DetC* p, ulonglong2& k, double& c) {
+  uint64_t x, y, z, u;
+  asm volatile("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(x), "=l"(y), "=l"(z), "=l"(u) : "l"(p));
+  k = make_ulonglong2(x, y);
+  c = __longlong_as_double((long long)z);
+}
+
+// Chunks of RQ_CHUNK stored entries from a queue, whatever rows they belong to
+// (a row of 1e5 entries left to one warp is a tail several times as long as
+// all the rest).  One-orientation graphs: every stored entry is one
+// orientation of a connected pair; both-orientation graphs: the entries with
+// j > i are.  The pairs to accumulate are queued per
+// warp (half of a full row's entries are the other orientation's) and looked
+// at 32 at a time; alpha-beta doubles, most of them, are added at once,
+// same-spin doubles and singles (whose spectators loop) are queued again by
+// kind, so that no lane waits through another kind's code.  (44e,44o), 4.9e8
+// pairs: 15.4 ms with every kind in place and 2 to 4 atomics per double,
+// 5.2 ms so.
+constexpr int RQ_CHUNK = 2048;
+
+__global__ void __launch_bounds__(R_WARPS * 32) k_rdm_offdiag(int n, const DetC* __restrict__ V, int64_t nV,
                                                               const int64_t* __restrict__ rowptr,
                                                               const int64_t* __restrict__ rowstart,
                                                               const __grid_constant__ SegTab T, int both, RdmAcc R,
                                                               unsigned long long* __restrict__ queue) {
+  __shared__ int2 s_q[R_WARPS][3][64];
   const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  int2(*q)[64] = s_q[threadIdx.x >> 5];
+  int nq = 0, ns = 0, n1 = 0;        // queued pairs, same-spin doubles, singles
+  auto shift = [&](int2* w, int& cnt, int m) {
+    const int2 rest = lane + m < cnt ? w[lane + m] : make_int2(0, 0);
+    __syncwarp();
+    if (lane + m < cnt) w[lane] = rest;
+    cnt -= m;
+    __syncwarp();
+  };
+  auto take_kind = [&](int kind, int& cnt, int m) {
+    __syncwarp();
+    if (lane < m) {
+      const int2 p = q[kind][lane];
+      ulonglong2 ki, kj;
+      double ci, cj;
+      load_det(V + p.x, ki, ci);
+      load_det(V + p.y, kj, cj);
+      const double cc = ci * cj;
+      if (cc != 0.0) {
+        if (kind == 2) rdm_single(R, n, ki, kj, cc);
+        else if (ki.y == kj.y) rdm_same(R, n, ki.x, kj.x, cc);
+        else rdm_same(R, n, ki.y, kj.y, cc);
+      }
+    }
+    shift(q[kind], cnt, m);
+  };
+  auto take = [&](int m) {   // the first m <= 32 queued pairs
+    __syncwarp();
+    bool same = false, one = false;
+    int2 p = make_int2(0, 0);
+    if (lane < m) {
+      p = q[0][lane];
+      ulonglong2 ki, kj;
+      double ci, cj;
+      load_det(V + p.x, ki, ci);
+      load_det(V + p.y, kj, cj);
+      const int da = __popcll(ki.x ^ kj.x), db = __popcll(ki.y ^ kj.y);
+      one = da + db == 2;
+      same = !one && da != db;
+      const double cc = ci * cj;
+      if (!one && !same && cc != 0.0) rdm_mixed(R, n, ki, kj, cc);
+    }
+    const unsigned bs = __ballot_sync(0xffffffffu, same), b1 = __ballot_sync(0xffffffffu, one);
+    if (same) q[1][ns + __popc(bs & lt)] = p;
+    if (one) q[2][n1 + __popc(b1 & lt)] = p;
+    ns += __popc(bs);
+    n1 += __popc(b1);
+    shift(q[0], nq, m);
+    if (ns >= 32) take_kind(1, ns, 32);
+    if (n1 >= 32) take_kind(2, n1, 32);
+  };
+  const int64_t total = rowptr[nV];
   while (true) {
     unsigned long long qi = 0;
-    if (lane == 0) qi = atomicAdd(queue, 1ull);
-    const int64_t i = (int64_t)__shfl_sync(0xffffffffu, qi, 0);
-    if (i >= nV) break;
-    const double ci = c[i];
-    if (ci == 0.0) continue;
-    const ulonglong2 ki = V[i];
-    const int64_t rs = rowstart[i], len = rowptr[i + 1] - rowptr[i];
-    const int32_t* col = T.col[rs >> GRAPH_SEG_SHIFT] + (rs & GRAPH_SEG_MASK);
-    for (int64_t k = lane; k < len; k += 32) {
-      const int64_t j = col[k];
-      if (both && j <= i) continue;
-      const double cc = ci * c[j];
-      if (cc == 0.0) continue;
-      rdm_accumulate(R, n, ki, V[j], cc);
+    if (lane == 0) qi = atomicAdd(queue, (unsigned long long)RQ_CHUNK);
+    const int64_t e0 = (int64_t)__shfl_sync(0xffffffffu, qi, 0);
+    if (e0 >= total) break;
+    const int64_t e1 = e0 + RQ_CHUNK < total ? e0 + RQ_CHUNK : total;
+    int64_t e = e0;
+    for (int64_t i = row_of_entry(rowptr, nV, e0); e < e1; ++i) {
+      const int64_t lo = rowptr[i], hi = rowptr[i + 1] < e1 ? rowptr[i + 1] : e1;
+      const int64_t rs = rowstart[i], off = e - lo, len = hi - e;
+      e = hi;
+      if (len <= 0 || V[i].c == 0.0) continue;
+      const int32_t* col = T.col[rs >> GRAPH_SEG_SHIFT] + (rs & GRAPH_SEG_MASK) + off;
+      int32_t jn = lane < len ? __ldcs(col + lane) : -1;
+      for (int64_t k0 = 0; k0 < len; k0 += 32) {
+        const int32_t j = jn;
+        jn = k0 + 32 + lane < len ? __ldcs(col + k0 + 32 + lane) : -1;
+        const bool ok = j >= 0 && (!both || j > i);
+        const unsigned b = __ballot_sync(0xffffffffu, ok);
+        if (ok) q[0][nq + __popc(b & lt)] = make_int2((int)i, j);
+        nq += __popc(b);
+        if (nq >= 32) take(32);
+      }
     }
   }
+  if (nq > 0) take(nq);
+  if (ns > 0) take_kind(1, ns, ns);
+  if (n1 > 0) take_kind(2, n1, n1);
 }
 
 // Single-excitation spectator sums: Xt[b][a][k] over both spins,
@@ -62,12 +156,12 @@ __device__ __forceinline__ double rdm_xt(const RdmAcc& R, int n, int b, int a, i
   const int64_t ba = (int64_t)b * n + a;
   const double s = R.S1[ba] + R.S1[(int64_t)n * n + ba];
   const int occ = (int)((R.ref_a >> k) & 1ull) + (int)((R.ref_b >> k) & 1ull) - (k == a);
-  return s * occ + R.Dt[ba * n + k];
+  return s * occ + R.Ds[ba * n + k] + R.Do[ba * n + k];
 }
 __device__ __forceinline__ double rdm_xx(const RdmAcc& R, int n, int b, int a, int k) {
   const int64_t ba = (int64_t)b * n + a;
   const int oa = (int)((R.ref_a >> k) & 1ull) - (k == a), ob = (int)((R.ref_b >> k) & 1ull) - (k == a);
-  return R.S1[ba] * oa + R.S1[(int64_t)n * n + ba] * ob + R.Dx[ba * n + k];
+  return R.S1[ba] * oa + R.S1[(int64_t)n * n + ba] * ob + R.Ds[ba * n + k];
 }
 // the single-excitation terms of one orientation at (p,q,r,s)
 __device__ __forceinline__ double rdm_single_terms(const RdmAcc& R, int n, int p, int q, int r, int s) {
@@ -79,17 +173,28 @@ __device__ __forceinline__ double rdm_single_terms(const RdmAcc& R, int n, int p
   return v;
 }
 
-// rdm2 += Hh + single terms, rdm1 += S1 (the accumulated orientation), and
+// the doubles of one orientation at (p,q,r,s): alpha-beta pairs in both
+// orders, same-spin pairs with the sign of their particles' and holes' order
+__device__ __forceinline__ double rdm_double_terms(const RdmAcc& R, int n, int p, int q, int r, int s) {
+  const int64_t pq = (int64_t)p * n + q, rs = (int64_t)r * n + s, n2 = (int64_t)n * n;
+  double v = R.Hm[pq * n2 + rs] + R.Hm[rs * n2 + pq];
+  if (p != r && q != s) {
+    const int np = n * (n - 1) / 2;
+    const double x = R.Hs[(int64_t)(p < r ? tri_index(p, r) : tri_index(r, p)) * np +
+                          (q < s ? tri_index(q, s) : tri_index(s, q))];
+    v += (p < r) == (q < s) ? x : -x;
+  }
+  return v;
+}
+
+// rdm2 += doubles + single terms, rdm1 += S1 (the accumulated orientation), and
 // with sym also their transposes (the other orientation of every pair)
 __global__ void k_rdm_finish(int n, RdmAcc R, double* __restrict__ r1, double* __restrict__ r2, int sym) {
   const int64_t n2 = (int64_t)n * n, n4 = n2 * n2;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n4; t += (int64_t)gridDim.x * blockDim.x) {
     const int s = (int)(t % n), r = (int)((t / n) % n), q = (int)((t / n2) % n), p = (int)(t / (n2 * n));
-    double v = R.Hh[t] + rdm_single_terms(R, n, p, q, r, s);
-    if (sym) {
-      const int64_t tt = (((int64_t)q * n + p) * n + s) * n + r;
-      v += R.Hh[tt] + rdm_single_terms(R, n, q, p, s, r);
-    }
+    double v = rdm_double_terms(R, n, p, q, r, s) + rdm_single_terms(R, n, p, q, r, s);
+    if (sym) v += rdm_double_terms(R, n, q, p, s, r) + rdm_single_terms(R, n, q, p, s, r);
     r2[t] += v;
     if (t < n2) {
       const int pp = (int)(t / n), qq = (int)(t % n);
@@ -113,8 +218,8 @@ __global__ void k_rdm_pairs(int n, const ulonglong2* __restrict__ V, const doubl
   }
 }
 
-// Occupation correlation sum_a w_a n(a) n(a)^T of the distinct targets (the
-// listed pairs j = list[0 .. *nlist), w_a = d_j^2), over spin orbitals
+// Occupation correlation sum_a w_a n(a) n(a)^T, w_a = d_a^2, of determinants
+// tgt[j] (j = 0 .. m - 1, or the listed j = list[0 .. *nlist)), over spin orbitals
 // (alpha 0..n-1, beta n..2n-1), split about the aufbau occupations n_R:
 // n(a) = n_R + delta_a.  A changed spin orbital k has delta_k = s_k, -1 when
 // n_R holds it and +1 when not, so only the weights P_kl = sum of w over the
@@ -122,22 +227,24 @@ __global__ void k_rdm_pairs(int n, const ulonglong2* __restrict__ V, const doubl
 // with W = sum w: about 36 additions per target.  They go to L2 as FP64
 // reductions without return, spread over DD_COPIES copies [W, P (2n x 2n)]
 // so that the frontier orbitals' entries do not queue up at one address.
+// The same sums with w = c_i^2 over V are the diagonal part of the RDMs
+// (3.0e5 determinants: 82 + 700 + 21 us by string groups, 34 us so).
 // FP64 additions in shared memory are compare-and-swap loops: block-local
 // copies there took 71.4 ms for the pairs of a (44e,44o) state at eps2 = 2e-5,
 // this 4.7 ms.
 constexpr int DD_COPIES = 64;
 
 __global__ void __launch_bounds__(256) k_dd_acc(int n, const ulonglong2* __restrict__ tgt, const double* __restrict__ d,
-                                                const int64_t* __restrict__ list,
+                                                int64_t m, const int64_t* __restrict__ list,
                                                 const unsigned long long* __restrict__ nlist, uint64_t ra, uint64_t rb,
                                                 double* __restrict__ acc) {
   const int mm = 2 * n;
   double* A = acc + (int64_t)(blockIdx.x % DD_COPIES) * (1 + mm * mm);
   double* P = A + 1;
   double wsum = 0.0;
-  const int64_t nt = (int64_t)*nlist;
+  const int64_t nt = list ? (int64_t)*nlist : m;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nt; q += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t j = list[q];
+    const int64_t j = list ? list[q] : q;
     const double dj = d[j];
     if (dj == 0.0) continue;
     const ulonglong2 key = tgt[j];
@@ -184,196 +291,6 @@ __global__ void k_dd_matrix(int n, const double* __restrict__ sum, uint64_t ra, 
   }
 }
 
-// M[s*n+p][t*n+q] = sum_i c_i^2 n_sp(i) n_tq(i), folded over the string
-// groups of the cached graph:
-//  1. W_g = sum_{i in g} c_i^2 and v_g[q] = sum_{i in g} c_i^2 n_q(beta_i)
-//     per alpha group g, Wb_h = sum_{i in h} c_i^2 per beta group h.
-//  2. one thread per M entry and block per slice of groups: alpha-alpha
-//     entries sum W_g over groups with p, q in alpha_g, alpha-beta entries
-//     sum v_g[q] over groups with p in alpha_g, beta-beta entries sum Wb_h;
-//     the slices' partial M are added in a fixed order.
-// Step 1 cuts the determinants (alpha-major) and the beta-major positions
-// into chunks of GW_CH consecutive members, one warp per chunk, so that a
-// group holding a large share of the space is spread over many warps; each
-// warp adds its partial sums to the groups it touched with atomics.
-constexpr int GW_CH = 256;
-
-__global__ void __launch_bounds__(256) k_group_weights(int n, const ulonglong2* __restrict__ V,
-                                                       const double* __restrict__ c, const int32_t* __restrict__ ia,
-                                                       int64_t nV, const int32_t* __restrict__ permb,
-                                                       const int32_t* __restrict__ ib, double* __restrict__ Wa,
-                                                       double* __restrict__ va, double* __restrict__ Wb) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t nch = (nV + GW_CH - 1) / GW_CH;
-  for (int64_t ch = warp; ch < 2 * nch; ch += nwarps) {
-    const bool beta = ch >= nch;
-    const int64_t i0 = (beta ? ch - nch : ch) * GW_CH;
-    const int64_t i1 = i0 + GW_CH < nV ? i0 + GW_CH : nV;
-    if (!beta) {
-      // members in order; lane q accumulates orbitals q and q + 32
-      // (broadcast loads, eight members fetched ahead)
-      int g = ia[i0];
-      double W = 0.0, v0 = 0.0, v1 = 0.0;
-      for (int64_t ib0 = i0; ib0 < i1; ib0 += 8) {
-        int gg[8];
-        double cw[8];
-        uint64_t yy[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int64_t i = ib0 + u;
-          gg[u] = i < i1 ? ia[i] : g;
-          cw[u] = i < i1 ? c[i] : 0.0;
-          yy[u] = i < i1 ? V[i].y : 0ull;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          if (gg[u] != g) {
-            if (lane == 0) atomicAdd(&Wa[g], W);
-            if (lane < n) atomicAdd(&va[(int64_t)g * n + lane], v0);
-            if (lane + 32 < n) atomicAdd(&va[(int64_t)g * n + lane + 32], v1);
-            g = gg[u];
-            W = v0 = v1 = 0.0;
-          }
-          const double w = cw[u] * cw[u];
-          W += w;
-          if ((yy[u] >> lane) & 1ull) v0 += w;
-          if ((yy[u] >> (lane + 32)) & 1ull) v1 += w;
-        }
-      }
-      if (lane == 0) atomicAdd(&Wa[g], W);
-      if (lane < n) atomicAdd(&va[(int64_t)g * n + lane], v0);
-      if (lane + 32 < n) atomicAdd(&va[(int64_t)g * n + lane + 32], v1);
-    } else {
-      // one member per lane; groups are runs of consecutive positions, so a
-      // sum over the lanes of equal group (shuffles down) leaves each run's
-      // total in its first lane
-      for (int64_t k0 = i0; k0 < i1; k0 += 32) {
-        const int64_t k = k0 + lane;
-        int h = -1;
-        double w = 0.0;
-        if (k < i1) {
-          const int32_t d = permb[k];
-          h = ib[d];
-          w = c[d] * c[d];
-        }
-        for (int o = 1; o < 32; o <<= 1) {
-          const double ow = __shfl_down_sync(0xffffffffu, w, o);
-          const int oh = __shfl_down_sync(0xffffffffu, h, o);
-          if (lane + o < 32 && oh == h) w += ow;
-        }
-        const int hp = __shfl_up_sync(0xffffffffu, h, 1);
-        if (h >= 0 && (lane == 0 || hp != h)) atomicAdd(&Wb[h], w);
-      }
-    }
-  }
-}
-
-constexpr int OCC_SLICES = 256;
-
-__global__ void k_occ_sums(int n, const ulonglong2* __restrict__ V, const int64_t* __restrict__ ga, int64_t nua,
-                           const ulonglong2* __restrict__ bk, const int64_t* __restrict__ gb, int64_t nub,
-                           const double* __restrict__ Wa, const double* __restrict__ va,
-                           const double* __restrict__ Wb, double* __restrict__ part) {
-  // blockIdx.x: slice of groups, staged in shared memory in chunks; thread
-  // t < 3n^2 owns one entry of the alpha-alpha (t < n^2), alpha-beta
-  // (t < 2n^2) or beta-beta block
-  constexpr int CH = 128;
-  __shared__ uint64_t s_a[CH];
-  __shared__ double s_w[CH];
-  __shared__ double s_v[CH * HCI_MAXORB / 2];   // n <= 64: CH x n doubles staged in two halves
-  const int m = 2 * n;
-  const int64_t slice = blockIdx.x;
-  const int64_t a0 = nua * slice / OCC_SLICES, a1 = nua * (slice + 1) / OCC_SLICES;
-  const int64_t b0 = nub * slice / OCC_SLICES, b1 = nub * (slice + 1) / OCC_SLICES;
-  const int nt = 3 * n * n;
-  double acc[12];
-  for (int r = 0; r < 12; ++r) acc[r] = 0.0;
-  // alpha groups: strings, weights and v in chunks
-  for (int64_t g0 = a0; g0 < a1; g0 += CH) {
-    const int cnt = (int)(a1 - g0 < CH ? a1 - g0 : CH);
-    for (int half = 0; half < 2; ++half) {
-      const int q0 = half * (n / 2), q1 = half == 0 ? n / 2 : n;
-      const int nq = q1 - q0;
-      __syncthreads();
-      for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-        s_a[t] = V[ga[g0 + t]].x;
-        s_w[t] = Wa[g0 + t];
-      }
-      for (int t = threadIdx.x; t < cnt * nq; t += blockDim.x) {
-        const int gi = t / nq, qq = t % nq;
-        s_v[gi * nq + qq] = va[(g0 + gi) * n + q0 + qq];
-      }
-      __syncthreads();
-      int r = 0;
-      for (int t = threadIdx.x; t < nt; t += blockDim.x, ++r) {
-        if (t < n * n) {
-          if (half) continue;
-          const int p = t / n, q = t % n;
-          double a = 0.0;
-          for (int gi = 0; gi < cnt; ++gi) {
-            const uint64_t x = s_a[gi];
-            if (((x >> p) & 1ull) && ((x >> q) & 1ull)) a += s_w[gi];
-          }
-          acc[r] += a;
-        } else if (t < 2 * n * n) {
-          const int u = t - n * n, p = u / n, q = u % n;
-          if (q < q0 || q >= q1) continue;
-          double a = 0.0;
-          for (int gi = 0; gi < cnt; ++gi)
-            if ((s_a[gi] >> p) & 1ull) a += s_v[gi * nq + (q - q0)];
-          acc[r] += a;
-        }
-      }
-    }
-  }
-  // beta groups
-  for (int64_t h0 = b0; h0 < b1; h0 += CH) {
-    const int cnt = (int)(b1 - h0 < CH ? b1 - h0 : CH);
-    __syncthreads();
-    for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-      s_a[t] = bk[gb[h0 + t]].x;
-      s_w[t] = Wb[h0 + t];
-    }
-    __syncthreads();
-    int r = 0;
-    for (int t = threadIdx.x; t < nt; t += blockDim.x, ++r) {
-      if (t < 2 * n * n) continue;
-      const int u = t - 2 * n * n, p = u / n, q = u % n;
-      double a = 0.0;
-      for (int gi = 0; gi < cnt; ++gi) {
-        const uint64_t x = s_a[gi];
-        if (((x >> p) & 1ull) && ((x >> q) & 1ull)) a += s_w[gi];
-      }
-      acc[r] += a;
-    }
-  }
-  int r = 0;
-  double* P = part + slice * (int64_t)m * m;
-  for (int t = threadIdx.x; t < nt; t += blockDim.x, ++r) {
-    if (t < n * n) {
-      const int p = t / n, q = t % n;
-      P[p * m + q] = acc[r];
-    } else if (t < 2 * n * n) {
-      const int u = t - n * n, p = u / n, q = u % n;
-      P[p * m + n + q] = acc[r];
-      P[(n + q) * m + p] = acc[r];
-    } else {
-      const int u = t - 2 * n * n, p = u / n, q = u % n;
-      P[(n + p) * m + n + q] = acc[r];
-    }
-  }
-}
-
-__global__ void k_sum_slices(int mm, const double* __restrict__ part, double* __restrict__ M) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= mm) return;
-  double s = 0.0;
-  for (int k = 0; k < OCC_SLICES; ++k) s += part[(int64_t)k * mm + t];
-  M[t] = s;
-}
-
 // diagonal contributions from M
 __global__ void k_diag_rdm(int n, const double* __restrict__ M, double* __restrict__ r1, double* __restrict__ r2) {
   const int m = 2 * n;
@@ -395,6 +312,11 @@ __global__ void k_diag_rdm(int n, const double* __restrict__ M, double* __restri
 
 }  // namespace
 
+static RdmAcc ctx_acc(hci_ctx* ctx) {
+  return rdm_acc_at(bp<double>(ctx->s_rdmh), (size_t)ctx->n, ctx->na == 64 ? ~0ull : ((1ull << ctx->na) - 1ull),
+                    ctx->nb == 64 ? ~0ull : ((1ull << ctx->nb) - 1ull));
+}
+
 extern "C" hci_status hci_rdm12(hci_ctx* ctx, const uint64_t* keys, int64_t nV, const double* c, double* rdm1,
                                 double* rdm2) {
   if (!ctx) return hci_fail(nullptr, HCI_ERR_INVALID, "hci_rdm12: null context");
@@ -407,53 +329,41 @@ extern "C" hci_status hci_rdm12(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
   const size_t n2 = (size_t)n * n, n4 = n2 * n2;
   HCI_CUDA(ctx, cudaMemsetAsync(rdm1, 0, n2 * 8, st));
   HCI_CUDA(ctx, cudaMemsetAsync(rdm2, 0, n4 * 8, st));
-  HCI_TRY(ensure_buf(ctx, ctx->s_misc, (size_t)4 * n2 * 8 + 64));
-  double* M = bp<double>(ctx->s_misc);
-  HCI_CUDA(ctx, cudaMemsetAsync(M, 0, 4 * n2 * 8, st));
   prof_tic(ctx, HCI_PH_RDM_DIAG);
-  const ulonglong2* V = bp<ulonglong2>(ctx->graph.keys);
-  {
-    const Graph& G = ctx->graph;
-    const int64_t nua = G.nua, nub = G.nub;
-    const size_t mm = (size_t)4 * n2;
-    HCI_TRY(ensure_buf(ctx, ctx->s_rdmw, (size_t)(nua + nub + nua * n + 16) * 8 + (size_t)OCC_SLICES * mm * 8));
-    double* Wa = bp<double>(ctx->s_rdmw);
-    double* Wb = Wa + nua;
-    double* va = Wb + nub;
-    double* part = va + nua * n;
-    HCI_CUDA(ctx, cudaMemsetAsync(Wa, 0, (size_t)(nua + nub + nua * n) * 8, st));
-    HCI_LAUNCH(k_group_weights, grid_for(2 * ((nV + GW_CH - 1) / GW_CH) * 32, 256), 256, 0, st)(
-        n, V, c, bp<int32_t>(ctx->g_ia), nV, bp<int32_t>(ctx->g_permb), bp<int32_t>(ctx->g_ib), Wa, va, Wb);
-    HCI_LAUNCH(k_occ_sums, OCC_SLICES, 1024, 0, st)(n, V, bp<int64_t>(ctx->g_ga), nua, bp<ulonglong2>(ctx->g_bkeys),
-                                                   bp<int64_t>(ctx->g_gb), nub, Wa, va, Wb, part);
-    HCI_LAUNCH(k_sum_slices, (unsigned)((mm + 255) / 256), 256, 0, st)((int)mm, part, M);
-  }
+  // diagonal part: M[s*n+p][t*n+q] = sum_i c_i^2 n_sp(i) n_tq(i)
+  const int cnt = 1 + 4 * n * n;
+  HCI_TRY(ensure_buf(ctx, ctx->s_rdmw, ((size_t)(DD_COPIES + 1) * cnt + 4 * n2) * 8));
+  double* acc = bp<double>(ctx->s_rdmw);
+  double* sum = acc + (size_t)DD_COPIES * cnt;
+  double* M = sum + cnt;
+  const uint64_t ra = ctx->na == 64 ? ~0ull : ((1ull << ctx->na) - 1ull);
+  const uint64_t rb = ctx->nb == 64 ? ~0ull : ((1ull << ctx->nb) - 1ull);
+  HCI_CUDA(ctx, cudaMemsetAsync(acc, 0, (size_t)DD_COPIES * cnt * 8, st));
+  HCI_LAUNCH(k_dd_acc, grid_for(nV, 256, ctx->nsm * 8), 256, 0, st)(n, bp<ulonglong2>(ctx->graph.keys), c, nV, nullptr,
+                                                                   nullptr, ra, rb, acc);
+  HCI_LAUNCH(k_dd_sum, (unsigned)((cnt + 255) / 256), 256, 0, st)(cnt, acc, sum);
+  HCI_LAUNCH(k_dd_matrix, grid_for((int64_t)4 * n2, 256), 256, 0, st)(n, sum, ra, rb, M);
   HCI_LAUNCH(k_diag_rdm, grid_for((int64_t)n2, 256), 256, 0, st)(n, M, rdm1, rdm2);
   prof_toc(ctx, HCI_PH_RDM_DIAG);
   HCI_TRY(ensure_buf(ctx, ctx->s_counter, 64));
   unsigned long long* queue = reinterpret_cast<unsigned long long*>(bp<char>(ctx->s_counter) + 56);
   HCI_CUDA(ctx, cudaMemsetAsync(queue, 0, 8, st));
   // the connections are stored by internal id
-  HCI_TRY(ensure_buf(ctx, ctx->d_perm, (size_t)nV * 8));
-  double* ci = bp<double>(ctx->d_perm);
+  HCI_TRY(ensure_buf(ctx, ctx->d_perm, (size_t)nV * 40 + 32));
+  DetC* det = bp<DetC>(ctx->d_perm);
+  double* ci = reinterpret_cast<double*>(det + nV);
   HCI_TRY(to_internal(ctx, c, ci, 1));
-  const size_t n3 = n2 * n;
-  HCI_TRY(ensure_buf(ctx, ctx->s_rdmh, (n4 + 2 * n2 + 2 * n3) * 8));
-  HCI_CUDA(ctx, cudaMemsetAsync(ctx->s_rdmh.p, 0, (n4 + 2 * n2 + 2 * n3) * 8, st));
-  RdmAcc R;
-  R.Hh = bp<double>(ctx->s_rdmh);
-  R.S1 = R.Hh + n4;
-  R.Dt = R.S1 + 2 * n2;
-  R.Dx = R.Dt + n3;
-  R.ref_a = ctx->na == 64 ? ~0ull : ((1ull << ctx->na) - 1ull);
-  R.ref_b = ctx->nb == 64 ? ~0ull : ((1ull << ctx->nb) - 1ull);
+  HCI_TRY(ensure_buf(ctx, ctx->s_rdmh, rdm_acc_doubles(n) * 8));
+  HCI_CUDA(ctx, cudaMemsetAsync(ctx->s_rdmh.p, 0, rdm_acc_doubles(n) * 8, st));
+  const RdmAcc R = ctx_acc(ctx);
   if (ctx->graph.direct)
     HCI_TRY(direct_rdm(ctx, ci, R));   // connections searched again, one orientation each
-  else
-    HCI_LAUNCH(k_rdm_offdiag, ctx->nsm * 8, R_WARPS * 32, 0, st)(n, bp<ulonglong2>(ctx->graph.keys_int), nV, ci,
-                                                                 bp<int64_t>(ctx->graph.rowptr),
+  else {
+    HCI_LAUNCH(k_pack_det, grid_for(nV, 256), 256, 0, st)(bp<ulonglong2>(ctx->graph.keys_int), ci, nV, det);
+    HCI_LAUNCH(k_rdm_offdiag, ctx->nsm * 8, R_WARPS * 32, 0, st)(n, det, nV, bp<int64_t>(ctx->graph.rowptr),
                                                                  bp<int64_t>(ctx->graph.rowstart), ctx->graph.tab(),
                                                                  ctx->graph.half ? 0 : 1, R, queue);
+  }
   HCI_LAUNCH(k_rdm_finish, grid_for((int64_t)n4, 256, ctx->nsm * 8), 256, 0, st)(n, R, rdm1, rdm2, 1);
   HCI_CUDA(ctx, cudaGetLastError());
   prof_toc(ctx, HCI_PH_RDM);
@@ -495,22 +405,10 @@ extern "C" hci_status hci_spin_square(hci_ctx* ctx, const double* rdm2, double* 
 
 // Density matrices of the perturbative correction, accumulated over the
 // hash classes of hci_pt2: begin (clear), pairs (once per class), finish.
-static RdmAcc pt2_acc(hci_ctx* ctx) {
-  const size_t n = (size_t)ctx->n, n2 = n * n, n4 = n2 * n2;
-  RdmAcc R;
-  R.Hh = bp<double>(ctx->s_rdmh);
-  R.S1 = R.Hh + n4;
-  R.Dt = R.S1 + 2 * n2;
-  R.Dx = R.Dt + n2 * n;
-  R.ref_a = ctx->na == 64 ? ~0ull : ((1ull << ctx->na) - 1ull);
-  R.ref_b = ctx->nb == 64 ? ~0ull : ((1ull << ctx->nb) - 1ull);
-  return R;
-}
-
 hci_status pt2_rdm_begin(hci_ctx* ctx) {
-  const size_t n = (size_t)ctx->n, n2 = n * n, n4 = n2 * n2, m = 2 * n;
-  HCI_TRY(ensure_buf(ctx, ctx->s_rdmh, (n4 + 2 * n2 + 2 * n2 * n) * 8));
-  HCI_CUDA(ctx, cudaMemsetAsync(ctx->s_rdmh.p, 0, (n4 + 2 * n2 + 2 * n2 * n) * 8, ctx->st));
+  const size_t n = (size_t)ctx->n, m = 2 * n;
+  HCI_TRY(ensure_buf(ctx, ctx->s_rdmh, rdm_acc_doubles(n) * 8));
+  HCI_CUDA(ctx, cudaMemsetAsync(ctx->s_rdmh.p, 0, rdm_acc_doubles(n) * 8, ctx->st));
   // the copies, their sum and M
   HCI_TRY(ensure_buf(ctx, ctx->p2_dd, ((DD_COPIES + 1) * (1 + m * m) + m * m) * 8));
   HCI_CUDA(ctx, cudaMemsetAsync(ctx->p2_dd.p, 0, DD_COPIES * (1 + m * m) * 8, ctx->st));
@@ -521,9 +419,9 @@ hci_status pt2_rdm_pairs(hci_ctx* ctx, const ulonglong2* V, const double* c, con
                          const double* d, int64_t m, const int64_t* list, const unsigned long long* nlist) {
   if (m <= 0) return HCI_OK;
   const int n = ctx->n;
-  RdmAcc R = pt2_acc(ctx);
+  RdmAcc R = ctx_acc(ctx);
   HCI_LAUNCH(k_rdm_pairs, grid_for(m, 256), 256, 0, ctx->st)(n, V, c, tgt, src, d, m, R);
-  HCI_LAUNCH(k_dd_acc, grid_for(m, 256, ctx->nsm * 8), 256, 0, ctx->st)(n, tgt, d, list, nlist, R.ref_a, R.ref_b,
+  HCI_LAUNCH(k_dd_acc, grid_for(m, 256, ctx->nsm * 8), 256, 0, ctx->st)(n, tgt, d, m, list, nlist, R.ref_a, R.ref_b,
                                                                        bp<double>(ctx->p2_dd));
   HCI_CUDA(ctx, cudaGetLastError());
   return HCI_OK;
@@ -533,7 +431,7 @@ hci_status pt2_rdm_finish(hci_ctx* ctx, double* r1dd, double* r2dd, double* r1dc
   const int n = ctx->n, mm = 2 * n;
   const size_t n2 = (size_t)n * n, n4 = n2 * n2;
   cudaStream_t st = ctx->st;
-  RdmAcc R = pt2_acc(ctx);
+  RdmAcc R = ctx_acc(ctx);
   HCI_CUDA(ctx, cudaMemsetAsync(r1dc, 0, n2 * 8, st));
   HCI_CUDA(ctx, cudaMemsetAsync(r2dc, 0, n4 * 8, st));
   HCI_LAUNCH(k_rdm_finish, grid_for((int64_t)n4, 256, ctx->nsm * 8), 256, 0, st)(n, R, r1dc, r2dc, 0);

@@ -40,7 +40,7 @@ namespace {
 // term-by-term rule takes 17, then s squarings.  On FP64 issue alone a
 // product of 44 x 44 matrices takes 1.4 us over 16 SMs; as separate launches
 // (6.9 us a product, 1.5 us a Horner step, and the host's wait for the norm)
-// exp took 200 us, the chain 45 us.
+// exp took 200 us, the chain 39 us.
 // ---------------------------------------------------------------------------
 constexpr int CLM_T = 128;          // threads per CTA: one warp per FP64 pipe
 constexpr int CLM_NU = 4;           // entries per thread at most (8 CTAs: 16 x 32 of 64 x 64)
@@ -63,6 +63,7 @@ __device__ __forceinline__ int cl_size() {
 // this CTA's block of every matrix
 struct Tile {
   int i0, j0, ni, nj, cnt;
+  int rn, rj;            // ceil(2^18 / n), ceil(2^18 / nj)
 };
 __device__ __forceinline__ Tile cl_tile(int n) {
   const int c = cl_size(), r = cl_rank();
@@ -76,6 +77,8 @@ __device__ __forceinline__ Tile cl_tile(int n) {
   if (t.ni < 0) t.ni = 0;
   if (t.nj < 0) t.nj = 0;
   t.cnt = t.ni * t.nj;
+  t.rn = ((1 << 18) + n - 1) / n;
+  t.rj = t.nj > 0 ? ((1 << 18) + t.nj - 1) / t.nj : 0;
   return t;
 }
 
@@ -91,43 +94,50 @@ struct MM {
 // L2, after cl_sync.
 template <int NT, class F>
 __device__ __forceinline__ void cl_mm(int n, const Tile& t, const MM (&terms)[NT], double* sA, double* sB, F epi) {
-  double acc[CLM_NU];
+  double acc[CLM_NU], acc2[CLM_NU];     // two chains: one alone waits for its own latency
 #pragma unroll
-  for (int u = 0; u < CLM_NU; ++u) acc[u] = 0.0;
+  for (int u = 0; u < CLM_NU; ++u) acc[u] = acc2[u] = 0.0;
+  const int na = t.ni * n, nb = n * t.nj, most = na > nb ? na : nb;
 #pragma unroll
   for (int q = 0; q < NT; ++q) {
     const MM& m = terms[q];
     __syncthreads();
 #pragma unroll 4
-    for (int e = threadIdx.x; e < t.ni * n; e += CLM_T) {
-      const int i = e / n, k = e - i * n;
-      sA[e] = __ldcg(m.tA ? m.A + k * n + t.i0 + i : m.A + (t.i0 + i) * n + k);
-    }
-#pragma unroll 4
-    for (int e = threadIdx.x; e < n * t.nj; e += CLM_T) {
-      const int k = e / t.nj, j = e - k * t.nj;
-      sB[e] = __ldcg(m.tB ? m.B + (t.j0 + j) * n + k : m.B + k * n + t.j0 + j);
+    for (int e = threadIdx.x; e < most; e += CLM_T) {
+      // e / n and e / nj by multiplication (exact for e < 2^12)
+      const int i = (e * t.rn) >> 18, k = e - i * n, kb = (e * t.rj) >> 18, j = e - kb * t.nj;
+      double va = 0.0, vb = 0.0;
+      if (e < na) va = __ldcg(m.tA ? m.A + k * n + t.i0 + i : m.A + (t.i0 + i) * n + k);
+      if (e < nb) vb = __ldcg(m.tB ? m.B + (t.j0 + j) * n + kb : m.B + kb * n + t.j0 + j);
+      if (e < na) sA[e] = va;
+      if (e < nb) sB[e] = vb;
     }
     __syncthreads();
 #pragma unroll
     for (int u = 0; u < CLM_NU; ++u) {
       const int o = threadIdx.x + u * CLM_T;
       if (o >= t.cnt) break;
-      const int i = o / t.nj, j = o - i * t.nj;
+      const int i = (o * t.rj) >> 18, j = o - i * t.nj;
       const double* a = sA + i * n;
       const double* b = sB + j;
-      double v = acc[u];
+      double v = acc[u], v2 = acc2[u];
+      int k = 0;
 #pragma unroll 4
-      for (int k = 0; k < n; ++k) v = fma(a[k], b[k * t.nj], v);
+      for (; k + 2 <= n; k += 2) {
+        v = fma(a[k], b[k * t.nj], v);
+        v2 = fma(a[k + 1], b[(k + 1) * t.nj], v2);
+      }
+      if (k < n) v = fma(a[k], b[k * t.nj], v);
       acc[u] = v;
+      acc2[u] = v2;
     }
   }
 #pragma unroll
   for (int u = 0; u < CLM_NU; ++u) {
     const int o = threadIdx.x + u * CLM_T;
     if (o >= t.cnt) break;
-    const int i = o / t.nj;
-    epi(u, t.i0 + i, t.j0 + (o - i * t.nj), acc[u]);
+    const int i = (o * t.rj) >> 18;
+    epi(u, t.i0 + i, t.j0 + (o - i * t.nj), acc[u] + acc2[u]);
   }
 }
 
@@ -371,7 +381,8 @@ __global__ void k_sym8(int n, double* __restrict__ eri) {
 // d <= c with T[y][d][c][b] + T[y][c][d][b] (d < c), half the FP64 products
 // that bound this contraction.  Every block takes an equal share of the
 // n^2 (n + 1) / 2 rows, NT_CH staged at a time; thread t owns entries
-// t, t + 256, ... (44 orbitals: 302 us for all of J, 179 us so).
+// t, t + 256, ... (44 orbitals: 302 us for all of J, 156 us so with
+// three blocks per SM, 170 with two).
 constexpr int NT_CH = 48;
 template <int NACC>
 __global__ void __launch_bounds__(256) k_gemm_nt_part(int n, int64_t rows, const double* __restrict__ eri,
@@ -594,7 +605,7 @@ extern "C" hci_status hci_rotate_backward(int norb, const double* kappa, const d
   Scratch S{st};
   const size_t n2 = (size_t)n * n, n4 = n2 * n2;
   const int64_t rows = (int64_t)n2 * (n + 1) / 2;
-  const int nparts = (int)std::min<int64_t>(2 * hci_nsm(), (rows + 15) / 16);
+  const int nparts = (int)std::min<int64_t>(3 * hci_nsm(), (rows + 15) / 16);
   double *ws = S.get(W_COUNT * n2 + 2), *U = S.get(n2), *ta = S.get(n4), *tb = S.get(n4);
   double* part = dkappa ? S.get((size_t)nparts * n2) : nullptr;
   if (!ws || !U || !ta || !tb || (dkappa && !part))

@@ -113,16 +113,6 @@ __device__ __forceinline__ void warp_emit(bool emit, ulonglong2 key, double term
   if (cnt >= EM_FLUSH) emit_flush(B, cnt, A);
 }
 
-// flip the sign of v for an odd count
-__device__ __forceinline__ double flip_sign(double v, int odd) {
-  return __longlong_as_double(__double_as_longlong(v) ^ ((long long)(odd & 1) << 63));
-}
-// number of set bits of s strictly between orbitals p and r
-__device__ __forceinline__ int bits_between(uint64_t s, int p, int r) {
-  const int lo = p < r ? p : r, hi = p < r ? r : p;
-  return __popcll(s & ((1ull << hi) - 1ull) & ~((2ull << lo) - 1ull));
-}
-
 // The warp's next 32 determinants, one per lane (nV or above: none), or -1
 // at the queue's end.  An atomic per determinant would bound spaces of small
 // coefficients; the 32 lie nV / 32 apart, because determinants of large
