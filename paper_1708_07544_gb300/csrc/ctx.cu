@@ -386,6 +386,7 @@ extern "C" hci_status hci_destroy(hci_ctx* ctx) {
                     &ctx->graph.keys_int, &ctx->graph.s2i, &ctx->graph.i2s,
                     &ctx->d_perm, &ctx->s_rdmh, &ctx->inc.scr, &ctx->inc.stage,
                     &ctx->inc.roff, &ctx->inc.ctl, &ctx->inc.left, &ctx->inc.samp,
+                    &ctx->inc.items, &ctx->inc.first, &ctx->inc.itp,
                     &ctx->p2_vals, &ctx->p2_vals2, &ctx->p2_ref,
                     &ctx->p2_src, &ctx->p2_src2, &ctx->p2_d, &ctx->p2_dd, &ctx->p2_tab,
                     &ctx->d_zv, &ctx->d_rel, &ctx->d_lock, &ctx->d_partner, &ctx->dkeep.Q, &ctx->dkeep.W, &ctx->ss_w, &ctx->ss_draw,

@@ -31,8 +31,10 @@ namespace {
 constexpr int G_WARPS = 8;
 // blocks of the row search: six per SM, all resident at 40 registers
 inline int rows_grid(const hci_ctx* ctx) { return ctx->nsm * 6; }
-constexpr int64_t ROW_SCR = 32768;   // scratch entries per warp of the staged row search
-constexpr int64_t ROW_SAMPLE = 2048; // rows counted to size the staging buffer
+constexpr int64_t ROW_SCR = 8192;    // scratch entries per warp of the staged row search
+constexpr int64_t ROW_SAMPLE = 2048; // work items counted to size the staging buffer
+// pair checks per work item of the row search (see k_item_count)
+constexpr int64_t ITEM_COST = 16384;
 
 __device__ __forceinline__ bool key_less(ulonglong2 a, ulonglong2 b) {
   return a.x < b.x || (a.x == b.x && a.y < b.y);
@@ -181,7 +183,7 @@ __device__ __forceinline__ double single_el(const HamView& H, uint64_t sj, uint6
   for (uint64_t m = rs & ~sj; m; m &= m - 1) v -= js[__ffsll((long long)m) - 1];
   for (uint64_t m = oj & ~ro; m; m &= m - 1) v += jo[__ffsll((long long)m) - 1];
   for (uint64_t m = ro & ~oj; m; m &= m - 1) v -= jo[__ffsll((long long)m) - 1];
-  return exc_phase(sj, p, r) * v;
+  return flip_sign(v, bits_between(sj, p, r));
 }
 
 __device__ __forceinline__ double same_double_el(const HamView& H, uint64_t sj, uint64_t x) {
@@ -190,10 +192,8 @@ __device__ __forceinline__ double same_double_el(const HamView& H, uint64_t sj, 
   int q = __ffsll((long long)holes) - 1;
   int r = __ffsll((long long)parts) - 1; parts &= parts - 1;
   int s = __ffsll((long long)parts) - 1;
-  double s1 = exc_phase(sj, p, r);
-  uint64_t t = sj ^ (1ull << p) ^ (1ull << r);
-  double s2 = exc_phase(t, q, s);
-  return s1 * s2 * (eri4(H, p, r, q, s) - eri4(H, p, s, q, r));
+  const uint64_t t = sj ^ (1ull << p) ^ (1ull << r);
+  return flip_sign(eri4(H, p, r, q, s) - eri4(H, p, s, q, r), bits_between(sj, p, r) + bits_between(t, q, s));
 }
 
 __device__ double connection_el(const HamView& H, ulonglong2 ki, ulonglong2 kj) {
@@ -215,7 +215,7 @@ __device__ double connection_el(const HamView& H, ulonglong2 ki, ulonglong2 kj) 
   }
   int p = __ffsll((long long)(kj.x & xa)) - 1, r = __ffsll((long long)(ki.x & xa)) - 1;
   int q = __ffsll((long long)(kj.y & xb)) - 1, s = __ffsll((long long)(ki.y & xb)) - 1;
-  return exc_phase(kj.x, p, r) * exc_phase(kj.y, q, s) * eri4(H, p, r, q, s);
+  return flip_sign(eri4(H, p, r, q, s), bits_between(kj.x, p, r) + bits_between(kj.y, q, s));
 }
 
 // ---------------------------------------------------------------------------
@@ -240,26 +240,24 @@ struct GraphArgs {
   const int32_t* bnbr;
   const int64_t* costa;    // cost of the alpha-side (C) search per distinct alpha string
   const int64_t* costb;
-  const int32_t* rowlist;  // rows to process (nullptr: all rows, in order)
-  int64_t nrows;
-  const int64_t* rowptr;   // fill pass: output offset per processed row
+  const int4* items;       // work items {row, its number in the row list, part, parts}
+  int64_t nitems;
+  const int64_t* offs;     // fill pass: output offset per item
   int32_t* col;
-  double* val;
-  int64_t* rowcnt;         // count / staged pass: entries per processed row
+  int64_t* cnt;            // count / staged pass: entries per item
   int32_t* scr;            // staged pass: scr_cap entries of scratch per warp of the grid
   int64_t scr_cap;
-  int32_t* stage;          // staged pass: rows, each contiguous, at rowoff[q]
+  int32_t* stage;          // staged pass: items, each contiguous, at itoff[q]
   int64_t stage_cap;
-  int64_t* rowoff;
-  unsigned long long* stage_ctl;  // [0] next free staging entry, [1] rows left to the fill pass
+  int64_t* itoff;
+  unsigned long long* stage_ctl;  // [0] next free staging entry, [1] items left to the fill pass
   const int32_t* s2i;      // sorted position -> internal id (columns are stored as internal ids)
   int lower;               // one-orientation form: a row keeps the connections with a smaller id
   unsigned long long* queue;
   HamView H;
   // direct traversals (no stored rows), vectors by sorted position
   const double* dc;             // input vector
-  double* dsig;                 // sigma: output
-  const double* ddiag;          // sigma: diagonal elements
+  double* dpart;                // sigma: each item's share of its row's sum
   unsigned long long* dnnz;     // sigma: connections visited (may be null)
   RdmAcc R;                     // RDMs: accumulators
 };
@@ -320,14 +318,19 @@ __device__ __forceinline__ void visit(const GraphArgs& A, ulonglong2 ki, int64_t
 template <int MODE, bool BETA>
 __device__ __forceinline__ void mixed_side(const GraphArgs& A, ulonglong2 ki, int g, int64_t& w, int32_t* out,
                                            int64_t* s_start, int64_t* s_pref, int64_t* s_size, const int* occ_o,
-                                           const int* vir_o, int nocc_o, int nvir_o, RowAcc& ra) {
+                                           const int* vir_o, int nocc_o, int nvir_o, RowAcc& ra, int part, int parts) {
   const int lane = threadIdx.x & 31;
   const int64_t* ptr = BETA ? A.bnbr_ptr : A.anbr_ptr;
   const int32_t* nbr = BETA ? A.bnbr : A.anbr;
   const int64_t* gs = BETA ? A.gb : A.ga;
   const uint64_t mine = BETA ? ki.x : ki.y;     // other-spin string of row i
   const int L = nocc_o * nvir_o;
-  const int64_t nb0 = ptr[g], nb1 = ptr[g + 1];
+  int64_t nb0 = ptr[g], nb1 = ptr[g + 1];
+  if (parts > 1) {
+    const int64_t len = nb1 - nb0, b = nb0;
+    nb0 = b + len * part / parts;
+    nb1 = b + len * (part + 1) / parts;
+  }
   for (int64_t c0 = nb0; c0 < nb1; c0 += 32) {
     const int64_t cidx = c0 + lane;
     int64_t st = 0, sz = 0;
@@ -418,13 +421,48 @@ __device__ __forceinline__ int occ_vir_lists(uint64_t s, int n, int* occ, int* v
   return bo;
 }
 
-// One warp per row taken from a queue.  ROWS_STAGED: the row goes to the
-// warp's scratch; at its end one atomic reserves the row's range of the
-// staging buffer and the row is copied there (rowoff[q] = its start, or -1
-// when the row outgrew the scratch or the staging buffer; rowcnt[q] is
-// exact either way).
+// Work items of the row search: a row whose search takes more than ITEM_COST
+// pair checks (the members of its alpha and beta groups and the cost of its
+// cheaper mixed side) is cut into parts, part p of P taking the p-th share
+// of both groups and of the neighbour list, so that no warp is left with the
+// search of the aufbau determinant's row when all others are done (half of
+// the direct product on 3e4 pentacene determinants).
+__global__ void k_item_count(GraphArgs A, const int32_t* __restrict__ rowlist, int64_t nrows, int64_t* __restrict__ cnt) {
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nrows; q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = rowlist ? (int64_t)rowlist[q] : q;
+    const int ga = A.ia[i], gb = A.ib[i];
+    const int64_t ca = A.costa[ga], cb = A.costb[gb];
+    const int64_t cost = (A.ga[ga + 1] - A.ga[ga]) + (A.gb[gb + 1] - A.gb[gb]) + (ca <= cb ? ca : cb);
+    const int64_t parts = (cost + ITEM_COST - 1) / ITEM_COST;
+    cnt[q] = parts < 1 ? 1 : parts > 4096 ? 4096 : parts;
+  }
+}
+__global__ void k_item_fill(const int32_t* __restrict__ rowlist, int64_t nrows, const int64_t* __restrict__ first,
+                            int4* __restrict__ items) {
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nrows; q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t f = first[q];
+    const int parts = (int)(first[q + 1] - f);
+    const int i = rowlist ? rowlist[q] : (int)q;
+    for (int p = 0; p < parts; ++p) items[f + p] = make_int4(i, (int)q, p, parts);
+  }
+}
+
+// One warp per item taken from a queue.  ROWS_STAGED: the entries go to the
+// warp's scratch; at the item's end one atomic reserves its range of the
+// staging buffer and they are copied there (itoff[q] = its start, or -1 when
+// the item outgrew the scratch or the staging buffer; cnt[q] is exact either
+// way).
+// the p-th of P shares of [b, e)
+__device__ __forceinline__ void share(int64_t& b, int64_t& e, int p, int P) {
+  if (P > 1) {
+    const int64_t len = e - b, b0 = b;
+    b = b0 + len * p / P;
+    e = b0 + len * (p + 1) / P;
+  }
+}
+
 template <int MODE>
-__global__ void __launch_bounds__(G_WARPS * 32) k_rows(GraphArgs A) {
+__global__ void __launch_bounds__(G_WARPS * 32, MODE <= ROWS_STAGED ? 6 : 5) k_rows(GraphArgs A) {
   __shared__ int64_t s_start[G_WARPS][32];
   __shared__ int64_t s_size[G_WARPS][32];
   __shared__ int64_t s_pref[G_WARPS][33];
@@ -435,10 +473,12 @@ __global__ void __launch_bounds__(G_WARPS * 32) k_rows(GraphArgs A) {
     unsigned long long qi = 0;
     if (lane == 0) qi = atomicAdd(A.queue, 1ull);
     const int64_t q = (int64_t)__shfl_sync(0xffffffffu, qi, 0);
-    if (q >= A.nrows) break;
-    const int64_t i = A.rowlist ? (int64_t)A.rowlist[q] : q;
+    if (q >= A.nitems) break;
+    const int4 it = A.items[q];
+    const int64_t i = it.x;
+    const int part = it.z, parts = it.w;
     const ulonglong2 ki = A.V[i];
-    int64_t w = MODE == ROWS_FILL ? A.rowptr[q] : 0;
+    int64_t w = MODE == ROWS_FILL ? A.offs[q] : 0;
     int32_t* out = MODE == ROWS_FILL ? A.col
                    : MODE == ROWS_STAGED ? A.scr + (int64_t)(blockIdx.x * G_WARPS + wid) * A.scr_cap
                                          : nullptr;
@@ -446,7 +486,8 @@ __global__ void __launch_bounds__(G_WARPS * 32) k_rows(GraphArgs A) {
     // (A) same alpha string
     {
       const int g = A.ia[i];
-      const int64_t b = A.ga[g], e = A.ga[g + 1];
+      int64_t b = A.ga[g], e = A.ga[g + 1];
+      share(b, e, part, parts);
       for (int64_t j0 = b; j0 < e; j0 += 64) {
         const int64_t j = j0 + lane, j2 = j + 32;
         const uint64_t x1 = j < e ? A.vb[j] : 0ull, x2 = j2 < e ? A.vb[j2] : 0ull;
@@ -466,7 +507,8 @@ __global__ void __launch_bounds__(G_WARPS * 32) k_rows(GraphArgs A) {
     // (B) same beta string
     {
       const int g = A.ib[i];
-      const int64_t b = A.gb[g], e = A.gb[g + 1];
+      int64_t b = A.gb[g], e = A.gb[g + 1];
+      share(b, e, part, parts);
       const int64_t mypos = A.posb[i];
       for (int64_t k0 = b; k0 < e; k0 += 64) {
         const int64_t k = k0 + lane, k2 = k + 32;
@@ -494,19 +536,19 @@ __global__ void __launch_bounds__(G_WARPS * 32) k_rows(GraphArgs A) {
       if (A.costa[ga_i] <= A.costb[gb_i]) {
         const int no = occ_vir_lists(ki.y, A.n, s_occ[wid], s_vir[wid]);
         mixed_side<MODE, false>(A, ki, ga_i, w, out, s_start[wid], s_pref[wid], s_size[wid], s_occ[wid],
-                                s_vir[wid], no, A.n - no, ra);
+                                s_vir[wid], no, A.n - no, ra, part, parts);
       } else {
         const int no = occ_vir_lists(ki.x, A.n, s_occ[wid], s_vir[wid]);
         mixed_side<MODE, true>(A, ki, gb_i, w, out, s_start[wid], s_pref[wid], s_size[wid], s_occ[wid],
-                               s_vir[wid], no, A.n - no, ra);
+                               s_vir[wid], no, A.n - no, ra, part, parts);
       }
     }
-    if (MODE == ROWS_COUNT && lane == 0) A.rowcnt[q] = w;
+    if (MODE == ROWS_COUNT && lane == 0) A.cnt[q] = w;
     if (MODE == ROWS_SIGMA) {
       double a = ra.acc;
       for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
       if (lane == 0) {
-        A.dsig[i] = fma(A.ddiag[i], ra.ci, a);
+        A.dpart[q] = a;
         if (A.dnnz) atomicAdd(A.dnnz, (unsigned long long)w);
       }
     }
@@ -514,13 +556,13 @@ __global__ void __launch_bounds__(G_WARPS * 32) k_rows(GraphArgs A) {
       __syncwarp();
       int64_t base = -1;
       if (lane == 0) {
-        A.rowcnt[q] = w;
+        A.cnt[q] = w;
         if (w <= A.scr_cap) {
           const int64_t b = (int64_t)atomicAdd(A.stage_ctl, (unsigned long long)w);
           if (b + w <= A.stage_cap) base = b;
         }
         if (base < 0) atomicAdd(A.stage_ctl + 1, 1ull);
-        A.rowoff[q] = base;
+        A.itoff[q] = base;
       }
       base = __shfl_sync(0xffffffffu, base, 0);
       if (base >= 0)
@@ -530,71 +572,113 @@ __global__ void __launch_bounds__(G_WARPS * 32) k_rows(GraphArgs A) {
   }
 }
 
-// rows[t] = list[t * n / ns], an evenly strided sample of ns entries of list
-__global__ void k_stride_sample(const int32_t* __restrict__ list, int64_t n, int64_t ns, int32_t* __restrict__ rows) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < ns) rows[t] = list[t * n / ns];
+// direct product: a row's sum is its items' shares in order
+__global__ void k_row_sums(const int64_t* __restrict__ first, int64_t nV, const double* __restrict__ part,
+                           const double* __restrict__ diag, const double* __restrict__ c, double* __restrict__ sigma) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nV; i += (int64_t)gridDim.x * blockDim.x) {
+    double s = 0.0;
+    for (int64_t q = first[i]; q < first[i + 1]; ++q) s += part[q];
+    sigma[i] = fma(diag[i], c[i], s);
+  }
 }
 
-// Staged rows placed: row q (rowoff[q] >= 0) copied from the staging buffer
-// to [rp[q], rp[q] + len) of col, len = lens[q] (or rp[q+1] - rp[q] when
-// lens is NULL, a dense CSR), one warp per row.
-__global__ void k_copy_staged(const int64_t* __restrict__ rowoff, const int64_t* __restrict__ rp,
-                              const int64_t* __restrict__ lens, int64_t nrows, const int32_t* __restrict__ stage,
+// out[t] = items[t * n / ns], an evenly strided sample of ns items
+__global__ void k_stride_sample(const int4* __restrict__ items, int64_t n, int64_t ns, int4* __restrict__ out) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < ns) out[t] = items[t * n / ns];
+}
+
+// row offsets from the items': rp[q] = itp[first[q]], q <= nrows; len[q] its
+// entries (or NULL)
+__global__ void k_row_offsets(const int64_t* __restrict__ first, const int64_t* __restrict__ itp, int64_t nrows,
+                              int64_t* __restrict__ rp, int64_t* __restrict__ len) {
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q <= nrows; q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t o = itp[first[q]];
+    rp[q] = o;
+    if (len && q < nrows) len[q] = itp[first[q + 1]] - o;
+  }
+}
+
+// where item u's entries go: its row's place plus its offset in the row
+__device__ __forceinline__ int64_t item_place(const int4* __restrict__ items, const int64_t* __restrict__ first,
+                                              const int64_t* __restrict__ itp, const int64_t* __restrict__ rowoff, int64_t u) {
+  const int q = items[u].y;
+  return rowoff[q] + itp[u] - itp[first[q]];
+}
+
+// Staged items placed (itoff >= 0), one warp per item: copied from the
+// staging buffer to their row's place in col
+__global__ void k_copy_staged(const int4* __restrict__ items, int64_t nitems, const int64_t* __restrict__ first,
+                              const int64_t* __restrict__ itp, const int64_t* __restrict__ itoff,
+                              const int64_t* __restrict__ rowoff, const int32_t* __restrict__ stage,
                               int32_t* __restrict__ col) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t q = warp; q < nrows; q += nwarps) {
-    const int64_t off = rowoff[q];
+  for (int64_t u = warp; u < nitems; u += nwarps) {
+    const int64_t off = itoff[u];
     if (off < 0) continue;
-    const int64_t b = rp[q], len = lens ? lens[q] : rp[q + 1] - b;
-    for (int64_t t = lane; t < len; t += 32) col[b + t] = stage[off + t];
+    const int64_t b = item_place(items, first, itp, rowoff, u), len = itp[u + 1] - itp[u];
+    int64_t t = lane;
+    for (; t + 96 < len; t += 128) {
+      const int32_t v0 = stage[off + t], v1 = stage[off + t + 32], v2 = stage[off + t + 64], v3 = stage[off + t + 96];
+      col[b + t] = v0; col[b + t + 32] = v1; col[b + t + 64] = v2; col[b + t + 96] = v3;
+    }
+    for (; t < len; t += 32) col[b + t] = stage[off + t];
   }
 }
 
-// rows the staged pass could not keep: their ids and CSR offsets, for the
-// fill pass (any order: each row is written at its own offset)
-__global__ void k_collect_left(const int64_t* __restrict__ rowoff, const int64_t* __restrict__ rp,
-                               const int32_t* __restrict__ rowlist, int64_t nrows,
-                               unsigned long long* __restrict__ counter, int32_t* __restrict__ left_rows,
-                               int64_t* __restrict__ left_off) {
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nrows; q += (int64_t)gridDim.x * blockDim.x)
-    if (rowoff[q] < 0) {
+// items the staged pass could not keep (or, with itoff NULL, every item) and
+// their places, for the fill pass (any order: each is written at its own)
+__global__ void k_collect_left(const int4* __restrict__ items, int64_t nitems, const int64_t* __restrict__ first,
+                               const int64_t* __restrict__ itp, const int64_t* __restrict__ itoff,
+                               const int64_t* __restrict__ rowoff, unsigned long long* __restrict__ counter,
+                               int4* __restrict__ left, int64_t* __restrict__ left_off) {
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < nitems; u += (int64_t)gridDim.x * blockDim.x)
+    if (!itoff || itoff[u] < 0) {
       const unsigned long long m = atomicAdd(counter, 1ull);
-      left_rows[m] = rowlist[q];
-      left_off[m] = rp[q];
+      left[m] = items[u];
+      left_off[m] = item_place(items, first, itp, rowoff, u);
     }
 }
 
-// Matrix elements of filled rows (the search only records the columns):
-// row q holds entries [start[q], start[q] + len) of col/val, with
-// len = start[q+1] - start[q] (DENSE) or lens[q]; four entries per lane in
-// flight.
-template <bool DENSE>
-__global__ void __launch_bounds__(256) k_row_values(const int32_t* __restrict__ rowlist, int64_t nrows,
-                                                    const int64_t* __restrict__ start,
-                                                    const int64_t* __restrict__ lens, const int32_t* __restrict__ col,
+// Matrix elements of filled rows (the search only records the columns): row
+// q has the logical entries [rowptr[q], rowptr[q+1]), kept from start[q] on
+// (start NULL: at rowptr[q]) in col/val.  Chunks of RV_CHUNK entries whatever
+// rows they belong to, four entries per lane in flight; bound by the latency
+// of the gathered keys and integrals.  Phases flip the sign bit: with FP64
+// products for them, and a warp per row, 1100 us for the 7e7 entries of a
+// pentacene space, 966 us so.
+constexpr int RV_CHUNK = 1024;
+__global__ void __launch_bounds__(256, 4) k_row_values(const int32_t* __restrict__ rowlist, int64_t nrows,
+                                                    const int64_t* __restrict__ rowptr,
+                                                    const int64_t* __restrict__ start, const int32_t* __restrict__ col,
                                                     double* __restrict__ val, const ulonglong2* __restrict__ Vrow,
                                                     const ulonglong2* __restrict__ V, HamView H) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t q = warp; q < nrows; q += nwarps) {
-    const int64_t i = rowlist ? (int64_t)rowlist[q] : q;
-    const ulonglong2 ki = Vrow[i];
-    const int64_t b = start[q];
-    const int64_t len = DENSE ? start[q + 1] - b : lens[q];
-    int64_t k = lane;
-    for (; k + 96 < len; k += 128) {
-      const ulonglong2 k0 = V[col[b + k]], k1 = V[col[b + k + 32]], k2 = V[col[b + k + 64]],
-                       k3 = V[col[b + k + 96]];
-      val[b + k] = connection_el(H, ki, k0);
-      val[b + k + 32] = connection_el(H, ki, k1);
-      val[b + k + 64] = connection_el(H, ki, k2);
-      val[b + k + 96] = connection_el(H, ki, k3);
+  const int64_t total = rowptr[nrows];
+  for (int64_t e0 = warp * RV_CHUNK; e0 < total; e0 += nwarps * RV_CHUNK) {
+    const int64_t e1 = e0 + RV_CHUNK < total ? e0 + RV_CHUNK : total;
+    int64_t e = e0;
+    for (int64_t q = row_of_entry(rowptr, nrows, e0); e < e1; ++q) {
+      const int64_t lo = rowptr[q], hi = rowptr[q + 1] < e1 ? rowptr[q + 1] : e1;
+      if (hi <= e) continue;
+      const ulonglong2 ki = Vrow[rowlist ? (int64_t)rowlist[q] : q];
+      const int64_t b = (start ? start[q] : lo) + (e - lo), len = hi - e;
+      e = hi;
+      int64_t k = lane;
+      for (; k + 96 < len; k += 128) {
+        const ulonglong2 k0 = V[col[b + k]], k1 = V[col[b + k + 32]], k2 = V[col[b + k + 64]],
+                         k3 = V[col[b + k + 96]];
+        val[b + k] = connection_el(H, ki, k0);
+        val[b + k + 32] = connection_el(H, ki, k1);
+        val[b + k + 64] = connection_el(H, ki, k2);
+        val[b + k + 96] = connection_el(H, ki, k3);
+      }
+      for (; k < len; k += 32) val[b + k] = connection_el(H, ki, V[col[b + k]]);
     }
-    for (; k < len; k += 32) val[b + k] = connection_el(H, ki, V[col[b + k]]);
   }
 }
 
@@ -1365,36 +1449,27 @@ static void space_args(hci_ctx* ctx, int64_t nV, GraphArgs& A) {
                 ctx->na == 64 ? ~0ull : ((1ull << ctx->na) - 1ull),
                 ctx->nb == 64 ? ~0ull : ((1ull << ctx->nb) - 1ull)};
   A.queue = reinterpret_cast<unsigned long long*>(bp<char>(ctx->s_counter) + 48);
-  A.rowlist = nullptr;
-  A.nrows = nV;
-  A.rowptr = nullptr; A.col = nullptr; A.val = nullptr; A.rowcnt = nullptr;
-  A.scr = nullptr; A.scr_cap = 0; A.stage = nullptr; A.stage_cap = 0; A.rowoff = nullptr; A.stage_ctl = nullptr;
   A.s2i = bp<int32_t>(ctx->graph.s2i);
-  A.lower = 0;
-  A.dc = nullptr; A.dsig = nullptr; A.ddiag = nullptr; A.dnnz = nullptr;
 }
 
-// Count the entries of the rows listed in A (A.rowlist / A.nrows) into cnt.
-static hci_status rows_count(hci_ctx* ctx, GraphArgs& A, DevBuf& cnt) {
-  HCI_TRY(ensure_buf(ctx, cnt, (size_t)(A.nrows + 1) * 8));
-  A.rowcnt = bp<int64_t>(cnt);
-  A.rowptr = nullptr; A.col = nullptr; A.val = nullptr;
+// Entries of A's items counted into cnt.
+static hci_status rows_count(hci_ctx* ctx, GraphArgs A, int64_t* cnt) {
+  A.cnt = cnt;
   HCI_CUDA(ctx, cudaMemsetAsync(A.queue, 0, 8, ctx->st));
   HCI_LAUNCH(k_rows<ROWS_COUNT>, rows_grid(ctx), G_WARPS * 32, 0, ctx->st)(A);
   HCI_CUDA(ctx, cudaGetLastError());
-  A.rowcnt = nullptr;
   return HCI_OK;
 }
 
-// Fill the listed rows, row q starting at offs[q] of col/val.
-static hci_status rows_fill(hci_ctx* ctx, GraphArgs& A, const int64_t* offs, int32_t* col, double* val) {
-  A.rowptr = offs; A.col = col; A.val = val;
+// The nitems items searched, item u's entries written from offs[u] of col.
+static hci_status rows_fill(hci_ctx* ctx, GraphArgs A, const int4* items, int64_t nitems, const int64_t* offs,
+                            int32_t* col) {
+  A.items = items; A.nitems = nitems; A.offs = offs; A.col = col;
   HCI_CUDA(ctx, cudaMemsetAsync(A.queue, 0, 8, ctx->st));
   HCI_LAUNCH(k_rows<ROWS_FILL>, rows_grid(ctx), G_WARPS * 32, 0, ctx->st)(A);
   HCI_CUDA(ctx, cudaGetLastError());
   return HCI_OK;
 }
-
 
 static int64_t read_i64(hci_ctx* ctx, const int64_t* d, hci_status* st) {
   int64_t v = 0;
@@ -1404,38 +1479,70 @@ static int64_t read_i64(hci_ctx* ctx, const int64_t* d, hci_status* st) {
   return v;
 }
 
-// The rows listed in A (rowlist, nrows; a list is required) searched once
-// into per-warp scratch and a staging buffer (sized from est entries):
-// counts into inc.cnt, their prefix sums into inc.rpN (inc.rpN[nrows] =
-// *total), rows that outgrew the scratch or the staging space marked for a
-// second search (*left of them).
-static hci_status stage_search(hci_ctx* ctx, GraphArgs& A, int64_t est, int64_t* total, int64_t* left) {
+// Work items of the rows in rowlist (NULL: rows 0 .. nrows-1) into
+// inc.items, each row's first into inc.first.
+static hci_status make_items(hci_ctx* ctx, GraphArgs& A, const int32_t* rowlist, int64_t nrows) {
   IncScratch& S = ctx->inc;
   cudaStream_t st = ctx->st;
-  const int64_t nrows = A.nrows;
   int64_t* dtot = reinterpret_cast<int64_t*>(bp<char>(ctx->s_counter) + 40);
   HCI_TRY(ensure_buf(ctx, S.cnt, (size_t)(nrows + 1) * 8));
-  HCI_TRY(ensure_buf(ctx, S.roff, (size_t)(nrows + 1) * 8));
+  HCI_TRY(ensure_buf(ctx, S.first, (size_t)(nrows + 1) * 8));
+  HCI_LAUNCH(k_item_count, grid_for(nrows, 256), 256, 0, st)(A, rowlist, nrows, bp<int64_t>(S.cnt));
+  HCI_TRY(scan_i64(ctx, bp<int64_t>(S.cnt), bp<int64_t>(S.first), nrows, dtot));
+  HCI_LAUNCH(k_store_at, 1, 1, 0, st)(bp<int64_t>(S.first), nrows, dtot);
+  hci_status hs = HCI_OK;
+  A.nitems = read_i64(ctx, dtot, &hs);
+  HCI_TRY(hs);
+  HCI_TRY(ensure_buf(ctx, S.items, (size_t)A.nitems * 16));
+  HCI_LAUNCH(k_item_fill, grid_for(nrows, 256), 256, 0, st)(rowlist, nrows, bp<int64_t>(S.first), bp<int4>(S.items));
+  HCI_CUDA(ctx, cudaGetLastError());
+  A.items = bp<int4>(S.items);
+  return HCI_OK;
+}
+
+// Items' counts (inc.cnt) to offsets: inc.itp per item, inc.rpN per row
+// (inc.rpN[nrows] = *total); the counts of the rows to len (or NULL).
+static hci_status item_offsets(hci_ctx* ctx, const GraphArgs& A, int64_t nrows, int64_t* len) {
+  IncScratch& S = ctx->inc;
+  int64_t* dtot = reinterpret_cast<int64_t*>(bp<char>(ctx->s_counter) + 40);
+  HCI_TRY(ensure_buf(ctx, S.itp, (size_t)(A.nitems + 1) * 8));
+  HCI_TRY(ensure_buf(ctx, S.rpN, (size_t)(nrows + 1) * 8));
+  HCI_TRY(scan_i64(ctx, bp<int64_t>(S.cnt), bp<int64_t>(S.itp), A.nitems, dtot));
+  HCI_LAUNCH(k_store_at, 1, 1, 0, ctx->st)(bp<int64_t>(S.itp), A.nitems, dtot);
+  HCI_LAUNCH(k_row_offsets, grid_for(nrows + 1, 256), 256, 0, ctx->st)(bp<int64_t>(S.first), bp<int64_t>(S.itp), nrows,
+                                                                      bp<int64_t>(S.rpN), len);
+  HCI_CUDA(ctx, cudaGetLastError());
+  return HCI_OK;
+}
+
+// A's items searched once into per-warp scratch and a staging buffer (sized
+// from est entries), their counts and offsets as item_offsets, items that
+// outgrew the scratch or the staging space marked for a second search (*left
+// of them).
+static hci_status stage_search(hci_ctx* ctx, GraphArgs& A, int64_t nrows, int64_t* len, int64_t est, int64_t* total,
+                               int64_t* left) {
+  IncScratch& S = ctx->inc;
+  cudaStream_t st = ctx->st;
+  int64_t* dtot = reinterpret_cast<int64_t*>(bp<char>(ctx->s_counter) + 40);
+  HCI_TRY(ensure_buf(ctx, S.cnt, (size_t)(A.nitems + 1) * 8));
+  HCI_TRY(ensure_buf(ctx, S.roff, (size_t)(A.nitems + 1) * 8));
   HCI_TRY(ensure_buf(ctx, S.scr, (size_t)rows_grid(ctx) * G_WARPS * ROW_SCR * 4));
   if (S.stage.bytes < (size_t)est * 4) HCI_TRY(ensure_buf(ctx, S.stage, (size_t)est * 4));
   HCI_TRY(ensure_buf(ctx, S.ctl, 32));
   HCI_CUDA(ctx, cudaMemsetAsync(S.ctl.p, 0, 32, st));
   unsigned long long* ctl = bp<unsigned long long>(S.ctl);
-  A.rowcnt = bp<int64_t>(S.cnt);
-  A.scr = bp<int32_t>(S.scr);
-  A.scr_cap = ROW_SCR;
-  A.stage = bp<int32_t>(S.stage);
-  A.stage_cap = (int64_t)(S.stage.bytes / 4);
-  A.rowoff = bp<int64_t>(S.roff);
-  A.stage_ctl = ctl;
-  HCI_CUDA(ctx, cudaMemsetAsync(A.queue, 0, 8, st));
-  HCI_LAUNCH(k_rows<ROWS_STAGED>, rows_grid(ctx), G_WARPS * 32, 0, st)(A);
+  GraphArgs B = A;
+  B.cnt = bp<int64_t>(S.cnt);
+  B.scr = bp<int32_t>(S.scr);
+  B.scr_cap = ROW_SCR;
+  B.stage = bp<int32_t>(S.stage);
+  B.stage_cap = (int64_t)(S.stage.bytes / 4);
+  B.itoff = bp<int64_t>(S.roff);
+  B.stage_ctl = ctl;
+  HCI_CUDA(ctx, cudaMemsetAsync(B.queue, 0, 8, st));
+  HCI_LAUNCH(k_rows<ROWS_STAGED>, rows_grid(ctx), G_WARPS * 32, 0, st)(B);
   HCI_CUDA(ctx, cudaGetLastError());
-  A.rowcnt = nullptr; A.scr = nullptr; A.scr_cap = 0; A.stage = nullptr; A.stage_cap = 0; A.rowoff = nullptr;
-  A.stage_ctl = nullptr;
-  HCI_TRY(ensure_buf(ctx, S.rpN, (size_t)(nrows + 1) * 8));
-  HCI_TRY(scan_i64(ctx, bp<int64_t>(S.cnt), bp<int64_t>(S.rpN), nrows, dtot));
-  HCI_LAUNCH(k_store_at, 1, 1, 0, st)(bp<int64_t>(S.rpN), nrows, dtot);
+  HCI_TRY(item_offsets(ctx, A, nrows, len));
   hci_status hs = HCI_OK;
   *total = read_i64(ctx, dtot, &hs);
   HCI_TRY(hs);
@@ -1444,35 +1551,35 @@ static hci_status stage_search(hci_ctx* ctx, GraphArgs& A, int64_t est, int64_t*
   return HCI_OK;
 }
 
-// Columns of the rows of stage_search written to col, row q at off[q]
-// (default inc.rpN[q]; lens[q] entries, default the dense rpN differences):
-// staged rows copied, the rows left searched again at their offsets (left <
-// 0: no row was staged, all are searched again).
-static hci_status stage_place(hci_ctx* ctx, GraphArgs& A, int64_t left, int32_t* col, const int64_t* off = nullptr,
-                              const int64_t* lens = nullptr) {
+// Columns of the rows of stage_new_rows written to col, row q at off[q]
+// (default inc.rpN[q]): staged items copied, the ones left searched again at
+// their places (left < 0: nothing was staged, all are searched again).
+static hci_status stage_place(hci_ctx* ctx, GraphArgs& A, int64_t left, int32_t* col, const int64_t* off = nullptr) {
   IncScratch& S = ctx->inc;
   cudaStream_t st = ctx->st;
-  const int64_t nrows = A.nrows;
   if (!off) off = bp<int64_t>(S.rpN);
-  if (left < 0) return rows_fill(ctx, A, off, col, nullptr);   // counted, not staged
-  HCI_LAUNCH(k_copy_staged, grid_for(nrows * 32, 256), 256, 0, st)(bp<int64_t>(S.roff), off, lens, nrows,
-                                                                    bp<int32_t>(S.stage), col);
-  HCI_CUDA(ctx, cudaGetLastError());
-  ctx->st_counts[HCI_ST_ROWS_REFILLED] += left;
+  const bool staged = left >= 0;
+  if (staged) {
+    HCI_LAUNCH(k_copy_staged, grid_for(A.nitems * 32, 256), 256, 0, st)(A.items, A.nitems, bp<int64_t>(S.first),
+                                                                       bp<int64_t>(S.itp), bp<int64_t>(S.roff), off,
+                                                                       bp<int32_t>(S.stage), col);
+    HCI_CUDA(ctx, cudaGetLastError());
+    ctx->st_counts[HCI_ST_ROWS_REFILLED] += left;
+  } else {
+    left = A.nitems;
+  }
   if (left > 0) {
-    unsigned long long* ctl = bp<unsigned long long>(S.ctl);
-    HCI_TRY(ensure_buf(ctx, S.left, (size_t)left * 12 + 16));
-    int64_t* left_off = bp<int64_t>(S.left);
-    int32_t* left_rows = reinterpret_cast<int32_t*>(left_off + left);
-    HCI_LAUNCH(k_collect_left, grid_for(nrows, 256), 256, 0, st)(bp<int64_t>(S.roff), off, A.rowlist, nrows, ctl + 2,
-                                                                  left_rows, left_off);
-    const int32_t* rl = A.rowlist;
-    A.rowlist = left_rows;
-    A.nrows = left;
-    hci_status fs = rows_fill(ctx, A, left_off, col, nullptr);
-    A.rowlist = rl;
-    A.nrows = nrows;
-    HCI_TRY(fs);
+    HCI_TRY(ensure_buf(ctx, S.ctl, 32));
+    unsigned long long* counter = bp<unsigned long long>(S.ctl) + 2;
+    HCI_CUDA(ctx, cudaMemsetAsync(counter, 0, 8, st));
+    HCI_TRY(ensure_buf(ctx, S.left, (size_t)left * 24 + 16));
+    int4* items = bp<int4>(S.left);
+    int64_t* offs = reinterpret_cast<int64_t*>(items + left);
+    HCI_LAUNCH(k_collect_left, grid_for(A.nitems, 256), 256, 0, st)(A.items, A.nitems, bp<int64_t>(S.first),
+                                                                   bp<int64_t>(S.itp),
+                                                                   staged ? bp<int64_t>(S.roff) : nullptr, off, counter,
+                                                                   items, offs);
+    HCI_TRY(rows_fill(ctx, A, items, left, offs, col));
   }
   return HCI_OK;
 }
@@ -1528,40 +1635,39 @@ static hci_status seg_alloc(hci_ctx* ctx, int64_t entries, int* seg) {
   return HCI_OK;
 }
 
-// The new rows listed in A searched once (stage_search), the staging space
-// sized from the mean length of a strided sample of them (the old rows'
-// lengths say little when the space grows many-fold).  When that space would
-// exceed an eighth of device memory the rows are only counted here (*left =
-// -1) and stage_place searches them a second time, straight into place.
-static hci_status stage_new_rows(hci_ctx* ctx, GraphArgs& A, int64_t nnew, int64_t nV, int64_t* total, int64_t* left) {
+// The nnew rows in rowlist (NULL: all of V in order) cut into items and
+// searched once (stage_search), the staging space sized from the mean count
+// of a strided sample of the items (the old rows' lengths say little when
+// the space grows many-fold).  When that space would exceed an eighth of
+// device memory the items are only counted here (*left = -1) and stage_place
+// searches them a second time, straight into place.  Rows' entries to len (or
+// NULL).
+static hci_status stage_new_rows(hci_ctx* ctx, GraphArgs& A, const int32_t* rowlist, int64_t nnew, int64_t nV,
+                                 int64_t* len, int64_t* total, int64_t* left) {
   IncScratch& S = ctx->inc;
   cudaStream_t st = ctx->st;
-  const int64_t ns = std::min<int64_t>(nnew, ROW_SAMPLE);
-  HCI_TRY(ensure_buf(ctx, S.samp, (size_t)ns * 12 + 16));
-  int64_t* samp_cnt = bp<int64_t>(S.samp);
-  int32_t* samp_rows = reinterpret_cast<int32_t*>(samp_cnt + ns);
-  HCI_LAUNCH(k_stride_sample, grid_for(ns, 256), 256, 0, st)(A.rowlist, nnew, ns, samp_rows);
+  HCI_TRY(make_items(ctx, A, rowlist, nnew));
+  const int64_t ns = std::min<int64_t>(A.nitems, ROW_SAMPLE);
+  HCI_TRY(ensure_buf(ctx, S.samp, (size_t)ns * 24 + 16));
+  int4* samp = bp<int4>(S.samp);
+  int64_t* samp_cnt = reinterpret_cast<int64_t*>(samp + ns);
+  HCI_LAUNCH(k_stride_sample, grid_for(ns, 256), 256, 0, st)(A.items, A.nitems, ns, samp);
   GraphArgs B = A;
-  B.rowlist = samp_rows;
-  B.nrows = ns;
-  B.rowcnt = samp_cnt;
-  HCI_CUDA(ctx, cudaMemsetAsync(B.queue, 0, 8, st));
-  HCI_LAUNCH(k_rows<ROWS_COUNT>, rows_grid(ctx), G_WARPS * 32, 0, st)(B);
-  HCI_CUDA(ctx, cudaGetLastError());
+  B.items = samp;
+  B.nitems = ns;
+  HCI_TRY(rows_count(ctx, B, samp_cnt));
   std::vector<int64_t> cnt((size_t)ns);
   HCI_CUDA(ctx, cudaMemcpyAsync(cnt.data(), samp_cnt, (size_t)ns * 8, cudaMemcpyDeviceToHost, st));
   HCI_CUDA(ctx, cudaStreamSynchronize(st));
   double sum = 0.0;
   for (int64_t v : cnt) sum += (double)v;
-  const double mean = ns > 0 ? sum / (double)ns : 0.0;
-  const double want = 1.5 * (double)nnew * mean;
-  const int64_t est = (int64_t)std::min((double)nnew * (double)nV, want) + ((int64_t)1 << 22);
+  const double mean = ns > 0 ? sum / (double)ns : 0.0, rows = (double)A.nitems * mean;
+  const int64_t est = (int64_t)std::min((double)nnew * (double)nV, 1.5 * rows) + ((int64_t)1 << 22);
   {
     // a graph that cannot fit device memory is refused before the search:
     // both orientations add the new rows, their transposes and slack to the
     // pool, one orientation adds the new rows
     const Graph& G = ctx->graph;
-    const double rows = (double)nnew * mean;
     const double need = G.half ? (double)G.nstored + rows : (double)G.pool_used + 2.5 * rows;
     if (need * 12.0 > 0.9 * (double)ctx->mem_total)
       return hci_fail(ctx, HCI_ERR_NOMEM, "graph: about %.3g bytes of stored connections would exceed device memory",
@@ -1571,17 +1677,19 @@ static hci_status stage_new_rows(hci_ctx* ctx, GraphArgs& A, int64_t nnew, int64
     // a staging buffer this large would crowd out the stored rows: count
     // the rows first and let stage_place search them again into place
     int64_t* dtot = reinterpret_cast<int64_t*>(bp<char>(ctx->s_counter) + 40);
-    HCI_TRY(rows_count(ctx, A, S.cnt));
-    HCI_TRY(ensure_buf(ctx, S.rpN, (size_t)(nnew + 1) * 8));
-    HCI_TRY(scan_i64(ctx, bp<int64_t>(S.cnt), bp<int64_t>(S.rpN), nnew, dtot));
-    HCI_LAUNCH(k_store_at, 1, 1, 0, st)(bp<int64_t>(S.rpN), nnew, dtot);
+    HCI_TRY(ensure_buf(ctx, S.cnt, (size_t)(A.nitems + 1) * 8));
+    HCI_TRY(rows_count(ctx, A, bp<int64_t>(S.cnt)));
+    HCI_TRY(item_offsets(ctx, A, nnew, len));
     hci_status hs = HCI_OK;
     *total = read_i64(ctx, dtot, &hs);
     *left = -1;
     return hs;
   }
-  return stage_search(ctx, A, est, total, left);
+  return stage_search(ctx, A, nnew, len, est, total, left);
 }
+
+// blocks of k_row_values: a warp per chunk, at most 16 blocks per SM
+static int values_grid(int64_t entries) { return grid_for((entries + RV_CHUNK - 1) / RV_CHUNK * 32, 256); }
 
 static hci_status graph_build_half(hci_ctx* ctx, const uint64_t* keys, int64_t nV) {
   Graph& G = ctx->graph;
@@ -1605,12 +1713,10 @@ static hci_status graph_build_half(hci_ctx* ctx, const uint64_t* keys, int64_t n
   A.s2i = bp<int32_t>(G.s2i);
   A.lower = 1;
   prof_tic(ctx, HCI_PH_GRAPH_ROWS);
-  // stored halves of the rows, each searched once (staged; the row list is
-  // the identity map), into one segment, then their elements
-  A.rowlist = bp<int32_t>(G.s2i);
-  A.nrows = nV;
+  // stored halves of the rows, each searched once (staged), into one segment,
+  // then their elements
   int64_t nst = 0, left = 0;
-  HCI_TRY(stage_new_rows(ctx, A, nV, nV, &nst, &left));
+  HCI_TRY(stage_new_rows(ctx, A, nullptr, nV, nV, nullptr, &nst, &left));
   HCI_TRY(ensure_buf(ctx, G.rowptr, (size_t)(nV + 1) * 8));
   HCI_TRY(ensure_buf(ctx, G.rowstart, (size_t)(nV + 1) * 8));
   HCI_CUDA(ctx, cudaMemcpyAsync(G.rowptr.p, ctx->inc.rpN.p, (size_t)(nV + 1) * 8, cudaMemcpyDeviceToDevice, ctx->st));
@@ -1619,8 +1725,7 @@ static hci_status graph_build_half(hci_ctx* ctx, const uint64_t* keys, int64_t n
   int32_t* col = bp<int32_t>(G.seg_col[seg]);
   double* val = bp<double>(G.seg_val[seg]);
   HCI_TRY(stage_place(ctx, A, left, col));
-  A.rowlist = nullptr;
-  HCI_LAUNCH(k_row_values<true>, grid_for(nV * 32, 256), 256, 0, ctx->st)(
+  HCI_LAUNCH(k_row_values, values_grid(nst), 256, 0, ctx->st)(
       nullptr, nV, bp<int64_t>(G.rowptr), nullptr, col, val, bp<ulonglong2>(G.keys), bp<ulonglong2>(G.keys_int), A.H);
   HCI_LAUNCH(k_append_rows, grid_for(nV + 1, 256), 256, 0, ctx->st)(0, nV, bp<int64_t>(G.rowptr), 0, seg,
                                                                      bp<int64_t>(G.rowptr), bp<int64_t>(G.rowstart));
@@ -1692,17 +1797,15 @@ static hci_status graph_extend_half(hci_ctx* ctx, const uint64_t* keys, int64_t 
   HCI_TRY(build_space(ctx, nV, A));
   A.s2i = bp<int32_t>(G.s2i);
   A.lower = 1;
-  A.rowlist = bp<int32_t>(S.newrows);
-  A.nrows = nnew;
   prof_tic(ctx, HCI_PH_GRAPH_ROWS);
   int64_t total = 0, left = 0;
-  HCI_TRY(stage_new_rows(ctx, A, nnew, nV, &total, &left));
+  HCI_TRY(stage_new_rows(ctx, A, bp<int32_t>(S.newrows), nnew, nV, nullptr, &total, &left));
   int seg = 0;
   HCI_TRY(seg_alloc(ctx, total, &seg));
   int32_t* col = bp<int32_t>(G.seg_col[seg]);
   double* val = bp<double>(G.seg_val[seg]);
   HCI_TRY(stage_place(ctx, A, left, col));
-  HCI_LAUNCH(k_row_values<true>, grid_for(nnew * 32, 256), 256, 0, st)(
+  HCI_LAUNCH(k_row_values, values_grid(total), 256, 0, st)(
       bp<int32_t>(S.newrows), nnew, bp<int64_t>(S.rpN), nullptr, col, val, bp<ulonglong2>(G.keys),
       bp<ulonglong2>(G.keys_int), A.H);
   HCI_CUDA(ctx, cudaGetLastError());
@@ -1760,15 +1863,12 @@ static hci_status graph_build_full(hci_ctx* ctx, const uint64_t* keys, int64_t n
   HCI_TRY(build_space(ctx, nV, A));
   A.s2i = bp<int32_t>(G.s2i);
   prof_tic(ctx, HCI_PH_GRAPH_ROWS);
-  // every row searched once (staged, as for the new rows of an extension;
-  // the row list is the identity map), lengths and logical offsets from it
-  A.rowlist = bp<int32_t>(G.s2i);
-  A.nrows = nV;
-  int64_t nnz = 0, left = 0;
-  HCI_TRY(stage_new_rows(ctx, A, nV, nV, &nnz, &left));
+  // every row searched once (staged, as for the new rows of an extension),
+  // lengths and logical offsets from it
   HCI_TRY(ensure_buf(ctx, G.rowlen, (size_t)(nV + 1) * 8));
+  int64_t nnz = 0, left = 0;
+  HCI_TRY(stage_new_rows(ctx, A, nullptr, nV, nV, bp<int64_t>(G.rowlen), &nnz, &left));
   HCI_TRY(ensure_buf(ctx, G.rowptr, (size_t)(nV + 1) * 8));
-  HCI_CUDA(ctx, cudaMemcpyAsync(G.rowlen.p, ctx->inc.cnt.p, (size_t)nV * 8, cudaMemcpyDeviceToDevice, ctx->st));
   HCI_CUDA(ctx, cudaMemcpyAsync(G.rowptr.p, ctx->inc.rpN.p, (size_t)(nV + 1) * 8, cudaMemcpyDeviceToDevice, ctx->st));
   // capacities with slack, starts = their prefix sums, pool with headroom
   HCI_TRY(ensure_buf(ctx, G.rowcap, (size_t)(nV + 1) * 8));
@@ -1785,10 +1885,9 @@ static hci_status graph_build_full(hci_ctx* ctx, const uint64_t* keys, int64_t n
   HCI_TRY(ensure_buf(ctx, G.seg_col[0], (size_t)cap * 4));
   HCI_TRY(ensure_buf(ctx, G.seg_val[0], (size_t)cap * 8));
   G.nseg = 1;
-  HCI_TRY(stage_place(ctx, A, left, bp<int32_t>(G.seg_col[0]), bp<int64_t>(G.rowstart), bp<int64_t>(G.rowlen)));
-  A.rowlist = nullptr;
-  HCI_LAUNCH(k_row_values<false>, grid_for(nV * 32, 256), 256, 0, ctx->st)(
-      nullptr, nV, bp<int64_t>(G.rowstart), bp<int64_t>(G.rowlen), bp<int32_t>(G.seg_col[0]),
+  HCI_TRY(stage_place(ctx, A, left, bp<int32_t>(G.seg_col[0]), bp<int64_t>(G.rowstart)));
+  HCI_LAUNCH(k_row_values, values_grid(nnz), 256, 0, ctx->st)(
+      nullptr, nV, bp<int64_t>(G.rowptr), bp<int64_t>(G.rowstart), bp<int32_t>(G.seg_col[0]),
       bp<double>(G.seg_val[0]), bp<ulonglong2>(G.keys), bp<ulonglong2>(G.keys_int), A.H);
   HCI_CUDA(ctx, cudaGetLastError());
   prof_toc(ctx, HCI_PH_GRAPH_ROWS);
@@ -1862,20 +1961,18 @@ static hci_status graph_extend_full(hci_ctx* ctx, const uint64_t* keys, int64_t 
   GraphArgs A;
   HCI_TRY(build_space(ctx, nV, A));
   A.s2i = bp<int32_t>(G.s2i);
-  A.rowlist = bp<int32_t>(S.newrows);
-  A.nrows = nnew;
   prof_tic(ctx, HCI_PH_GRAPH_ROWS);
   // staging space from the mean length of a strided sample of the new rows
   // (the old rows' lengths say little when the space grows many-fold)
   int64_t nnzN = 0;
   {
     int64_t left = 0;
-    HCI_TRY(stage_new_rows(ctx, A, nnew, nV, &nnzN, &left));
+    HCI_TRY(stage_new_rows(ctx, A, bp<int32_t>(S.newrows), nnew, nV, nullptr, &nnzN, &left));
     HCI_TRY(ensure_buf(ctx, S.colN, (size_t)(nnzN + 1) * 4));
     HCI_TRY(ensure_buf(ctx, S.valN, (size_t)(nnzN + 1) * 8));
     HCI_TRY(stage_place(ctx, A, left, bp<int32_t>(S.colN)));
   }
-  HCI_LAUNCH(k_row_values<true>, grid_for(nnew * 32, 256), 256, 0, st)(
+  HCI_LAUNCH(k_row_values, values_grid(nnzN), 256, 0, st)(
       bp<int32_t>(S.newrows), nnew, bp<int64_t>(S.rpN), nullptr, bp<int32_t>(S.colN), bp<double>(S.valN),
       bp<ulonglong2>(G.keys), bp<ulonglong2>(G.keys_int), A.H);
   HCI_CUDA(ctx, cudaGetLastError());
@@ -1885,6 +1982,7 @@ static hci_status graph_extend_full(hci_ctx* ctx, const uint64_t* keys, int64_t 
   HCI_TRY(ensure_buf(ctx, S.hist, (size_t)(nV + 1) * 8));
   HCI_CUDA(ctx, cudaMemsetAsync(S.hist.p, 0, (size_t)(nV + 1) * 8, st));
   const int gw = grid_for(nnew * 32, 256);
+  HCI_TRY(ensure_buf(ctx, S.cnt, (size_t)(nnew + 1) * 8));
   HCI_LAUNCH(k_count_old_cols, gw, 256, 0, st)(bp<int64_t>(S.rpN), bp<int32_t>(S.colN), nnew, nold,
                                                 bp<int64_t>(S.cnt), bp<int64_t>(S.hist));
   HCI_TRY(ensure_buf(ctx, S.tbase, (size_t)(nnew + 1) * 8));
@@ -1997,6 +2095,10 @@ static hci_status graph_build_direct(hci_ctx* ctx, const uint64_t* keys, int64_t
   HCI_LAUNCH(k_iota, grid_for(nV, 256), 256, 0, ctx->st)(bp<int32_t>(G.s2i), bp<int32_t>(G.i2s), nV);
   GraphArgs A;
   HCI_TRY(build_space(ctx, nV, A));
+  // the work items of every traversal, and their shares of the rows' sums
+  HCI_TRY(make_items(ctx, A, nullptr, nV));
+  ctx->inc.nitems = A.nitems;
+  HCI_TRY(ensure_buf(ctx, ctx->inc.itp, (size_t)A.nitems * 8));
   HCI_TRY(ensure_buf(ctx, G.diag, (size_t)nV * 8));
   HCI_TRY(compute_diag(ctx, nV, bp<ulonglong2>(G.keys_int), bp<double>(G.diag)));
   prof_toc(ctx, HCI_PH_GRAPH);
@@ -2017,7 +2119,7 @@ static void release_stored(hci_ctx* ctx) {
   IncScratch& S = ctx->inc;
   free_segments(ctx);
   DevBuf* bufs[] = {&G.rowptr, &G.rowstart, &G.rowlen, &G.rowcap, &S.scr, &S.stage, &S.grow, &S.col_old,
-                    &S.val_old, &S.colN, &S.valN, &S.T, &S.T2};
+                    &S.val_old, &S.colN, &S.valN, &S.T, &S.T2, &S.items, &S.first, &S.itp};
   for (DevBuf* b : bufs) free_buf(ctx->st, *b);
   cudaStreamSynchronize(ctx->st);
 }
@@ -2086,15 +2188,18 @@ static hci_status sigma_direct(hci_ctx* ctx, const double* c, double* sigma, int
   Graph& G = ctx->graph;
   GraphArgs A;
   space_args(ctx, G.nV, A);
-  A.ddiag = bp<double>(G.diag);
+  A.items = bp<int4>(ctx->inc.items);
+  A.nitems = ctx->inc.nitems;
+  A.dpart = bp<double>(ctx->inc.itp);
   unsigned long long* cnt = reinterpret_cast<unsigned long long*>(bp<char>(ctx->s_counter) + 56);
   for (int v = 0; v < nvec; ++v) {
     A.dc = c + (int64_t)v * G.nV;
-    A.dsig = sigma + (int64_t)v * G.nV;
     A.dnnz = G.nnz < 0 ? cnt : nullptr;
     if (A.dnnz) HCI_CUDA(ctx, cudaMemsetAsync(cnt, 0, 8, ctx->st));
     HCI_CUDA(ctx, cudaMemsetAsync(A.queue, 0, 8, ctx->st));
     HCI_LAUNCH(k_rows<ROWS_SIGMA>, rows_grid(ctx), G_WARPS * 32, 0, ctx->st)(A);
+    HCI_LAUNCH(k_row_sums, grid_for(G.nV, 256), 256, 0, ctx->st)(bp<int64_t>(ctx->inc.first), G.nV, A.dpart,
+                                                                bp<double>(G.diag), A.dc, sigma + (int64_t)v * G.nV);
     HCI_CUDA(ctx, cudaGetLastError());
     if (A.dnnz) {
       unsigned long long h = 0;
@@ -2110,6 +2215,8 @@ hci_status direct_rdm(hci_ctx* ctx, const double* c, const RdmAcc& R) {
   Graph& G = ctx->graph;
   GraphArgs A;
   space_args(ctx, G.nV, A);
+  A.items = bp<int4>(ctx->inc.items);
+  A.nitems = ctx->inc.nitems;
   A.dc = c;
   A.R = R;
   HCI_CUDA(ctx, cudaMemsetAsync(A.queue, 0, 8, ctx->st));

@@ -98,6 +98,8 @@ struct IncScratch {
   DevBuf pos_old, mark, flag, newrows, rpN, cnt, keys_old, s2i_old, grow;
   DevBuf colN, valN, hist, tbase, T, T2, tstart, len, rp_old, col_old, val_old, len_old, cap_old;  // both orientations
   DevBuf scr, stage, roff, ctl, left, samp;   // staged row search
+  DevBuf items, first, itp;                   // its work items, each row's first, the items' offsets
+  int64_t nitems = 0;                         // direct form: work items of a traversal
 };
 
 // Per-phase CUDA-event timers (enabled by hci_profile).
