@@ -371,7 +371,7 @@ extern "C" hci_status hci_destroy(hci_ctx* ctx) {
                     &ctx->lists.list_max, &ctx->lists.f_ref, &ctx->s_items,
                     &ctx->lists.same_mag, &ctx->lists.same_tgt, &ctx->lists.single_bound, &ctx->lists.single_pr, &ctx->lists.single_bf,
                     &ctx->lists.single_f32, &ctx->lists.single_max,
-                    &ctx->graph.rowptr, &ctx->graph.rowstart, &ctx->graph.diag, &ctx->graph.keys,
+                    &ctx->graph.rowptr, &ctx->graph.rowstart, &ctx->graph.diag, &ctx->graph.sig_plan, &ctx->graph.keys,
                     &ctx->s_cand, &ctx->s_cand2, &ctx->s_flags, &ctx->s_scan, &ctx->s_misc, &ctx->s_counter,
                     &ctx->s_hist, &ctx->g_ua, &ctx->g_ga, &ctx->g_ia, &ctx->g_ub, &ctx->g_gb, &ctx->g_ib,
                     &ctx->g_permb, &ctx->g_bkeys, &ctx->g_bkeys2, &ctx->g_nbr_ptr, &ctx->g_nbr, &ctx->g_cnt,

@@ -582,10 +582,17 @@ __global__ void k_row_sums(const int64_t* __restrict__ first, int64_t nV, const 
   }
 }
 
-// out[t] = items[t * n / ns], an evenly strided sample of ns items
+// out[t] = a SAMP_SHARE-th of items[t * n / ns], an evenly strided sample of ns
+// items (a whole one of ITEM_COST checks keeps its warp for 200 us)
+constexpr int SAMP_SHARE = 8;
 __global__ void k_stride_sample(const int4* __restrict__ items, int64_t n, int64_t ns, int4* __restrict__ out) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < ns) out[t] = items[t * n / ns];
+  if (t < ns) {
+    int4 it = items[t * n / ns];
+    it.z = it.z * SAMP_SHARE + (int)(t % SAMP_SHARE);
+    it.w *= SAMP_SHARE;
+    out[t] = it;
+  }
 }
 
 // row offsets from the items': rp[q] = itp[first[q]], q <= nrows; len[q] its
@@ -1031,75 +1038,120 @@ __global__ void k_diag(int n, const double* __restrict__ h, const double* __rest
   }
 }
 
-// Both-orientation form: sigma = diag .* c + offdiag * c ; one warp per row.  In the single-vector
-// path each warp owns a contiguous range of rows holding an equal share of
-// the connections and keeps four (col, val, c[col]) loads per lane in
-// flight; the CSR stream is read with evict-first hints so that c stays in
-// L2.  Rows are summed four at a time, so that the cross-lane reduction
-// costs 1.5 FP64 additions per row instead of 8 (the FP64 pipe, 2 DFMA per
-// clock per SM, bounds this kernel).
-// blocks of k_sigma1 per SM, all resident (the grid is this many per SM)
+// Both-orientation form: sigma = diag .* c + offdiag * c.  Every warp takes an
+// equal share of the connections (logical entries [w, w + 1) x chunk), whatever
+// rows they belong to: it owns the rows that start in its share and sums the
+// last one up to the share's end; the share's head, the rest of a row that
+// started earlier, goes to head[w], which k_sigma_heads adds to the row in the
+// order of the shares.  (With whole rows per warp the aufbau
+// determinant's row, connected to most of a small space, was all of the
+// product: 221 us on a 2.8e4-determinant (24e,24o) space, 97 us so; 2940 and
+// 2518 us on 3.0e5 (44e,44o) determinants.)  Four
+// (col, val, c[col]) loads per lane in flight; the connections are read with
+// evict-first hints so that c stays in L2.  Rows are summed four at a time,
+// so that the cross-lane reduction costs 1.5 FP64 additions per row instead
+// of 8 (the FP64 pipe, 2 DFMA per clock per SM, and the L1's address stage,
+// one gathered entry per clock per SM, bound this kernel).
+// blocks of k_sigma1 per SM at most, all resident
 constexpr int SIGMA_BLOCKS_PER_SM = 5;
+constexpr int64_t SIGMA_SHARE = 512;     // entries per warp at least
+
+// plan[w] = the first row that starts at or after entry w x chunk, w <= warps
+__global__ void k_sigma_plan(const int64_t* __restrict__ rowptr, int64_t nV, int64_t warps, int64_t chunk,
+                             int32_t* __restrict__ plan) {
+  const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (w > warps) return;
+  int64_t lo = 0, hi = nV;
+  const int64_t x = w * chunk;
+  while (lo < hi) {
+    const int64_t mid = (lo + hi) >> 1;
+    if (rowptr[mid] < x) lo = mid + 1;
+    else hi = mid;
+  }
+  plan[w] = (int32_t)(w == warps ? nV : lo);
+}
+
+// sum over k < len of val[k] c[col[k]] (a lane's share)
+__device__ __forceinline__ double row_dot(const int32_t* __restrict__ col, const double* __restrict__ val, int len,
+                                          const double* __restrict__ c) {
+  double a = 0.0, a2 = 0.0;   // two chains, so consecutive FMAs do not wait on each other
+  int k = threadIdx.x & 31;
+  for (; k + 96 < len; k += 128) {
+    const int32_t j0 = __ldcs(col + k), j1 = __ldcs(col + k + 32), j2 = __ldcs(col + k + 64), j3 = __ldcs(col + k + 96);
+    const double v0 = __ldcs(val + k), v1 = __ldcs(val + k + 32), v2 = __ldcs(val + k + 64), v3 = __ldcs(val + k + 96);
+    a = fma(v0, c[j0], a);
+    a2 = fma(v1, c[j1], a2);
+    a = fma(v2, c[j2], a);
+    a2 = fma(v3, c[j3], a2);
+  }
+  for (; k < len; k += 32) a = fma(__ldcs(val + k), c[__ldcs(col + k)], a);
+  return a + a2;
+}
 
 __global__ void __launch_bounds__(256, SIGMA_BLOCKS_PER_SM) k_sigma1(const int64_t* __restrict__ rowptr,
                                                   const int64_t* __restrict__ rowstart, const int32_t* __restrict__ col,
                                                const double* __restrict__ val, const double* __restrict__ diag,
-                                               int64_t nV, const double* __restrict__ c, double* __restrict__ sigma,
-                                               int nvec_unused) {
+                                               int64_t nV, const int32_t* __restrict__ plan, int64_t chunk,
+                                               const double* __restrict__ c, double* __restrict__ sigma,
+                                               double* __restrict__ head) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int r0 = plan[warp], r1 = plan[warp + 1];
+  const int64_t e0 = warp * chunk, e1 = e0 + chunk;
   {
-    // contiguous row ranges holding an equal share of the connections
-    const int64_t tot = rowptr[nV];
-    const int64_t chunk = (tot + nwarps - 1) / nwarps;
-    int64_t r0, r1;
-    {
-      int64_t lo = 0, hi = nV, x = warp * chunk;
-      while (lo < hi) { const int64_t mid = (lo + hi) >> 1; if (rowptr[mid] < x) lo = mid + 1; else hi = mid; }
-      r0 = lo;
-      lo = r0; hi = nV; x = (warp + 1) * chunk;
-      while (lo < hi) { const int64_t mid = (lo + hi) >> 1; if (rowptr[mid] < x) lo = mid + 1; else hi = mid; }
-      r1 = warp == nwarps - 1 ? nV : lo;
+    // the head: row r0 - 1 from e0 on
+    const int64_t hi = rowptr[r0];
+    double a = 0.0;
+    if (hi > e0) {
+      const int i = r0 - 1;
+      const int64_t b = rowstart[i] + (e0 - rowptr[i]);
+      a = row_dot(col + b, val + b, (int)((hi < e1 ? hi : e1) - e0), c);
+      for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     }
-    for (int64_t g = r0; g < r1; g += 4) {
-      double acc[4];
+    if (lane == 0) head[warp] = a;
+  }
+  for (int g = r0; g < r1; g += 4) {
+    double acc[4];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        double a = 0.0, a2 = 0.0;   // two chains, so consecutive FMAs do not wait on each other
-        const int64_t i = g + r;
-        if (i < r1) {
-          const int64_t b = rowstart[i], e = b + (rowptr[i + 1] - rowptr[i]);
-          int64_t k = b + lane;
-          for (; k + 96 < e; k += 128) {
-            const int32_t j0 = __ldcs(col + k), j1 = __ldcs(col + k + 32), j2 = __ldcs(col + k + 64),
-                          j3 = __ldcs(col + k + 96);
-            const double v0 = __ldcs(val + k), v1 = __ldcs(val + k + 32), v2 = __ldcs(val + k + 64),
-                         v3 = __ldcs(val + k + 96);
-            a = fma(v0, c[j0], a);
-            a2 = fma(v1, c[j1], a2);
-            a = fma(v2, c[j2], a);
-            a2 = fma(v3, c[j3], a2);
-          }
-          for (; k < e; k += 32) a = fma(__ldcs(val + k), c[__ldcs(col + k)], a);
-        }
-        acc[r] = a + a2;
+    for (int r = 0; r < 4; ++r) {
+      const int i = g + r;
+      acc[r] = 0.0;
+      if (i < r1) {
+        const int64_t b = rowstart[i], lo = rowptr[i], hi = rowptr[i + 1];
+        acc[r] = row_dot(col + b, val + b, (int)((hi < e1 ? hi : e1) - lo), c);
       }
-      // four row sums at once: halve the values held per lane across lanes
-      // 16 apart, then 8 apart, then a plain tree over the last 8 lanes
-      const bool h16 = lane & 16, h8 = lane & 8;
-      const double w0 = (h16 ? acc[2] : acc[0]) + __shfl_xor_sync(0xffffffffu, h16 ? acc[0] : acc[2], 16);
-      const double w1 = (h16 ? acc[3] : acc[1]) + __shfl_xor_sync(0xffffffffu, h16 ? acc[1] : acc[3], 16);
-      double u = (h8 ? w1 : w0) + __shfl_xor_sync(0xffffffffu, h8 ? w0 : w1, 8);
-      u += __shfl_xor_sync(0xffffffffu, u, 4);
-      u += __shfl_xor_sync(0xffffffffu, u, 2);
-      u += __shfl_xor_sync(0xffffffffu, u, 1);
-      if ((lane & 7) == 0) {
-        const int64_t i = g + (h16 ? 2 : 0) + (h8 ? 1 : 0);
-        if (i < r1) sigma[i] = fma(diag[i], c[i], u);
-      }
+    }
+    // four row sums at once: halve the values held per lane across lanes
+    // 16 apart, then 8 apart, then a plain tree over the last 8 lanes
+    const bool h16 = lane & 16, h8 = lane & 8;
+    const double w0 = (h16 ? acc[2] : acc[0]) + __shfl_xor_sync(0xffffffffu, h16 ? acc[0] : acc[2], 16);
+    const double w1 = (h16 ? acc[3] : acc[1]) + __shfl_xor_sync(0xffffffffu, h16 ? acc[1] : acc[3], 16);
+    double u = (h8 ? w1 : w0) + __shfl_xor_sync(0xffffffffu, h8 ? w0 : w1, 8);
+    u += __shfl_xor_sync(0xffffffffu, u, 4);
+    u += __shfl_xor_sync(0xffffffffu, u, 2);
+    u += __shfl_xor_sync(0xffffffffu, u, 1);
+    if ((lane & 7) == 0) {
+      const int i = g + (h16 ? 2 : 0) + (h8 ? 1 : 0);
+      if (i < r1) sigma[i] = fma(diag[i], c[i], u);
     }
   }
+}
+
+// The heads added to their rows: the first share of a run of heads of one row
+// adds them all, in order.  A thread per share in a launch of its own: left to
+// the last block of k_sigma1 its dependent loads took 25 us.
+__global__ void __launch_bounds__(128) k_sigma_heads(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ plan,
+                                                     int64_t warps, int64_t chunk, const double* __restrict__ head,
+                                                     double* __restrict__ sigma) {
+  const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (w >= warps) return;
+  const int64_t row = (int64_t)plan[w] - 1;
+  if (row < 0) return;
+  const int64_t lo = rowptr[row], hi = rowptr[row + 1];
+  if (hi <= w * chunk || lo < (w - 1) * chunk) return;      // no head, or not the row's first
+  double s = sigma[row];
+  for (int64_t v = w; v < warps && hi > v * chunk; ++v) s += head[v];
+  sigma[row] = s;
 }
 
 // several vectors at once (one pass over the connections per 4 vectors)
@@ -1661,7 +1713,7 @@ static hci_status stage_new_rows(hci_ctx* ctx, GraphArgs& A, const int32_t* rowl
   HCI_CUDA(ctx, cudaStreamSynchronize(st));
   double sum = 0.0;
   for (int64_t v : cnt) sum += (double)v;
-  const double mean = ns > 0 ? sum / (double)ns : 0.0, rows = (double)A.nitems * mean;
+  const double mean = ns > 0 ? SAMP_SHARE * sum / (double)ns : 0.0, rows = (double)A.nitems * mean;
   const int64_t est = (int64_t)std::min((double)nnew * (double)nV, 1.5 * rows) + ((int64_t)1 << 22);
   {
     // a graph that cannot fit device memory is refused before the search:
@@ -2130,6 +2182,8 @@ static bool want_half(const hci_ctx* ctx) {
   return ctx->sigma_mode == HCI_SIGMA_HALF || (ctx->sigma_mode == HCI_SIGMA_AUTO && ctx->half_fallback);
 }
 
+static hci_status plan_sigma(hci_ctx* ctx);
+
 static hci_status graph_stored(hci_ctx* ctx, const uint64_t* keys, int64_t nV) {
   Graph& G = ctx->graph;
   const bool half = want_half(ctx);
@@ -2143,6 +2197,7 @@ static hci_status graph_stored(hci_ctx* ctx, const uint64_t* keys, int64_t nV) {
     G.direct = false;
     s = half ? graph_build_half(ctx, keys, nV) : graph_build_full(ctx, keys, nV);
   }
+  if (s == HCI_OK && !half) s = plan_sigma(ctx);
   return s;
 }
 
@@ -2225,6 +2280,22 @@ hci_status direct_rdm(hci_ctx* ctx, const double* c, const RdmAcc& R) {
   return HCI_OK;
 }
 
+// plan of k_sigma1 for the cached both-orientation graph: the shares' first
+// rows, then the heads
+static double* sig_head(Graph& G) { return reinterpret_cast<double*>(bp<char>(G.sig_plan) + ((size_t)(G.sig_warps + 2) * 4 + 7) / 8 * 8); }
+static hci_status plan_sigma(hci_ctx* ctx) {
+  Graph& G = ctx->graph;
+  const int64_t most = (int64_t)ctx->nsm * SIGMA_BLOCKS_PER_SM;
+  const int64_t blocks = std::max<int64_t>(1, std::min(most, G.nstored / (8 * SIGMA_SHARE)));
+  G.sig_warps = blocks * 8;
+  G.sig_chunk = std::max<int64_t>(1, (G.nstored + G.sig_warps - 1) / G.sig_warps);
+  HCI_TRY(ensure_buf(ctx, G.sig_plan, (size_t)(G.sig_warps + 2) * 4 + 8 + (size_t)G.sig_warps * 8 + 16));
+  HCI_LAUNCH(k_sigma_plan, (unsigned)((G.sig_warps + 256) / 256), 256, 0, ctx->st)(
+      bp<int64_t>(G.rowptr), G.nV, G.sig_warps, G.sig_chunk, bp<int32_t>(G.sig_plan));
+  HCI_CUDA(ctx, cudaGetLastError());
+  return HCI_OK;
+}
+
 hci_status sigma_apply(hci_ctx* ctx, const double* c, double* sigma, int nvec) {
   Graph& G = ctx->graph;
   if (G.direct) {
@@ -2259,9 +2330,11 @@ hci_status sigma_apply(hci_ctx* ctx, const double* c, double* sigma, int nvec) {
       HCI_LAUNCH(k_sigma_half, grid_for(G.nV * 32, 256, ctx->nsm * 16), 256, 0, ctx->st)(
           bp<int64_t>(G.rowptr), bp<int64_t>(G.rowstart), T, bp<double>(G.diag), G.nV, c, sigma, nvec);
   } else if (nvec == 1) {
-    HCI_LAUNCH(k_sigma1, ctx->nsm * SIGMA_BLOCKS_PER_SM, 256, 0, ctx->st)(bp<int64_t>(G.rowptr), bp<int64_t>(G.rowstart),
-                                                        bp<int32_t>(G.seg_col[0]), bp<double>(G.seg_val[0]),
-                                                        bp<double>(G.diag), G.nV, c, sigma, 1);
+    HCI_LAUNCH(k_sigma1, (unsigned)(G.sig_warps / 8), 256, 0, ctx->st)(
+        bp<int64_t>(G.rowptr), bp<int64_t>(G.rowstart), bp<int32_t>(G.seg_col[0]), bp<double>(G.seg_val[0]),
+        bp<double>(G.diag), G.nV, bp<int32_t>(G.sig_plan), G.sig_chunk, c, sigma, sig_head(G));
+    HCI_LAUNCH(k_sigma_heads, (unsigned)((G.sig_warps + 127) / 128), 128, 0, ctx->st)(
+        bp<int64_t>(G.rowptr), bp<int32_t>(G.sig_plan), G.sig_warps, G.sig_chunk, sig_head(G), sigma);
   } else {
     HCI_LAUNCH(k_sigma, grid_for(G.nV * 32, 256, ctx->nsm * 16), 256, 0, ctx->st)(
         bp<int64_t>(G.rowptr), bp<int64_t>(G.rowstart), bp<int32_t>(G.seg_col[0]), bp<double>(G.seg_val[0]),

@@ -1,0 +1,58 @@
+"""The stored product where a warp's equal share of the connections cuts rows:
+spaces from one determinant up, rows longer than several shares (a determinant
+connected to the whole space), unconnected determinants (empty rows, the last
+ones among them), against the oracle's rows."""
+import numpy as np
+import pytest
+import torch
+
+import hci_inputs as hi
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(inst, keys, seed=1, grow=0):
+    import paper_1708_07544_gb300 as pkg
+
+    dev = lambda k: torch.tensor(np.ascontiguousarray(k).astype(np.int64), device="cuda")  # noqa: E731
+    c = hi.random_vector(len(keys), seed)
+    ref = oracle.sigma_rows(inst, keys, c, np.arange(len(keys)))
+    with pkg.HCISolver(inst.norb, inst.nalpha, inst.nbeta, torch.tensor(inst.h, device="cuda"),
+                       torch.tensor(inst.eri, device="cuda"), inst.e_core) as s:
+        if grow:      # the graph extended from a part of the space
+            part = np.sort(np.random.default_rng(2).choice(len(keys), grow, replace=False))
+            s.sigma(dev(keys[part]), torch.ones(grow, dtype=torch.float64, device="cuda"))
+        out = s.sigma(dev(keys), torch.tensor(c, device="cuda"))
+        again = s.sigma(dev(keys), torch.tensor(c, device="cuda"))
+    assert torch.equal(out, again)
+    assert np.abs(out.cpu().numpy() - ref).max() <= 1e-11 * max(1.0, np.abs(ref).max())
+
+
+@pytest.mark.parametrize("nV", [1, 2, 3, 5, 33, 100, 700, 4000])
+@pytest.mark.parametrize("grow", [0, 1])
+def test_random_spaces(nV, grow):
+    inst = hi.random_tiny(10, 5, 4, 77)
+    _check(inst, hi.random_det_keys(10, 5, 4, nV, 5), grow=grow if nV > 1 else 0)
+
+
+# every single and double of one determinant: its row holds the whole space
+@pytest.mark.parametrize("n,na,nb", [(8, 4, 4), (12, 6, 5)])
+def test_one_long_row(n, na, nb):
+    inst = hi.random_tiny(n, na, nb, 9)
+    k0 = hi.aufbau_key(na, nb)
+    new, _, _ = oracle.select(inst, k0, np.ones(1), 0.0)
+    keys = np.concatenate([k0, new])
+    _check(inst, keys[np.lexsort((keys[:, 1], keys[:, 0]))])
+
+
+# determinants three or more electrons apart: every row empty, or only a few
+@pytest.mark.parametrize("linked", [0, 3])
+def test_empty_rows(linked):
+    inst = hi.random_tiny(16, 4, 4, 4)
+    blocks = [0b1111, 0b11110000, 0b111100000000, 0b1111000000000000]
+    keys = [(a, b) for a in blocks for b in blocks if (a, b) != (15, 15)]
+    keys = [(a, b) for a, b in keys]
+    keys += [(0b1111, (0b111 | (1 << (4 + k)))) for k in range(linked)]
+    keys = np.array(sorted(set(keys)), dtype=np.uint64)
+    _check(inst, keys)
