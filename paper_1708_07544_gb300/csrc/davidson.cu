@@ -14,12 +14,19 @@ constexpr int MAXSUB = 24;          // subspace size before restart (<= 32)
 constexpr int DAV_KEEP = 4;         // Ritz vectors kept for the next, grown space
 constexpr int LDG = 32;             // leading dimension of the subspace matrix
 constexpr int DBLOCK = 256;
+// Iterations queued before the host waits for their reports.  A wait leaves
+// the GPU idle for about 35 us (the copy back, the host, the next launches),
+// as long as an iteration's own kernels on a small space; the kernels queued
+// behind the converged one return at once (about 14 us per iteration).
+constexpr int DAV_AHEAD = 4;
 
 // what the host reads of an iteration
 struct DavReport {
   double theta;           // Ritz value
   double ols[3];          // |r|^2, x . M^-1 r, x . M^-1 x (Olsen correction)
   int stall;              // a correction fell inside the subspace
+  int stop;               // chained iterations: nothing queued after this is to run
+  int it, k;              // Ritz steps taken, the last one's subspace size
 };
 
 struct DavDev {
@@ -173,7 +180,7 @@ __global__ void __launch_bounds__(DBLOCK) k_dots(const double* __restrict__ V, i
 //   NORM:  V_k <- t - sum_j dots_j V_j, nrm2 = |V_k|^2
 //   GCOL:  after W_k = H V_k: V_k and W_k scaled by 1 / sqrt(nrm2), then
 //          G[j][k] = G[k][j] = V_j . W_k, j <= k.  A correction of norm^2 at
-//          most 1e-26 lies in the subspace: V_k = W_k = 0 and stall = 1.
+//          most 1e-26 lies in the subspace: V_k = W_k = 0, stall = stop = 1.
 // Bound by FP64 issue (2 k + 1 operations per element) at 1e5 elements, by
 // the k vectors' bytes beyond L2.  (12e,12o) space, 1.4e5 elements, k <= 24,
 // per iteration: 4 x 24 us (products, norm), 2 x 5 (subtractions), 7 (Olsen)
@@ -185,6 +192,7 @@ __global__ void __launch_bounds__(DBLOCK, 2) k_pass(double* __restrict__ V, doub
                                                     int64_t n, double* __restrict__ t, const double* __restrict__ u,
                                                     DavDev* __restrict__ d, double* __restrict__ partial) {
   __shared__ double cs[LDG];
+  if (d->rep.stop) return;
   if (threadIdx.x < LDG) cs[threadIdx.x] = d->dots[threadIdx.x];
   __syncthreads();
   double eps = 0.0, f = 0.0;
@@ -239,7 +247,7 @@ __global__ void __launch_bounds__(DBLOCK, 2) k_pass(double* __restrict__ V, doub
       d->G[j * LDG + k] = s;
       d->G[k * LDG + j] = s;
     }
-    if (j == 0 && f == 0.0) d->rep.stall = 1;
+    if (j == 0 && f == 0.0) d->rep.stall = d->rep.stop = 1;
   } else if (j < k) {
     d->dots[j] = s;
   }
@@ -525,6 +533,7 @@ __global__ void __launch_bounds__(LW_T) k_lowest(DavDev* d, int k) {
   __shared__ double rc[LDG / 2], rs[LDG / 2];
   __shared__ int rp[LDG / 2], rq[LDG / 2];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (NV == 1 && d->rep.stop) return;
   const double sh = d->G[0];
   const int kx = (d->kx == k || d->kx == k - 1) ? d->kx : 0, ky = d->ky;
   for (int e = tid; e < LDG * LDG; e += LW_T) {
@@ -741,8 +750,9 @@ __global__ void __launch_bounds__(DBLOCK) k_ritz(const double* __restrict__ V, c
                                                  int k, DavDev* __restrict__ d, const double* __restrict__ diag,
                                                  int64_t n, double* __restrict__ x, double* __restrict__ wy,
                                                  double* __restrict__ t, double* __restrict__ u,
-                                                 double* __restrict__ partial) {
+                                                 double* __restrict__ partial, int chained, double tol) {
   __shared__ double ys[LDG];
+  if (d->rep.stop) return;
   if (threadIdx.x < LDG) ys[threadIdx.x] = d->y[threadIdx.x];
   __syncthreads();
   const double theta = d->rep.theta;
@@ -785,6 +795,12 @@ __global__ void __launch_bounds__(DBLOCK) k_ritz(const double* __restrict__ V, c
   double s;
   if (!grid_sums<4>(acc, 0, 3, partial, &d->ticket, &s)) return;
   if (threadIdx.x < 3) d->rep.ols[threadIdx.x] = s;
+  if (threadIdx.x == 0) {
+    d->rep.it += 1;
+    d->rep.k = k;
+    // a residual that is not finite ends the chain too
+    if (chained && (!(sqrt(s) > tol) || !isfinite(s) || !isfinite(theta))) d->rep.stop = 1;
+  }
 }
 
 // The kk <= DAV_KEEP lowest Ritz vectors of the current subspace (ascending Ritz value)
@@ -1026,7 +1042,9 @@ struct Dav {
     HCI_CUDA(ctx, cudaGetLastError());
     return HCI_OK;
   }
-  hci_status sigma(int slot) { return sigma_apply(ctx, V + (int64_t)slot * ld, W + (int64_t)slot * ld, 1); }
+  hci_status sigma(int slot) {
+    return sigma_apply(ctx, V + (int64_t)slot * ld, W + (int64_t)slot * ld, 1, &d->rep.stop);
+  }
 };
 
 }  // namespace
@@ -1131,10 +1149,7 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
   // start vector, in the graph's internal order (after the kept vectors)
   double* V0 = D.V + (int64_t)kwarm * D.ld;
   HCI_TRY(to_internal(ctx, c_inout, V0, 1));
-  HCI_TRY(D.dots(V0, 1, V0, &D.d->nrm2));
-  double nrm2 = 0.0;
-  HCI_CUDA(ctx, cudaMemcpyAsync(&nrm2, &D.d->nrm2, 8, cudaMemcpyDeviceToHost, st));
-  HCI_CUDA(ctx, cudaStreamSynchronize(st));
+  double nrm2 = c0n2;
   if (ctx->spin_parity != 0 && nrm2 > 0.0 && std::isfinite(nrm2)) {
     // the start vector's part of the requested spin parity
     parity_project(ctx, V0, nV, D.nblk);
@@ -1202,58 +1217,42 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
   bool converged = false;
   double theta = 0.0, rn = 0.0;
   int it = 0;
-  // one host synchronisation per iteration: the Ritz value, the residual
-  // and whether the previous correction fell inside the subspace
-  auto ritz = [&](double& th, double& r, int& stall) -> hci_status {
+  // Without locked vectors or spin parity an iteration is one chain of
+  // launches, and several are queued at a time: a kernel of the chain returns
+  // at once when an earlier one found convergence, an unusable residual or a
+  // correction inside the subspace (rep.stop).  The one-orientation and
+  // direct products do not look at the flag and go one at a time.
+  const bool plain = m == 0 && ctx->spin_parity == 0;
+  const int ahead = plain && !G.half && !G.direct ? DAV_AHEAD : 1;
+  DavReport rep = {};
+  auto ritz = [&]() -> hci_status {
     HCI_LAUNCH(k_lowest<1>, 1, LW_T, 0, st)(D.d, k);
-    HCI_LAUNCH(k_ritz, D.rblk2, DBLOCK, 0, st)(D.V, D.W, D.ld, k, D.d, diag, nV, D.x, D.wy, D.t, D.u, D.part);
+    HCI_LAUNCH(k_ritz, D.rblk2, DBLOCK, 0, st)(D.V, D.W, D.ld, k, D.d, diag, nV, D.x, D.wy, D.t, D.u, D.part,
+                                              plain ? 1 : 0, tol);
     HCI_CUDA(ctx, cudaGetLastError());
-    DavReport h;
-    HCI_CUDA(ctx, cudaMemcpyAsync(&h, &D.d->rep, sizeof h, cudaMemcpyDeviceToHost, st));
-    HCI_CUDA(ctx, cudaStreamSynchronize(st));
-    th = h.theta;
-    r = std::sqrt(h.ols[0]);
-    stall = h.stall;
     return HCI_OK;
   };
-  for (; it < maxit; ++it) {
-    int stall = 0;
-    HCI_TRY(ritz(theta, rn, stall));
-    if (stall) {
-      // the last correction lay in the subspace (it was added as zeros):
-      // drop it, take the Ritz pair of the subspace before it and stop
-      --k;
-      HCI_TRY(ritz(theta, rn, stall));
-      if (!std::isfinite(theta) || !std::isfinite(rn))
-        return hci_fail(ctx, HCI_ERR_CUDA, "hci_davidson: non-finite Ritz value or residual");
-      converged = rn <= tol;
-      break;
-    }
+  auto report = [&]() -> hci_status {
+    HCI_CUDA(ctx, cudaMemcpyAsync(&rep, &D.d->rep, sizeof rep, cudaMemcpyDeviceToHost, st));
+    HCI_CUDA(ctx, cudaStreamSynchronize(st));
+    theta = rep.theta;
+    rn = std::sqrt(rep.ols[0]);
     if (!std::isfinite(theta) || !std::isfinite(rn))
       return hci_fail(ctx, HCI_ERR_CUDA, "hci_davidson: non-finite Ritz value or residual");
-    if (rn <= tol) {
-      converged = true;
-      break;
-    }
-    if (k == MAXSUB) {
-      // restart from the current Ritz vector
-      HCI_CUDA(ctx, cudaMemcpyAsync(D.V, D.x, (size_t)nV * 8, cudaMemcpyDeviceToDevice, st));
-      HCI_CUDA(ctx, cudaMemcpyAsync(D.W, D.wy, (size_t)nV * 8, cudaMemcpyDeviceToDevice, st));
-      HCI_TRY(D.dots(D.V, 1, D.V, &D.d->nrm2));
-      HCI_LAUNCH(k_scale_by, D.nblk, DBLOCK, 0, st)(D.V, D.W, nV, &D.d->nrm2);
-      HCI_TRY(D.dots(D.V, 1, D.W, D.d->dots, 0));
-      k = 1;
-    }
-    // orthogonalise the correction twice, normalise
-    if (m == 0 && ctx->spin_parity == 0) {
-      HCI_TRY(D.pass<PASS_OLSEN>(k));
-      HCI_TRY(D.pass<PASS_ORTH>(k));
-      HCI_TRY(D.pass<PASS_NORM>(k));
-      HCI_TRY(D.sigma(k));
-      HCI_TRY(D.pass<PASS_GCOL>(k));
-      ++k;
-      continue;
-    }
+    return HCI_OK;
+  };
+  // the correction of the last Ritz step, orthogonalised twice and
+  // normalised, as vector k, with its product
+  auto expand = [&]() -> hci_status {
+    HCI_TRY(D.pass<PASS_OLSEN>(k));
+    HCI_TRY(D.pass<PASS_ORTH>(k));
+    HCI_TRY(D.pass<PASS_NORM>(k));
+    HCI_TRY(D.sigma(k));
+    HCI_TRY(D.pass<PASS_GCOL>(k));
+    ++k;
+    return HCI_OK;
+  };
+  auto expand_locked = [&]() -> hci_status {
     HCI_LAUNCH(k_olsen, D.nblk, DBLOCK, 0, st)(D.d, nV, D.u, D.t);
     parity_project(ctx, D.t, nV, D.nblk);
     for (int pass = 0; pass < 2; ++pass) {
@@ -1265,13 +1264,60 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
       }
     }
     HCI_TRY(D.dots(D.t, 1, D.t, &D.d->nrm2));
-    double* slot = D.V + (int64_t)k * D.ld;
-    HCI_LAUNCH(k_scale_unit, D.nblk, DBLOCK, 0, st)(D.t, nV, D.d, slot);
+    HCI_LAUNCH(k_scale_unit, D.nblk, DBLOCK, 0, st)(D.t, nV, D.d, D.V + (int64_t)k * D.ld);
     HCI_TRY(D.sigma(k));
     HCI_TRY(D.dots(D.V, k + 1, D.W + (int64_t)k * D.ld, D.d->dots, k));
     ++k;
+    return HCI_OK;
+  };
+  while (it < maxit) {
+    const int before = it;
+    int queued = 1;
+    HCI_TRY(ritz());
+    for (; queued < ahead && it + queued < maxit && k < MAXSUB; ++queued) {
+      HCI_TRY(expand());
+      HCI_TRY(ritz());
+    }
+    HCI_TRY(report());
+    it = plain ? rep.it : it + 1;
+    if (plain && rep.stop) {
+      // products queued behind the stop did not run
+      const int64_t skipped = (queued - 1) - (it - before - (rep.stall ? 0 : 1));
+      ctx->st_counts[HCI_ST_SIGMA_CALLS] -= skipped;
+      ctx->st_counts[HCI_ST_SIGMA_ROWS] -= skipped * G.nV;
+      ctx->st_counts[HCI_ST_SIGMA_NNZ] -= skipped * G.nnz;
+      // a correction inside the subspace: the Ritz pair before it is final
+      k = rep.k;
+      converged = rn <= tol;
+      HCI_CUDA(ctx, cudaMemsetAsync(&D.d->rep.stop, 0, sizeof(int), st));
+      break;
+    }
+    if (!plain && rep.stall) {
+      // the last correction lay in the subspace (it was added as zeros):
+      // drop it, take the Ritz pair of the subspace before it and stop
+      --k;
+      HCI_TRY(ritz());
+      HCI_TRY(report());
+      converged = rn <= tol;
+      break;
+    }
+    if (rn <= tol) {
+      converged = true;
+      break;
+    }
+    if (it >= maxit) break;
+    if (k == MAXSUB) {
+      // restart from the current Ritz vector
+      HCI_CUDA(ctx, cudaMemcpyAsync(D.V, D.x, (size_t)nV * 8, cudaMemcpyDeviceToDevice, st));
+      HCI_CUDA(ctx, cudaMemcpyAsync(D.W, D.wy, (size_t)nV * 8, cudaMemcpyDeviceToDevice, st));
+      HCI_TRY(D.dots(D.V, 1, D.V, &D.d->nrm2));
+      HCI_LAUNCH(k_scale_by, D.nblk, DBLOCK, 0, st)(D.V, D.W, nV, &D.d->nrm2);
+      HCI_TRY(D.dots(D.V, 1, D.W, D.d->dots, 0));
+      k = 1;
+    }
+    HCI_TRY(plain ? expand() : expand_locked());
   }
-  if (iters) *iters = it + (converged ? 1 : 0);
+  if (iters) *iters = it;
   // the lowest Ritz vectors for a later run on this space or a grown one
   K.valid = false;
   if (m == 0 && converged) {

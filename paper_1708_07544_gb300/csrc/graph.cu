@@ -1043,7 +1043,7 @@ __global__ void k_diag(int n, const double* __restrict__ h, const double* __rest
 // rows they belong to: it owns the rows that start in its share and sums the
 // last one up to the share's end; the share's head, the rest of a row that
 // started earlier, goes to head[w], which k_sigma_heads adds to the row in the
-// order of the shares.  (With whole rows per warp the aufbau
+// order of the shares.  Nothing is done when *stop is set.  (With whole rows per warp the aufbau
 // determinant's row, connected to most of a small space, was all of the
 // product: 221 us on a 2.8e4-determinant (24e,24o) space, 97 us so; 2940 and
 // 2518 us on 3.0e5 (44e,44o) determinants.)  Four
@@ -1093,7 +1093,8 @@ __global__ void __launch_bounds__(256, SIGMA_BLOCKS_PER_SM) k_sigma1(const int64
                                                const double* __restrict__ val, const double* __restrict__ diag,
                                                int64_t nV, const int32_t* __restrict__ plan, int64_t chunk,
                                                const double* __restrict__ c, double* __restrict__ sigma,
-                                               double* __restrict__ head) {
+                                               double* __restrict__ head, const int* __restrict__ stop) {
+  if (stop && *stop) return;
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int r0 = plan[warp], r1 = plan[warp + 1];
@@ -1142,9 +1143,9 @@ __global__ void __launch_bounds__(256, SIGMA_BLOCKS_PER_SM) k_sigma1(const int64
 // the last block of k_sigma1 its dependent loads took 25 us.
 __global__ void __launch_bounds__(128) k_sigma_heads(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ plan,
                                                      int64_t warps, int64_t chunk, const double* __restrict__ head,
-                                                     double* __restrict__ sigma) {
+                                                     double* __restrict__ sigma, const int* __restrict__ stop) {
   const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (w >= warps) return;
+  if (w >= warps || (stop && *stop)) return;
   const int64_t row = (int64_t)plan[w] - 1;
   if (row < 0) return;
   const int64_t lo = rowptr[row], hi = rowptr[row + 1];
@@ -2296,7 +2297,7 @@ static hci_status plan_sigma(hci_ctx* ctx) {
   return HCI_OK;
 }
 
-hci_status sigma_apply(hci_ctx* ctx, const double* c, double* sigma, int nvec) {
+hci_status sigma_apply(hci_ctx* ctx, const double* c, double* sigma, int nvec, const int* stop) {
   Graph& G = ctx->graph;
   if (G.direct) {
     prof_tic(ctx, HCI_PH_SIGMA);
@@ -2332,9 +2333,9 @@ hci_status sigma_apply(hci_ctx* ctx, const double* c, double* sigma, int nvec) {
   } else if (nvec == 1) {
     HCI_LAUNCH(k_sigma1, (unsigned)(G.sig_warps / 8), 256, 0, ctx->st)(
         bp<int64_t>(G.rowptr), bp<int64_t>(G.rowstart), bp<int32_t>(G.seg_col[0]), bp<double>(G.seg_val[0]),
-        bp<double>(G.diag), G.nV, bp<int32_t>(G.sig_plan), G.sig_chunk, c, sigma, sig_head(G));
+        bp<double>(G.diag), G.nV, bp<int32_t>(G.sig_plan), G.sig_chunk, c, sigma, sig_head(G), stop);
     HCI_LAUNCH(k_sigma_heads, (unsigned)((G.sig_warps + 127) / 128), 128, 0, ctx->st)(
-        bp<int64_t>(G.rowptr), bp<int32_t>(G.sig_plan), G.sig_warps, G.sig_chunk, sig_head(G), sigma);
+        bp<int64_t>(G.rowptr), bp<int32_t>(G.sig_plan), G.sig_warps, G.sig_chunk, sig_head(G), sigma, stop);
   } else {
     HCI_LAUNCH(k_sigma, grid_for(G.nV * 32, 256, ctx->nsm * 16), 256, 0, ctx->st)(
         bp<int64_t>(G.rowptr), bp<int64_t>(G.rowstart), bp<int32_t>(G.seg_col[0]), bp<double>(G.seg_val[0]),

@@ -247,8 +247,10 @@ hci_status check_sorted(hci_ctx* ctx, const uint64_t* keys, int64_t n, int* ok_h
 
 // graph.cu
 hci_status graph_ensure(hci_ctx* ctx, const uint64_t* keys, int64_t nV);
-// sigma on vectors in internal order (rows/columns of the cached graph)
-hci_status sigma_apply(hci_ctx* ctx, const double* c, double* sigma, int nvec);
+// sigma on vectors in internal order (rows/columns of the cached graph); with
+// stop given (device) the both-orientation product of one vector does nothing
+// when it is set
+hci_status sigma_apply(hci_ctx* ctx, const double* c, double* sigma, int nvec, const int* stop = nullptr);
 // out[i] = sum_j H_ij c_j for the rows i in [r0, nV) of the cached stored
 // graph, off-diagonal entries only, for a c that vanishes on those rows
 hci_status sigma_tail(hci_ctx* ctx, int64_t r0, const double* c, double* out);
