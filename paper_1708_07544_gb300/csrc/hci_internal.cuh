@@ -20,6 +20,7 @@
 struct DevBuf {
   void* p = nullptr;
   size_t bytes = 0;
+  bool slab = false;   // part of its context's slab: nothing to free
 };
 
 // Stored connections are kept in segments (one per build or extension of
@@ -128,6 +129,8 @@ struct hci_ctx {
   int n = 0, na = 0, nb = 0;
   double ecore = 0;
   cudaStream_t st = nullptr;
+  void* slab = nullptr;              // the small buffers' memory (ensure_buf)
+  size_t slab_used = 0;
   DevBuf h, eri;                     // device copies
   DevBuf jk_same, j_opp;             // n^3 tables for single excitations
   Lists lists;

@@ -5,8 +5,10 @@
 //   c^{mu+1}, E^{mu+1} = Davidson on V^{mu+1} warm-started from the padded c.
 // hci_solve_batch runs many such solves concurrently, one context and one
 // stream per in-flight instance, driven by a pool of host threads.
+#include <algorithm>
 #include <atomic>
 #include <mutex>
+#include <numeric>
 #include <thread>
 #include <vector>
 
@@ -266,6 +268,12 @@ extern "C" hci_status hci_solve_batch(int count, const int* norb, const int* nal
   int dev = 0;
   cudaError_t ce = cudaGetDevice(&dev);
   if (ce != cudaSuccess) return hci_fail(nullptr, HCI_ERR_CUDA, "hci_solve_batch: %s", cudaGetErrorString(ce));
+  // The instances with most orbitals start first: a solve is a serial chain of
+  // launches that cannot be split over streams, so the call lasts at least as
+  // long as its longest one after that one starts.
+  std::vector<int> order((size_t)count);
+  std::iota(order.begin(), order.end(), 0);
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return norb[a] > norb[b]; });
   std::atomic<int> next{0};
   std::atomic<int> first_err{HCI_OK};
   g_batch_err[0] = 0;
@@ -277,7 +285,8 @@ extern "C" hci_status hci_solve_batch(int count, const int* norb, const int* nal
       first_err.compare_exchange_strong(z, HCI_ERR_CUDA);
       return;
     }
-    for (int k = next.fetch_add(1); k < count; k = next.fetch_add(1)) {
+    for (int q = next.fetch_add(1); q < count; q = next.fetch_add(1)) {
+      const int k = order[(size_t)q];
       hci_ctx* ctx = nullptr;
       hci_status s = hci_create(&ctx, norb[k], nalpha[k], nbeta[k], h[k], eri[k], e_core ? e_core[k] : 0.0, st);
       DevBuf kr, cr;
