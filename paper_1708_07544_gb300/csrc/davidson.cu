@@ -37,6 +37,7 @@ struct DavDev {
   double dots[LDG];
   DavReport rep;
   double nrm2;
+  double eps, unit;           // k_pass: the Olsen step, 1 / norm of the correction (0: it lies in the subspace)
   int kx, ky;             // sizes of X and of y (0: none)
   unsigned int ticket;    // blocks of the running reduction that have finished
 };
@@ -172,84 +173,86 @@ __global__ void __launch_bounds__(DBLOCK) k_dots(const double* __restrict__ V, i
 }
 
 // The vector passes of one iteration between the Ritz step and the next
-// product, each one launch over the k subspace vectors (NA >= their number):
+// product, each one launch over the k subspace vectors (NA >= the number of
+// sums):
 //   OLSEN: t <- t - eps u (the Olsen correction, see k_ritz), dots_j = V_j . t
 //   ORTH:  t <- t - sum_j dots_j V_j, dots_j = V_j . t of the result (the
 //          second Gram-Schmidt pass's products, from the values of V_j that
-//          the first one's subtraction has in registers)
-//   NORM:  V_k <- t - sum_j dots_j V_j, nrm2 = |V_k|^2
-//   GCOL:  after W_k = H V_k: V_k and W_k scaled by 1 / sqrt(nrm2), then
-//          G[j][k] = G[k][j] = V_j . W_k, j <= k.  A correction of norm^2 at
-//          most 1e-26 lies in the subspace: V_k = W_k = 0, stall = stop = 1.
+//          the first one's subtraction has in registers), and with |t|^2 of
+//          it |t|^2 - sum_j dots_j^2, the norm^2 that the second subtraction
+//          leaves (dots_j is rounding beside t, the V_j are orthonormal):
+//          unit = 1 / the norm.  A correction of norm^2 at most 1e-26 lies in
+//          the subspace: unit = 0
+//   UNIT:  V_k <- (t - sum_j dots_j V_j) unit, no sums
+//   GCOL:  after W_k = H V_k: G[j][k] = G[k][j] = V_j . W_k, j <= k, and with
+//          unit = 0 stall = stop = 1.
 // Bound by FP64 issue (2 k + 1 operations per element) at 1e5 elements, by
-// the k vectors' bytes beyond L2.  (12e,12o) space, 1.4e5 elements, k <= 24,
-// per iteration: 4 x 24 us (products, norm), 2 x 5 (subtractions), 7 (Olsen)
-// and 6 (scaling) as separate passes with plain shuffle trees, 53 us so.
-enum { PASS_OLSEN = 0, PASS_ORTH = 1, PASS_NORM = 2, PASS_GCOL = 3 };
+// the k vectors' bytes beyond L2, and by their launch and reduction (6.3 us)
+// on small spaces.  (12e,12o) space, 1.4e5 elements, k from 17 to 24: 15.1,
+// 20.7, 9.8 and 15.1 us; with |V_k|^2 summed in a pass of its own and the
+// scaling left to GCOL 17.0, 22.9, 11.5 and 22.8.
+enum { PASS_OLSEN = 0, PASS_ORTH = 1, PASS_UNIT = 2, PASS_GCOL = 3 };
 
 template <int OP, int NA>
-__global__ void __launch_bounds__(DBLOCK, 2) k_pass(double* __restrict__ V, double* __restrict__ W, int64_t ld, int k,
-                                                    int64_t n, double* __restrict__ t, const double* __restrict__ u,
-                                                    DavDev* __restrict__ d, double* __restrict__ partial) {
+__global__ void __launch_bounds__(DBLOCK, OP == PASS_UNIT ? 2 : 1) k_pass(double* __restrict__ V, const double* __restrict__ W, int64_t ld,
+                                                    int k, int64_t n, double* __restrict__ t,
+                                                    const double* __restrict__ u, DavDev* __restrict__ d,
+                                                    double* __restrict__ partial) {
   __shared__ double cs[LDG];
   if (d->rep.stop) return;
   if (threadIdx.x < LDG) cs[threadIdx.x] = d->dots[threadIdx.x];
   __syncthreads();
-  double eps = 0.0, f = 0.0;
-  if (OP == PASS_OLSEN) {
-    const double den = d->rep.ols[2];
-    eps = den != 0.0 ? d->rep.ols[1] / den : 0.0;
-  }
-  if (OP == PASS_GCOL) {
-    const double n2 = d->nrm2;
-    f = n2 > 1e-26 ? 1.0 / sqrt(n2) : 0.0;
-  }
-  constexpr int NS = OP == PASS_NORM ? 1 : NA;
+  const double eps = OP == PASS_OLSEN ? d->eps : 0.0, f = d->unit;
+  const int nv = OP == PASS_GCOL ? k + 1 : k;            // vectors read
+  const int ns = OP == PASS_ORTH ? NA : nv;              // sums; ORTH (k < NA): the last is |t|^2
+  constexpr int NS = OP == PASS_UNIT ? 1 : NA;
   double acc[NS];
 #pragma unroll
   for (int j = 0; j < NS; ++j) acc[j] = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     double v[NA];
 #pragma unroll
-    for (int j = 0; j < NA; ++j) v[j] = j < k ? V[(int64_t)j * ld + i] : 0.0;
-    double w, vk = 0.0;
+    for (int j = 0; j < NA; ++j) v[j] = j < nv && (OP != PASS_ORTH || j < NA - 1) ? V[(int64_t)j * ld + i] : 0.0;
+    double w;
     if (OP == PASS_OLSEN) {
       w = fma(-eps, u[i], t[i]);
       t[i] = w;
     } else if (OP == PASS_GCOL) {
-      vk = f != 0.0 ? V[(int64_t)k * ld + i] * f : 0.0;
-      w = f != 0.0 ? W[(int64_t)k * ld + i] * f : 0.0;
-      V[(int64_t)k * ld + i] = vk;
-      W[(int64_t)k * ld + i] = w;
+      w = W[(int64_t)k * ld + i];
     } else {
       w = t[i];
 #pragma unroll
       for (int j = 0; j < NA; ++j)
         if (j < k) w = fma(-cs[j], v[j], w);
       if (OP == PASS_ORTH) t[i] = w;
-      else V[(int64_t)k * ld + i] = w;
+      else V[(int64_t)k * ld + i] = f != 0.0 ? w * f : 0.0;
     }
-    if (OP == PASS_NORM) {
-      acc[0] = fma(w, w, acc[0]);
-    } else {
+    if (OP != PASS_UNIT) {
 #pragma unroll
       for (int j = 0; j < NS; ++j)
-        if (j < k + (OP == PASS_GCOL)) acc[j] = fma(OP == PASS_GCOL && j >= k ? vk : v[j], w, acc[j]);
+        if (OP == PASS_ORTH && j == NA - 1) acc[j] = fma(w, w, acc[j]);
+        else if (j < nv) acc[j] = fma(v[j], w, acc[j]);
     }
   }
+  if (OP == PASS_UNIT) return;
   double s;
-  if (!grid_sums<NS>(acc, 0, OP == PASS_NORM ? 1 : OP == PASS_GCOL ? k + 1 : k, partial, &d->ticket, &s)) return;
+  if (!grid_sums<NS>(acc, 0, ns, partial, &d->ticket, &s)) return;
   const int j = threadIdx.x;
-  if (OP == PASS_NORM) {
-    if (j == 0) d->nrm2 = s;
-  } else if (OP == PASS_GCOL) {
+  if (OP == PASS_GCOL) {
     if (j <= k) {
       d->G[j * LDG + k] = s;
       d->G[k * LDG + j] = s;
     }
     if (j == 0 && f == 0.0) d->rep.stall = d->rep.stop = 1;
-  } else if (j < k) {
-    d->dots[j] = s;
+    return;
+  }
+  if (j < k) d->dots[j] = s;
+  if (OP == PASS_ORTH && j < 32) {
+    double q = j < k ? -s * s : j == NA - 1 ? s : 0.0;
+    for (int o = 16; o; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    // here and not in every thread of UNIT: a warp's FP64 root and division
+    // cost as much as its share of the pass
+    if (j == 0) d->unit = q > 1e-26 ? 1.0 / sqrt(q) : 0.0;
   }
 }
 
@@ -795,7 +798,10 @@ __global__ void __launch_bounds__(DBLOCK) k_ritz(const double* __restrict__ V, c
   double s;
   if (!grid_sums<4>(acc, 0, 3, partial, &d->ticket, &s)) return;
   if (threadIdx.x < 3) d->rep.ols[threadIdx.x] = s;
+  if (threadIdx.x >= 32) return;
+  const double num = __shfl_sync(0xffffffffu, s, 1), den = __shfl_sync(0xffffffffu, s, 2);
   if (threadIdx.x == 0) {
+    d->eps = den != 0.0 ? num / den : 0.0;
     d->rep.it += 1;
     d->rep.k = k;
     // a residual that is not finite ends the chain too
@@ -1016,10 +1022,9 @@ struct Dav {
   DavDev* d;
   int nblk;     // blocks of the elementwise passes
   // blocks of the reducing passes: each warp pays the reduction once, so few
-  // blocks (one per SM: 18.6 / 24.8 / 13.4 us for OLSEN / ORTH / NORM at
-  // 1.2e5 elements and k = 22, two 20.6 / 28.1 / 14.3, three 30.7 / 37.8 /
-  // 16.5); k_ritz and GCOL, which also store two to four vectors, take two
-  // (GCOL 24.7, one 28.9; k_ritz 65.9 at 5e5 elements, one 84.2)
+  // blocks (one per SM: 18.6 / 24.8 us for OLSEN / ORTH at 1.2e5 elements
+  // and k = 22, two 20.6 / 28.1, three 30.7 / 37.8); k_ritz, which also
+  // stores four vectors, takes two (65.9 us at 5e5 elements, one 84.2)
   int rblk, rblk2;
 
   // out[j] = Vb_j . w, j < k; with gcol >= 0 also column gcol of G
@@ -1031,8 +1036,8 @@ struct Dav {
   }
   template <int OP>
   hci_status pass(int k) {
-    const int na = k + (OP == PASS_GCOL);
-    const int g = OP == PASS_GCOL ? rblk2 : rblk;
+    const int na = k + (OP == PASS_ORTH || OP == PASS_GCOL);
+    const int g = OP == PASS_UNIT ? nblk : rblk;
     if (na <= 8)
       HCI_LAUNCH((k_pass<OP, 8>), g, DBLOCK, 0, ctx->st)(V, W, ld, k, n, t, u, d, part);
     else if (na <= 16)
@@ -1246,7 +1251,7 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
   auto expand = [&]() -> hci_status {
     HCI_TRY(D.pass<PASS_OLSEN>(k));
     HCI_TRY(D.pass<PASS_ORTH>(k));
-    HCI_TRY(D.pass<PASS_NORM>(k));
+    HCI_TRY(D.pass<PASS_UNIT>(k));
     HCI_TRY(D.sigma(k));
     HCI_TRY(D.pass<PASS_GCOL>(k));
     ++k;
