@@ -48,15 +48,6 @@ __device__ __forceinline__ int64_t lower_bound_k(const ulonglong2* __restrict__ 
   }
   return lo;
 }
-__device__ __forceinline__ int64_t lower_bound_u(const uint64_t* __restrict__ arr, int64_t n, uint64_t key) {
-  int64_t lo = 0, hi = n;
-  while (lo < hi) {
-    int64_t mid = (lo + hi) >> 1;
-    if (arr[mid] < key) lo = mid + 1;
-    else hi = mid;
-  }
-  return lo;
-}
 
 // ---------------------------------------------------------------------------
 // grouping
@@ -897,60 +888,59 @@ __global__ void k_assign_starts(int64_t* __restrict__ start2, const int64_t* __r
     if (start2[i] < 0) start2[i] = base + rel[i];
 }
 
-// old rows (internal ids below nold): copied when they move (repack or
-// outgrown slack), then the transposes of the new rows' entries appended;
-// columns are stable internal ids, so rows that gain nothing are untouched
-__global__ void k_move_old_rows(const int64_t* __restrict__ start_old, const int64_t* __restrict__ len_old,
-                                int64_t nold, const int32_t* col_src, const double* val_src,
-                                const int64_t* __restrict__ start2, int32_t* col_dst, double* val_dst,
-                                const ulonglong2* __restrict__ T, const int64_t* __restrict__ tstart,
-                                const int64_t* __restrict__ hist, const double* __restrict__ valN) {
+// Rows copied to their places: row r's entries from start_src[r] of the source
+// to start_dst[r] of the destination, unless that is where they are (columns
+// are stable internal ids).  Bound by the 24 bytes per entry it moves; every
+// warp takes MOVE_CHUNK consecutive entries (logical offsets rowptr), whatever
+// rows they belong to: with a row per warp the aufbau determinant's row was
+// all of it on a small space (113 and 19 us for the old and the new rows of
+// an extension of 10 to 24 orbital spaces, 17 us each so).
+constexpr int64_t MOVE_CHUNK = 1024;
+
+__global__ void __launch_bounds__(256) k_move_rows(const int64_t* __restrict__ rowptr, int64_t nrows,
+                                                   const int64_t* __restrict__ start_src, const int32_t* col_src,
+                                                   const double* val_src, const int64_t* __restrict__ start_dst,
+                                                   int32_t* col_dst, double* val_dst) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r = warp; r < nold; r += nwarps) {
-    const int64_t src = start_old[r], dst = start2[r], len = len_old[r];
-    const int64_t tn = hist[r];
-    const bool moved = (dst != src) || (col_dst != col_src);
-    if (!moved && tn == 0) continue;
-    if (moved) {
-      int64_t k = lane;
-      for (; k + 96 < len; k += 128) {
-        const int32_t j0 = col_src[src + k], j1 = col_src[src + k + 32], j2 = col_src[src + k + 64],
-                      j3 = col_src[src + k + 96];
-        const double v0 = val_src[src + k], v1 = val_src[src + k + 32], v2 = val_src[src + k + 64],
-                     v3 = val_src[src + k + 96];
-        col_dst[dst + k] = j0; col_dst[dst + k + 32] = j1; col_dst[dst + k + 64] = j2; col_dst[dst + k + 96] = j3;
-        val_dst[dst + k] = v0; val_dst[dst + k + 32] = v1; val_dst[dst + k + 64] = v2; val_dst[dst + k + 96] = v3;
+  const int64_t total = rowptr[nrows];
+  for (int64_t c0 = warp * MOVE_CHUNK; c0 < total; c0 += nwarps * MOVE_CHUNK) {
+    const int64_t c1 = c0 + MOVE_CHUNK < total ? c0 + MOVE_CHUNK : total;
+    int64_t r = row_of_entry(rowptr, nrows, c0), lo = rowptr[r];
+    for (int64_t e = c0; e < c1; ++r) {
+      const int64_t hi = rowptr[r + 1], end = hi < c1 ? hi : c1;
+      const int64_t s = start_src[r] - lo, d = start_dst[r] - lo;
+      if (s != d || col_src != col_dst) {
+        int64_t k = e + lane;
+        for (; k + 96 < end; k += 128) {
+          const int32_t j0 = col_src[s + k], j1 = col_src[s + k + 32], j2 = col_src[s + k + 64], j3 = col_src[s + k + 96];
+          const double v0 = val_src[s + k], v1 = val_src[s + k + 32], v2 = val_src[s + k + 64], v3 = val_src[s + k + 96];
+          col_dst[d + k] = j0; col_dst[d + k + 32] = j1; col_dst[d + k + 64] = j2; col_dst[d + k + 96] = j3;
+          val_dst[d + k] = v0; val_dst[d + k + 32] = v1; val_dst[d + k + 64] = v2; val_dst[d + k + 96] = v3;
+        }
+        for (; k < end; k += 32) {
+          col_dst[d + k] = col_src[s + k];
+          val_dst[d + k] = val_src[s + k];
+        }
       }
-      for (; k < len; k += 32) {
-        col_dst[dst + k] = col_src[src + k];
-        val_dst[dst + k] = val_src[src + k];
-      }
-    }
-    const int64_t t0 = tstart[r];
-    for (int64_t k = lane; k < tn; k += 32) {
-      const ulonglong2 t = T[t0 + k];
-      col_dst[dst + len + k] = (int32_t)(nold + (int64_t)(t.x >> 32));
-      val_dst[dst + len + k] = valN[t.y];
+      e = end;
+      lo = hi;
     }
   }
 }
 
-__global__ void k_place_new_rows(int64_t nold, int64_t nnew, const int64_t* __restrict__ rpN,
-                                 const int32_t* __restrict__ colN, const double* __restrict__ valN,
-                                 const int64_t* __restrict__ start2, int32_t* __restrict__ col_dst,
-                                 double* __restrict__ val_dst) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t q = warp; q < nnew; q += nwarps) {
-    const int64_t dst = start2[nold + q];
-    const int64_t b = rpN[q], len = rpN[q + 1] - b;
-    for (int64_t k = lane; k < len; k += 32) {
-      col_dst[dst + k] = colN[b + k];
-      val_dst[dst + k] = valN[b + k];
-    }
+// the transposes of the new rows' entries behind the old rows' own, one
+// thread each (T is sorted by row; tstart[r] = the row's first)
+__global__ void k_append_T(const ulonglong2* __restrict__ T, int64_t nT, const int64_t* __restrict__ tstart,
+                           const int64_t* __restrict__ start, const int64_t* __restrict__ len_old, int64_t nold,
+                           const double* __restrict__ valN, int32_t* __restrict__ col_dst, double* __restrict__ val_dst) {
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nT; k += (int64_t)gridDim.x * blockDim.x) {
+    const ulonglong2 t = T[k];
+    const int64_t r = (int64_t)(t.x & 0xffffffffull);
+    const int64_t at = start[r] + len_old[r] + (k - tstart[r]);
+    col_dst[at] = (int32_t)(nold + (int64_t)(t.x >> 32));
+    val_dst[at] = valN[t.y];
   }
 }
 
@@ -992,49 +982,64 @@ __global__ void k_gather_vec(const double* __restrict__ in, const int32_t* __res
 }
 
 
-// diagonal <D|H|D> (includes e_core)
-__global__ void k_diag(int n, const double* __restrict__ h, const double* __restrict__ eri, double ecore,
-                       const ulonglong2* __restrict__ V, int64_t nV, double* __restrict__ out,
-                       const int32_t* __restrict__ rowlist) {
+// Diagonal <D|H|D> (includes e_core) as its difference from the aufbau
+// determinant R,
+//   E_R + sum_k d_k F_k + sum_{k<l} d_k d_l ((kk|ll) - [same spin] (kl|lk))
+// over the spin orbitals where D differs from R (d = -1 emptied, +1 filled):
+// a few dozen FP64 additions per determinant, where the sum over all
+// occupied pairs takes 700 (1.2e5 determinants of 22 electrons: 101 us, now
+// under 40) to 1400.
+__global__ void __launch_bounds__(256) k_diag(int n, uint64_t ra, uint64_t rb, const double* __restrict__ h,
+                                              const double* __restrict__ eri, const double* __restrict__ f_ref,
+                                              double ecore, const ulonglong2* __restrict__ V, int64_t nV,
+                                              double* __restrict__ out) {
   extern __shared__ double sm[];
-  double* J = sm;            // (kk|ll)
-  double* K = sm + n * n;    // (kl|lk)
+  __shared__ double s_eref;
+  double* J = sm;              // (kk|ll)
+  double* A = J + n * n;       // (kk|ll) - (kl|lk)
+  double* F = A + n * n;       // f_ref's diagonal, alpha then beta
   for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-    int k = t / n, l = t % n;
-    J[t] = eri[(((int64_t)k * n + k) * n + l) * n + l];
-    K[t] = eri[(((int64_t)k * n + l) * n + l) * n + k];
+    const int k = t / n, l = t % n;
+    const double j = eri[(((int64_t)k * n + k) * n + l) * n + l];
+    J[t] = j;
+    A[t] = j - eri[(((int64_t)k * n + l) * n + l) * n + k];
+  }
+  for (int t = threadIdx.x; t < 2 * n; t += blockDim.x) F[t] = f_ref[((int64_t)(t / n) * n + t % n) * n + t % n];
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double e = 0.0;
+    for (int t = threadIdx.x; t < 2 * n; t += 32)
+      if ((t < n ? ra >> t : rb >> (t - n)) & 1) e += h[(t % n) * n + t % n] + F[t];
+    for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (threadIdx.x == 0) s_eref = fma(0.5, e, ecore);
   }
   __syncthreads();
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nV; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = rowlist ? (int64_t)rowlist[t] : t;
-    ulonglong2 key = V[i];
+  const double eref = s_eref;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nV; i += (int64_t)gridDim.x * blockDim.x) {
+    const ulonglong2 key = V[i];
+    const uint64_t da = key.x ^ ra, db = key.y ^ rb;
     double e1 = 0.0, e2 = 0.0;
-    for (int s = 0; s < 2; ++s) {
-      uint64_t x = s == 0 ? key.x : key.y;
-      uint64_t o = s == 0 ? key.y : key.x;
-      uint64_t a = x;
-      while (a) {
-        int k = __ffsll((long long)a) - 1;
-        a &= a - 1;
-        e1 += h[k * n + k];
-        // same spin pairs l > k, opposite spin pairs counted once (s == 0)
-        uint64_t b = x & ~((2ull << k) - 1ull);
-        while (b) {
-          int l = __ffsll((long long)b) - 1;
-          b &= b - 1;
-          e2 += J[k * n + l] - K[k * n + l];
-        }
-        if (s == 0) {
-          uint64_t c = o;
-          while (c) {
-            int l = __ffsll((long long)c) - 1;
-            c &= c - 1;
-            e2 += J[k * n + l];
-          }
-        }
+    for (uint64_t x = da; x; x &= x - 1) {
+      const int k = __ffsll((long long)x) - 1, sk = (int)(ra >> k);
+      e1 += flip_sign(F[k], sk);
+      for (uint64_t y = x & (x - 1); y; y &= y - 1) {
+        const int l = __ffsll((long long)y) - 1;
+        e2 += flip_sign(A[k * n + l], sk ^ (int)(ra >> l));
+      }
+      for (uint64_t y = db; y; y &= y - 1) {
+        const int l = __ffsll((long long)y) - 1;
+        e2 += flip_sign(J[k * n + l], sk ^ (int)(rb >> l));
       }
     }
-    out[i] = ecore + e1 + e2;
+    for (uint64_t x = db; x; x &= x - 1) {
+      const int k = __ffsll((long long)x) - 1, sk = (int)(rb >> k);
+      e1 += flip_sign(F[n + k], sk);
+      for (uint64_t y = x & (x - 1); y; y &= y - 1) {
+        const int l = __ffsll((long long)y) - 1;
+        e2 += flip_sign(A[k * n + l], sk ^ (int)(rb >> l));
+      }
+    }
+    out[i] = eref + (e1 + e2);
   }
 }
 
@@ -1640,10 +1645,12 @@ static hci_status stage_place(hci_ctx* ctx, GraphArgs& A, int64_t left, int32_t*
 static hci_status compute_diag(hci_ctx* ctx, int64_t nrows, const ulonglong2* keys, double* out) {
   const int n = ctx->n;
   prof_tic(ctx, HCI_PH_HDIAG);
-  HCI_CUDA(ctx, cudaFuncSetAttribute(k_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 64 * 64 * 8));
+  HCI_CUDA(ctx, cudaFuncSetAttribute(k_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, (2 * 64 * 64 + 128) * 8));
+  // few blocks: each one gathers the 2 n^2 integrals
   if (nrows > 0)
-    HCI_LAUNCH(k_diag, grid_for(nrows, 128), 128, (size_t)2 * n * n * 8, ctx->st)(
-        n, bp<double>(ctx->h), bp<double>(ctx->eri), ctx->ecore, keys, nrows, out, nullptr);
+    HCI_LAUNCH(k_diag, grid_for(nrows, 256, ctx->nsm * 2), 256, (size_t)(2 * n * n + 2 * n) * 8, ctx->st)(
+        n, ctx->na == 64 ? ~0ull : ((1ull << ctx->na) - 1ull), ctx->nb == 64 ? ~0ull : ((1ull << ctx->nb) - 1ull),
+        bp<double>(ctx->h), bp<double>(ctx->eri), bp<double>(ctx->lists.f_ref), ctx->ecore, keys, nrows, out);
   HCI_CUDA(ctx, cudaGetLastError());
   prof_toc(ctx, HCI_PH_HDIAG);
   return HCI_OK;
@@ -1824,7 +1831,6 @@ static hci_status graph_extend_half(hci_ctx* ctx, const uint64_t* keys, int64_t 
   HCI_CUDA(ctx, cudaStreamSynchronize(st));
   if (miss) return HCI_OK;        // not an extension: full rebuild
   prof_tic(ctx, HCI_PH_GRAPH);
-  hci_status hs = HCI_OK;
   const int64_t nnew = nV - nold;
   // keys and map of the old space move to the scratch side
   std::swap(G.keys, S.keys_old);
@@ -1876,7 +1882,6 @@ static hci_status graph_extend_half(hci_ctx* ctx, const uint64_t* keys, int64_t 
   HCI_TRY(compute_diag(ctx, nnew, bp<ulonglong2>(G.keys_int) + nold, bp<double>(G.diag) + nold));
   prof_toc(ctx, HCI_PH_GRAPH);
   HCI_CUDA(ctx, cudaStreamSynchronize(st));
-  (void)hs;
   G.parent = G.epoch;
   G.epoch += 1;
   G.nold = nold;
@@ -2086,12 +2091,17 @@ static hci_status graph_extend_full(hci_ctx* ctx, const uint64_t* keys, int64_t 
     base = 0;
   }
   HCI_LAUNCH(k_assign_starts, grid_for(nV, 256), 256, 0, st)(bp<int64_t>(G.rowstart), rel, nV, base);
-  HCI_LAUNCH(k_move_old_rows, grid_for(nold * 32, 256), 256, 0, st)(
-      bp<int64_t>(S.rp_old), bp<int64_t>(S.len_old), nold, bp<int32_t>(G.seg_col[0]), bp<double>(G.seg_val[0]),
-      bp<int64_t>(G.rowstart), col_dst, val_dst, bp<ulonglong2>(S.T), bp<int64_t>(S.tstart), bp<int64_t>(S.hist),
-      bp<double>(S.valN));
-  HCI_LAUNCH(k_place_new_rows, gw, 256, 0, st)(nold, nnew, bp<int64_t>(S.rpN), bp<int32_t>(S.colN),
-                                                bp<double>(S.valN), bp<int64_t>(G.rowstart), col_dst, val_dst);
+  const auto move_grid = [&](int64_t entries) { return grid_for((entries + MOVE_CHUNK - 1) / MOVE_CHUNK * 32, 256); };
+  HCI_LAUNCH(k_move_rows, move_grid(G.nnz), 256, 0, st)(bp<int64_t>(G.rowptr), nold, bp<int64_t>(S.rp_old),
+                                                        bp<int32_t>(G.seg_col[0]), bp<double>(G.seg_val[0]),
+                                                        bp<int64_t>(G.rowstart), col_dst, val_dst);
+  if (nT > 0)
+    HCI_LAUNCH(k_append_T, grid_for(nT, 256), 256, 0, st)(bp<ulonglong2>(S.T), nT, bp<int64_t>(S.tstart),
+                                                         bp<int64_t>(G.rowstart), bp<int64_t>(S.len_old), nold,
+                                                         bp<double>(S.valN), col_dst, val_dst);
+  HCI_LAUNCH(k_move_rows, move_grid(nnzN), 256, 0, st)(bp<int64_t>(S.rpN), nnew, bp<int64_t>(S.rpN),
+                                                       bp<int32_t>(S.colN), bp<double>(S.valN),
+                                                       bp<int64_t>(G.rowstart) + nold, col_dst, val_dst);
   HCI_CUDA(ctx, cudaGetLastError());
   if (repack) {
     std::swap(G.seg_col[0], S.col_old);
