@@ -1043,23 +1043,29 @@ __global__ void __launch_bounds__(256) k_diag(int n, uint64_t ra, uint64_t rb, c
   }
 }
 
-// Both-orientation form: sigma = diag .* c + offdiag * c.  Every warp takes an
-// equal share of the connections (logical entries [w, w + 1) x chunk), whatever
-// rows they belong to: it owns the rows that start in its share and sums the
-// last one up to the share's end; the share's head, the rest of a row that
-// started earlier, goes to head[w], which k_sigma_heads adds to the row in the
-// order of the shares.  Nothing is done when *stop is set.  (With whole rows per warp the aufbau
-// determinant's row, connected to most of a small space, was all of the
-// product: 221 us on a 2.8e4-determinant (24e,24o) space, 97 us so; 2940 and
-// 2518 us on 3.0e5 (44e,44o) determinants.)  Four
-// (col, val, c[col]) loads per lane in flight; the connections are read with
-// evict-first hints so that c stays in L2.  Rows are summed four at a time,
-// so that the cross-lane reduction costs 1.5 FP64 additions per row instead
-// of 8 (the FP64 pipe, 2 DFMA per clock per SM, and the L1's address stage,
-// one gathered entry per clock per SM, bound this kernel).
-// blocks of k_sigma1 per SM at most, all resident
-constexpr int SIGMA_BLOCKS_PER_SM = 5;
+// Both-orientation form: sigma = diag .* c + offdiag * c.  The connections are
+// cut into equal shares (logical entries [w, w + 1) x chunk), whatever rows
+// they belong to, and a block's warps take its shares in turn.  A warp owns
+// the rows that start in a share and sums the last one up to the share's end;
+// the share's head, the rest of a row that started earlier, goes to head[w],
+// which k_sigma_heads adds to the row in the order of the shares.  Nothing is
+// done when *stop is set.  (With whole rows per warp the aufbau determinant's
+// row, connected to most of a small space, was all of the product.)
+//
+// Connections come from HBM, c from L2 one 32-byte sector per entry unless L1
+// has it: the loads' latency bounds the product (80% of the stalls, FP64 pipe
+// 70% and HBM 60% busy).  So a batch of 128 connections is loaded while the
+// batch before it gathers c, across the ends of rows, and neighbouring rows
+// are worked on side by side.  Rows are summed four at a time, so that the
+// cross-lane reduction costs 1.5 FP64 additions per row instead of 8.
+// Connections are read with evict-first hints so that c stays in L2.
+//
+// us per product, whole rows per warp / shares / shares and batches ahead:
+// (24e,24o) 2.8e4 determinants 221 / 97 / 85, (22e,22o) 1.2e5 181 / 184 /
+// 150, (44e,44o) 3.0e5 2940 / 2521 / 2252 and 4.3e5 3753 / 3777 / 3009.
+constexpr int SIGMA_WARPS_PER_SM = 32;   // of k_sigma1, all resident
 constexpr int64_t SIGMA_SHARE = 512;     // entries per warp at least
+constexpr int64_t SIGMA_SUB = 16384;     // entries per share where a warp has several
 
 // plan[w] = the first row that starts at or after entry w x chunk, w <= warps
 __global__ void k_sigma_plan(const int64_t* __restrict__ rowptr, int64_t nV, int64_t warps, int64_t chunk,
@@ -1076,69 +1082,113 @@ __global__ void k_sigma_plan(const int64_t* __restrict__ rowptr, int64_t nV, int
   plan[w] = (int32_t)(w == warps ? nV : lo);
 }
 
-// sum over k < len of val[k] c[col[k]] (a lane's share)
-__device__ __forceinline__ double row_dot(const int32_t* __restrict__ col, const double* __restrict__ val, int len,
-                                          const double* __restrict__ c) {
-  double a = 0.0, a2 = 0.0;   // two chains, so consecutive FMAs do not wait on each other
-  int k = threadIdx.x & 31;
-  for (; k + 96 < len; k += 128) {
-    const int32_t j0 = __ldcs(col + k), j1 = __ldcs(col + k + 32), j2 = __ldcs(col + k + 64), j3 = __ldcs(col + k + 96);
-    const double v0 = __ldcs(val + k), v1 = __ldcs(val + k + 32), v2 = __ldcs(val + k + 64), v3 = __ldcs(val + k + 96);
-    a = fma(v0, c[j0], a);
-    a2 = fma(v1, c[j1], a2);
-    a = fma(v2, c[j2], a);
-    a2 = fma(v3, c[j3], a2);
+// A row's entries, or those in a share
+struct RowPiece {
+  const int32_t* col;
+  const double* val;
+  int len;
+};
+// 128 of its entries, four per lane, zeros past its end
+struct RowBatch {
+  int32_t j[4];
+  double v[4];
+  __device__ __forceinline__ void load(const RowPiece& p, int at) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int k = at + 32 * u + (int)(threadIdx.x & 31);
+      const bool in = k < p.len;
+      j[u] = in ? __ldcs(p.col + k) : -1;
+      v[u] = in ? __ldcs(p.val + k) : 0.0;
+    }
   }
-  for (; k < len; k += 32) a = fma(__ldcs(val + k), c[__ldcs(col + k)], a);
-  return a + a2;
-}
+};
 
-__global__ void __launch_bounds__(256, SIGMA_BLOCKS_PER_SM) k_sigma1(const int64_t* __restrict__ rowptr,
+template <int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, SIGMA_WARPS_PER_SM / WARPS) k_sigma1(const int64_t* __restrict__ rowptr,
                                                   const int64_t* __restrict__ rowstart, const int32_t* __restrict__ col,
                                                const double* __restrict__ val, const double* __restrict__ diag,
-                                               int64_t nV, const int32_t* __restrict__ plan, int64_t chunk,
+                                               int64_t nV, const int32_t* __restrict__ plan, int rounds, int64_t chunk,
                                                const double* __restrict__ c, double* __restrict__ sigma,
                                                double* __restrict__ head, const int* __restrict__ stop) {
   if (stop && *stop) return;
   const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int r0 = plan[warp], r1 = plan[warp + 1];
-  const int64_t e0 = warp * chunk, e1 = e0 + chunk;
-  {
-    // the head: row r0 - 1 from e0 on
-    const int64_t hi = rowptr[r0];
-    double a = 0.0;
-    if (hi > e0) {
-      const int i = r0 - 1;
-      const int64_t b = rowstart[i] + (e0 - rowptr[i]);
-      a = row_dot(col + b, val + b, (int)((hi < e1 ? hi : e1) - e0), c);
-      for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    }
-    if (lane == 0) head[warp] = a;
-  }
-  for (int g = r0; g < r1; g += 4) {
-    double acc[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int i = g + r;
-      acc[r] = 0.0;
-      if (i < r1) {
-        const int64_t b = rowstart[i], lo = rowptr[i], hi = rowptr[i + 1];
-        acc[r] = row_dot(col + b, val + b, (int)((hi < e1 ? hi : e1) - lo), c);
+  // the block's warps take its shares in turn
+  const int64_t w0 = (int64_t)blockIdx.x * WARPS * rounds + (threadIdx.x >> 5);
+  for (int t = 0; t < rounds; ++t) {
+    const int64_t w = w0 + WARPS * t;
+    const int r0 = plan[w], r1 = plan[w + 1];
+    const int64_t e0 = w * chunk, e1 = e0 + chunk;
+    // row i's entries of this share
+    auto piece = [&](int i) {
+      const int64_t lo = rowptr[i], hi = rowptr[i + 1];
+      const int64_t b = lo > e0 ? lo : e0, at = rowstart[i] + (b - lo);
+      return RowPiece{col + at, val + at, (int)((hi < e1 ? hi : e1) - b)};
+    };
+    RowPiece next{col, val, 0};
+    RowBatch q;
+    // the sum of the row whose first batch q holds; leaves q with the first
+    // batch of `next`
+    auto row = [&](const RowPiece& p) {
+      double a = 0.0, a2 = 0.0;   // two chains, so consecutive FMAs do not wait on each other
+      for (int at = 0;; at += 128) {
+        double x[4], v[4];
+  #pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          x[u] = q.j[u] >= 0 ? c[q.j[u]] : 0.0;
+          v[u] = q.v[u];
+        }
+        const bool last = at + 128 >= p.len;
+        if (last) q.load(next, 0);
+        else q.load(p, at + 128);
+        const int left = p.len - at;
+        if (left > 0) a = fma(v[0], x[0], a);
+        if (left > 32) a2 = fma(v[1], x[1], a2);
+        if (left > 64) a = fma(v[2], x[2], a);
+        if (left > 96) a2 = fma(v[3], x[3], a2);
+        if (last) break;
       }
+      return a + a2;
+    };
+    const bool has_head = rowptr[r0] > e0;
+    const int first = has_head ? r0 - 1 : r0;
+    if (first < r1) next = piece(first);
+    q.load(next, 0);
+    {
+      // the head: row r0 - 1 from e0 on
+      double a = 0.0;
+      if (has_head) {
+        const RowPiece p = next;
+        next = r0 < r1 ? piece(r0) : RowPiece{col, val, 0};
+        a = row(p);
+        for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      }
+      if (lane == 0) head[w] = a;
     }
-    // four row sums at once: halve the values held per lane across lanes
-    // 16 apart, then 8 apart, then a plain tree over the last 8 lanes
-    const bool h16 = lane & 16, h8 = lane & 8;
-    const double w0 = (h16 ? acc[2] : acc[0]) + __shfl_xor_sync(0xffffffffu, h16 ? acc[0] : acc[2], 16);
-    const double w1 = (h16 ? acc[3] : acc[1]) + __shfl_xor_sync(0xffffffffu, h16 ? acc[1] : acc[3], 16);
-    double u = (h8 ? w1 : w0) + __shfl_xor_sync(0xffffffffu, h8 ? w0 : w1, 8);
-    u += __shfl_xor_sync(0xffffffffu, u, 4);
-    u += __shfl_xor_sync(0xffffffffu, u, 2);
-    u += __shfl_xor_sync(0xffffffffu, u, 1);
-    if ((lane & 7) == 0) {
-      const int i = g + (h16 ? 2 : 0) + (h8 ? 1 : 0);
-      if (i < r1) sigma[i] = fma(diag[i], c[i], u);
+    for (int g = r0; g < r1; g += 4) {
+      double acc[4];
+  #pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int i = g + r;
+        acc[r] = 0.0;
+        if (i < r1) {
+          const RowPiece p = next;
+          next = i + 1 < r1 ? piece(i + 1) : RowPiece{col, val, 0};
+          acc[r] = row(p);
+        }
+      }
+      // four row sums at once: halve the values held per lane across lanes
+      // 16 apart, then 8 apart, then a plain tree over the last 8 lanes
+      const bool h16 = lane & 16, h8 = lane & 8;
+      const double s0 = (h16 ? acc[2] : acc[0]) + __shfl_xor_sync(0xffffffffu, h16 ? acc[0] : acc[2], 16);
+      const double s1 = (h16 ? acc[3] : acc[1]) + __shfl_xor_sync(0xffffffffu, h16 ? acc[1] : acc[3], 16);
+      double u = (h8 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, h8 ? s0 : s1, 8);
+      u += __shfl_xor_sync(0xffffffffu, u, 4);
+      u += __shfl_xor_sync(0xffffffffu, u, 2);
+      u += __shfl_xor_sync(0xffffffffu, u, 1);
+      if ((lane & 7) == 0) {
+        const int i = g + (h16 ? 2 : 0) + (h8 ? 1 : 0);
+        if (i < r1) sigma[i] = fma(diag[i], c[i], u);
+      }
     }
   }
 }
@@ -2296,9 +2346,16 @@ hci_status direct_rdm(hci_ctx* ctx, const double* c, const RdmAcc& R) {
 static double* sig_head(Graph& G) { return reinterpret_cast<double*>(bp<char>(G.sig_plan) + ((size_t)(G.sig_warps + 2) * 4 + 7) / 8 * 8); }
 static hci_status plan_sigma(hci_ctx* ctx) {
   Graph& G = ctx->graph;
-  const int64_t most = (int64_t)ctx->nsm * SIGMA_BLOCKS_PER_SM;
-  const int64_t blocks = std::max<int64_t>(1, std::min(most, G.nstored / (8 * SIGMA_SHARE)));
-  G.sig_warps = blocks * 8;
+  // Warps per block: with a share per warp, 8 (22 orbitals, 8e6 connections
+  // 50.5 us, 16 warps 52.1; 12 orbitals, 4e5: 16.3 and 19.6).  With several,
+  // a block's warps work on neighbouring rows and so find each other's c in
+  // L1: 16 (44 orbitals, 1.3e9: 3302 us with 8, 3009 with 16, 3070 with 32;
+  // 28 orbitals, 9.7e7: 242, 236, 241).
+  const int64_t most = (int64_t)ctx->nsm * SIGMA_WARPS_PER_SM;
+  G.sig_block = G.nstored >= most * SIGMA_SUB ? 16 : 8;
+  const int64_t warps = std::max<int64_t>(1, std::min(most, G.nstored / SIGMA_SHARE) / G.sig_block) * G.sig_block;
+  G.sig_rounds = (int)std::max<int64_t>(1, (G.nstored + warps * SIGMA_SUB / 2) / (warps * SIGMA_SUB));
+  G.sig_warps = warps * G.sig_rounds;
   G.sig_chunk = std::max<int64_t>(1, (G.nstored + G.sig_warps - 1) / G.sig_warps);
   HCI_TRY(ensure_buf(ctx, G.sig_plan, (size_t)(G.sig_warps + 2) * 4 + 8 + (size_t)G.sig_warps * 8 + 16));
   HCI_LAUNCH(k_sigma_plan, (unsigned)((G.sig_warps + 256) / 256), 256, 0, ctx->st)(
@@ -2341,9 +2398,10 @@ hci_status sigma_apply(hci_ctx* ctx, const double* c, double* sigma, int nvec, c
       HCI_LAUNCH(k_sigma_half, grid_for(G.nV * 32, 256, ctx->nsm * 16), 256, 0, ctx->st)(
           bp<int64_t>(G.rowptr), bp<int64_t>(G.rowstart), T, bp<double>(G.diag), G.nV, c, sigma, nvec);
   } else if (nvec == 1) {
-    HCI_LAUNCH(k_sigma1, (unsigned)(G.sig_warps / 8), 256, 0, ctx->st)(
+    auto* k = G.sig_block == 16 ? k_sigma1<16> : k_sigma1<8>;
+    HCI_LAUNCH(k, (unsigned)(G.sig_warps / (G.sig_block * G.sig_rounds)), G.sig_block * 32, 0, ctx->st)(
         bp<int64_t>(G.rowptr), bp<int64_t>(G.rowstart), bp<int32_t>(G.seg_col[0]), bp<double>(G.seg_val[0]),
-        bp<double>(G.diag), G.nV, bp<int32_t>(G.sig_plan), G.sig_chunk, c, sigma, sig_head(G), stop);
+        bp<double>(G.diag), G.nV, bp<int32_t>(G.sig_plan), G.sig_rounds, G.sig_chunk, c, sigma, sig_head(G), stop);
     HCI_LAUNCH(k_sigma_heads, (unsigned)((G.sig_warps + 127) / 128), 128, 0, ctx->st)(
         bp<int64_t>(G.rowptr), bp<int32_t>(G.sig_plan), G.sig_warps, G.sig_chunk, sig_head(G), sigma, stop);
   } else {

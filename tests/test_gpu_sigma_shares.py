@@ -56,3 +56,29 @@ def test_empty_rows(linked):
     keys += [(0b1111, (0b111 | (1 << (4 + k)))) for k in range(linked)]
     keys = np.array(sorted(set(keys)), dtype=np.uint64)
     _check(inst, keys)
+
+
+# more connections than a share per warp: blocks of 16 warps with one and with
+# several shares each, on every determinant of 8 electrons
+@pytest.mark.parametrize("n", [11, 12])
+def test_several_shares(n):
+    import paper_1708_07544_gb300 as pkg
+    from itertools import combinations
+
+    inst = hi.random_tiny(n, 4, 4, 5)
+    strings = sorted(sum(1 << p for p in o) for o in combinations(range(n), 4))
+    keys = np.array([(a, b) for a in strings for b in strings], dtype=np.uint64)
+    c, d = hi.random_vector(len(keys), 1), hi.random_vector(len(keys), 2)
+    rows = np.unique(np.concatenate([np.arange(4), np.random.default_rng(3).integers(0, len(keys), 24),
+                                     len(keys) - 1 - np.arange(4)]))
+    ref = oracle.sigma_rows(inst, keys, c, rows)
+    kt = torch.tensor(keys.astype(np.int64), device="cuda")
+    ct, dt = torch.tensor(c, device="cuda"), torch.tensor(d, device="cuda")
+    with pkg.HCISolver(inst.norb, inst.nalpha, inst.nbeta, torch.tensor(inst.h, device="cuda"),
+                       torch.tensor(inst.eri, device="cuda"), inst.e_core) as s:
+        hc, hd = s.sigma(kt, ct), s.sigma(kt, dt)
+        assert s.stats()["graph_nnz"] > 8e7
+    assert np.abs(hc.cpu().numpy()[rows] - ref).max() <= 1e-11 * max(1.0, np.abs(ref).max())
+    # H is symmetric: every row and column
+    a, b = float(dt @ hc), float(ct @ hd)
+    assert abs(a - b) <= 1e-12 * float(dt.norm() * hc.norm() + ct.norm() * hd.norm())
