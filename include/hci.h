@@ -402,7 +402,8 @@ hci_status hci_rotate_noalloc(int norb, const double* kappa, const double* h, co
  *   HCI_ST_GRAPH_BUILDS     connection graphs built
  *   HCI_ST_WALK_ENTRIES     list entries examined by the heat-bath walks
  *   HCI_ST_SINGLES_EXACT    single excitations evaluated exactly
- *   HCI_ST_ROWS_REFILLED    new graph rows too long for the one-pass search,
+ *   HCI_ST_ROWS_REFILLED    new graph rows, or parts of long ones, with more
+ *                           entries than the one-pass search's scratch holds,
  *                           filled by a second search
  *   HCI_ST_SIGMA_DIRECT     1 when the cached graph is direct (connections
  *                           searched again by every traversal), else 0

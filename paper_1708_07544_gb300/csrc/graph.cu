@@ -1053,10 +1053,12 @@ __global__ void __launch_bounds__(256) k_diag(int n, uint64_t ra, uint64_t rb, c
 // row, connected to most of a small space, was all of the product.)
 //
 // Connections come from HBM, c from L2 one 32-byte sector per entry unless L1
-// has it: the loads' latency bounds the product (80% of the stalls, FP64 pipe
-// 70% and HBM 60% busy).  So a batch of 128 connections is loaded while the
-// batch before it gathers c, across the ends of rows, and neighbouring rows
-// are worked on side by side.  Rows are summed four at a time, so that the
+// has it: the loads' latency bounded the product (52 cycles of stall per
+// instruction, FP64 pipe 70% and HBM 60% busy at 9.7e7 connections).  So a
+// batch of 128 connections is loaded while the batch before it gathers c,
+// across the ends of rows, and neighbouring rows are worked on side by side
+// (16 cycles, 75% and 64%; the FP64 pipe, HBM and L1 share the bound).  Rows
+// are summed four at a time, so that the
 // cross-lane reduction costs 1.5 FP64 additions per row instead of 8.
 // Connections are read with evict-first hints so that c stays in L2.
 //
@@ -1103,6 +1105,30 @@ struct RowBatch {
   }
 };
 
+// The sum of val c[col] over row p (a lane's share), whose first batch q holds;
+// leaves q with the first batch of `next`.
+__device__ __forceinline__ double row_sum(const RowPiece& p, const RowPiece& next, RowBatch& q,
+                                          const double* __restrict__ c) {
+  double a = 0.0, a2 = 0.0;   // two chains, so consecutive FMAs do not wait on each other
+  for (int at = 0;; at += 128) {
+    double x[4], v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      x[u] = q.j[u] >= 0 ? c[q.j[u]] : 0.0;
+      v[u] = q.v[u];
+    }
+    const bool last = at + 128 >= p.len;
+    if (last) q.load(next, 0);
+    else q.load(p, at + 128);
+    const int left = p.len - at;
+    if (left > 0) a = fma(v[0], x[0], a);
+    if (left > 32) a2 = fma(v[1], x[1], a2);
+    if (left > 64) a = fma(v[2], x[2], a);
+    if (left > 96) a2 = fma(v[3], x[3], a2);
+    if (last) return a + a2;
+  }
+}
+
 template <int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, SIGMA_WARPS_PER_SM / WARPS) k_sigma1(const int64_t* __restrict__ rowptr,
                                                   const int64_t* __restrict__ rowstart, const int32_t* __restrict__ col,
@@ -1126,29 +1152,6 @@ __global__ void __launch_bounds__(WARPS * 32, SIGMA_WARPS_PER_SM / WARPS) k_sigm
     };
     RowPiece next{col, val, 0};
     RowBatch q;
-    // the sum of the row whose first batch q holds; leaves q with the first
-    // batch of `next`
-    auto row = [&](const RowPiece& p) {
-      double a = 0.0, a2 = 0.0;   // two chains, so consecutive FMAs do not wait on each other
-      for (int at = 0;; at += 128) {
-        double x[4], v[4];
-  #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          x[u] = q.j[u] >= 0 ? c[q.j[u]] : 0.0;
-          v[u] = q.v[u];
-        }
-        const bool last = at + 128 >= p.len;
-        if (last) q.load(next, 0);
-        else q.load(p, at + 128);
-        const int left = p.len - at;
-        if (left > 0) a = fma(v[0], x[0], a);
-        if (left > 32) a2 = fma(v[1], x[1], a2);
-        if (left > 64) a = fma(v[2], x[2], a);
-        if (left > 96) a2 = fma(v[3], x[3], a2);
-        if (last) break;
-      }
-      return a + a2;
-    };
     const bool has_head = rowptr[r0] > e0;
     const int first = has_head ? r0 - 1 : r0;
     if (first < r1) next = piece(first);
@@ -1159,7 +1162,7 @@ __global__ void __launch_bounds__(WARPS * 32, SIGMA_WARPS_PER_SM / WARPS) k_sigm
       if (has_head) {
         const RowPiece p = next;
         next = r0 < r1 ? piece(r0) : RowPiece{col, val, 0};
-        a = row(p);
+        a = row_sum(p, next, q, c);
         for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
       }
       if (lane == 0) head[w] = a;
@@ -1173,7 +1176,7 @@ __global__ void __launch_bounds__(WARPS * 32, SIGMA_WARPS_PER_SM / WARPS) k_sigm
         if (i < r1) {
           const RowPiece p = next;
           next = i + 1 < r1 ? piece(i + 1) : RowPiece{col, val, 0};
-          acc[r] = row(p);
+          acc[r] = row_sum(p, next, q, c);
         }
       }
       // four row sums at once: halve the values held per lane across lanes
@@ -1357,21 +1360,31 @@ __global__ void __launch_bounds__(256, SIGMA_HALF_BLOCKS_PER_SM) k_sigma1_half(c
 // Rows r0 .. nV-1 of H c for a vector that vanishes on them (the rows a
 // space gained in its last extension): out[i] = sum of the row's stored
 // entries times c (both forms store every connection of such a row to an
-// earlier determinant in the row itself); one warp per row.
-__global__ void __launch_bounds__(256) k_sigma_tail(const int64_t* __restrict__ rowptr,
-                                                    const int64_t* __restrict__ rowstart,
-                                                    const __grid_constant__ SegTab T, int64_t r0, int64_t nV,
-                                                    const double* __restrict__ c, double* __restrict__ out) {
+// earlier determinant in the row itself); one warp per row, batches loaded
+// ahead as in k_sigma1 (the last extensions of a 4.3e5-determinant (44e,44o)
+// solve: 227 -> 169 us).
+__global__ void __launch_bounds__(256, 4) k_sigma_tail(const int64_t* __restrict__ rowptr,
+                                                       const int64_t* __restrict__ rowstart,
+                                                       const __grid_constant__ SegTab T, int64_t r0, int64_t nV,
+                                                       const double* __restrict__ c, double* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  auto piece = [&](int64_t i) {
+    RowPiece p{nullptr, nullptr, 0};
+    if (i < nV) {
+      row_entries(T, rowstart[i], p.col, p.val);
+      p.len = (int)(rowptr[i + 1] - rowptr[i]);
+    }
+    return p;
+  };
+  RowPiece next = piece(r0 + warp);
+  RowBatch q;
+  q.load(next, 0);
   for (int64_t i = r0 + warp; i < nV; i += nwarps) {
-    const int64_t len = rowptr[i + 1] - rowptr[i];
-    const int32_t* col;
-    const double* val;
-    row_entries(T, rowstart[i], col, val);
-    double a = 0.0;
-    for (int64_t k = lane; k < len; k += 32) a = fma(__ldcs(val + k), c[__ldcs(col + k)], a);
+    const RowPiece p = next;
+    next = piece(i + nwarps);
+    double a = row_sum(p, next, q, c);
     for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     if (lane == 0) out[i] = a;
   }
