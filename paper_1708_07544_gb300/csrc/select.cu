@@ -113,18 +113,24 @@ __device__ __forceinline__ void warp_emit(bool emit, ulonglong2 key, double term
   if (cnt >= EM_FLUSH) emit_flush(B, cnt, A);
 }
 
-// The warp's next 32 determinants, one per lane (nV or above: none), or -1
-// at the queue's end.  An atomic per determinant would bound spaces of small
-// coefficients; the 32 lie nV / 32 apart, because determinants of large
-// coefficients are neighbours (32 consecutive ones: 3.9 ms of k_singles where
-// these take 0.3).
+// The warp's next determinants, one per lane (nV or above: none), or -1 at
+// the queue's end: 32 of them, or about nV / warps where that is less, so that
+// a small set of large coefficients (a sample's draws, a first selection) is
+// spread over every warp.  An atomic per determinant would bound spaces of
+// small coefficients; those of a fetch lie far apart, because determinants of
+// large coefficients are neighbours (32 consecutive ones: 3.9 ms of k_singles
+// where these take 0.3).  Fourteen selections of (12e,12o) spaces: 1.75 ms of
+// k_walk_plan with 32 always, 1.23 so.
 __device__ __forceinline__ int64_t next_dets(const WalkArgs& A) {
   const int lane = threadIdx.x & 31;
-  const int64_t stride = (A.nV + 31) >> 5;
+  const int64_t warps = (int64_t)gridDim.x * SEL_WARPS, each = (A.nV + warps - 1) / warps;
+  const int per = each < 1 ? 1 : each < 32 ? (int)each : 32;
+  const int64_t stride = (A.nV + per - 1) / per;
   unsigned long long q = 0;
   if (lane == 0) q = atomicAdd(&A.counter[1], 1ull);
   q = __shfl_sync(0xffffffffu, q, 0);
-  return (int64_t)q < stride ? (int64_t)q + lane * stride : -1;
+  if ((int64_t)q >= stride) return -1;
+  return lane < per ? (int64_t)q + lane * stride : A.nV;
 }
 
 // Compact the occupied orbitals of a spin string into smem (ascending).

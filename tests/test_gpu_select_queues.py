@@ -61,3 +61,16 @@ def test_screened_pairs(space, eps2):
         got = s.pt2(_dev(keys), _dev(c), eps2, e0)
     assert got[1] == n
     assert abs(got[0] - e2) <= 1e-11 * max(abs(e2), 1e-12)
+
+
+# several determinants per fetch, fewer than 32: about one fetch per warp of
+# the chip (9728 warps on 152 multiprocessors)
+@pytest.mark.parametrize("nV", [9000, 9729, 20000, 60001])
+def test_selection_of_wider_queues(nV):
+    inst, keys, c = _problem(12, 6, 5, nV)
+    want, _, ties = oracle.select(inst, keys, c, 0.3)
+    with _solver(inst) as s:
+        got = s.select(0.3, _dev(keys), _dev(c)).cpu().numpy().view(np.uint64).reshape(-1, 2)
+    as_set = lambda k: set(map(tuple, np.asarray(k).tolist()))  # noqa: E731
+    assert as_set(got) - as_set(ties) == as_set(want) - as_set(ties)
+    assert len(as_set(got)) == len(got)
