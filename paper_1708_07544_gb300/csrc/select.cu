@@ -1265,42 +1265,42 @@ __global__ void k_ss_gather(int64_t j0, int64_t j1, int64_t ndist, int64_t m, co
   }
 }
 
-// On the first pair of every target (grouped pairs; element H_aj and
-// source j on each pair): targets in V give 0, the others their estimate
-// with the eps2 screen (every emitted pair) and with eps2_det.
-__global__ void k_ss_terms(const ulonglong2* __restrict__ t, const double* __restrict__ v,
-                           const int32_t* __restrict__ src, int64_t m, uint64_t gmask,
-                           const ulonglong2* __restrict__ V, const int32_t* __restrict__ tab, uint64_t tmask,
-                           const double* __restrict__ sc, const double* __restrict__ sf, double eps2_det,
-                           double nd, int n, const double* __restrict__ ref, uint64_t ra, uint64_t rb, double e0,
-                           double* __restrict__ out_t, double* __restrict__ out_d) {
+// One listed target per thread (grouped pairs; element H_aj and source j on
+// each pair): its estimate with the eps2 screen (every emitted pair) and with
+// eps2_det, on its first pair; the other pairs' places are zero beforehand.
+// FP64 issue bounds it, so the targets are listed first as for k_pt2_terms:
+// taken in place, where only the first pair of a run works, ten samples of
+// 1000 draws from 3.4e4 (22e,22o) determinants took 50 ms, 16.8 so.
+__global__ void __launch_bounds__(256) k_ss_terms(const ulonglong2* __restrict__ t, const double* __restrict__ v,
+                                                  const int32_t* __restrict__ src, int64_t m, uint64_t gmask,
+                                                  const int64_t* __restrict__ list,
+                                                  const unsigned long long* __restrict__ count,
+                                                  const double* __restrict__ sc, const double* __restrict__ sf,
+                                                  double eps2_det, double nd, int n, const double* __restrict__ ref,
+                                                  uint64_t ra, uint64_t rb, double e0, double* __restrict__ out_t,
+                                                  double* __restrict__ out_d) {
   extern __shared__ double s_ref[];
   const int nref = 1 + 2 * n + 4 * n * n;
   for (int u = threadIdx.x; u < nref; u += blockDim.x) s_ref[u] = ref[u];
   __syncthreads();
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    double et = 0.0, ed = 0.0;
+  const int64_t nt = (int64_t)*count;
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < nt; q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = list[q];
     const ulonglong2 key = t[i];
-    if (first_of_key(t, i, key, gmask)) {
-      if (!in_space(V, tab, tmask, key)) {
-        double S[2] = {0.0, 0.0}, T[2] = {0.0, 0.0}, U[2] = {0.0, 0.0};
-        for (int64_t e = i; e < m; e = next_of_key(t, e, m, key, gmask)) {
-          const int32_t j = src[e];
-          const double x = v[e] * sc[j], f = sf[j];
-          for (int k = 0; k < 2; ++k) {
-            if (k == 1 && !(fabs(x) > eps2_det)) break;
-            S[k] += f * x;
-            T[k] += (f * x) * (f * x);
-            U[k] += f * x * x;
-          }
-        }
-        const double den = nd * (nd - 1.0) * (e0 - pt2_diag(s_ref, n, key, ra, rb));
-        et = (S[0] * S[0] - T[0] + (nd - 1.0) * U[0]) / den;
-        ed = (S[1] * S[1] - T[1] + (nd - 1.0) * U[1]) / den;
+    double S[2] = {0.0, 0.0}, T[2] = {0.0, 0.0}, U[2] = {0.0, 0.0};
+    for (int64_t e = i; e < m; e = next_of_key(t, e, m, key, gmask)) {
+      const int32_t j = src[e];
+      const double x = v[e] * sc[j], f = sf[j];
+      for (int k = 0; k < 2; ++k) {
+        if (k == 1 && !(fabs(x) > eps2_det)) break;
+        S[k] += f * x;
+        T[k] += (f * x) * (f * x);
+        U[k] += f * x * x;
       }
     }
-    out_t[i] = et;
-    out_d[i] = ed;
+    const double den = nd * (nd - 1.0) * (e0 - pt2_diag(s_ref, n, key, ra, rb));
+    out_t[i] = (S[0] * S[0] - T[0] + (nd - 1.0) * U[0]) / den;
+    out_d[i] = (S[1] * S[1] - T[1] + (nd - 1.0) * U[1]) / den;
   }
 }
 
@@ -1434,10 +1434,18 @@ extern "C" hci_status hci_pt2_stochastic(hci_ctx* ctx, const uint64_t* keys, con
                         bp<double>(ctx->p2_vals2), bp<int32_t>(ctx->p2_src), bp<int32_t>(ctx->p2_src2), mp, &gbits));
     double* ct = bp<double>(ctx->p2_vals2);
     double* cd = bp<double>(ctx->p2_d);
-    HCI_LAUNCH(k_ss_terms, grid_for(mp, 256), 256, smref, st)(bp<ulonglong2>(ctx->s_cand), bp<double>(ctx->p2_vals),
-                                                              bp<int32_t>(ctx->p2_src), mp, ((uint64_t)1 << gbits) - 1, Vk,
-                                                              bp<int32_t>(ctx->p2_tab), tsize - 1, sc, sf, eps2_det,
-                                                              (double)nd, n, ref, A.ref_a, A.ref_b, e0, ct, cd);
+    const uint64_t gmask = ((uint64_t)1 << gbits) - 1;
+    HCI_TRY(ensure_buf(ctx, ctx->s_flags, (size_t)(1 + mp) * 8));
+    unsigned long long* count = bp<unsigned long long>(ctx->s_flags);
+    int64_t* list = reinterpret_cast<int64_t*>(count + 1);
+    HCI_CUDA(ctx, cudaMemsetAsync(count, 0, 8, st));
+    HCI_LAUNCH(k_pt2_targets, grid_for(mp, 256), 256, 0, st)(bp<ulonglong2>(ctx->s_cand), mp, gmask, Vk,
+                                                           bp<int32_t>(ctx->p2_tab), tsize - 1, list, count, nullptr);
+    HCI_CUDA(ctx, cudaMemsetAsync(ct, 0, (size_t)mp * 8, st));
+    HCI_CUDA(ctx, cudaMemsetAsync(cd, 0, (size_t)mp * 8, st));
+    HCI_LAUNCH(k_ss_terms, grid_for(mp, 256, ctx->nsm * 8), 256, smref, st)(
+        bp<ulonglong2>(ctx->s_cand), bp<double>(ctx->p2_vals), bp<int32_t>(ctx->p2_src), mp, gmask, list, count, sc, sf,
+        eps2_det, (double)nd, n, ref, A.ref_a, A.ref_b, e0, ct, cd);
     HCI_LAUNCH(k_sum_slices_d, PT2_SUM_BLOCKS, 256, 0, st)(ct, mp, part);
     HCI_LAUNCH(k_sum_parts_d, 1, 32, 0, st)(part, PT2_SUM_BLOCKS, dsum);
     HCI_LAUNCH(k_sum_slices_d, PT2_SUM_BLOCKS, 256, 0, st)(cd, mp, part);
