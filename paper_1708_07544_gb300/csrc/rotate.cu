@@ -46,8 +46,12 @@ constexpr int CLM_T = 128;          // threads per CTA: one warp per FP64 pipe
 constexpr int CLM_NU = 4;           // entries per thread at most (8 CTAs: 16 x 32 of 64 x 64)
 constexpr int CLM_BI = 16, CLM_BJ = 32;
 
+// Without .aligned, which asks that a warp's threads execute the barrier
+// together: cl_mm's loops and epilogues end thread by thread (a block of
+// 5 x 5 entries, the triangle of h), and nothing says where the warp meets
+// again.
 __device__ __forceinline__ void cl_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 __device__ __forceinline__ int cl_rank() {
   int r;

@@ -72,3 +72,29 @@ def test_infinite_kappa_refused():
         pkg.hci_rotate(k, h, e)
     with pytest.raises(pkg.HCIError):
         pkg.hci_rotate_backward(k, h, e, h, e)
+
+
+# blocks of a CTA that end in the middle of a warp (5 x 5 to 16 x 16 less a
+# ragged edge): every product's loop ends thread by thread before the
+# cluster's barrier.  Without two-electron integrals the whole gradient comes
+# from the chains: dE/dU = h U g1^T + h^T U g1, dkappa = L_exp(kappa^T, dE/dU).
+@pytest.mark.parametrize("n", [18, 21, 26, 31, 37, 50, 63])
+@pytest.mark.parametrize("sigma", [0.01, 0.4])
+def test_ragged_blocks(n, sigma):
+    import paper_1708_07544_gb300 as pkg
+
+    g = np.random.default_rng(n)
+    kap = hi.random_kappa(n, seed=n, sigma=sigma)
+    h, r1 = g.standard_normal((n, n)), g.standard_normal((n, n))
+    h, r1 = h + h.T, r1 + r1.T
+    t = lambda a: torch.tensor(np.ascontiguousarray(a), device="cuda")  # noqa: E731
+    zero = torch.zeros((n,) * 4, dtype=torch.float64, device="cuda")
+    U, h2, _ = (x.cpu().numpy() for x in pkg.hci_rotate(t(kap), t(h), zero))
+    dh, _, dk = (x.cpu().numpy() for x in pkg.hci_rotate_backward(t(kap), t(h), zero, t(r1), zero))
+    ref = sl.expm(kap)
+    assert np.abs(U - ref).max() <= 1e-14 * n * max(1.0, np.abs(kap).sum(0).max())
+    assert np.abs(h2 - ref.T @ h @ ref).max() <= 1e-13 * n * np.abs(h).max()
+    assert np.abs(dh - ref @ r1 @ ref.T).max() <= 1e-13 * n * np.abs(r1).max()
+    G = h @ ref @ r1.T + h.T @ ref @ r1
+    want = sl.expm_frechet(kap.T, G, compute_expm=False)
+    assert np.abs(dk - want).max() <= 1e-13 * n * max(1.0, np.abs(kap).sum(0).max()) * np.abs(want).max()
