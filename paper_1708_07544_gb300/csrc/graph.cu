@@ -2272,6 +2272,9 @@ static hci_status graph_stored(hci_ctx* ctx, const uint64_t* keys, int64_t nV) {
     s = half ? graph_build_half(ctx, keys, nV) : graph_build_full(ctx, keys, nV);
   }
   if (s == HCI_OK && !half) s = plan_sigma(ctx);
+  // a failure behind the build leaves a graph without its plan, and under the
+  // hash of the space before it
+  if (s != HCI_OK) G.valid = false;
   return s;
 }
 
@@ -2365,12 +2368,15 @@ static hci_status plan_sigma(hci_ctx* ctx) {
   // L1: 16 (44 orbitals, 1.3e9: 3302 us with 8, 3009 with 16, 3070 with 32;
   // 28 orbitals, 9.7e7: 242, 236, 241).
   const int64_t most = (int64_t)ctx->nsm * SIGMA_WARPS_PER_SM;
-  G.sig_block = G.nstored >= most * SIGMA_SUB ? 16 : 8;
-  const int64_t warps = std::max<int64_t>(1, std::min(most, G.nstored / SIGMA_SHARE) / G.sig_block) * G.sig_block;
-  G.sig_rounds = (int)std::max<int64_t>(1, (G.nstored + warps * SIGMA_SUB / 2) / (warps * SIGMA_SUB));
-  G.sig_warps = warps * G.sig_rounds;
-  G.sig_chunk = std::max<int64_t>(1, (G.nstored + G.sig_warps - 1) / G.sig_warps);
-  HCI_TRY(ensure_buf(ctx, G.sig_plan, (size_t)(G.sig_warps + 2) * 4 + 8 + (size_t)G.sig_warps * 8 + 16));
+  const int block = G.nstored >= most * SIGMA_SUB ? 16 : 8;
+  const int64_t warps = std::max<int64_t>(1, std::min(most, G.nstored / SIGMA_SHARE) / block) * block;
+  const int64_t rounds = std::max<int64_t>(1, (G.nstored + warps * SIGMA_SUB / 2) / (warps * SIGMA_SUB));
+  const int64_t shares = warps * rounds;
+  HCI_TRY(ensure_buf(ctx, G.sig_plan, (size_t)(shares + 2) * 4 + 8 + (size_t)shares * 8 + 16));
+  G.sig_block = block;
+  G.sig_rounds = (int)rounds;
+  G.sig_warps = shares;
+  G.sig_chunk = std::max<int64_t>(1, (G.nstored + shares - 1) / shares);
   HCI_LAUNCH(k_sigma_plan, (unsigned)((G.sig_warps + 256) / 256), 256, 0, ctx->st)(
       bp<int64_t>(G.rowptr), G.nV, G.sig_warps, G.sig_chunk, bp<int32_t>(G.sig_plan));
   HCI_CUDA(ctx, cudaGetLastError());

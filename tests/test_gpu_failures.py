@@ -220,3 +220,62 @@ def test_resume_rejects_unsorted_start(pkg, inst):
         with pytest.raises(pkg.HCIError) as ei:
             s.solve_from(keys.flip(0).contiguous(), c, 1e-3)
         assert ei.value.status == pkg._abi.HCI_ERR_INVALID
+
+
+def test_refused_build_leaves_no_graph_of_another_space(pkg, inst):
+    """Space A in use, then space B of the same size, connected enough to
+    need larger buffers, refused at its first, second, ... allocation, the
+    product's plan among them: A afterwards is A or out of memory, never B's
+    connections (the cached graph is found again by size and content hash)."""
+    import oracle
+
+    n, nV = inst.norb, 300
+    # A: spread over the whole space; B: the determinants nearest the aufbau one
+    every = hi.random_det_keys(n, inst.nalpha, inst.nbeta, 4000, seed=5)
+    ref = [(1 << inst.nalpha) - 1, (1 << inst.nbeta) - 1]
+    far = [bin(int(a) ^ ref[0]).count("1") + bin(int(b) ^ ref[1]).count("1") for a, b in every]
+    order = np.argsort(far, kind="stable")
+    pick = {"A": every[np.sort(np.random.default_rng(2).choice(len(every), nV, False))],
+            "B": every[np.sort(order[:nV])]}
+    t = {k: torch.from_numpy(np.ascontiguousarray(v).view(np.int64).reshape(-1, 2)).cuda() for k, v in pick.items()}
+    c = torch.randn(nV, dtype=torch.float64, generator=torch.Generator().manual_seed(3))
+    c = (c / c.norm()).cuda()
+    want = oracle.hamiltonian(inst, pick["A"]) @ c.cpu().numpy()
+    r1, r2 = oracle.rdm12(n, pick["A"], c.cpu().numpy())
+    b_refused = a_after = 0
+    try:
+        for k in range(0, 2000):
+            os.environ[ENV] = str(k)
+            s = None
+            try:
+                s = _solver(pkg, inst)
+                s.set_sigma_mode(pkg._abi.SIGMA_STORED)
+                s.sigma(t["A"], c)
+                s.rdm12(t["A"], c)
+            except pkg.HCIError as e:
+                assert e.status == pkg._abi.HCI_ERR_NOMEM
+                if s is not None:
+                    s.close()
+                continue
+            try:
+                s.sigma(t["B"], c)
+                break
+            except pkg.HCIError as e:
+                assert e.status == pkg._abi.HCI_ERR_NOMEM
+                b_refused += 1
+                for call, ref_out in ((lambda: [s.sigma(t["A"], c)], [want]), (lambda: s.rdm12(t["A"], c), [r1, r2])):
+                    try:
+                        got = call()
+                    except pkg.HCIError as e2:
+                        assert e2.status == pkg._abi.HCI_ERR_NOMEM
+                        continue
+                    a_after += 1
+                    for g, w in zip(got, ref_out):
+                        np.testing.assert_allclose(g.cpu().numpy(), w, rtol=0, atol=1e-11)
+            finally:
+                s.close()
+        else:
+            pytest.fail("B was never built")
+    finally:
+        os.environ.pop(ENV, None)
+    assert b_refused >= 3
