@@ -214,8 +214,10 @@ int64_t hci_fail_alloc_env();
 // M[a][p] for J < n^3 (qtrans_tc.cu): exact digit products on the bf16
 // tensor cores, rounded once to FP64.  A launch that gives up waiting for its
 // products sets *timeout (device), or with NULL a flag that qtrans_tc_check()
-// reports and clears (it reads the flag on st and synchronises st).
-hci_status qtrans_tc(cudaStream_t st, int n, const double* in, const double* M, double* out, int* timeout);
+// reports and clears (it reads the flag on st and synchronises st).  Nothing
+// is done, and out is left as it is, when skip is given (device) and set.
+hci_status qtrans_tc(cudaStream_t st, int n, const double* in, const double* M, double* out, int* timeout,
+                     const int* skip = nullptr);
 hci_status qtrans_tc_check(cudaStream_t st);
 
 inline int grid_for(int64_t work, int block, int max_blocks = -1) {

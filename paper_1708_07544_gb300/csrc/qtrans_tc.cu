@@ -270,8 +270,10 @@ __device__ __forceinline__ void issue_products(uint32_t tmem, uint32_t As_a, uin
 template <int NP>
 __global__ void __launch_bounds__(QtcCfg<NP>::THREADS, 1) k_qtrans_tc(int n, const double* __restrict__ in,
                                                              const double* __restrict__ M, double* __restrict__ out,
-                                                             int64_t ntiles, int* __restrict__ timeout) {
+                                                             int64_t ntiles, int* __restrict__ timeout,
+                                                             const int* __restrict__ skip) {
   using C = QtcCfg<NP>;
+  if (skip && *skip) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* As = sm;
@@ -451,7 +453,8 @@ __global__ void __launch_bounds__(QtcCfg<NP>::THREADS, 1) k_qtrans_tc(int n, con
 int g_qtc_nsm[HCI_MAXORB];   // SM count per device ordinal (0: not looked up)
 
 template <int NP>
-hci_status launch(cudaStream_t st, int n, const double* in, const double* M, double* out, int* timeout) {
+hci_status launch(cudaStream_t st, int n, const double* in, const double* M, double* out, int* timeout,
+                  const int* skip) {
   using C = QtcCfg<NP>;
   static bool attr_set[HCI_MAXORB] = {};
   int dev = 0;
@@ -470,18 +473,19 @@ hci_status launch(cudaStream_t st, int n, const double* in, const double* M, dou
   const int64_t N3 = (int64_t)n * n * n;
   const int64_t ntiles = (N3 + QTC_M - 1) / QTC_M;
   const int grid = (int)(ntiles < g_qtc_nsm[dev] ? ntiles : g_qtc_nsm[dev]);
-  HCI_LAUNCH(k_qtrans_tc<NP>, grid, C::THREADS, C::SMEM, st)(n, in, M, out, ntiles, timeout);
+  HCI_LAUNCH(k_qtrans_tc<NP>, grid, C::THREADS, C::SMEM, st)(n, in, M, out, ntiles, timeout, skip);
   return cudaGetLastError() == cudaSuccess ? HCI_OK : HCI_ERR_CUDA;
 }
 
 }  // namespace
 
-hci_status qtrans_tc(cudaStream_t st, int n, const double* in, const double* M, double* out, int* timeout) {
+hci_status qtrans_tc(cudaStream_t st, int n, const double* in, const double* M, double* out, int* timeout,
+                     const int* skip) {
   if (n < 1 || n > HCI_MAXORB) return HCI_ERR_INVALID;
-  if (n <= 16) return launch<16>(st, n, in, M, out, timeout);
-  if (n <= 32) return launch<32>(st, n, in, M, out, timeout);
-  if (n <= 48) return launch<48>(st, n, in, M, out, timeout);
-  return launch<64>(st, n, in, M, out, timeout);
+  if (n <= 16) return launch<16>(st, n, in, M, out, timeout, skip);
+  if (n <= 32) return launch<32>(st, n, in, M, out, timeout, skip);
+  if (n <= 48) return launch<48>(st, n, in, M, out, timeout, skip);
+  return launch<64>(st, n, in, M, out, timeout, skip);
 }
 
 hci_status qtrans_tc_check(cudaStream_t st) {

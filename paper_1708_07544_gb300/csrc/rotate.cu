@@ -155,7 +155,8 @@ __device__ constexpr double INV_FACT[17] = {
 enum { W_X = 0, W_X2, W_X3, W_X4, W_S0, W_S1, W_S2, W_E, W_F, W_T, W_T2, W_UT, W_UTH, W_GU, W_FWD_COUNT = W_T + 1,
        W_D1 = W_GU + 1, W_D2, W_D3, W_D4, W_DS0, W_DS1, W_DS2, W_DE, W_DF, W_COUNT };
 struct RotStatus {
-  int nonfinite;     // |kappa|_1 is not finite
+  int nonfinite;     // |kappa|_1 is not finite: every later kernel of the call returns at once, so that the
+                     // outputs stay as they were
   int timeout;       // a quarter transform gave up waiting for its products
   int squarings;
   int bad_gradient;  // dE/dU is infinite
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(CLM_T) k_exp_chain(ChainArgs A) {
 
 // dkappa = L_exp(kappa^T, G), G = W_GU: the derivative of every step of the
 // chain above at X^T (whose powers are the stored ones transposed) along
-// dX = G / 2^s; 12 products.
+// dX = G / 2^s; 12 products.  dkappa is left as it is when G is infinite.
 __global__ void __launch_bounds__(CLM_T) k_exp_adjoint(ChainArgs A, double* __restrict__ dkappa) {
   __shared__ double sA[CLM_BI * HCI_MAXORB], sB[HCI_MAXORB * CLM_BJ];
   if (A.status->nonfinite) return;
@@ -320,6 +321,7 @@ __global__ void __launch_bounds__(CLM_T) k_exp_adjoint(ChainArgs A, double* __re
     W(W_D2)[i * n + j] = d2[u];
   });
   cl_sync();
+  if (__ldcg(&A.status->bad_gradient)) return;   // written before the barrier only: the same in every CTA
   const MM p3[2] = {{W(W_X2), W(W_D1), 1, 0}, {W(W_D2), W(W_X), 0, 1}};
   cl_mm(n, t, p3, sA, sB, [&](int u, int i, int j, double v) { d3[u] = v; });
   const MM p4[2] = {{W(W_X2), W(W_D2), 1, 0}, {W(W_D2), W(W_X2), 0, 1}};
@@ -367,7 +369,8 @@ __global__ void __launch_bounds__(CLM_T) k_exp_adjoint(ChainArgs A, double* __re
 // representative ((a,b) = sorted (p,q), (c,d) = sorted (r,s), pairs ordered
 // so that (a,b) <= (c,d)), and h_pq = h_qp takes the value of h_min,max.  In
 // place: a representative is only ever rewritten with its own value.
-__global__ void k_sym8(int n, double* __restrict__ eri) {
+__global__ void k_sym8(int n, double* __restrict__ eri, const RotStatus* __restrict__ status) {
+  if (status->nonfinite) return;
   const int64_t n2 = (int64_t)n * n, n4 = n2 * n2;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n4; t += (int64_t)gridDim.x * blockDim.x) {
     const int s = (int)(t % n), r = (int)((t / n) % n), q = (int)((t / n2) % n), p = (int)(t / (n2 * n));
@@ -540,9 +543,9 @@ cudaError_t launch_chain(cudaStream_t st, int n, void (*k)(P...), Q... args) {
 }
 
 // out[J*n + p] = sum_a in[a*N3 + J] * M[a*n + p], J < N3 = n^3
-#define QTRANS(who, in, M, out, flag)                                                        \
+#define QTRANS(who, in, M, out, flag, skip)                                                  \
   do {                                                                                       \
-    if (qtrans_tc(st, n, in, M, out, flag) != HCI_OK)                                            \
+    if (qtrans_tc(st, n, in, M, out, flag, skip) != HCI_OK)                                      \
       return hci_fail(nullptr, HCI_ERR_CUDA, who ": quarter transform launch failed: %s",     \
                       cudaGetErrorString(cudaGetLastError()));                               \
   } while (0)
@@ -570,12 +573,12 @@ hci_status rotate_core(const char* who, cudaStream_t st, int n, const double* ka
   cudaError_t e = cudaMemsetAsync(status, 0, sizeof(RotStatus), st);
   if (e == cudaSuccess) e = launch_chain(st, n, k_exp_chain<false>, A);
   if (e != cudaSuccess) return hci_fail(nullptr, HCI_ERR_CUDA, "%s: %s", who, cudaGetErrorString(e));
-  QTRANS("hci_rotate", eri, U, t4, &status->timeout);
-  QTRANS("hci_rotate", t4, U, eri_out, &status->timeout);
-  QTRANS("hci_rotate", eri_out, U, t4, &status->timeout);
-  QTRANS("hci_rotate", t4, U, eri_out, &status->timeout);
+  QTRANS("hci_rotate", eri, U, t4, &status->timeout, &status->nonfinite);
+  QTRANS("hci_rotate", t4, U, eri_out, &status->timeout, &status->nonfinite);
+  QTRANS("hci_rotate", eri_out, U, t4, &status->timeout, &status->nonfinite);
+  QTRANS("hci_rotate", t4, U, eri_out, &status->timeout, &status->nonfinite);
   // exact permutational symmetry of the rotated integrals (see k_sym8)
-  HCI_LAUNCH(k_sym8, (unsigned)std::min<int64_t>(blocks((int64_t)n * n * n * n), 4096), 256, 0, st)(n, eri_out);
+  HCI_LAUNCH(k_sym8, (unsigned)std::min<int64_t>(blocks((int64_t)n * n * n * n), 4096), 256, 0, st)(n, eri_out, status);
   return chain_status(who, st, status);
 }
 
@@ -626,9 +629,9 @@ extern "C" hci_status hci_rotate_backward(int norb, const double* kappa, const d
   // transforms leave T[y][d][c][b] in ta, the fourth is dE/d(dc|ba)
   const double *Ut = ws + (size_t)W_UT * n2, *Uth = ws + (size_t)W_UTH * n2;
   if (deri || dkappa) {
-    QTRANS("hci_rotate_backward", rdm2, Uth, ta, &status->timeout);
-    QTRANS("hci_rotate_backward", ta, Ut, tb, &status->timeout);
-    QTRANS("hci_rotate_backward", tb, Ut, ta, &status->timeout);
+    QTRANS("hci_rotate_backward", rdm2, Uth, ta, &status->timeout, &status->nonfinite);
+    QTRANS("hci_rotate_backward", ta, Ut, tb, &status->timeout, &status->nonfinite);
+    QTRANS("hci_rotate_backward", tb, Ut, ta, &status->timeout, &status->nonfinite);
   }
   if (dkappa) {
     const size_t sm = (size_t)NT_CH * (2 * n + 1) * 8;
@@ -642,7 +645,7 @@ extern "C" hci_status hci_rotate_backward(int norb, const double* kappa, const d
     e = launch_chain(st, n, k_exp_adjoint, A, dkappa);
     if (e != cudaSuccess) return hci_fail(nullptr, HCI_ERR_CUDA, "hci_rotate_backward: %s", cudaGetErrorString(e));
   }
-  if (deri) QTRANS("hci_rotate_backward", ta, Ut, deri, &status->timeout);
+  if (deri) QTRANS("hci_rotate_backward", ta, Ut, deri, &status->timeout, &status->nonfinite);
   return chain_status("hci_rotate_backward", st, status);
 }
 
@@ -652,7 +655,7 @@ extern "C" hci_status hci_qtrans(int norb, const double* in, const double* M, do
   if (n < 1 || n > HCI_MAXORB) return hci_fail(nullptr, HCI_ERR_INVALID, "hci_qtrans: norb=%d outside [1,64]", n);
   if (!in || !M || !out) return hci_fail(nullptr, HCI_ERR_INVALID, "hci_qtrans: null pointer");
   cudaStream_t st = (cudaStream_t)stream;
-  QTRANS("hci_qtrans", in, M, out, nullptr);
+  QTRANS("hci_qtrans", in, M, out, nullptr, nullptr);
   if (check && qtrans_tc_check(st) != HCI_OK)
     return hci_fail(nullptr, HCI_ERR_CUDA, "hci_qtrans: a quarter transform gave up waiting for its tensor-core products");
   return HCI_OK;

@@ -98,3 +98,34 @@ def test_ragged_blocks(n, sigma):
     G = h @ ref @ r1.T + h.T @ ref @ r1
     want = sl.expm_frechet(kap.T, G, compute_expm=False)
     assert np.abs(dk - want).max() <= 1e-13 * n * max(1.0, np.abs(kap).sum(0).max()) * np.abs(want).max()
+
+
+# a refused call leaves its outputs as they were (eri_out may be eri itself)
+@pytest.mark.parametrize("n", [5, 20])
+@pytest.mark.parametrize("noalloc", [False, True])
+def test_refused_rotation_keeps_its_outputs(n, noalloc):
+    from paper_1708_07544_gb300 import _abi
+
+    L = _abi.load()
+    dev = {"dtype": torch.float64, "device": "cuda"}
+    k = torch.zeros(n, n, **dev)
+    k[1, 2] = float("inf")
+    h, eri = torch.randn(n, n, **dev), torch.randn(n, n, n, n, **dev)
+    outs = [torch.full((n, n), 7.0, **dev), torch.full((n, n), 7.0, **dev), eri]
+    keep = [o.clone() for o in outs]
+    torch.cuda.synchronize()
+    f = L.hci_rotate_noalloc if noalloc else L.hci_rotate
+    assert f(n, k.data_ptr(), h.data_ptr(), eri.data_ptr(), *[o.data_ptr() for o in outs], None) == _abi.HCI_ERR_INVALID
+    for o, w in zip(outs, keep):
+        assert torch.equal(o, w)
+    # backward: an infinite kappa, then an infinite dE/dU (dh and deri are done by then)
+    g = [torch.full((n, n), 7.0, **dev), torch.full((n,) * 4, 7.0, **dev), torch.full((n, n), 7.0, **dev)]
+    r1, r2 = torch.randn(n, n, **dev), torch.randn(n, n, n, n, **dev)
+    torch.cuda.synchronize()
+    back = lambda kap, rdm1: L.hci_rotate_backward(n, kap.data_ptr(), h.data_ptr(), eri.data_ptr(), rdm1.data_ptr(),  # noqa: E731
+                                                   r2.data_ptr(), *[o.data_ptr() for o in g], None)
+    assert back(k, r1) == _abi.HCI_ERR_INVALID
+    assert all(bool((o == 7.0).all()) for o in g)
+    r1[0, 0] = float("inf")
+    assert back(torch.zeros(n, n, **dev), r1) == _abi.HCI_ERR_INVALID
+    assert bool((g[2] == 7.0).all())
