@@ -36,7 +36,7 @@ hci_status hci_fail(hci_ctx* ctx, hci_status code, const char* fmt, ...) {
 // 10 to 24 orbitals: 3133 calls and 53 ms without, 45 ms so).
 constexpr size_t SLAB_BYTES = (size_t)4 << 20, SLAB_MAX = (size_t)64 << 10, ROUND_MAX = (size_t)16 << 20;
 
-hci_status ensure_buf(hci_ctx* ctx, DevBuf& b, size_t bytes) {
+hci_status ensure_buf(hci_ctx* ctx, DevBuf& b, size_t bytes, bool exact) {
   if (bytes <= b.bytes && b.p) return HCI_OK;
   if (ctx->fail_alloc_after >= 0) {
     if (ctx->fail_alloc_after == 0)
@@ -46,16 +46,16 @@ hci_status ensure_buf(hci_ctx* ctx, DevBuf& b, size_t bytes) {
   }
   free_buf(ctx->st, b);
   size_t want = 256;
-  if (bytes <= ROUND_MAX)
+  if (!exact && bytes <= ROUND_MAX)
     while (want < bytes) want *= 2;
   else
     want = (bytes + 255) & ~(size_t)255;
-  if (want <= SLAB_MAX && !ctx->slab && cudaMallocAsync(&ctx->slab, SLAB_BYTES, ctx->st) != cudaSuccess) {
+  if (!exact && want <= SLAB_MAX && !ctx->slab && cudaMallocAsync(&ctx->slab, SLAB_BYTES, ctx->st) != cudaSuccess) {
     cudaGetLastError();
     ctx->slab = nullptr;
   }
   cudaError_t e = cudaSuccess;
-  if (want <= SLAB_MAX && ctx->slab && ctx->slab_used + want <= SLAB_BYTES) {
+  if (!exact && want <= SLAB_MAX && ctx->slab && ctx->slab_used + want <= SLAB_BYTES) {
     b.p = (char*)ctx->slab + ctx->slab_used;
     b.slab = true;
     ctx->slab_used += want;

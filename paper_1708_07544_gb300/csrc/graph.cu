@@ -1743,6 +1743,12 @@ static void free_segments(hci_ctx* ctx) {
   G.pool_used = G.pool_cap = 0;
 }
 
+// Buffers of stored connections: the pool grows in place up to what they
+// hold, so under a budget they hold what was admitted and no more.
+static hci_status conn_buf(hci_ctx* ctx, DevBuf& b, int64_t bytes) {
+  return ensure_buf(ctx, b, (size_t)bytes, ctx->graph_budget > 0);
+}
+
 // A new segment of `entries` stored connections; HCI_ERR_NOMEM when the
 // stored connections would exceed the context's budget.
 static hci_status seg_alloc(hci_ctx* ctx, int64_t entries, int* seg) {
@@ -1752,8 +1758,8 @@ static hci_status seg_alloc(hci_ctx* ctx, int64_t entries, int* seg) {
   if (ctx->graph_budget > 0 && bytes > ctx->graph_budget)
     return hci_fail(ctx, HCI_ERR_NOMEM, "graph: %lld bytes of stored connections exceed the budget of %lld",
                     (long long)bytes, (long long)ctx->graph_budget);
-  HCI_TRY(ensure_buf(ctx, G.seg_col[G.nseg], (size_t)(entries + 1) * 4));
-  HCI_TRY(ensure_buf(ctx, G.seg_val[G.nseg], (size_t)(entries + 1) * 8));
+  HCI_TRY(conn_buf(ctx, G.seg_col[G.nseg], (entries + 1) * 4));
+  HCI_TRY(conn_buf(ctx, G.seg_val[G.nseg], (entries + 1) * 8));
   *seg = G.nseg++;
   return HCI_OK;
 }
@@ -2003,8 +2009,8 @@ static hci_status graph_build_full(hci_ctx* ctx, const uint64_t* keys, int64_t n
   if (ctx->graph_budget > 0 && cap * 12 > ctx->graph_budget)
     return hci_fail(ctx, HCI_ERR_NOMEM, "graph: a pool of %lld bytes exceeds the budget of %lld", (long long)(cap * 12),
                     (long long)ctx->graph_budget);
-  HCI_TRY(ensure_buf(ctx, G.seg_col[0], (size_t)cap * 4));
-  HCI_TRY(ensure_buf(ctx, G.seg_val[0], (size_t)cap * 8));
+  HCI_TRY(conn_buf(ctx, G.seg_col[0], cap * 4));
+  HCI_TRY(conn_buf(ctx, G.seg_val[0], cap * 8));
   G.nseg = 1;
   HCI_TRY(stage_place(ctx, A, left, bp<int32_t>(G.seg_col[0]), bp<int64_t>(G.rowstart)));
   HCI_LAUNCH(k_row_values, values_grid(nnz), 256, 0, ctx->st)(
@@ -2147,8 +2153,8 @@ static hci_status graph_extend_full(hci_ctx* ctx, const uint64_t* keys, int64_t 
     if (ctx->graph_budget > 0 && (cap + G.pool_cap) * 12 > ctx->graph_budget)
       return hci_fail(ctx, HCI_ERR_NOMEM, "graph: repacking into %lld bytes exceeds the budget of %lld",
                       (long long)(cap * 12), (long long)ctx->graph_budget);
-    HCI_TRY(ensure_buf(ctx, S.col_old, (size_t)cap * 4));
-    HCI_TRY(ensure_buf(ctx, S.val_old, (size_t)cap * 8));
+    HCI_TRY(conn_buf(ctx, S.col_old, cap * 4));
+    HCI_TRY(conn_buf(ctx, S.val_old, cap * 8));
     col_dst = bp<int32_t>(S.col_old);
     val_dst = bp<double>(S.val_old);
     base = 0;

@@ -193,8 +193,9 @@ hci_status hci_fail(hci_ctx* ctx, hci_status code, const char* fmt, ...);
     if (_s != HCI_OK) return _s;      \
   } while (0)
 
-// Ensure buf holds at least `bytes` (contents are NOT preserved on growth).
-hci_status ensure_buf(hci_ctx* ctx, DevBuf& b, size_t bytes);
+// Ensure buf holds at least `bytes` (contents are NOT preserved on growth);
+// exact: no more is allocated than asked for (to the next 256 bytes).
+hci_status ensure_buf(hci_ctx* ctx, DevBuf& b, size_t bytes, bool exact = false);
 void free_buf(cudaStream_t st, DevBuf& b);
 
 template <class T>

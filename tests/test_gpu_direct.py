@@ -126,3 +126,67 @@ def test_auto_falls_back_under_a_budget(pkg):
             s.set_sigma_mode(7)
         with pytest.raises(pkg.HCIError):
             s.set_sigma_mode(_abi.SIGMA_AUTO, -1)
+
+
+def _near(ref, norb):
+    """Determinants within two excitations of ref, ascending."""
+    from itertools import combinations
+
+    def moved(s, k):
+        occ = [p for p in range(norb) if s >> p & 1]
+        vir = [p for p in range(norb) if not s >> p & 1]
+        return [s ^ sum(1 << p for p in h + t) for h in combinations(occ, k) for t in combinations(vir, k)]
+
+    a, b = ref
+    out = [(x, y) for i in range(3) for j in range(3 - i) for x in moved(a, i) for y in moved(b, j)]
+    return np.array(sorted(out), np.uint64)
+
+
+def _row_slots(keys):
+    """Connections of each determinant and the slots its stored row takes."""
+    d = sum(np.bitwise_count(keys[:, None, k] ^ keys[None, :, k]).astype(int) for k in (0, 1))
+    n = ((d == 2) | (d == 4)).sum(1)
+    return n, n + n // 4 + 8
+
+
+@pytest.mark.parametrize("nv", [300, 360, 430, 510, 600])
+def test_budget_holds_while_a_space_grows(pkg, nv):
+    """A pool admitted by its budget takes what the rest of it holds and no
+    more: a far group of determinants (no connections to the first) is
+    appended in place while its rows fit the pool, and refused, not put into
+    what an allocation was rounded up to, when they do not."""
+    from paper_1708_07544_gb300 import _abi
+
+    inst = hi.df_12o()
+    low, high = _near((0o77, 0o77), 12), _near((0o7700, 0o7700), 12)
+    g = np.random.default_rng(nv)
+    A = low[np.sort(g.choice(len(low), nv, False))]
+    used = _row_slots(A)[1].sum()
+    cap = int(used + used // 4 + 1024)
+    order = g.permutation(len(high))
+
+    def with_far(m):
+        K = np.concatenate([A, high[order[:m]]])
+        return K[np.lexsort((K[:, 1], K[:, 0]))]
+
+    def far_slots(m):
+        return _row_slots(high[order[:m]])[1].sum()
+
+    fits = max(m for m in range(1, nv) if used + far_slots(m) <= cap)
+    exceeds = min(m for m in range(fits, len(high), 8) if used + far_slots(m) > 1.1 * cap)
+    c = torch.ones(nv + exceeds, dtype=torch.float64, device="cuda")
+    for m, ok in ((fits, True), (exceeds, False)):
+        K = with_far(m)
+        with solver(pkg, inst, _abi.SIGMA_STORED, 12 * cap) as s:
+            s.sigma(dev_keys(A), c[:nv])
+            if ok:
+                s.sigma(dev_keys(K), c[:len(K)])
+                assert s.stats()["graph_half"] == 0
+            else:
+                with pytest.raises(pkg.HCIError) as ei:
+                    s.sigma(dev_keys(K), c[:len(K)])
+                assert ei.value.status == _abi.HCI_ERR_NOMEM
+        with solver(pkg, inst, _abi.SIGMA_AUTO, 12 * cap) as s:
+            s.sigma(dev_keys(A), c[:nv])
+            s.sigma(dev_keys(K), c[:len(K)])
+            assert (s.stats()["graph_half"], s.stats()["sigma_direct"]) == ((0, 0) if ok else (1, 0))
