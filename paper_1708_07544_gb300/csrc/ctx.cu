@@ -28,13 +28,40 @@ hci_status hci_fail(hci_ctx* ctx, hci_status code, const char* fmt, ...) {
 }
 
 // A context has some 110 buffers, and on a small space nearly all of them
-// stay below a page and grow with every extension.  Those up to SLAB_MAX come
-// out of one slab per context, given back as a whole with the context, and
-// sizes up to ROUND_MAX are rounded up to powers of two, so that a buffer
-// grows a few times in all and not with every extension: on eight streams the
-// runtime's allocator takes 29 us per call, one call at a time (15 solves of
-// 10 to 24 orbitals: 3133 calls and 53 ms without, 45 ms so).
-constexpr size_t SLAB_BYTES = (size_t)4 << 20, SLAB_MAX = (size_t)64 << 10, ROUND_MAX = (size_t)16 << 20;
+// stay below a page and grow with every extension.  Those up to SLAB_MAX are
+// pieces of one slab per context, which goes back to the runtime with the
+// context, and sizes up to ROUND_MAX are rounded up to powers of two, so that
+// a buffer grows a few times in all and not with every extension: on eight
+// streams the runtime's allocator takes 29 us per call, one call at a time (15
+// solves of 10 to 24 orbitals: 3133 calls and 53 ms without, 45 ms so).  A
+// piece given back is the next one of its size (all of a context's work is
+// on one stream, in order), so that repeated calls stay on the slab.
+constexpr size_t SLAB_BYTES = SLAB_UNIT * SLAB_UNITS, SLAB_MAX = SLAB_UNIT << (SLAB_CLASSES - 1),
+                 ROUND_MAX = (size_t)16 << 20;
+
+// a piece of want = SLAB_UNIT << k bytes, or false
+static bool slab_take(hci_ctx* ctx, DevBuf& b, size_t want) {
+  if (!ctx->slab && cudaMallocAsync(&ctx->slab, SLAB_BYTES, ctx->st) != cudaSuccess) {
+    cudaGetLastError();
+    ctx->slab = nullptr;
+    return false;
+  }
+  int k = 0;
+  while ((SLAB_UNIT << k) < want) ++k;
+  size_t unit = 0;
+  if (ctx->slab_free[k]) {
+    unit = ctx->slab_free[k] - 1u;
+    ctx->slab_free[k] = ctx->slab_next[unit];
+  } else if (ctx->slab_used + want <= SLAB_BYTES) {
+    unit = ctx->slab_used / SLAB_UNIT;
+    ctx->slab_used += want;
+  } else {
+    return false;
+  }
+  b.p = (char*)ctx->slab + unit * SLAB_UNIT;
+  b.slab = true;
+  return true;
+}
 
 hci_status ensure_buf(hci_ctx* ctx, DevBuf& b, size_t bytes, bool exact) {
   if (bytes <= b.bytes && b.p) return HCI_OK;
@@ -44,24 +71,14 @@ hci_status ensure_buf(hci_ctx* ctx, DevBuf& b, size_t bytes, bool exact) {
                       bytes);
     --ctx->fail_alloc_after;
   }
-  free_buf(ctx->st, b);
+  free_buf(ctx, b);
   size_t want = 256;
   if (!exact && bytes <= ROUND_MAX)
     while (want < bytes) want *= 2;
   else
     want = (bytes + 255) & ~(size_t)255;
-  if (!exact && want <= SLAB_MAX && !ctx->slab && cudaMallocAsync(&ctx->slab, SLAB_BYTES, ctx->st) != cudaSuccess) {
-    cudaGetLastError();
-    ctx->slab = nullptr;
-  }
   cudaError_t e = cudaSuccess;
-  if (!exact && want <= SLAB_MAX && ctx->slab && ctx->slab_used + want <= SLAB_BYTES) {
-    b.p = (char*)ctx->slab + ctx->slab_used;
-    b.slab = true;
-    ctx->slab_used += want;
-  } else {
-    e = cudaMallocAsync(&b.p, want, ctx->st);
-  }
+  if (exact || want > SLAB_MAX || !slab_take(ctx, b, want)) e = cudaMallocAsync(&b.p, want, ctx->st);
   if (e != cudaSuccess) {
     cudaGetLastError();
     b = DevBuf();
@@ -72,8 +89,16 @@ hci_status ensure_buf(hci_ctx* ctx, DevBuf& b, size_t bytes, bool exact) {
   return HCI_OK;
 }
 
-void free_buf(cudaStream_t st, DevBuf& b) {
-  if (b.p && !b.slab) cudaFreeAsync(b.p, st);
+void free_buf(hci_ctx* ctx, DevBuf& b) {
+  if (b.p && b.slab) {
+    const size_t unit = (size_t)((char*)b.p - (char*)ctx->slab) / SLAB_UNIT;
+    int k = 0;
+    while ((SLAB_UNIT << k) < b.bytes) ++k;
+    ctx->slab_next[unit] = ctx->slab_free[k];
+    ctx->slab_free[k] = (uint16_t)(unit + 1);
+  } else if (b.p) {
+    cudaFreeAsync(b.p, ctx->st);
+  }
   b = DevBuf();
 }
 
@@ -410,10 +435,10 @@ extern "C" hci_status hci_destroy(hci_ctx* ctx) {
                     &ctx->d_zv, &ctx->d_rel, &ctx->d_lock, &ctx->d_partner, &ctx->dkeep.Q, &ctx->dkeep.W, &ctx->ss_w, &ctx->ss_draw,
                     &ctx->ss_draw2, &ctx->ss_run, &ctx->ss_src};
   for (int k = 0; k < GRAPH_MAXSEG; ++k) {
-    free_buf(st, ctx->graph.seg_col[k]);
-    free_buf(st, ctx->graph.seg_val[k]);
+    free_buf(ctx, ctx->graph.seg_col[k]);
+    free_buf(ctx, ctx->graph.seg_val[k]);
   }
-  for (DevBuf* b : bufs) free_buf(st, *b);
+  for (DevBuf* b : bufs) free_buf(ctx, *b);
   if (ctx->slab) cudaFreeAsync(ctx->slab, st);
   prof_release(ctx);
   cudaStreamSynchronize(st);

@@ -1727,15 +1727,15 @@ static hci_status grow_keep(hci_ctx* ctx, DevBuf& b, size_t bytes, size_t keep) 
   HCI_TRY(ensure_buf(ctx, t, bytes + bytes / 4));
   if (keep > 0 && b.p) HCI_CUDA(ctx, cudaMemcpyAsync(t.p, b.p, keep, cudaMemcpyDeviceToDevice, ctx->st));
   std::swap(b, t);
-  free_buf(ctx->st, t);
+  free_buf(ctx, t);
   return HCI_OK;
 }
 
 static void free_segments(hci_ctx* ctx) {
   Graph& G = ctx->graph;
   for (int k = 0; k < GRAPH_MAXSEG; ++k) {
-    free_buf(ctx->st, G.seg_col[k]);
-    free_buf(ctx->st, G.seg_val[k]);
+    free_buf(ctx, G.seg_col[k]);
+    free_buf(ctx, G.seg_val[k]);
   }
   G.nseg = 0;
   G.nstored = 0;
@@ -2175,8 +2175,8 @@ static hci_status graph_extend_full(hci_ctx* ctx, const uint64_t* keys, int64_t 
   if (repack) {
     std::swap(G.seg_col[0], S.col_old);
     std::swap(G.seg_val[0], S.val_old);
-    free_buf(st, S.col_old);
-    free_buf(st, S.val_old);
+    free_buf(ctx, S.col_old);
+    free_buf(ctx, S.val_old);
     G.pool_cap = pool_entries(G);
     G.pool_used = total;
   } else {
@@ -2252,7 +2252,7 @@ static void release_stored(hci_ctx* ctx) {
   free_segments(ctx);
   DevBuf* bufs[] = {&G.rowptr, &G.rowstart, &G.rowlen, &G.rowcap, &S.scr, &S.stage, &S.grow, &S.col_old,
                     &S.val_old, &S.colN, &S.valN, &S.T, &S.T2, &S.items, &S.first, &S.itp};
-  for (DevBuf* b : bufs) free_buf(ctx->st, *b);
+  for (DevBuf* b : bufs) free_buf(ctx, *b);
   cudaStreamSynchronize(ctx->st);
 }
 

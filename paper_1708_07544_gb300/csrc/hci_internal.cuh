@@ -20,8 +20,12 @@
 struct DevBuf {
   void* p = nullptr;
   size_t bytes = 0;
-  bool slab = false;   // part of its context's slab: nothing to free
+  bool slab = false;   // a piece of its context's slab
 };
+
+// Slab of small buffers (ensure_buf): pieces of 256 << k bytes, k < SLAB_CLASSES
+constexpr int SLAB_CLASSES = 9;
+constexpr size_t SLAB_UNIT = 256, SLAB_UNITS = 16384;
 
 // Stored connections are kept in segments (one per build or extension of
 // the space); a row's first entry is addressed as segment << GRAPH_SEG_SHIFT
@@ -131,7 +135,9 @@ struct hci_ctx {
   double ecore = 0;
   cudaStream_t st = nullptr;
   void* slab = nullptr;              // the small buffers' memory (ensure_buf)
-  size_t slab_used = 0;
+  size_t slab_used = 0;              // pieces handed out from the slab's start
+  uint16_t slab_free[SLAB_CLASSES] = {};   // pieces given back, by size: lists through slab_next of
+  uint16_t slab_next[SLAB_UNITS] = {};     // unit + 1 (0: end)
   DevBuf h, eri;                     // device copies
   DevBuf jk_same, j_opp;             // n^3 tables for single excitations
   Lists lists;
@@ -196,7 +202,7 @@ hci_status hci_fail(hci_ctx* ctx, hci_status code, const char* fmt, ...);
 // Ensure buf holds at least `bytes` (contents are NOT preserved on growth);
 // exact: no more is allocated than asked for (to the next 256 bytes).
 hci_status ensure_buf(hci_ctx* ctx, DevBuf& b, size_t bytes, bool exact = false);
-void free_buf(cudaStream_t st, DevBuf& b);
+void free_buf(hci_ctx* ctx, DevBuf& b);
 
 template <class T>
 inline T* bp(DevBuf& b) { return reinterpret_cast<T*>(b.p); }

@@ -45,8 +45,8 @@ static hci_status solve_core(hci_ctx* ctx, double eps1, int max_iter, double dav
   HCI_TRY(hci_build_lists(ctx));
   DevBuf kb[2], cb[2], nk;
   auto cleanup = [&]() {
-    for (int i = 0; i < 2; ++i) { free_buf(st, kb[i]); free_buf(st, cb[i]); }
-    free_buf(st, nk);
+    for (int i = 0; i < 2; ++i) { free_buf(ctx, kb[i]); free_buf(ctx, cb[i]); }
+    free_buf(ctx, nk);
   };
   int cur = 0;
   int64_t nV = keys0 ? nV0 : 1;
@@ -141,8 +141,8 @@ static hci_status solve_entry(const char* name, hci_ctx* ctx, double eps1, int m
   *nV_out = nV;
   *energy = e;
   if (nV > cap) {
-    free_buf(st, kr);
-    free_buf(st, cr);
+    free_buf(ctx, kr);
+    free_buf(ctx, cr);
     return hci_fail(ctx, HCI_ERR_CAPACITY, "%s: %lld determinants exceed cap %lld", name, (long long)nV,
                     (long long)cap);
   }
@@ -150,8 +150,8 @@ static hci_status solve_entry(const char* name, hci_ctx* ctx, double eps1, int m
   if (keys_out) ce = cudaMemcpyAsync(keys_out, kr.p, (size_t)nV * 16, cudaMemcpyDeviceToDevice, st);
   if (ce == cudaSuccess && c_out) ce = cudaMemcpyAsync(c_out, cr.p, (size_t)nV * 8, cudaMemcpyDeviceToDevice, st);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
-  free_buf(st, kr);
-  free_buf(st, cr);
+  free_buf(ctx, kr);
+  free_buf(ctx, cr);
   if (ce != cudaSuccess) return hci_fail(ctx, HCI_ERR_CUDA, "%s: %s", name, cudaGetErrorString(ce));
   return HCI_OK;
 }
@@ -187,9 +187,9 @@ extern "C" hci_status hci_solve_roots(hci_ctx* ctx, int nroots, double eps1, int
   HCI_TRY(hci_build_lists(ctx));
   DevBuf kb[2], cb[2], nk, ce;
   auto cleanup = [&]() {
-    for (int i = 0; i < 2; ++i) { free_buf(st, kb[i]); free_buf(st, cb[i]); }
-    free_buf(st, nk);
-    free_buf(st, ce);
+    for (int i = 0; i < 2; ++i) { free_buf(ctx, kb[i]); free_buf(ctx, cb[i]); }
+    free_buf(ctx, nk);
+    free_buf(ctx, ce);
   };
   hci_status s;
   if ((s = ensure_buf(ctx, kb[0], 16)) != HCI_OK || (s = ensure_buf(ctx, ce, 8)) != HCI_OK) { cleanup(); return s; }
@@ -307,8 +307,8 @@ extern "C" hci_status hci_solve_batch(int count, const int* norb, const int* nal
         }
       }
       if (ctx) {
-        free_buf(st, kr);
-        free_buf(st, cr);
+        free_buf(ctx, kr);
+        free_buf(ctx, cr);
         hci_destroy(ctx);
       }
     }
