@@ -1304,6 +1304,7 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
       HCI_TRY(ritz());
       HCI_TRY(report());
       converged = rn <= tol;
+      if (!converged) --it;   // not a step of its own: counted as the chain above counts
       break;
     }
     if (rn <= tol) {

@@ -145,3 +145,19 @@ def test_spin_parity_refusals(pkg):
         with pytest.raises(pkg.HCIError) as ei:
             s.davidson(dev_keys(oracle.aufbau(4, 4)), None)
         assert "no state" in str(ei.value)
+
+
+@pytest.mark.parametrize("parity,nstr", [(1, 2), (1, 3), (-1, 3), (-1, 4)])
+def test_iterations_up_to_an_exhausted_sector(pkg, parity, nstr):
+    """tol = 0 in a sector of d states: Davidson takes one step per state and
+    stops when the next correction lies in the subspace; that correction is
+    not a step."""
+    inst = hi.random_tiny(4, 2, 2, 13)
+    strings = [0b0011, 0b0101, 0b0110, 0b1001][:nstr]
+    keys = np.array(sorted((a, b) for a in strings for b in strings), np.uint64)
+    d = nstr * (nstr + 1) // 2 if parity > 0 else nstr * (nstr - 1) // 2
+    e_or, _ = oracle.parity_ground_state(inst, keys, parity)
+    with solver(pkg, inst, parity) as s:
+        e, _, it = s.davidson(dev_keys(keys), None, tol=0.0, maxit=60, allow_unconverged=True)
+    assert abs(e - e_or) < 1e-11
+    assert it == d
