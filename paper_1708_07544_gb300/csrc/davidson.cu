@@ -804,8 +804,9 @@ __global__ void __launch_bounds__(DBLOCK) k_ritz(const double* __restrict__ V, c
     d->eps = den != 0.0 ? num / den : 0.0;
     d->rep.it += 1;
     d->rep.k = k;
-    // a residual that is not finite ends the chain too
-    if (chained && (!(sqrt(s) > tol) || !isfinite(s) || !isfinite(theta))) d->rep.stop = 1;
+    // a residual that is not finite ends the chain too; a tolerance that is not
+    // a number is never met, here as on the host
+    if (chained && (sqrt(s) <= tol || !isfinite(s) || !isfinite(theta))) d->rep.stop = 1;
   }
 }
 

@@ -66,3 +66,19 @@ def test_energy_offset(offset):
     with _solver(inst) as s:
         e, c, _ = s.davidson(kt, None, max(1e-10, 1e-13 * abs(offset)), 2000)
     assert abs(e - np.linalg.eigvalsh(H)[0]) <= 1e-12 * max(1.0, abs(offset)) * 10
+
+
+@pytest.mark.parametrize("maxit", [1, 3, 4, 5, 9])
+def test_tolerance_never_met(maxit):
+    # neither a negative tolerance nor NaN is met by any residual: maxit steps,
+    # and the same Ritz pair from both
+    inst = hi.random_tiny(6, 3, 3, 9)
+    keys = hi.random_det_keys(6, 3, 3, 200, 4)
+    kt = torch.tensor(keys.astype(np.int64), device="cuda")
+    out = {}
+    for tol in (-1.0, float("nan")):
+        with _solver(inst) as s:
+            out[str(tol)] = s.davidson(kt, None, tol, maxit, allow_unconverged=True)
+    (e0, c0, i0), (e1, c1, i1) = out.values()
+    assert i0 == i1 == maxit
+    assert e0 == e1 and torch.equal(c0, c1)
