@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(SEL_WARPS * 32) k_singles(WalkArgs A) {
           bool ok = e < L && ((s >> p) & 1ull) && !((s >> r) & 1ull);
           if (!A.accept_all) {
             const float t = __fmaf_ru(spin == 0 ? da : db, mx.z, __fmaf_ru(spin == 0 ? db : da, mx.w, spin == 0 ? mx.x : mx.y));
-            ok = ok && __fmul_ru(t, cf) > epsf;
+            ok = ok && !(__fmul_ru(t, cf) <= epsf);   // not a number: 0 changed orbitals of a term beyond FP32
           }
           const unsigned b = __ballot_sync(0xffffffffu, ok);
           if (A.accept_all && !A.vals) {

@@ -74,3 +74,24 @@ def test_selection_of_wider_queues(nV):
     as_set = lambda k: set(map(tuple, np.asarray(k).tolist()))  # noqa: E731
     assert as_set(got) - as_set(ties) == as_set(want) - as_set(ties)
     assert len(as_set(got)) == len(got)
+
+
+# integrals beyond FP32's range (the screens' bounds are FP32, rounded up):
+# (pr|kk) of an orbital k that is empty in the determinant does not matter to
+# its single p -> r, and one that is occupied decides it
+@pytest.mark.parametrize("k", [1, 3])
+@pytest.mark.parametrize("big", [1e38, 1e39, 1e300])
+def test_integrals_beyond_fp32(k, big):
+    inst = hi.random_tiny(4, 2, 1, 7)
+    inst.h, inst.eri = np.zeros((4, 4)), np.zeros((4,) * 4)
+    inst.h[0, 2] = inst.h[2, 0] = 0.1
+    for p, r in ((0, 2), (2, 0)):
+        inst.eri[p, r, k, k] = inst.eri[k, k, p, r] = big
+    for c, eps1 in ((1.0, 1e-3), (1e-40, 1e-43), (1e-40, 1e-39), (1.0, 0.2)):
+        for keys in (np.array([[0b0011, 0b0001]], np.uint64), np.array([[0b0011, 0b0010]], np.uint64)):
+            cv = np.array([c])
+            want, _, ties = oracle.select(inst, keys, cv, eps1)
+            with _solver(inst) as s:
+                got = s.select(eps1, _dev(keys), _dev(cv)).cpu().numpy().view(np.uint64).reshape(-1, 2)
+            assert sorted(map(tuple, got.tolist())) == sorted(map(tuple, np.asarray(want).reshape(-1, 2).tolist()))
+            assert len(ties) == 0
