@@ -300,20 +300,6 @@ __global__ void k_max_first(const double* __restrict__ mag, int nlists, int L, d
   }
 }
 
-__global__ void k_max_vec(const double* __restrict__ v, int n, double* out) {
-  double m = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) m = fmax(m, v[i]);
-  for (int o = 16; o; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  __shared__ double w[32];
-  if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double r = 0.0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) r = fmax(r, w[k]);
-    *out = r;
-  }
-}
-
 int next_pow2(int x) {
   int p = 1;
   while (p < x) p <<= 1;
@@ -507,14 +493,12 @@ extern "C" hci_status hci_build_lists(hci_ctx* ctx) {
   HCI_LAUNCH(k_max_first, 1, 1024, 0, ctx->st)(bp<double>(L.opp_mag), n * n, L.len_opp, dm + 0);
   if (L.npair_same > 0)
     HCI_LAUNCH(k_max_first, 1, 1024, 0, ctx->st)(bp<double>(L.same_mag), L.npair_same, L.len_same, dm + 1);
-  HCI_LAUNCH(k_max_vec, 1, 1024, 0, ctx->st)(bp<double>(L.single_bound), n * n, dm + 2);
   HCI_CUDA(ctx, cudaGetLastError());
-  double hm[3];
-  HCI_CUDA(ctx, cudaMemcpyAsync(hm, dm, 24, cudaMemcpyDeviceToHost, ctx->st));
+  double hm[2];
+  HCI_CUDA(ctx, cudaMemcpyAsync(hm, dm, 16, cudaMemcpyDeviceToHost, ctx->st));
   HCI_CUDA(ctx, cudaStreamSynchronize(ctx->st));
   L.max_opp = hm[0];
   L.max_same = hm[1];
-  L.max_single = hm[2];
   L.built = true;
   prof_toc(ctx, HCI_PH_LISTS);
   return HCI_OK;

@@ -214,7 +214,6 @@ __device__ double connection_el(const HamView& H, ulonglong2 ki, ulonglong2 kj) 
 // ---------------------------------------------------------------------------
 struct GraphArgs {
   const ulonglong2* V;     // alpha-major keys
-  const ulonglong2* bk;    // beta-major swapped keys (beta, alpha)
   int64_t nV;
   int n, na, nb;
   const int32_t* ia;       // alpha group of each det
@@ -303,7 +302,7 @@ __device__ __forceinline__ void visit(const GraphArgs& A, ulonglong2 ki, int64_t
 // (C) from one side.  BETA == false: neighbours are alpha strings, groups are
 // alpha groups (members j = position, other-spin value V[j].y); BETA == true:
 // neighbours are beta strings, groups live in beta-major order (members
-// j = permb[pos], other-spin value bk[pos].y).  Small groups are scanned
+// j = permb[pos], other-spin value ba[pos]).  Small groups are scanned
 // (flattened, 32 groups at a time); large groups are probed with binary
 // searches for the L single excitations of the other-spin string.
 template <int MODE, bool BETA>
@@ -1549,7 +1548,6 @@ static void space_args(hci_ctx* ctx, int64_t nV, GraphArgs& A) {
   const int n = ctx->n;
   A = GraphArgs{};
   A.V = bp<ulonglong2>(ctx->graph.keys);
-  A.bk = bp<ulonglong2>(ctx->g_bkeys);
   A.nV = nV;
   A.n = n; A.na = ctx->na; A.nb = ctx->nb;
   A.ia = bp<int32_t>(ctx->g_ia); A.ga = bp<int64_t>(ctx->g_ga);

@@ -98,7 +98,7 @@ struct Lists {
   DevBuf single_f32;                 // |jk_same|, |j_opp| [n^3 each] and |f_ref| [2 n^2] rounded up to FP32
   DevBuf list_max;                   // [n*n + npair_same] first (largest) magnitude of each list
   DevBuf f_ref;                      // [2][n][n] single-excitation rows of the aufbau determinant (set at create)
-  double max_opp = 0, max_same = 0, max_single = 0;
+  double max_opp = 0, max_same = 0;
 };
 
 // Scratch of the incremental graph update (V' = V + new determinants).
@@ -315,15 +315,6 @@ __device__ __forceinline__ int64_t next_of_key(const ulonglong2* __restrict__ t,
     if ((group_hash(k) & mask) != h) return m;
   }
   return m;
-}
-
-__device__ __forceinline__ int popc64(uint64_t x) { return __popcll(x); }
-
-// (-1)^(number of set bits of s strictly between orbitals p and r)
-__device__ __forceinline__ double exc_phase(uint64_t s, int p, int r) {
-  int lo = p < r ? p : r, hi = p < r ? r : p;
-  uint64_t mask = ((hi >= 64) ? ~0ull : ((1ull << hi) - 1ull)) & ~((2ull << lo) - 1ull);
-  return (__popcll(s & mask) & 1) ? -1.0 : 1.0;
 }
 
 // flip the sign of v for an odd count

@@ -36,7 +36,6 @@ struct WalkArgs {
   const float* single_bf;          // tight bound rounded up to FP32
   const float* single_f32;
   const float4* single_max;        // per sorted single: |F_R| alpha, beta, largest same- and other-spin term
-  double max_single;
   ulonglong2* out;
   int64_t cap;
   unsigned long long* counter;     // [0] candidates, [1] next det (work queue)
@@ -53,7 +52,6 @@ struct WalkArgs {
   int32_t* srcs;         // perturbative mode with sources: source determinant of each pair; vals then
                          // holds the element H_ai instead of the term H_ai c_i
   int npart, part;
-  const double* eri;
 };
 
 // perturbative mode: keep the term and the target?
@@ -654,14 +652,14 @@ extern "C" hci_status hci_select(hci_ctx* ctx, double eps1, const uint64_t* keys
   A.same_mag = bp<double>(L.same_mag); A.same_tgt = bp<uint16_t>(L.same_tgt); A.Ls = L.len_same;
   A.max_dbl = L.max_opp > L.max_same ? L.max_opp : L.max_same;
   A.h = bp<double>(ctx->h); A.jk_same = bp<double>(ctx->jk_same); A.j_opp = bp<double>(ctx->j_opp);
-  A.single_bound = bp<double>(L.single_bound); A.max_single = L.max_single;
+  A.single_bound = bp<double>(L.single_bound);
   A.single_pr = bp<uint16_t>(L.single_pr); A.single_bf = bp<float>(L.single_bf);
   A.single_f32 = bp<float>(L.single_f32); A.single_max = bp<float4>(L.single_max);
   A.list_max = bp<double>(L.list_max);
   A.f_ref = bp<double>(L.f_ref);
   A.ref_a = ctx->na == 64 ? ~0ull : ((1ull << ctx->na) - 1ull);
   A.ref_b = ctx->nb == 64 ? ~0ull : ((1ull << ctx->nb) - 1ull);
-  A.vals = nullptr; A.srcs = nullptr; A.npart = 1; A.part = 0; A.eri = bp<double>(ctx->eri);
+  A.vals = nullptr; A.srcs = nullptr; A.npart = 1; A.part = 0;
   HCI_TRY(ensure_buf(ctx, ctx->s_counter, 64));
   A.counter = bp<unsigned long long>(ctx->s_counter);
   // candidate buffer: grow and rerun when the first guess overflows
@@ -966,14 +964,13 @@ static hci_status pt_walk_args(hci_ctx* ctx, WalkArgs& A, const uint64_t* keys, 
   A.same_mag = bp<double>(L.same_mag); A.same_tgt = bp<uint16_t>(L.same_tgt); A.Ls = L.len_same;
   A.max_dbl = L.max_opp > L.max_same ? L.max_opp : L.max_same;
   A.h = bp<double>(ctx->h); A.jk_same = bp<double>(ctx->jk_same); A.j_opp = bp<double>(ctx->j_opp);
-  A.single_bound = bp<double>(L.single_bound); A.max_single = L.max_single;
+  A.single_bound = bp<double>(L.single_bound);
   A.single_pr = bp<uint16_t>(L.single_pr); A.single_bf = bp<float>(L.single_bf);
   A.single_f32 = bp<float>(L.single_f32); A.single_max = bp<float4>(L.single_max);
   A.list_max = bp<double>(L.list_max);
   A.f_ref = bp<double>(L.f_ref);
   A.ref_a = ctx->na == 64 ? ~0ull : ((1ull << ctx->na) - 1ull);
   A.ref_b = ctx->nb == 64 ? ~0ull : ((1ull << ctx->nb) - 1ull);
-  A.eri = bp<double>(ctx->eri);
   A.srcs = nullptr;
   A.vals = nullptr;
   A.npart = 1;
