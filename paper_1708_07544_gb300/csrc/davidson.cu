@@ -3,7 +3,9 @@
 // normalisation multiplier (Sec. II.A: after each enlargement of V the new
 // ground state is found with Davidson's method).  Vector operations, the
 // subspace eigenproblem (one block) and the phase convention all run on the
-// GPU; the host only reads the Ritz value and the residual norm per iteration.
+// GPU; the host reads one report (Ritz value, residual norm, why a chain ended)
+// per DAV_AHEAD iterations, or per iteration where products cannot be queued
+// ahead (locked roots, a spin parity, one-orientation and direct graphs).
 #include <cmath>
 
 #include "hci_internal.cuh"
@@ -288,7 +290,11 @@ __global__ void __launch_bounds__(DBLOCK, OP == PASS_UNIT ? 2 : 1) k_pass(double
 //
 // (12e,12o) space, k up to 24, about 840 calls: 219 us per call with an
 // FP64 Jacobi started from the last eigenvectors, 45 us by the second way,
-// 12.4 us by the first.
+// 12.4 us by the first.  Against a Jacobi in quad precision, 2700 calls of
+// Davidson runs on 240 random matrices (gaps from 0.02 to 1 of a spectrum of
+// 6, offsets of -40 and -8000): vector error at most 5e-16 and residual 1e-15 (the FP64 Jacobi 2e-14
+// and 4e-14, with the offset 2e-12 and 3e-12), since only the residual is
+// rounded in FP64 and it is formed on the shifted matrix.
 constexpr int LW_X = 160;             // threads below: 2 x 2 blocks of A; from here on: rows of X
 constexpr int LW_T = 320;
 constexpr float LW_SKIP = 1e-6f;      // rotations below this angle are skipped

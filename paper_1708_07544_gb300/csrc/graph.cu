@@ -437,11 +437,6 @@ __global__ void k_item_fill(const int32_t* __restrict__ rowlist, int64_t nrows, 
   }
 }
 
-// One warp per item taken from a queue.  ROWS_STAGED: the entries go to the
-// warp's scratch; at the item's end one atomic reserves its range of the
-// staging buffer and they are copied there (itoff[q] = its start, or -1 when
-// the item outgrew the scratch or the staging buffer; cnt[q] is exact either
-// way).
 // the p-th of P shares of [b, e)
 __device__ __forceinline__ void share(int64_t& b, int64_t& e, int p, int P) {
   if (P > 1) {
@@ -451,6 +446,11 @@ __device__ __forceinline__ void share(int64_t& b, int64_t& e, int p, int P) {
   }
 }
 
+// One warp per item taken from a queue.  ROWS_STAGED: the entries go to the
+// warp's scratch; at the item's end one atomic reserves its range of the
+// staging buffer and they are copied there (itoff[q] = its start, or -1 when
+// the item outgrew the scratch or the staging buffer; cnt[q] is exact either
+// way).
 template <int MODE>
 __global__ void __launch_bounds__(G_WARPS * 32, MODE <= ROWS_STAGED ? 6 : 5) k_rows(GraphArgs A) {
   __shared__ int64_t s_start[G_WARPS][32];

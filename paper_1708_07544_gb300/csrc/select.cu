@@ -871,8 +871,10 @@ __global__ void __launch_bounds__(256) k_pt2_targets(const ulonglong2* __restric
 }
 
 // One listed target per thread: its terms summed, sum^2 / (e0 - H_aa) added
-// to the block's part_e (threads in order, then a fixed tree), and with dpair
-// the first-order coefficient d_a on every pair of the target.  Bound by FP64
+// to the block's part_e, and with dpair the first-order coefficient d_a on
+// every pair of the target.  The list's order and that of a target's pairs
+// come from atomic counters, so E2 is a sum of the same terms in an order that
+// differs from run to run.  Bound by FP64
 // issue (about 55 operations per target, most of them H_aa's), so the targets
 // are listed first: taken in place, where only the first pair of a run works,
 // 2 to 3 lanes of 4 idle through all of them.

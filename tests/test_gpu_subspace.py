@@ -82,3 +82,23 @@ def test_tolerance_never_met(maxit):
     (e0, c0, i0), (e1, c1, i1) = out.values()
     assert i0 == i1 == maxit
     assert e0 == e1 and torch.equal(c0, c1)
+
+
+@pytest.mark.parametrize("offset", [0.0, -1e3, 1e6, -3e7])
+def test_energy_offset_to_rounding(offset):
+    # the subspace problem is shifted by its first element, so an offset costs
+    # the rounding of the diagonal, the products and the Rayleigh quotient
+    # (some ulps of the offset) and no more: against the spectrum without it
+    inst = hi.random_tiny(6, 3, 3, 9)
+    keys = hi.random_det_keys(6, 3, 3, 200, 4)
+    H = oracle.hamiltonian(inst, keys).toarray()
+    w = np.linalg.eigvalsh(H)
+    inst.e_core += offset
+    kt = torch.tensor(keys.astype(np.int64), device="cuda")
+    tol = max(1e-10, 1e-13 * abs(offset))
+    with _solver(inst) as s:
+        e, c, _ = s.davidson(kt, None, tol, 2000)
+    c = c.cpu().numpy()
+    assert abs((e - offset) - w[0]) <= 1e-14 * abs(offset) + 1e-11
+    r = np.linalg.norm(H @ c - (e - offset) * c)
+    assert r <= tol + 1e-14 * max(1.0, abs(offset)) * np.sqrt(len(keys))
