@@ -333,7 +333,8 @@ hci_status hci_solve_batch(int count, const int* norb, const int* nalpha, const 
  * The outputs are made exactly symmetric, as hci_create requires: every
  * permutation of (pq|rs)' in its 8-fold orbit, and h'_qp, hold the bits of
  * the orbit's representative (p <= q, r <= s, pq <= rs) and of h'_pq, p < q.
- * All pointers device; U, h_out, eri_out are outputs (n*n, n*n, n^4).
+ * All pointers device; U, h_out, eri_out are outputs (n*n, n*n, n^4), left
+ * as they were when kappa's 1-norm is infinite (HCI_ERR_INVALID).
  * stream: cudaStream_t or NULL. */
 hci_status hci_rotate(int norb, const double* kappa, const double* h, const double* eri, double* U,
                       double* h_out, double* eri_out, void* stream);
