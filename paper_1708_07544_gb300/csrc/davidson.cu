@@ -1285,8 +1285,12 @@ static hci_status davidson_core(hci_ctx* ctx, const uint64_t* keys, int64_t nV, 
   while (it < maxit) {
     const int before = it;
     int queued = 1;
+    // Vectors kept from this very space have usually converged on it: nothing
+    // is queued behind the first step then (a converged call 361 us with three
+    // iterations queued in vain, 325 us so).
+    const int most = same && kwarm > 0 && it == 0 ? 1 : ahead;
     HCI_TRY(ritz());
-    for (; queued < ahead && it + queued < maxit && k < MAXSUB; ++queued) {
+    for (; queued < most && it + queued < maxit && k < MAXSUB; ++queued) {
       HCI_TRY(expand());
       HCI_TRY(ritz());
     }

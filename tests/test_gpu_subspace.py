@@ -102,3 +102,22 @@ def test_energy_offset_to_rounding(offset):
     assert abs((e - offset) - w[0]) <= 1e-14 * abs(offset) + 1e-11
     r = np.linalg.norm(H @ c - (e - offset) * c)
     assert r <= tol + 1e-14 * max(1.0, abs(offset)) * np.sqrt(len(keys))
+
+
+def test_converged_start_queues_nothing():
+    # a call from the converged state takes one step and launches no iteration
+    # behind it (8 kernels each)
+    from paper_1708_07544_gb300 import _abi
+
+    inst = hi.random_tiny(6, 3, 3, 9)
+    keys = hi.random_det_keys(6, 3, 3, 200, 4)
+    kt = torch.tensor(keys.astype(np.int64), device="cuda")
+    with _solver(inst) as s:
+        e, c, _ = s.davidson(kt)
+        before = _abi.hci_launch_count()
+        e2, c2, it = s.davidson(kt, c)
+        launches = _abi.hci_launch_count() - before
+        # a tighter tolerance goes on from there
+        e3, c3, it3 = s.davidson(kt, c, 1e-12)
+    assert it == 1 and launches <= 30
+    assert abs(e2 - e) <= 1e-12 and it3 > 1 and abs(e3 - e) <= 1e-11
