@@ -1047,8 +1047,9 @@ __global__ void __launch_bounds__(256) k_diag(int n, uint64_t ra, uint64_t rb, c
 // they belong to, and a block's warps take its shares in turn.  A warp owns
 // the rows that start in a share and sums the last one up to the share's end;
 // the share's head, the rest of a row that started earlier, goes to head[w],
-// which k_sigma_heads adds to the row in the order of the shares.  Nothing is
-// done when *stop is set.  (With whole rows per warp the aufbau determinant's
+// which k_sigma_heads adds to the row in the order of the shares.  (WHOLE: a
+// share takes its last row to the row's end, and there are no heads.)  Nothing
+// is done when *stop is set.  (With whole rows per warp the aufbau determinant's
 // row, connected to most of a small space, was all of the product.)
 //
 // Connections come from HBM, c from L2 one 32-byte sector per entry unless L1
@@ -1067,6 +1068,14 @@ __global__ void __launch_bounds__(256) k_diag(int n, uint64_t ra, uint64_t rb, c
 constexpr int SIGMA_WARPS_PER_SM = 32;   // of k_sigma1, all resident
 constexpr int64_t SIGMA_SHARE = 512;     // entries per warp at least
 constexpr int64_t SIGMA_SUB = 16384;     // entries per share where a warp has several
+// Spaces of up to SIGMA_WHOLE determinants keep their rows whole, each in the
+// share where it starts, with a share of SIGMA_WHOLE_SHARE entries per warp: no
+// row is longer than 16 batches, and the launch that adds the heads is saved.
+// hci_sigma with cut rows / whole ones, us by determinants: 41.8 / 37.4 (33),
+// 45.9 / 37.8 (443), 43.8 / 39.0 (1225), 45.7 / 41.4 (1765), 43.9 / 44.1 (2296),
+// 46.7 / 47.1 (3482), 48.3 / 51.2 (3807), 57.5 / 96.3 (10020); 64 or 256 entries
+// per share change nothing.
+constexpr int64_t SIGMA_WHOLE = 2048, SIGMA_WHOLE_SHARE = 128;
 
 // plan[w] = the first row that starts at or after entry w x chunk, w <= warps
 __global__ void k_sigma_plan(const int64_t* __restrict__ rowptr, int64_t nV, int64_t warps, int64_t chunk,
@@ -1128,7 +1137,7 @@ __device__ __forceinline__ double row_sum(const RowPiece& p, const RowPiece& nex
   }
 }
 
-template <int WARPS>
+template <int WARPS, bool WHOLE>
 __global__ void __launch_bounds__(WARPS * 32, SIGMA_WARPS_PER_SM / WARPS) k_sigma1(const int64_t* __restrict__ rowptr,
                                                   const int64_t* __restrict__ rowstart, const int32_t* __restrict__ col,
                                                const double* __restrict__ val, const double* __restrict__ diag,
@@ -1142,7 +1151,7 @@ __global__ void __launch_bounds__(WARPS * 32, SIGMA_WARPS_PER_SM / WARPS) k_sigm
   for (int t = 0; t < rounds; ++t) {
     const int64_t w = w0 + WARPS * t;
     const int r0 = plan[w], r1 = plan[w + 1];
-    const int64_t e0 = w * chunk, e1 = e0 + chunk;
+    const int64_t e0 = WHOLE ? rowptr[r0] : w * chunk, e1 = WHOLE ? rowptr[r1] : e0 + chunk;
     // row i's entries of this share
     auto piece = [&](int i) {
       const int64_t lo = rowptr[i], hi = rowptr[i + 1];
@@ -1151,11 +1160,11 @@ __global__ void __launch_bounds__(WARPS * 32, SIGMA_WARPS_PER_SM / WARPS) k_sigm
     };
     RowPiece next{col, val, 0};
     RowBatch q;
-    const bool has_head = rowptr[r0] > e0;
+    const bool has_head = !WHOLE && rowptr[r0] > e0;
     const int first = has_head ? r0 - 1 : r0;
     if (first < r1) next = piece(first);
     q.load(next, 0);
-    {
+    if (!WHOLE) {
       // the head: row r0 - 1 from e0 on
       double a = 0.0;
       if (has_head) {
@@ -2372,11 +2381,14 @@ static hci_status plan_sigma(hci_ctx* ctx) {
   // L1: 16 (44 orbitals, 1.3e9: 3302 us with 8, 3009 with 16, 3070 with 32;
   // 28 orbitals, 9.7e7: 242, 236, 241).
   const int64_t most = (int64_t)ctx->nsm * SIGMA_WARPS_PER_SM;
-  const int block = G.nstored >= most * SIGMA_SUB ? 16 : 8;
-  const int64_t warps = std::max<int64_t>(1, std::min(most, G.nstored / SIGMA_SHARE) / block) * block;
+  const bool whole = G.nV <= SIGMA_WHOLE;
+  const int block = !whole && G.nstored >= most * SIGMA_SUB ? 16 : 8;
+  const int64_t share = whole ? SIGMA_WHOLE_SHARE : SIGMA_SHARE;
+  const int64_t warps = std::max<int64_t>(1, std::min(most, G.nstored / share) / block) * block;
   const int64_t rounds = std::max<int64_t>(1, (G.nstored + warps * SIGMA_SUB / 2) / (warps * SIGMA_SUB));
   const int64_t shares = warps * rounds;
   HCI_TRY(ensure_buf(ctx, G.sig_plan, (size_t)(shares + 2) * 4 + 8 + (size_t)shares * 8 + 16));
+  G.sig_whole = whole;
   G.sig_block = block;
   G.sig_rounds = (int)rounds;
   G.sig_warps = shares;
@@ -2421,12 +2433,13 @@ hci_status sigma_apply(hci_ctx* ctx, const double* c, double* sigma, int nvec, c
       HCI_LAUNCH(k_sigma_half, grid_for(G.nV * 32, 256, ctx->nsm * 16), 256, 0, ctx->st)(
           bp<int64_t>(G.rowptr), bp<int64_t>(G.rowstart), T, bp<double>(G.diag), G.nV, c, sigma, nvec);
   } else if (nvec == 1) {
-    auto* k = G.sig_block == 16 ? k_sigma1<16> : k_sigma1<8>;
+    auto* k = G.sig_whole ? k_sigma1<8, true> : G.sig_block == 16 ? k_sigma1<16, false> : k_sigma1<8, false>;
     HCI_LAUNCH(k, (unsigned)(G.sig_warps / (G.sig_block * G.sig_rounds)), G.sig_block * 32, 0, ctx->st)(
         bp<int64_t>(G.rowptr), bp<int64_t>(G.rowstart), bp<int32_t>(G.seg_col[0]), bp<double>(G.seg_val[0]),
         bp<double>(G.diag), G.nV, bp<int32_t>(G.sig_plan), G.sig_rounds, G.sig_chunk, c, sigma, sig_head(G), stop);
-    HCI_LAUNCH(k_sigma_heads, (unsigned)((G.sig_warps + 127) / 128), 128, 0, ctx->st)(
-        bp<int64_t>(G.rowptr), bp<int32_t>(G.sig_plan), G.sig_warps, G.sig_chunk, sig_head(G), sigma, stop);
+    if (!G.sig_whole)
+      HCI_LAUNCH(k_sigma_heads, (unsigned)((G.sig_warps + 127) / 128), 128, 0, ctx->st)(
+          bp<int64_t>(G.rowptr), bp<int32_t>(G.sig_plan), G.sig_warps, G.sig_chunk, sig_head(G), sigma, stop);
   } else {
     HCI_LAUNCH(k_sigma, grid_for(G.nV * 32, 256, ctx->nsm * 16), 256, 0, ctx->st)(
         bp<int64_t>(G.rowptr), bp<int64_t>(G.rowstart), bp<int32_t>(G.seg_col[0]), bp<double>(G.seg_val[0]),

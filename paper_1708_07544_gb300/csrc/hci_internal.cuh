@@ -67,6 +67,7 @@ struct Graph {
   DevBuf sig_plan;           // both orientations: first row of each warp's share of H c, heads (k_sigma1)
   int64_t sig_warps = 0, sig_chunk = 0;
   int sig_rounds = 1, sig_block = 8;
+  bool sig_whole = false;    // shares end where rows end: no heads
   DevBuf keys;               // copy of the space's keys [nV][2], sorted
   DevBuf keys_int;           // the same keys by internal id (insertion order)
   DevBuf s2i, i2s;           // int32 maps sorted position <-> internal id

@@ -82,3 +82,41 @@ def test_several_shares(n):
     # H is symmetric: every row and column
     a, b = float(dt @ hc), float(ct @ hd)
     assert abs(a - b) <= 1e-12 * float(dt.norm() * hc.norm() + ct.norm() * hd.norm())
+
+
+# around the size from which rows are cut across shares: the determinant whose
+# row holds nearly the whole space, and four empty rows, the last of the space
+# among them
+@pytest.mark.parametrize("nV", [2047, 2048, 2049, 2600])
+@pytest.mark.parametrize("grow", [0, 40, 2000])
+def test_long_and_empty_rows_where_rows_are_first_cut(nV, grow):
+    inst = hi.random_tiny(16, 6, 5, 6)
+    k0 = hi.aufbau_key(6, 5)
+    new, _, _ = oracle.select(inst, k0, np.ones(1), 0.0)
+    # more than two electrons from one another and from the aufbau determinant's neighbours
+    far = [(0b111111 << 10, b << 6) for b in (0b11111, 0b1111100000)]
+    far = np.array(far + [(a, 0b11111 << 11) for a in (0b111111 << 6, 0b111 << 13 | 0b111 << 6)], np.uint64)
+    near = new[np.sort(np.random.default_rng(nV).choice(len(new), nV - 1 - len(far), replace=False))]
+    keys = np.unique(np.concatenate([k0, near, far]), axis=0)
+    lens = np.diff(oracle.hamiltonian(inst, keys).indptr) - 1
+    assert len(keys) == nV and lens.max() == nV - 1 - len(far) and (lens == 0).sum() == 4 and lens[-1] == 0
+    _check(inst, keys, grow=grow)
+
+
+# a product on a small space with its graph cached: the content hash, the two
+# orders of the vectors and the product itself
+@pytest.mark.parametrize("nV", [1, 30, 400, 2048])
+def test_launches_of_a_small_product(nV):
+    import paper_1708_07544_gb300 as pkg
+    from paper_1708_07544_gb300 import _abi
+
+    inst = hi.random_tiny(10, 5, 4, 77)
+    keys = hi.random_det_keys(10, 5, 4, nV, 5)
+    kt = torch.tensor(keys.astype(np.int64), device="cuda")
+    c = torch.ones(nV, dtype=torch.float64, device="cuda")
+    with pkg.HCISolver(inst.norb, inst.nalpha, inst.nbeta, torch.tensor(inst.h, device="cuda"),
+                       torch.tensor(inst.eri, device="cuda"), inst.e_core) as s:
+        s.sigma(kt, c)
+        before = _abi.hci_launch_count()
+        s.sigma(kt, c)
+        assert _abi.hci_launch_count() - before == 4
