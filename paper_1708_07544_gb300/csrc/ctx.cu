@@ -213,26 +213,6 @@ __global__ void k_build_lists(int n, const double* __restrict__ eri, int same, i
   }
 }
 
-// The single excitations p -> r by descending bound (one block), packed
-// p | r << 8 with the bound rounded up to FP32
-__global__ void k_sort_singles(int n, const double* __restrict__ bound, int P, uint16_t* __restrict__ pr,
-                               float* __restrict__ bf) {
-  extern __shared__ double sm_d[];
-  double* m = sm_d;
-  int* id = reinterpret_cast<int*>(m + P);
-  const int L = n * n;
-  for (int e = threadIdx.x; e < P; e += blockDim.x) {
-    m[e] = e < L ? bound[e] : -1.0;
-    id[e] = e < L ? e : INT_MAX;
-  }
-  __syncthreads();
-  bitonic_desc(m, id, P);
-  for (int e = threadIdx.x; e < L; e += blockDim.x) {
-    pr[e] = (uint16_t)((id[e] / n) | ((id[e] % n) << 8));
-    bf[e] = __double2float_ru(m[e]);
-  }
-}
-
 // |jk_same|, |j_opp| and |f_ref| rounded up to FP32: [n^3][n^3][2 n^2]
 __global__ void k_single_f32(int n, const double* __restrict__ jk_same, const double* __restrict__ j_opp,
                              const double* __restrict__ f_ref, float* __restrict__ out) {
@@ -243,26 +223,53 @@ __global__ void k_single_f32(int n, const double* __restrict__ jk_same, const do
   }
 }
 
-// For each sorted single the parts of a bound that needs only the numbers of
-// orbitals in which a determinant differs from the aufbau one, rounded up:
-// |F_R| (alpha, beta) with the margin of the FP64 sums' rounding, and the
-// largest same-spin and other-spin term
-__global__ void k_single_max(int n, const uint16_t* __restrict__ pr, const float* __restrict__ f32,
-                             const float* __restrict__ bf, float4* __restrict__ out) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n * n) return;
+// The single excitations p -> r by descending bound (ties by p, then r; a bound
+// that is not a number last): packed p | r << 8, the bound rounded up to FP32,
+// and the parts of a bound that needs only the numbers of orbitals in which a
+// determinant differs from the aufbau one, rounded up: |F_R| (alpha, beta) with
+// the margin of the FP64 sums' rounding, and the largest same-spin and
+// other-spin term.  A single's place is the number of singles before it,
+// counted by SR_LANES lanes over all of them as integers (a non-negative
+// double's bits order like its value, and an FP64 comparison would take 64
+// cycles of a sub-partition): 8 us at 44 orbitals, where one block's bitonic
+// sort and a launch for the sums took 102.
+constexpr int SR_LANES = 8, SR_T = 256;
+
+__global__ void __launch_bounds__(SR_T) k_rank_singles(int n, const double* __restrict__ bound,
+                                                       const float* __restrict__ f32, uint16_t* __restrict__ pr,
+                                                       float* __restrict__ bf, float4* __restrict__ mx) {
+  extern __shared__ uint64_t s_key[];
+  const int L = n * n, sub = threadIdx.x % SR_LANES;
+  for (int t = threadIdx.x; t < L; t += SR_T) {
+    const double b = bound[t];
+    s_key[t] = b == b ? (uint64_t)__double_as_longlong(b) + 1 : 0;
+  }
+  __syncthreads();
+  const int e = (blockIdx.x * SR_T + threadIdx.x) / SR_LANES;
+  const int at = e < L ? e : L - 1;            // whole warps below
+  const uint64_t key = s_key[at];
+  int rank = 0;
+  for (int t = sub; t < L; t += SR_LANES) rank += s_key[t] > key || (s_key[t] == key && t < at);
+  const int p = at / n, r = at % n;
   const int64_t n3 = (int64_t)n * n * n;
-  const int p = pr[e] & 63, r = pr[e] >> 8;
   const float* js = f32 + ((int64_t)p * n + r) * n;
   float ms = 0.0f, mo = 0.0f;
-  for (int k = 0; k < n; ++k) {
+  for (int k = sub; k < n; k += SR_LANES) {
     ms = fmaxf(ms, js[k]);
     mo = fmaxf(mo, js[n3 + k]);
   }
-  const float add = __fmul_ru(2e-13f, bf[e]), up = 1.000002f;
-  out[e] = make_float4(__fmul_ru(__fadd_ru(f32[2 * n3 + p * n + r], add), up),
-                       __fmul_ru(__fadd_ru(f32[2 * n3 + (int64_t)n * n + p * n + r], add), up), __fmul_ru(ms, up),
-                       __fmul_ru(mo, up));
+  for (int o = SR_LANES / 2; o; o >>= 1) {
+    rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    ms = fmaxf(ms, __shfl_xor_sync(0xffffffffu, ms, o));
+    mo = fmaxf(mo, __shfl_xor_sync(0xffffffffu, mo, o));
+  }
+  if (sub != 0 || e >= L) return;
+  const float b = __double2float_ru(bound[e]), add = __fmul_ru(2e-13f, b), up = 1.000002f;
+  pr[rank] = (uint16_t)(p | (r << 8));
+  bf[rank] = b;
+  mx[rank] = make_float4(__fmul_ru(__fadd_ru(f32[2 * n3 + p * n + r], add), up),
+                         __fmul_ru(__fadd_ru(f32[2 * n3 + (int64_t)n * n + p * n + r], add), up), __fmul_ru(ms, up),
+                         __fmul_ru(mo, up));
 }
 
 // f_ref[s][p][r] = h_pr + sum_{k occ in spin s of R} ((pr|kk) - (pk|kr))
@@ -476,15 +483,12 @@ extern "C" hci_status hci_build_lists(hci_ctx* ctx) {
     HCI_TRY(ensure_buf(ctx, L.single_pr, (size_t)n * n * 2));
     HCI_TRY(ensure_buf(ctx, L.single_bf, (size_t)n * n * 4));
     HCI_TRY(ensure_buf(ctx, L.single_f32, (size_t)(2 * n3 + 2 * n * n) * 4));
-    const int P = next_pow2(n * n);
-    HCI_CUDA(ctx, cudaFuncSetAttribute(k_sort_singles, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
-    HCI_LAUNCH(k_sort_singles, 1, 1024, (size_t)P * 12, ctx->st)(n, bp<double>(L.single_bound), P,
-                                                                bp<uint16_t>(L.single_pr), bp<float>(L.single_bf));
+    HCI_TRY(ensure_buf(ctx, L.single_max, (size_t)n * n * 16));
     HCI_LAUNCH(k_single_f32, grid_for(2 * n3, 256), 256, 0, ctx->st)(n, bp<double>(ctx->jk_same), bp<double>(ctx->j_opp),
                                                                     bp<double>(L.f_ref), bp<float>(L.single_f32));
-    HCI_TRY(ensure_buf(ctx, L.single_max, (size_t)n * n * 16));
-    HCI_LAUNCH(k_single_max, (n * n + 127) / 128, 128, 0, ctx->st)(n, bp<uint16_t>(L.single_pr), bp<float>(L.single_f32),
-                                                                  bp<float>(L.single_bf), bp<float4>(L.single_max));
+    HCI_LAUNCH(k_rank_singles, (n * n * SR_LANES + SR_T - 1) / SR_T, SR_T, (size_t)n * n * 8, ctx->st)(
+        n, bp<double>(L.single_bound), bp<float>(L.single_f32), bp<uint16_t>(L.single_pr), bp<float>(L.single_bf),
+        bp<float4>(L.single_max));
     HCI_CUDA(ctx, cudaGetLastError());
   }
   HCI_TRY(ensure_buf(ctx, ctx->s_misc, 64));

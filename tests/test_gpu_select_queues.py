@@ -95,3 +95,25 @@ def test_integrals_beyond_fp32(k, big):
                 got = s.select(eps1, _dev(keys), _dev(cv)).cpu().numpy().view(np.uint64).reshape(-1, 2)
             assert sorted(map(tuple, got.tolist())) == sorted(map(tuple, np.asarray(want).reshape(-1, 2).tolist()))
             assert len(ties) == 0
+
+
+# the singles sorted by their bounds, at every width and with many equal bounds
+# (integrals from a few values): the singles within a threshold are a prefix
+@pytest.mark.parametrize("n,na,nb", [(1, 1, 0), (2, 1, 1), (3, 2, 1), (5, 3, 2), (16, 5, 4), (31, 3, 3), (33, 3, 2), (48, 3, 3),
+                                     (64, 3, 2)])
+def test_singles_of_every_width(n, na, nb):
+    inst = hi.random_tiny(n, na, nb, 5)
+    g = np.random.default_rng(n)
+    h = g.choice([0.0, 0.125, -0.25, 0.5, 3.0], (n, n))
+    inst.h = np.triu(h) + np.triu(h, 1).T
+    inst.eri = np.zeros((n,) * 4)
+    a0, b0 = (1 << na) - 1, (1 << nb) - 1
+    k1 = (a0 ^ 1 ^ (1 << (n - 1))) if n > na else a0
+    keys = np.array(sorted({(a0, b0), (k1, b0)}), np.uint64)
+    c = np.array([1.0, -0.3])[: len(keys)]
+    for eps1 in (1e-3, 0.124, 0.2, 0.4, 1.0, 4.0):
+        want, _, ties = oracle.select(inst, keys, c, eps1)
+        with _solver(inst) as s:
+            got = s.select(eps1, _dev(keys), _dev(c)).cpu().numpy().view(np.uint64).reshape(-1, 2)
+        assert len(ties) == 0
+        assert sorted(map(tuple, got.tolist())) == sorted(map(tuple, np.asarray(want).reshape(-1, 2).tolist()))
