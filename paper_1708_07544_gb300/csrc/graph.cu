@@ -247,9 +247,7 @@ struct GraphArgs {
   HamView H;
   // direct traversals (no stored rows), vectors by sorted position
   const double* dc;             // input vector
-  double* dpart;                // sigma: each item's share of its row's sum, or, where
-  double* dsig;                 // every row is one item, the output itself
-  const double* ddiag;          // and the diagonal elements for it
+  double* dpart;                // sigma: each item's share of its row's sum
   unsigned long long* dnnz;     // sigma: connections visited (may be null)
   RdmAcc R;                     // RDMs: accumulators
 };
@@ -540,8 +538,7 @@ __global__ void __launch_bounds__(G_WARPS * 32, MODE <= ROWS_STAGED ? 6 : 5) k_r
       double a = ra.acc;
       for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
       if (lane == 0) {
-        if (A.dsig) A.dsig[i] = fma(A.ddiag[i], ra.ci, a);
-        else A.dpart[q] = a;
+        A.dpart[q] = a;
         if (A.dnnz) atomicAdd(A.dnnz, (unsigned long long)w);
       }
     }
@@ -2338,21 +2335,16 @@ static hci_status sigma_direct(hci_ctx* ctx, const double* c, double* sigma, int
   space_args(ctx, G.nV, A);
   A.items = bp<int4>(ctx->inc.items);
   A.nitems = ctx->inc.nitems;
-  // no row cut (a small space): no second launch for the rows' sums
-  const bool cut = A.nitems != G.nV;
   A.dpart = bp<double>(ctx->inc.itp);
-  A.ddiag = bp<double>(G.diag);
   unsigned long long* cnt = reinterpret_cast<unsigned long long*>(bp<char>(ctx->s_counter) + 56);
   for (int v = 0; v < nvec; ++v) {
     A.dc = c + (int64_t)v * G.nV;
-    A.dsig = cut ? nullptr : sigma + (int64_t)v * G.nV;
     A.dnnz = G.nnz < 0 ? cnt : nullptr;
     if (A.dnnz) HCI_CUDA(ctx, cudaMemsetAsync(cnt, 0, 8, ctx->st));
     HCI_CUDA(ctx, cudaMemsetAsync(A.queue, 0, 8, ctx->st));
     HCI_LAUNCH(k_rows<ROWS_SIGMA>, rows_grid(ctx), G_WARPS * 32, 0, ctx->st)(A);
-    if (cut)
-      HCI_LAUNCH(k_row_sums, grid_for(G.nV, 256), 256, 0, ctx->st)(bp<int64_t>(ctx->inc.first), G.nV, A.dpart,
-                                                                  A.ddiag, A.dc, sigma + (int64_t)v * G.nV);
+    HCI_LAUNCH(k_row_sums, grid_for(G.nV, 256), 256, 0, ctx->st)(bp<int64_t>(ctx->inc.first), G.nV, A.dpart,
+                                                                bp<double>(G.diag), A.dc, sigma + (int64_t)v * G.nV);
     HCI_CUDA(ctx, cudaGetLastError());
     if (A.dnnz) {
       unsigned long long h = 0;

@@ -190,44 +190,3 @@ def test_budget_holds_while_a_space_grows(pkg, nv):
             s.sigma(dev_keys(A), c[:nv])
             s.sigma(dev_keys(K), c[:len(K)])
             assert (s.stats()["graph_half"], s.stats()["sigma_direct"]) == ((0, 0) if ok else (1, 0))
-
-
-# rows of one work item each: written by the search itself, without a launch
-# for the rows' sums
-@pytest.mark.parametrize("nv", [1, 40, 900, 40000])
-def test_direct_rows_whole(pkg, nv):
-    from paper_1708_07544_gb300 import _abi
-
-    inst = hi.df_12o()
-    keys = hi.random_det_keys(12, 6, 6, nv, seed=nv)
-    c = np.stack([hi.random_vector(len(keys), seed=1), hi.random_vector(len(keys), seed=2)])
-    rows = np.unique(np.random.default_rng(3).integers(0, len(keys), 60))
-    kd, cd = dev_keys(keys), torch.tensor(c).cuda()
-    with solver(pkg, inst, _abi.SIGMA_DIRECT) as s:
-        got = s.sigma(kd, cd).cpu().numpy()
-        before = _abi.hci_launch_count()
-        one = s.sigma(kd, cd[0].contiguous()).cpu().numpy()
-        # content hash, the two orders of the vector, the search
-        assert _abi.hci_launch_count() - before == 4
-    for x, v in zip((one, got[0], got[1]), (c[0], c[0], c[1])):
-        ref = oracle.sigma_rows(inst, keys, v, rows)
-        assert np.abs(x[rows] - ref).max() <= 1e-11 * np.abs(ref).max()
-
-
-# rows cut into several items, summed behind the search: the (22e,22o) space of
-# a solve, whose aufbau row takes far more pair checks than an item holds
-def test_direct_rows_cut(pkg):
-    from paper_1708_07544_gb300 import _abi
-
-    inst = hi.ppp_pentacene()
-    with solver(pkg, inst) as s:
-        out = s.solve(1e-4)
-        c = torch.stack([out["c"], torch.linspace(-1, 1, out["c"].shape[0], dtype=torch.float64, device="cuda")])
-        want = s.sigma(out["keys"], c)
-        s.set_sigma_mode(_abi.SIGMA_DIRECT)
-        got = s.sigma(out["keys"], c)
-        before = _abi.hci_launch_count()
-        one = s.sigma(out["keys"], c[1].contiguous())
-        assert _abi.hci_launch_count() - before == 5
-    assert (got - want).abs().max().item() <= 1e-12 * want.abs().max().item()
-    assert torch.equal(one, got[1])
